@@ -149,9 +149,12 @@ typedef enum {
   JFNK_FORMAL_SWEEP_THREAD = 2,  /* mixed: thread per frequency, all angles        */
   JFNK_FORMAL_SWEEP_WARP = 3,    /* mixed: warp per frequency pair, lane per ray   */
   JFNK_FORMAL_MOVING = 4,        /* moving columns: thread per ray, per-ray opacity */
-  JFNK_FORMAL_SWEEP_THREAD_FUSED = 5 /* mixed: thread per frequency, the tangent sweep
+  JFNK_FORMAL_SWEEP_THREAD_FUSED = 5, /* mixed: thread per frequency, the tangent sweep
                                     forming the JVP evaluations' opacity tangent itself
                                     (at most 8 transitions overlap at any frequency) */
+  JFNK_FORMAL_CACHED = 6         /* FP64, static columns: opacity, formal solution and rate
+                                    integrals per tile of frequencies, a base evaluation's
+                                    coefficients kept for the products of its Newton step */
 } jfnk_formal_kernel;
 
 /* Jacobian-vector products inside GMRES (Sect. 2.4, Fig. 2). The default is
@@ -236,7 +239,7 @@ typedef struct {
                            (mixed mode: of the base-type sweep launches)           */
   int formal_launches;  /* profile: number of timed launches (active ticks)        */
   int kernel_launches;  /* CUDA kernels launched by the solve (graph nodes included) */
-  int formal_qb;        /* fused kernel: frequencies per block (0 for the others)   */
+  int formal_qb;        /* fused and cached kernels: frequencies per block (0 for the others) */
   int formal_threads;   /* threads per block (warps per block: JFNK_FORMAL_SWEEP_WARP) */
   int formal_kernel;    /* jfnk_formal_kernel that ran the formal solution          */
   double formal_tan_ms; /* profile, mixed mode: summed duration of the tangent-sweep

@@ -46,6 +46,7 @@ JFNK_FORMAL_SWEEP_THREAD = 2
 JFNK_FORMAL_SWEEP_WARP = 3
 JFNK_FORMAL_MOVING = 4
 JFNK_FORMAL_SWEEP_THREAD_FUSED = 5
+JFNK_FORMAL_CACHED = 6
 
 _dp = C.POINTER(C.c_double)
 _ip = C.POINTER(C.c_int)

@@ -246,6 +246,7 @@ static int run_to_completion(Batch* b, const jfnk_options* o, cudaStream_t s) {
   const int nfull = b->ncols;
   ColDesc* dfull = b->d_cols;
   const int fz = b->max_nz, fq = b->max_nq, ft = b->max_nt, fN = b->max_N, fm = b->max_nmu;
+  const int ftiles = b->max_tiles;
   const int fvariant = b->sweep_variant, fthreads = b->formal_threads;
   std::vector<int> view(nfull);
   for (int c = 0; c < nfull; ++c) view[c] = c;
@@ -283,12 +284,13 @@ static int run_to_completion(Batch* b, const jfnk_options* o, cudaStream_t s) {
     if (running.empty()) break;
     if (b->ncols > 1 && (int)running.size() * 2 <= b->ncols) {
       std::vector<ColDesc> hv;
-      int mz = 0, mq = 0, mt = 0, mN = 0, mm = 0;
+      int mz = 0, mq = 0, mt = 0, mN = 0, mm = 0, mtl = 0;
       for (int c : running) {
         const ColDesc& d = b->h_cols[c];
         hv.push_back(d);
         mz = std::max(mz, d.t.nz); mq = std::max(mq, d.t.nq); mt = std::max(mt, d.t.nt);
         mN = std::max(mN, d.t.nz * d.t.nl); mm = std::max(mm, d.t.nmu);
+        if (d.w.cf) mtl = std::max(mtl, (d.t.nq + d.w.cq - 1) / d.w.cq);
       }
       std::vector<int> ones(running.size(), 1);
       if (cudaMemcpyAsync(b->d_view, hv.data(), sizeof(ColDesc) * hv.size(), cudaMemcpyHostToDevice, s) != cudaSuccess ||
@@ -297,6 +299,7 @@ static int run_to_completion(Batch* b, const jfnk_options* o, cudaStream_t s) {
       b->d_cols = b->d_view;
       b->ncols = (int)running.size();
       b->max_nz = mz; b->max_nq = mq; b->max_nt = mt; b->max_N = mN; b->max_nmu = mm;
+      b->max_tiles = mtl;
       // a few columns: one thread per frequency leaves most SMs idle, and the
       // warp-per-frequency-pair sweep (same results) finishes each tick sooner
       if (b->formal_kind == FORMAL_SWEEP && b->sweep_variant == 1 &&
@@ -314,6 +317,7 @@ static int run_to_completion(Batch* b, const jfnk_options* o, cudaStream_t s) {
   b->d_cols = dfull;
   b->ncols = nfull;
   b->max_nz = fz; b->max_nq = fq; b->max_nt = ft; b->max_N = fN; b->max_nmu = fm;
+  b->max_tiles = ftiles;
   b->sweep_variant = fvariant;
   b->formal_threads = fthreads;
   return rc;
@@ -407,7 +411,7 @@ static int prepare_solve(Batch* b, const std::vector<const jfnk_atmos*>& cols,
     if (fuse && b->max_overlap > kQMetaT)
       return fail(JFNK_E_INVALID, "JFNK_FORMAL_SWEEP_THREAD_FUSED: more than 8 transitions overlap at a frequency");
     if ((rc = set_sweep_config(b, v, size, fuse))) return rc;
-  } else if (!b->tuned && b->formal_kind != FORMAL_UNFUSED) {
+  } else if (!b->tuned && (b->formal_kind == FORMAL_SWEEP || b->formal_kind == FORMAL_FUSED)) {
     // tune the formal kernel once per batch, on its own columns: a base
     // evaluation at the initial state, then tangent data along v = n
     if ((rc = batch_set_forced_mode(b, EV_BASE, s))) return rc;
@@ -487,12 +491,13 @@ static int finish_solve(Batch* b, const std::vector<const jfnk_atmos*>& cols, do
       S.formal_fuse = b->formal_kind == FORMAL_SWEEP && sweep_fused(*b) ? b->sweep_fuse : 0;
       S.formal_launches = active;
       S.kernel_launches = (int)(b->replays * b->graph_kernels) + 2;   // + state init, mode reset
-      S.formal_qb = b->formal_kind == FORMAL_FUSED ? b->formal_qb : 0;
+      S.formal_qb = b->formal_kind == FORMAL_FUSED || b->formal_kind == FORMAL_CACHED ? b->formal_qb : 0;
       S.formal_threads = b->formal_threads;
       S.formal_kernel = b->formal_kind == FORMAL_SWEEP
                             ? (b->sweep_variant == 2 ? JFNK_FORMAL_SWEEP_WARP
                                : (sweep_fused(*b) ? JFNK_FORMAL_SWEEP_THREAD_FUSED : JFNK_FORMAL_SWEEP_THREAD))
-                            : (b->formal_kind == FORMAL_FUSED ? JFNK_FORMAL_FUSED
+                            : (b->formal_kind == FORMAL_CACHED ? JFNK_FORMAL_CACHED
+                               : b->formal_kind == FORMAL_FUSED ? JFNK_FORMAL_FUSED
                                : (b->formal_kind == FORMAL_MOVING ? JFNK_FORMAL_MOVING : JFNK_FORMAL_PER_RAY));
     }
     if (status != JFNK_OK && *worst == JFNK_OK) *worst = status;

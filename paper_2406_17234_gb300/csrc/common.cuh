@@ -48,6 +48,11 @@ enum Phase : int {
   PH_DONE = 4,
 };
 
+// Constants of an angle.
+struct Ang64 {
+  double inv2mu, hw, two_mu, pad;   // 1/(2 mu), w_mu/2, 2 mu
+};
+
 // Immutable tables of one column (device pointers), built at atmosphere creation.
 struct ColTables {
   int nz, nq, nl, nt, nmu, nwin;  // nwin = sum over transitions of window points
@@ -96,6 +101,7 @@ struct ColTables {
   const double* wmu;      // [nmu]
   const double* Vd;       // [2 nmu][nwin][nz] V_ij seen along each direction (outgoing
                           // mu_1..mu_n, then ingoing): a moving column; null when static
+  const Ang64* ang64;     // [nmu]
   const float4* ang32;    // [nmu] (1/(2 mu), w_mu/2, 2 mu, 0), each the FP64 value rounded once
   const float2* dz32;     // [nz-1] (|dz|, 1/|dz|) likewise
   const double* chi_c;    // [nq][nz]
@@ -224,6 +230,10 @@ struct ColWork {
   double* mdI;      // its tangent
   double* mLX;      // dI^k/dchi^k of each ray (base evaluations)
   double* mLE;      // dI^k/deta^k
+  // FP64 static columns, cached formal solution (formal_cached.cu); w.chi holds 1/chi there
+  double* cf;       // coefficient planes [tile][nz-1][5][n_mu][qb] (null with another formal kernel)
+  int cq;           // frequencies per tile (the column's own: its results are the same in any batch)
+  double* rpart;    // parts of the rate integrals [(transition, tile)][kPartFixed + nl][nz]
   double* dJdn;     // [nq][nz][nl] lagged d J/d n_j of the second preconditioner
                     // solution (null until a solve asks for it)
   SolverState* st;
@@ -276,6 +286,11 @@ __device__ __forceinline__ const double* eval_pops(const ColDesc& cd, int mode) 
 // [3] sum W chi_t Psi eta_bg, [4 + s] sum W chi_t Psi U_s.
 constexpr int kRhFixed = 4;
 constexpr int kRhStride = kRhFixed + kMaxT;
+// Slots of a tile's part of a transition's integrals in the cached FP64
+// evaluation: [0, 1] R_ij, R_ji, then base: [2 + j] preconditioner sums of
+// level j; RH92: [2, 3] Jeff sums, [4] constant part, [5 + j] sum W chi_t Psi
+// U_j of every level j (its transitions' [4 + s] above added).
+constexpr int kPartFixed = 5;
 
 // ---- error handling --------------------------------------------------------
 void set_error(const std::string& msg);

@@ -1,0 +1,873 @@
+// FP64 evaluation of static columns in one kernel per tile of frequencies
+// (steps a1 to a3: opacity, formal solution, angle and frequency integrals),
+// with the formal solution's coefficients kept for the Newton step's tangents.
+//
+// What bounds it: GB300 issues one FP64 warp instruction per SM every 16
+// cycles, so an evaluation costs the FP64 instructions of its ray-points,
+// whatever else it does. Three things lower that count:
+//   - a layer's coefficients e = exp(-dtau), w, a, b (App. A.1) depend on the
+//     opacity of the layer and on |mu| only: one set serves the ray going out
+//     through the layer and the one coming in;
+//   - they do not change while n is fixed. A base evaluation leaves e, w and
+//     the slope of each ray's intensity on its own dtau,
+//       g = -(e D^u + bq (S^u - S^k))/(2 mu),
+//     in device memory (L2 for one column), and every Jacobian-vector product
+//     of that Newton step is the recurrence
+//       dD^k = dD^u e + g |dz|(dchi^k + dchi^u) + w (dS^u - dS^k):
+//     three FMAs per ray-point instead of an exponential and about 40 others;
+//   - the ray sums take one FMA per ray and quantity, and the re-anchoring of
+//     D = I - S on the better-conditioned form compares exponent words.
+// The opacity of the tile and the rate integrals over it are formed in the
+// same block (two launches and the round trips of chi, dJ and the Lambda
+// diagonals fewer); a tile leaves its part of each integral it meets, and
+// k_rates_reduce adds the parts in tile order (no atomics).
+//
+// A block takes Qb frequencies (cached_default_qb) of one column: all threads
+// form the coefficients, one thread per ray runs the recurrences over chunks
+// of kChunk layers (loads a batch of layers ahead), all threads add the rays
+// of the chunk. Lanes run over frequencies first, so the coefficient planes
+// [tile][layer][5][angle][Qb] are read in contiguous rows.
+//
+// Measured (kernel time, warm L2), against the fused kernel with its separate
+// opacity and rate kernels: 82 depths x 1,005 frequencies x 5 angles, base
+// 244 + 11 + 59 -> 87 + 8 us, tangent 149 + 11 + 12 -> 26 + 8 us; 101 x 41 x 5,
+// base 126 + 8 + 18 -> 50 + 10 us, tangent 48 + 8 + 11 -> 18 + 10 us. A base
+// evaluation is bound by its FP64 instructions (half of it the coefficients),
+// a tangent by the chain of chunks.
+#include <algorithm>
+#include <cmath>
+
+#include "formal_coef.cuh"
+
+namespace jfnk {
+
+constexpr int kPlanes = 5;    // e, w, P_up (later g_up), P_dn (later g_dn), bq dS
+constexpr int kChunk = 8;     // layers between two ray sums
+constexpr int kMaxQb = 8;
+constexpr int kItems = 3;     // ray steps of a chunk per helper thread: kChunk 128 <= kItems (kEvalThreads - 128)
+constexpr int kBufRows = 8 * kChunk + 2 * (2 * kChunk + 1) + kChunk;
+static_assert(kChunk * 128 <= kItems * (kEvalThreads - 128), "a chunk's ray steps fit the helpers");
+constexpr int kExpTab = 256;
+constexpr size_t kCachedSmem = (size_t)222 * 1024;   // beside the static shared memory
+
+// 2^(-j/256) and 1 - 2^(-j/256), for neg_exp
+__device__ double2 d_exp_tab[kExpTab];
+
+__host__ __device__ inline int pad_qb(int qb) { return qb | 1; }   // odd row stride: no bank conflicts over depths
+
+// Doubles shared in turn by the recurrence's buffers (two chunks of e, X, P, Y
+// in, two of D, I out with the D before them, one of g) and by the level sums
+// of at least 32 depths.
+__host__ __device__ inline size_t chunk_doubles(int qb, int nmu, int nl) {
+  const size_t rays = (size_t)kBufRows * 2 * nmu * qb, zeta = (size_t)qb * nl * 32;
+  return rays > zeta ? rays : zeta;
+}
+
+size_t cached_smem_bytes(int qb, int nz, int nmu, int nl) {
+  const size_t Z = (size_t)nz * pad_qb(qb);
+  return sizeof(double) * (7 * Z + chunk_doubles(qb, nmu, nl)) + sizeof(int) * ((size_t)qb * kMaxT);
+}
+
+// Doubles of the coefficient planes and of the rate parts of one column.
+size_t cached_planes(int qb, int nz, int nq, int nmu) {
+  return (size_t)((nq + qb - 1) / qb) * (nz - 1) * kPlanes * qb * nmu;
+}
+size_t cached_parts(int qb, int nz, int nl, int nwin, int nt) {
+  // a transition's window of nw points meets at most (nw - 1)/qb + 2 tiles
+  return ((size_t)nwin / qb + 2 * (size_t)nt) * (kPartFixed + nl) * nz;
+}
+
+// Frequencies per block of a column: the smallest (waves of blocks) x (FP64
+// warp instructions of a block per layer), at 2 n_mu qb/32 full warps' worth
+// of about 18 (coefficients, ray sums) plus 7 per warp of rays (recurrences,
+// partly filled), for the column alone on the device: 7 for 1,005 frequencies
+// (144 blocks on 152 SMs), 1 for 41. It sets the order of the rate sums, so it
+// must not depend on the batch: a column's result is the same alone and in any
+// batch.
+int cached_default_qb(int nq, int nz, int nmu, int nl, int n_sm) {
+  int best = 0;
+  double cost = 0.0;
+  for (int qb = 1; qb <= kMaxQb; ++qb) {
+    if (cached_smem_bytes(qb, nz, nmu, nl) > kCachedSmem || 2 * nmu * qb > 128) break;
+    const long blocks = (nq + qb - 1) / qb;
+    const double waves = blocks <= 4L * n_sm ? (double)((blocks + n_sm - 1) / n_sm) : (double)blocks / n_sm;
+    const int rays = 2 * nmu * qb;
+    const double c = waves * (18.0 * rays / 32.0 + 7.0 * ((rays + 31) / 32));
+    if (!best || c < cost) {
+      best = qb;
+      cost = c;
+    }
+  }
+  return best;
+}
+
+namespace {
+
+__device__ __forceinline__ int mode_of(const ColDesc& cd) { return eval_mode_f(cd); }
+
+__device__ __forceinline__ const double* dir_of(const ColDesc& cd) {
+  if (cd.forced_mode >= 0) return cd.w.v;
+  const int N = cd.t.nz * cd.t.nl;
+  return cd.w.st->phase == PH_RESTART ? cd.w.x : cd.w.Vb + (size_t)cd.w.st->j * N;
+}
+
+// e = e^(-x) and om = 1 - e for x >= 1e-5 (e = 0 from x = 700 on) in ten FP64
+// instructions: x = n ln2/256 + r, |r| < 1.4e-3, 2^(-n/256) from a table, p =
+// e^(-r) - 1 to the fourth order (the next term is below 4e-17): the table
+// method of Tang (ACM Trans. Math. Softw. 15, 144, 1989). Below ln 2 the sum is
+// formed for om, from tabulated 1 - 2^(-j/256), and e = 1 - om: w = om/x then
+// keeps full relative accuracy in thin layers, where 1 - e cancels.
+__device__ __forceinline__ void neg_exp(double x, const double2* tab, double& e, double& om) {
+  const double magic = 6755399441055744.0;   // 1.5 2^52: n in the low word
+  const double t = fma(x, 369.32993046757464, magic);
+  const int n = __double2loint(t);
+  const double tn = t - magic;
+  double r = fma(tn, -0.0027076061740622863, x);
+  r = fma(tn, -9.0587766165870294e-20, r);
+  double q = fma(r, 1.0 / 24, -1.0 / 6);
+  q = fma(q, r, 0.5);
+  q = fma(q, r, -1.0);
+  const double2 T0 = tab[n & (kExpTab - 1)];
+  const double T = __hiloint2double(__double2hiint(T0.x) - ((n >> 8) << 20), __double2loint(T0.x));
+  const bool small = n < kExpTab;
+  const double u = fma(small ? -T : T, q * r, small ? T0.y : T), v = 1.0 - u;
+  e = small ? v : u;
+  om = small ? u : v;
+  if (__double2hiint(x) >= 0x4085e000) {   // x >= 700
+    e = 0.0;
+    om = 1.0;
+  }
+}
+
+// Coefficients of one step of optical depth x, r = 1/x (App. A.1): e, w, bq =
+// (w - e)/x, a = 1 - w and om = 1 - e = a + bq x. With om from neg_exp the
+// direct forms lose 1e-16/x relative in a and bq (which enter every sum times
+// x or x dS), so the series (truncated below 4e-17) is needed from x = 1e-5
+// down only; it skips the exponential.
+__device__ __forceinline__ void step_coef(double x, double r, const double2* tab, double& e, double& w, double& a,
+                                          double& bq, double& om) {
+  if (x < 1e-5) {
+    if (x > -1e-5) {
+      w = fma(fma(fma(-1.0 / 24, x, 1.0 / 6), x, -0.5), x, 1.0);
+      bq = fma(fma(1.0 / 8, x, -1.0 / 3), x, 0.5);
+      om = x * w;
+      e = 1.0 - om;
+      a = fma(-bq, x, om);
+    } else {   // inverted populations
+      pl_series64(x, w, a, bq);
+      e = exp(-x);
+      om = fma(bq, x, a);
+    }
+  } else {
+    neg_exp(x, tab, e, om);
+    w = om * r;
+    a = 1.0 - w;
+    bq = (w - e) * r;
+  }
+}
+
+// |x| to float by its words (no FP64 instruction), 0 below the float range.
+__device__ __forceinline__ float abs_float(double x) {
+  const int h = (__double2hiint(x) & 0x7fffffff) - (896 << 20);
+  return h <= 0 ? 0.f : __int_as_float((h << 3) | ((unsigned)__double2loint(x) >> 29));
+}
+
+__device__ __forceinline__ int mag(double x) { return __double2hiint(x) & 0x7fffffff; }
+
+// First part slot of transition t in ColWork::rpart and its number of tiles,
+// for the lane's transition (warp-wide; lanes past nt get 0).
+__device__ __forceinline__ int part_offset(const ColTables& T, int qb, int lane, int& tile0, int& ntile) {
+  tile0 = ntile = 0;
+  if (lane < T.nt) {
+    tile0 = T.t_q0[lane] / qb;
+    ntile = T.t_q1[lane] / qb - tile0 + 1;
+  }
+  int s = ntile;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int v = __shfl_up_sync(0xffffffffu, s, o);
+    if (lane >= o) s += v;
+  }
+  return s - ntile;
+}
+
+struct Tile {
+  int qb0, nqb, Qb, Qp, R5;   // first frequency, frequencies, tile size, padded size, Qb n_mu
+  int tile;
+};
+
+// The transitions active at each frequency of the tile: window point << 8 |
+// lower << 4 | upper, in list order, -1 past the last.
+__device__ __forceinline__ void stage_lists(const ColTables& T, const Tile& g, int* s_list) {
+  const bool packed = T.max_overlap <= kQMetaT;
+  for (int i = threadIdx.x; i < g.nqb * kMaxT; i += blockDim.x) {
+    const int ql = i / kMaxT, j = i - ql * kMaxT, q = g.qb0 + ql;
+    int m = -1;
+    if (packed) {
+      if (j < kQMetaT) m = __ldg(T.qmeta + (size_t)j * T.nq + q);
+    } else if (T.q_off[q] + j < T.q_off[q + 1]) {
+      const int s = T.q_off[q] + j;
+      const int t = T.q_t[s];
+      m = ((T.t_base[t] + q - T.t_q0[t]) << 8) | (T.t_lo[t] << 4) | T.t_up[t];
+    }
+    s_list[i] = m;
+  }
+}
+
+// sum V x_lo and sum g V x_up over the transitions active at a frequency (list
+// L), at depth k: the loads of two transitions are issued together.
+__device__ __forceinline__ void line_sums(const ColTables& T, const int* L, int k, const double* __restrict__ x,
+                                          double& sl, double& su) {
+  sl = su = 0.0;
+  const double* xk = x + (size_t)k * T.nl;
+  for (int j = 0; j < kMaxT; j += 2) {
+    const int m0 = L[j], m1 = L[j + 1];
+    if (m0 < 0) break;
+    const size_t p0 = (size_t)(m0 >> 8) * T.nz + k, p1 = (size_t)((m1 < 0 ? m0 : m1) >> 8) * T.nz + k;
+    const double v0 = T.V[p0], g0 = T.gV[p0], v1 = T.V[p1], g1 = T.gV[p1];
+    const double l0 = xk[(m0 >> 4) & 15], u0 = xk[m0 & 15];
+    const double l1 = xk[(m1 < 0 ? m0 : m1) >> 4 & 15], u1 = xk[(m1 < 0 ? m0 : m1) & 15];
+    sl = fma(v0, l0, sl);
+    su = fma(g0, u0, su);
+    if (m1 < 0) break;
+    sl = fma(v1, l1, sl);
+    su = fma(g1, u1, su);
+  }
+}
+
+// Parts of the rate integrals of transition t at depth k over the tile's
+// frequencies: sum W V J and sum W g V J (J: dJ in tangent evaluations).
+__device__ __forceinline__ void rate_parts(const ColTables& T, const Tile& g, int t, int k, const double* s_J,
+                                           double* part) {
+  const int q0 = T.t_q0[t], qa = max(q0, g.qb0), n = min(T.t_q1[t], g.qb0 + g.nqb - 1) - qa + 1;
+  const size_t pk = (size_t)(T.t_base[t] + qa - q0) * T.nz + k;
+  double wv[kMaxQb], wg[kMaxQb];
+#pragma unroll
+  for (int i = 0; i < kMaxQb; ++i) {
+    const size_t p = pk + (size_t)min(i, n - 1) * T.nz;
+    wv[i] = T.WV[p];
+    wg[i] = T.WgV[p];
+  }
+  double a0 = 0.0, a1 = 0.0;
+#pragma unroll
+  for (int i = 0; i < kMaxQb; ++i)
+    if (i < n) {
+      const double J = s_J[k * g.Qp + qa - g.qb0 + i];
+      a0 = fma(wv[i], J, a0);
+      a1 = fma(wg[i], J, a1);
+    }
+  part[k] = a0;
+  part[T.nz + k] = a1;
+}
+
+// Barrier of the threads from ``first`` on (the warps without rays).
+__device__ __forceinline__ void helper_sync(int first) {
+  asm volatile("bar.sync 1, %0;" ::"r"((int)blockDim.x - first) : "memory");
+}
+
+}  // namespace
+
+// One F-class evaluation of one tile of frequencies (grid: tiles x columns).
+//
+// Each SM sub-partition starts an FP64 warp instruction every 64 cycles, so a
+// warp that carries rays must do little else: the first warps (one lane per
+// ray) run the recurrences alone, D' = D e + X and I' = I e + P, over chunks of
+// kChunk layers, while the others form e, X, P of the next chunk in shared
+// memory (from planes loaded a chunk before) and add the rays of the previous
+// one. One block barrier per chunk.
+// MU: angles of every column of the launch (0: read from the column).
+template <int MU>
+__global__ void __launch_bounds__(kEvalThreads) k_eval64(const ColDesc* __restrict__ cols, const SolverOpts* bopts) {
+  extern __shared__ __align__(16) double sm[];
+  __shared__ double s_inv2mu[kMaxMu], s_hw[kMaxMu], s_2mu[kMaxMu];
+  __shared__ float s_hwf[kMaxMu];
+  __shared__ double2 s_tab[kExpTab];
+  __shared__ int s_act[kMaxT], s_off[kMaxT], s_nact;
+  const ColDesc& cd = cols[blockIdx.y];
+  const int mode = mode_of(cd);
+  if (mode == EV_SKIP) return;
+  const ColTables& T = cd.t;
+  const int nz = T.nz, nq = T.nq, nmu = MU ? MU : T.nmu, nl = T.nl, Qb = cd.w.cq;
+  Tile g;
+  g.tile = blockIdx.x;
+  g.Qb = Qb;
+  g.qb0 = g.tile * Qb;
+  if (g.qb0 >= nq) return;
+  g.nqb = min(Qb, nq - g.qb0);
+  g.Qp = pad_qb(Qb);
+  g.R5 = Qb * nmu;
+  const int Qp = g.Qp, nqb = g.nqb, qb0 = g.qb0, R5 = g.R5;
+  const int nray = 2 * R5;
+  const size_t Z = (size_t)nz * Qp;
+  double* s_S = sm;               // S^k
+  double* s_chi = s_S + Z;        // chi^k; then sum w I; then J
+  double* s_tz = s_chi + Z;       // sum w D; then Lambda_chi
+  double* s_rs = s_tz + Z;        // sum w |D| (float)
+  double* s_dS = s_rs + Z;        // S^{k+1} - S^k; then Lambda_eta
+  double* s_A = s_dS + Z;         // per layer, sum over the angles of w a
+  double* s_G = s_A + Z;          // sum of w dI/dchi without the local term
+  double* s_buf = s_G + Z;        // the recurrence's chunks; then the level sums
+  double* s_in = s_buf;                               // [2][4][kChunk][nray]: e, X, P, Y
+  double* s_out = s_buf + (size_t)8 * kChunk * nray;  // [2][2 kChunk + 1][nray]: D before the chunk, D, I
+  double* s_g = s_out + (size_t)2 * (2 * kChunk + 1) * nray;   // [kChunk][nray]: g
+  int* s_list = reinterpret_cast<int*>(s_buf + chunk_doubles(Qb, nmu, nl));
+  double* cf = cd.w.cf + (size_t)g.tile * (nz - 1) * kPlanes * R5;
+  const bool tan = (mode == EV_TANGENT), der = (mode == EV_BASE || mode == EV_RH92), base = (mode == EV_BASE);
+
+  stage_lists(T, g, s_list);
+  for (int m = threadIdx.x; m < nmu; m += blockDim.x) {
+    const Ang64 a = T.ang64[m];
+    s_inv2mu[m] = a.inv2mu;
+    s_hw[m] = a.hw;
+    s_2mu[m] = a.two_mu;
+    s_hwf[m] = (float)a.hw;
+  }
+  if (!tan)
+    for (int i = threadIdx.x; i < kExpTab; i += blockDim.x) s_tab[i] = d_exp_tab[i];
+  if (threadIdx.x < 32) {
+    // the transitions whose windows meet the tile, and their part slots
+    int tile0, ntile;
+    const int off = part_offset(T, Qb, threadIdx.x, tile0, ntile);
+    const bool on = g.tile >= tile0 && g.tile < tile0 + ntile;
+    const unsigned b = __ballot_sync(0xffffffffu, on);
+    if (on) {
+      const int i = __popc(b & ((1u << threadIdx.x) - 1));
+      s_act[i] = threadIdx.x;
+      s_off[i] = off + g.tile - tile0;
+    }
+    if (threadIdx.x == 0) s_nact = __popc(b);
+  }
+  __syncthreads();
+  const int nslot = kPartFixed + nl;
+
+  // this thread's ray, or its place among the warps without rays
+  const int ray = threadIdx.x;
+  const int hfirst = (nray + 31) & ~31;   // first helper thread (2 n_mu Qb <= 128)
+  const bool up = ray >= R5;
+  const int rr = up ? ray - R5 : ray;
+  const int rm = rr / Qb, rq = rr - rm * Qb;
+  const bool run = ray < nray && rq < nqb, helper = (int)threadIdx.x >= hfirst;
+  const int nch = (nz - 2) / kChunk + 1;   // chunks of the nz - 1 layers
+  // this helper's ray steps of every chunk: their row, layer and planes in chunk 0
+  const int t0 = threadIdx.x - hfirst, nh = blockDim.x - hfirst;
+  int ir[kItems], il[kItems];
+  double* ip[kItems];
+  double be[kItems], bw[kItems], bp[kItems], by[kItems];
+#pragma unroll
+  for (int j = 0; j < kItems; ++j) {
+    const int i = t0 + j * nh, r = i / nray, y = i - r * nray;
+    const bool u = y >= R5;
+    const int yr = u ? y - R5 : y;
+    ir[j] = !helper || r >= kChunk || yr % Qb >= nqb ? nz : r;   // nz: never
+    il[j] = u ? nz - 2 - r : r;
+    ip[j] = cf + (ptrdiff_t)il[j] * kPlanes * R5 + yr;
+  }
+  // this helper's place in the ray sums of every chunk: hemisphere, row and
+  // frequency (the last warps take them, the first ones carry more ray steps)
+  const int si = nh - 1 - t0, sh = si / (kChunk * Qb), sr = (si - sh * kChunk * Qb) / Qb, sq = si % Qb;
+  const bool sums = helper && sh < 2 && sq < nqb;
+  auto item_up = [&](int j) { return t0 + j * nh - ir[j] * nray >= R5; };
+  // the planes of chunk c, into registers
+  auto load = [&](int c) {
+#pragma unroll
+    for (int j = 0; j < kItems; ++j)
+      if (c * kChunk + ir[j] < nz - 1) {
+        const bool u = item_up(j);
+        const double* p = ip[j] + (u ? -1 : 1) * (ptrdiff_t)c * kChunk * kPlanes * R5;
+        be[j] = p[0];
+        bw[j] = p[R5];
+        if (tan || der) bp[j] = p[(u ? 2 : 3) * R5];
+        if (base) by[j] = p[4 * R5];
+      }
+  };
+  // the inputs of chunk c, from registers into its buffer
+  auto store = [&](int c) {
+    double* in = s_in + (size_t)(c & 1) * 4 * kChunk * nray;
+#pragma unroll
+    for (int j = 0; j < kItems; ++j)
+      if (c * kChunk + ir[j] < nz - 1) {
+        const bool u = item_up(j);
+        const int i = t0 + j * nh, l = il[j] + (u ? -c * kChunk : c * kChunk);
+        const int e = l * Qp + (u ? i - ir[j] * nray - R5 : i - ir[j] * nray) % Qb;
+        const double x = bw[j] * s_dS[e];
+        in[i] = be[j];
+        if (tan) {
+          // s_dS: dS^{k+1} - dS^k, s_tz: |dz|(dchi^k + dchi^{k+1})
+          in[kChunk * nray + i] = fma(bp[j], s_tz[e], u ? x : -x);
+        } else {
+          in[kChunk * nray + i] = u ? x : -x;
+          if (der) in[2 * kChunk * nray + i] = bp[j];
+          if (base) in[3 * kChunk * nray + i] = by[j];
+        }
+      }
+  };
+
+  if (tan) {
+    load(0);   // the base evaluation's planes, while the opacity's tangent is formed
+    double* s_dc = s_S;      // dchi^k; then dJ
+    double* s_dT = s_chi;    // dS^k
+    double* s_acc = s_rs;    // sum over the rays of w dD
+    const double* v = dir_of(cd);
+    const double* rchi = reinterpret_cast<const double*>(cd.w.chi);
+    for (int i = threadIdx.x; i < nqb * nz; i += blockDim.x) {
+      const int ql = i / nz, k = i - ql * nz;
+      const size_t o = (size_t)(qb0 + ql) * nz + k;
+      const double S = cd.w.S[o], rc = rchi[o];
+      double dl, de;
+      line_sums(T, s_list + ql * kMaxT, k, v, dl, de);
+      const double dc = dl - de;
+      s_dc[k * Qp + ql] = dc;
+      s_dT[k * Qp + ql] = fma(-S, dc, de) * rc;
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < nqb * nz; i += blockDim.x) {
+      const int k = i / nqb, ql = i - k * nqb, e = k * Qp + ql;
+      // the boundary rays start from dD = -dS at the bottom (outgoing) and the top (ingoing)
+      double acc = 0.0;
+      if (k == 0 || k == nz - 1)
+        for (int m = 0; m < nmu; ++m) acc = fma(-s_hw[m], s_dT[e], acc);
+      s_acc[e] = acc;
+      if (k < nz - 1) {
+        s_tz[e] = T.dz[k] * (s_dc[e] + s_dc[e + Qp]);
+        s_dS[e] = s_dT[e + Qp] - s_dT[e];
+      }
+    }
+    __syncthreads();
+    store(0);
+    load(1);
+    double dD = run ? -s_dT[(up ? nz - 1 : 0) * Qp + rq] : 0.0;
+    __syncthreads();
+    for (int c = 0; c <= nch; ++c) {
+      if (!helper) {
+        if (c < nch && run) {
+          const int rows = min(kChunk, nz - 1 - c * kChunk);
+          const double* in = s_in + (size_t)(c & 1) * 4 * kChunk * nray + ray;
+          double* out = s_out + (size_t)(c & 1) * (2 * kChunk + 1) * nray + ray;
+          double e[kChunk], X[kChunk];
+#pragma unroll
+          for (int r = 0; r < kChunk; ++r) {
+            const int q = min(r, rows - 1) * nray;
+            e[r] = in[q];
+            X[r] = in[kChunk * nray + q];
+          }
+#pragma unroll
+          for (int r = 0; r < kChunk; ++r) X[r] = dD = r < rows ? fma(dD, e[r], X[r]) : dD;
+#pragma unroll
+          for (int r = 0; r < kChunk; ++r)
+            if (r < rows) out[r * nray] = X[r];
+        }
+      } else {
+        if (c > 0) {
+          const int c0 = (c - 1) * kChunk, rows = min(kChunk, nz - 1 - c0);
+          const double* out = s_out + (size_t)((c - 1) & 1) * (2 * kChunk + 1) * nray;
+          // a depth can be reached by both hemispheres in one chunk (the middle
+          // of the column): its two sums are then added one after the other
+          const bool apart = c0 + rows < nz - 1 - c0 - rows || c0 + 1 > nz - 2 - c0;
+          for (int h = 0; h < (apart ? 1 : 2); ++h) {
+            if (sums && sr < rows && (apart || h == sh)) {
+              const int e = (sh ? nz - 2 - (c0 + sr) : c0 + sr + 1) * Qp + sq;
+              const double* x = out + sr * nray + sh * R5 + sq;
+              double a = s_acc[e];
+#pragma unroll
+              for (int m = 0; m < nmu; ++m) a = fma(s_hw[m], x[m * Qb], a);
+              s_acc[e] = a;
+            }
+            if (!apart) helper_sync(hfirst);
+          }
+        }
+        if (c + 1 < nch) {
+          store(c + 1);
+          load(c + 2);
+        }
+      }
+      __syncthreads();
+    }
+    for (int i = threadIdx.x; i < nqb * nz; i += blockDim.x) {
+      const int k = i / nqb, ql = i - k * nqb, e = k * Qp + ql;
+      s_dc[e] = (s_dT[e] + s_acc[e]) * T.c2[qb0 + ql];
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < s_nact * nz; i += blockDim.x) {
+      const int a = i / nz, k = i - a * nz;
+      rate_parts(T, g, s_act[a], k, s_dc, cd.w.rpart + (size_t)s_off[a] * nslot * nz);
+    }
+    return;
+  }
+
+  // ---- values: opacity and source function (Eqs. chi, eta) ------------------
+  const double* n = eval_pops(cd, mode);
+  const double* Jd = jdag_ptr(cd);
+  for (int i = threadIdx.x; i < nqb * nz; i += blockDim.x) {
+    const int ql = i / nz, k = i - ql * nz;
+    const size_t o = (size_t)(qb0 + ql) * nz + k;
+    const double sca = T.chi_sca[k], chib = T.chi_c[o] + sca;
+    const double eta_bg = T.eta_c[o] + sca * Jd[o];
+    const double c2 = T.c2[qb0 + ql];
+    double chl, el;
+    line_sums(T, s_list + ql * kMaxT, k, n, chl, el);
+    const double chi = chib + (chl - el), eta = fma(c2, el, eta_bg);
+    // S = eta/(chi 2 h nu^3/c^2), rounded once (quotient plus its remainder)
+    const double d = chi * c2, rd = 1.0 / d, q0 = eta * rd, S = fma(fma(-q0, d, eta), rd, q0), rc = c2 * rd;
+    s_chi[k * Qp + ql] = chi;
+    s_S[k * Qp + ql] = S;
+    s_A[k * Qp + ql] = 0.0;
+    if (der) {
+      reinterpret_cast<double*>(cd.w.chi)[o] = rc;   // 1/chi: all that later steps need
+      cd.w.S[o] = S;
+      if (mode == EV_RH92) cd.w.eta[o] = eta;
+    }
+  }
+  __syncthreads();
+  // ---- coefficients of every (layer, angle), for both hemispheres ------------
+  for (int i = threadIdx.x; i < nqb * (nz - 1); i += blockDim.x) {
+    const int l = i / nqb, ql = i - l * nqb, e0 = l * Qp + ql;
+    const double tz = T.dz[l] * (s_chi[e0] + s_chi[e0 + Qp]), rs = 1.0 / tz;
+    const double S0 = s_S[e0], S1 = s_S[e0 + Qp], dS = S1 - S0;
+    s_dS[e0] = dS;
+    double* c = cf + (size_t)l * kPlanes * R5 + ql;
+    double A = 0.0;
+#pragma unroll
+    for (int m = 0; m < nmu; ++m, c += Qb) {
+      const double x = tz * s_inv2mu[m];
+      double e, w, a, bq, om;
+      step_coef(x, rs * s_2mu[m], s_tab, e, w, a, bq, om);
+      c[0] = e;
+      c[R5] = w;
+      if (der) {
+        // outgoing a S^k + b S^{k+1}, ingoing a S^{k+1} + b S^k, b = bq x = om - a
+        const double Y = bq * dS, yx = Y * x;
+        c[2 * R5] = fma(om, S0, yx);
+        c[3 * R5] = fma(om, S1, -yx);
+        c[4 * R5] = Y;
+        A = fma(s_hw[m], a, A);
+      }
+    }
+    s_A[e0] = A;
+  }
+  // ---- recurrences ------------------------------------------------------------
+  __syncthreads();
+  double* s_I = s_chi;
+  double* s_D = s_tz;
+  float* s_aD = reinterpret_cast<float*>(s_rs);   // only compared
+  double* s_Le = s_dS;
+  for (int i = threadIdx.x; i < nqb * nz; i += blockDim.x) {
+    const int k = i / nqb, ql = i - k * nqb, e = k * Qp + ql;
+    double d = 0.0, in = 0.0;
+    float ad = 0.f;
+    if (k == 0 || k == nz - 1) {
+      const double Ib = k == 0 ? 0.0 : T.Bn[(size_t)(qb0 + ql) * nz + nz - 1] / T.c2[qb0 + ql];
+      const double D = Ib - s_S[e];
+      for (int m = 0; m < nmu; ++m) {
+        d = fma(s_hw[m], D, d);
+        ad = fmaf(s_hwf[m], abs_float(D), ad);
+        in = fma(s_hw[m], Ib, in);
+      }
+    }
+    s_I[e] = in;
+    s_D[e] = d;
+    s_aD[e] = ad;
+    s_G[e] = 0.0;
+  }
+  double D = 0.0, I = 0.0;
+  int M = 0;   // exponent word of the attenuated bound of |D| upstream
+  if (run) {
+    I = up ? T.Bn[(size_t)(qb0 + rq) * nz + nz - 1] / T.c2[qb0 + rq] : 0.0;
+    D = I - s_S[(up ? nz - 1 : 0) * Qp + rq];
+    M = mag(D);
+  }
+  load(0);
+  store(0);
+  load(1);
+  __syncthreads();
+  for (int c = 0; c <= nch; ++c) {
+    if (!helper) {
+      if (c < nch && run) {
+        const int c0 = c * kChunk, rows = min(kChunk, nz - 1 - c0);
+        const double* in = s_in + (size_t)(c & 1) * 4 * kChunk * nray + ray;
+        double* out = s_out + (size_t)(c & 1) * (2 * kChunk + 1) * nray + ray;   // D before, D after each step, I
+        out[0] = D;
+        double e[kChunk], X[kChunk], P[kChunk], Sk[kChunk];
+#pragma unroll
+        for (int r = 0; r < kChunk; ++r) {
+          const int rq_ = min(r, rows - 1), q = rq_ * nray;
+          e[r] = in[q];
+          X[r] = in[kChunk * nray + q];
+          if (der) {
+            P[r] = in[2 * kChunk * nray + q];
+            Sk[r] = s_S[(up ? nz - 2 - c0 - rq_ : c0 + rq_ + 1) * Qp + rq];
+          }
+        }
+#pragma unroll
+        for (int r = 0; r < kChunk; ++r)
+          if (r < rows) {
+            double Dn = fma(D, e[r], X[r]);
+            if (der) {
+              I = fma(I, e[r], P[r]);
+              // D carries an absolute error of the order of the largest |D| met
+              // upstream (attenuated), I - S one of the order of |I| + |S|: take the
+              // better-conditioned form (a factor of two does not matter here, so
+              // the comparison is one of exponent words)
+              M = max(M + __double2hiint(e[r]) - 0x3ff00000, mag(Dn));
+              const int anchor = max(mag(I), mag(Sk[r]));
+              if (anchor < M) {
+                Dn = I - Sk[r];
+                M = anchor;
+              }
+              P[r] = I;
+            }
+            X[r] = D = Dn;
+          }
+#pragma unroll
+        for (int r = 0; r < kChunk; ++r)
+          if (r < rows) {
+            out[(r + 1) * nray] = X[r];
+            if (der) out[(kChunk + 1 + r) * nray] = P[r];
+          }
+      }
+    } else {
+      if (base && c > 0) {
+        // the slope of each ray's intensity on its dtau, kept for the tangents
+        const double* in = s_in + (size_t)((c - 1) & 1) * 4 * kChunk * nray;
+        const double* out = s_out + (size_t)((c - 1) & 1) * (2 * kChunk + 1) * nray;
+#pragma unroll
+        for (int j = 0; j < kItems; ++j)
+          if ((c - 1) * kChunk + ir[j] < nz - 1) {
+            const bool u = item_up(j);
+            const int i = t0 + j * nh;
+            const double Y = in[3 * kChunk * nray + i];
+            const int yr = u ? i - ir[j] * nray - R5 : i - ir[j] * nray;
+            const double gm = -s_inv2mu[yr / Qb] * fma(in[i], out[i], u ? Y : -Y);
+            ip[j][(u ? -1 : 1) * (ptrdiff_t)(c - 1) * kChunk * kPlanes * R5 + (u ? 2 : 3) * R5] = gm;
+            s_g[i] = gm;
+          }
+      }
+      if (c + 1 < nch) {   // into the buffer whose e, Y this thread has just read
+        store(c + 1);
+        load(c + 2);
+      }
+      if (base) helper_sync(hfirst);
+      if (c > 0) {
+        const int c0 = (c - 1) * kChunk, rows = min(kChunk, nz - 1 - c0);
+        const double* out = s_out + (size_t)((c - 1) & 1) * (2 * kChunk + 1) * nray;
+        const bool apart = c0 + rows < nz - 1 - c0 - rows || c0 + 1 > nz - 2 - c0;   // as above
+        for (int h = 0; h < (apart ? 1 : 2); ++h) {
+          if (sums && sr < rows && (apart || h == sh)) {
+            const int k = sh ? nz - 2 - (c0 + sr) : c0 + sr + 1, l = sh ? k : k - 1;
+            const int y = sr * nray + sh * R5 + sq, e = k * Qp + sq;
+            double d = s_D[e], in = s_I[e], gs = 0.0;
+            float ad = s_aD[e];
+#pragma unroll
+            for (int m = 0; m < nmu; ++m) {
+              const double hw = s_hw[m], Dk = out[nray + y + m * Qb];
+              d = fma(hw, Dk, d);
+              if (der) {
+                ad = fmaf(s_hwf[m], abs_float(Dk), ad);
+                in = fma(hw, out[(kChunk + 1) * nray + y + m * Qb], in);
+                if (base) gs = fma(hw, s_g[y + m * Qb], gs);
+              }
+            }
+            s_D[e] = d;
+            if (der) {
+              s_aD[e] = ad;
+              s_I[e] = in;
+              if (base) s_G[e] = fma(T.dz[l], gs, s_G[e]);
+            }
+          }
+          if (!apart) helper_sync(hfirst);
+        }
+      }
+    }
+    __syncthreads();
+  }
+  if (run && up && der) cd.w.Iem[(size_t)(qb0 + rq) * nmu + rm] = I * T.c2[qb0 + rq];
+
+  // ---- J and the Lambda diagonals (App. A.2 with S^u - I^u = -D^u) ------------
+  for (int i = threadIdx.x; i < nqb * nz; i += blockDim.x) {
+    const int ql = i / nz, k = i - ql * nz, e = k * Qp + ql;
+    const size_t o = (size_t)(qb0 + ql) * nz + k;
+    const double c2 = T.c2[qb0 + ql], S = s_S[e];
+    double J = (S + s_D[e]) * c2, Lx = 0.0, Le = 0.0;
+    if (der) {
+      // the representation with the smaller rounding error (intensities are >= 0)
+      if (abs_float(s_I[e]) < s_aD[e]) J = s_I[e] * c2;
+      const double rc = reinterpret_cast<const double*>(cd.w.chi)[o];
+      const double A = (k < nz - 1 ? s_A[e] : 0.0) + (k > 0 ? s_A[e - Qp] : 0.0);
+      Le = rc * A;
+      jnew_ptr(cd)[o] = J;
+      if (base) {
+        Lx = fma(-S, Le, s_G[e]) * c2;
+        cd.w.Lchi[o] = Lx;
+        cd.w.Leta[o] = Le;
+      }
+    }
+    s_I[e] = J;
+    s_D[e] = Lx;
+    s_Le[e] = Le;
+  }
+  __syncthreads();
+
+  // ---- rate integrals over the tile (Eqs. Rij, Rji) ---------------------------
+  if (!der) {
+    for (int i = threadIdx.x; i < s_nact * nz; i += blockDim.x) {
+      const int a = i / nz, k = i - a * nz;
+      rate_parts(T, g, s_act[a], k, s_I, cd.w.rpart + (size_t)s_off[a] * nslot * nz);
+    }
+    return;
+  }
+  // with the preconditioner sums sum_nu W chi_t zeta_j (Sect. 2.5.1),
+  // zeta_j = beta_j Lchi + gamma_j Leta, or the RH92 sums with
+  // zeta_j = Psi* sum_{s: up = j} 2 h nu^3/c^2 g_s V_s: zeta is formed once per
+  // (nu, depth) and level, as many depths at a time as the buffer holds
+  const int pv = base ? precond_variant(cd, bopts) : 1;
+  const int kt = min(nz, (int)(chunk_doubles(Qb, nmu, nl) / ((size_t)Qb * nl)));
+  double* s_z = s_buf;   // [Qb][nl][kt]
+  for (int k0 = 0; k0 < nz; k0 += kt) {
+    const int nk = min(kt, nz - k0);
+    for (int i = threadIdx.x; i < nqb * nk; i += blockDim.x) {
+      const int ql = i / nk, kk = i - ql * nk, k = k0 + kk, e = k * Qp + ql;
+      double* z = s_z + (size_t)ql * nl * kt + kk;
+      const double Lx = s_D[e], Le = s_Le[e], c2 = T.c2[qb0 + ql], sca = T.chi_sca[k];
+      for (int j = 0; j < nl; ++j)
+        z[j * kt] = (pv == 2) ? sca * Le * cd.w.dJdn[((size_t)(qb0 + ql) * nz + k) * nl + j] : 0.0;
+      const double cu = base ? fma(c2, Le, -Lx) : c2 * Le;
+      const int* L = s_list + ql * kMaxT;
+      for (int j = 0; j < kMaxT; ++j) {
+        const int m = L[j];
+        if (m < 0) break;
+        const size_t p = (size_t)(m >> 8) * nz + k;
+        if (base) {
+          double& zl = z[((m >> 4) & 15) * kt];
+          zl = fma(T.V[p], Lx, zl);
+        }
+        double& zu = z[(m & 15) * kt];
+        zu = fma(T.gV[p], cu, zu);
+      }
+      if (pv == 3) {
+        const double f = 1.0 / (1.0 - sca * Le);
+        for (int j = 0; j < nl; ++j) z[j * kt] *= f;
+      }
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < s_nact * nk; i += blockDim.x) {
+      const int a = i / nk, kk = i - a * nk, k = k0 + kk, t = s_act[a];
+      const int q0 = T.t_q0[t], qa = max(q0, qb0), nw = min(T.t_q1[t], qb0 + nqb - 1) - qa + 1;
+      const double nlo = n[k * nl + T.t_lo[t]], nup = n[k * nl + T.t_up[t]];
+      const size_t pk = (size_t)(T.t_base[t] + qa - q0) * nz + k;
+      double wv[kMaxQb], wg[kMaxQb];
+#pragma unroll
+      for (int q = 0; q < kMaxQb; ++q) {
+        const size_t p = pk + (size_t)min(q, nw - 1) * nz;
+        wv[q] = T.WV[p];
+        wg[q] = T.WgV[p];
+      }
+      double* part = cd.w.rpart + (size_t)s_off[a] * nslot * nz + k;
+      double a0 = 0.0, a1 = 0.0, r0 = 0.0, r1 = 0.0, r3 = 0.0;
+#pragma unroll
+      for (int q = 0; q < kMaxQb; ++q)
+        if (q < nw) {
+          const int e = k * Qp + qa - qb0 + q;
+          const double J = s_I[e];
+          a0 = fma(wv[q], J, a0);
+          a1 = fma(wg[q], J, a1);
+          const double Wc = fma(wv[q], nlo, -wg[q] * nup);   // W chi_t
+          if (!base) {
+            const size_t o = (size_t)(qa + q) * nz + k;
+            const double Le = s_Le[e], Je = fma(-Le, cd.w.eta[o], J);   // Jeff = J - Psi* eta
+            r0 = fma(wv[q], Je, r0);
+            r1 = fma(wg[q], Je, r1);
+            r3 = fma(Wc * Le, T.eta_c[o] + T.chi_sca[k] * Jd[o], r3);
+          }
+          wv[q] = Wc;
+        }
+      part[0] = a0;
+      part[nz] = a1;
+      if (!base) {
+        part[2 * (size_t)nz] = r0;
+        part[3 * (size_t)nz] = r1;
+        part[4 * (size_t)nz] = r3;
+      }
+      const double* z = s_z + (size_t)(qa - qb0) * nl * kt + kk;
+      part += (size_t)(base ? 2 : kPartFixed) * nz;
+      for (int j = 0; j < nl; ++j, z += kt, part += nz) {
+        double acc = 0.0;
+#pragma unroll
+        for (int q = 0; q < kMaxQb; ++q)
+          if (q < nw) acc = fma(wv[q], z[q * nl * kt], acc);
+        part[0] = acc;
+      }
+    }
+    __syncthreads();
+  }
+}
+
+// Adds the tiles' parts of every rate integral in tile order and writes the
+// rates, the preconditioner sums or the RH92 sums where the assembly and the
+// RH92 update read them; thread per (transition, slot, depth).
+__global__ void __launch_bounds__(128) k_rates_reduce(const ColDesc* __restrict__ cols) {
+  const ColDesc& cd = cols[blockIdx.z];
+  const int mode = mode_of(cd);
+  if (mode == EV_SKIP) return;
+  const ColTables& T = cd.t;
+  const int nz = T.nz, nl = T.nl, t = blockIdx.y;
+  const bool base = (mode == EV_BASE), rh = (mode == EV_RH92);
+  const int ns = base ? 2 + nl : rh ? kPartFixed + nl : 2;
+  if (t >= T.nt || (int)(blockIdx.x * blockDim.x) >= ns * nz) return;
+  __shared__ int s_off, s_nt;
+  if (threadIdx.x < 32) {
+    int tile0, ntile;
+    const int off = part_offset(T, cd.w.cq, threadIdx.x, tile0, ntile);
+    if ((int)threadIdx.x == t) {
+      s_off = off;
+      s_nt = ntile;
+    }
+  }
+  __syncthreads();
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= ns * nz) return;
+  const int sl = i / nz, k = i - sl * nz;
+  const size_t stride = (size_t)(kPartFixed + nl) * nz;
+  const double* p = cd.w.rpart + (size_t)s_off * stride + (size_t)sl * nz + k;
+  double s = 0.0;
+#pragma unroll 8
+  for (int a = 0; a < s_nt; ++a) s += p[(size_t)a * stride];
+  const size_t o = (size_t)t * nz + k;
+  if (mode == EV_TANGENT) {
+    (sl == 0 ? cd.w.dRup : cd.w.dRdn)[o] = s;
+    return;
+  }
+  const double rsp = T.Rsp[o];
+  if (sl == 0) cd.w.Rup[o] = s;
+  else if (sl == 1) {
+    cd.w.Rdn[o] = s + rsp;
+    if (rh) cd.w.rh[o * kRhStride + 2] = rsp;
+  } else if (base) cd.w.Apart[o * nl + sl - 2] = s;
+  else if (sl < kPartFixed) cd.w.rh[o * kRhStride + (sl == 4 ? 3 : sl - 2)] = s;   // Jeff sums, constant part
+  else cd.w.rh[o * kRhStride + kRhFixed + sl - kPartFixed] = s;                     // per level
+}
+
+int cached_prepare() {
+  double2 tab[kExpTab];
+  for (int j = 0; j < kExpTab; ++j)
+    tab[j] = make_double2(std::exp2(-j / (double)kExpTab), -std::expm1(-j / (double)kExpTab * 0.69314718055994530942));
+  JFNK_CUDA(cudaMemcpyToSymbol(d_exp_tab, tab, sizeof(tab)));
+  JFNK_CUDA(cudaFuncSetAttribute(k_eval64<5>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCachedSmem));
+  JFNK_CUDA(cudaFuncSetAttribute(k_eval64<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCachedSmem));
+  return JFNK_OK;
+}
+
+int launch_eval64(const Batch& b, cudaStream_t s) {
+  const dim3 g(b.max_tiles, b.ncols);
+  if (b.eval_mu == 5) k_eval64<5><<<g, kEvalThreads, b.eval_smem, s>>>(b.d_cols, b.d_opts);
+  else k_eval64<0><<<g, kEvalThreads, b.eval_smem, s>>>(b.d_cols, b.d_opts);
+  JFNK_CUDA(cudaGetLastError());
+  return JFNK_OK;
+}
+
+int launch_rates_reduce(const Batch& b, cudaStream_t s) {
+  const int slots = kPartFixed + b.max_nl;
+  k_rates_reduce<<<dim3((slots * b.max_nz + 127) / 128, b.max_nt, b.ncols), 128, 0, s>>>(b.d_cols);
+  JFNK_CUDA(cudaGetLastError());
+  return JFNK_OK;
+}
+
+}  // namespace jfnk

@@ -256,8 +256,8 @@ __global__ void __launch_bounds__(kFusedThreads) k_formal_fused(const ColDesc* _
 int fused_prepare(Batch* b) {
   if (b->formal_qb <= 0) return JFNK_OK;
   if (b->formal_threads <= 0) b->formal_threads = kFusedThreads;
-  const size_t bytes = fused_smem_bytes(b->formal_qb, b->max_nz, b->max_nmu, b->mixed != 0);
-  JFNK_CUDA(cudaFuncSetAttribute(k_formal_fused<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
+  // the attribute is the kernel's, not this batch's: always the largest size
+  JFNK_CUDA(cudaFuncSetAttribute(k_formal_fused<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
   return JFNK_OK;
 }
 
@@ -291,7 +291,6 @@ int fused_autotune(Batch* b, cudaStream_t s) {
     const int nray = qb * 2 * b->max_nmu;
     for (int threads : {64, 128, 256}) {
       if (threads < nray) continue;
-      JFNK_CUDA(cudaFuncSetAttribute(k_formal_fused<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
       int rc = launch_fused_cfg(*b, s, qb, threads);   // warm-up
       if (rc) return rc;
       JFNK_CUDA(cudaEventRecord(e0, s));

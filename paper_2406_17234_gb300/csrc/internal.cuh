@@ -99,7 +99,8 @@ int build_atmosphere(jfnk_ctx* ctx, int lane, const AtomData& A, const jfnk_atmo
 
 // Formal-solution kernels: per-ray buffers + ray-sum kernel (any size),
 // in-block fused kernel (FP64), per-frequency sweep kernel (mixed precision).
-enum FormalKind { FORMAL_UNFUSED = 0, FORMAL_FUSED = 1, FORMAL_SWEEP = 2, FORMAL_MOVING = 3 };
+// whole evaluation per frequency tile with cached coefficients (FP64).
+enum FormalKind { FORMAL_UNFUSED = 0, FORMAL_FUSED = 1, FORMAL_SWEEP = 2, FORMAL_MOVING = 3, FORMAL_CACHED = 4 };
 
 // A batch of columns with their work buffers, resident on the device.
 struct Batch {
@@ -118,8 +119,8 @@ struct Batch {
   cudaGraphExec_t graph = nullptr;    // captured tick sequence
   int graph_ticks = 0;
   bool graph_profiled = false;
-  int formal_kind = 0;                // FORMAL_UNFUSED, FORMAL_FUSED or FORMAL_SWEEP
-  int formal_qb = 0;                  // frequencies per block of the fused formal kernel
+  int formal_kind = 0;                // FormalKind
+  int formal_qb = 0;                  // frequencies per block of the fused and cached formal kernels
   int formal_threads = 0;             // fused: threads per block; sweep: threads (variant 1) or warps (2)
   int sweep_variant = 0;              // sweep kernel: 1 thread per frequency, 2 warp per frequency pair
   int sweep_fuse = 0;                 // thread variant: the tangent sweep forms the opacity tangent itself
@@ -130,6 +131,9 @@ struct Batch {
                                                           // replace it for a solve)
   int max_overlap = 0;                // most transitions active at one frequency over the batch
   int n_sm = 1;                       // multiprocessors of the batch's device
+  int max_tiles = 0;                  // cached FP64 evaluation: most tiles of a column of the view
+  int eval_mu = 0;                    // ... the angle count shared by every column (0: several)
+  size_t eval_smem = 0;               // ... and its blocks' dynamic shared memory
   bool tuned = false;                 // autotuner has run on this batch
   int graph_kernels = 0;              // kernel nodes in the captured tick graph
   long replays = 0;                   // graph replays of the last solve
@@ -156,8 +160,9 @@ struct Batch {
 // Work buffers of one column: bytes of its block (256-byte aligned parts), and
 // the descriptor of a column whose block starts at ``base``.
 struct ColLayout;
-size_t column_bytes(const AtmosData& M, int kind, int mixed, int kmax, ColLayout* out);
-void column_bind(char* base, const AtmosData& M, int kind, int mixed, int kmax, SolverState* st, ColDesc* d);
+// qb: frequencies per tile of the cached kind.
+size_t column_bytes(const AtmosData& M, int kind, int mixed, int kmax, ColLayout* out, int qb = 0);
+void column_bind(char* base, const AtmosData& M, int kind, int mixed, int kmax, SolverState* st, ColDesc* d, int qb = 0);
 
 // Allocates work buffers for columns ``tabs`` (precision: mixed or FP64).
 int batch_create(Batch* b, const std::vector<const AtmosData*>& cols, int mixed, int kmax);
@@ -182,6 +187,15 @@ int fused_default_qb(int max_nz, int max_nmu, bool mixed);
 int fused_prepare(Batch* b);
 int launch_formal_fused(const Batch& b, cudaStream_t s);
 int fused_autotune(Batch* b, cudaStream_t s);
+// Cached FP64 evaluation (formal_cached.cu).
+int cached_default_qb(int nq, int nz, int nmu, int nl, int n_sm);
+size_t cached_smem_bytes(int qb, int nz, int nmu, int nl);
+size_t cached_planes(int qb, int nz, int nq, int nmu);
+size_t cached_parts(int qb, int nz, int nl, int nwin, int nt);
+constexpr int kEvalThreads = 512;   // threads per block of the cached evaluation
+int cached_prepare();
+int launch_eval64(const Batch& b, cudaStream_t s);
+int launch_rates_reduce(const Batch& b, cudaStream_t s);
 // Per-frequency sweep kernel of the mixed mode (formal_sweep.cu).
 size_t sweep_scratch_bytes(int nq, int nz);
 int sweep_prepare(Batch* b);

@@ -974,7 +974,7 @@ int prepare_kernels() {
   const int max_smem = (int)((size_t)kRateWarps * 32 * ((2 + kRhFixed + kMaxT) * sizeof(double) +
                                                        std::max(kMaxT, kMaxL) * sizeof(float)));
   JFNK_CUDA(cudaFuncSetAttribute(k_rates, cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem));
-  return JFNK_OK;
+  return cached_prepare();
 }
 
 static int launch_rates(const Batch& b, cudaStream_t s) {
@@ -1309,6 +1309,19 @@ int launch_evaluation(const Batch& b, cudaStream_t s, cudaEvent_t ev0, cudaEvent
     return JFNK_OK;
   }
   if (int rm = mark(0)) return rm;
+  if (b.formal_kind == FORMAL_CACHED) {
+    // opacity, formal solution and the tiles' rate integrals in one kernel
+    if (ev0) JFNK_CUDA(cudaEventRecordWithFlags(ev0, s, cudaEventRecordExternal));
+    int rc = launch_eval64(b, s);
+    if (rc) return rc;
+    if (ev1) JFNK_CUDA(cudaEventRecordWithFlags(ev1, s, cudaEventRecordExternal));
+    if ((rc = launch_rates_reduce(b, s))) return rc;
+    launch_dJdn_update(b, s);
+    if ((rc = mark(1))) return rc;
+    launch_assemble(b, s);
+    JFNK_CUDA(cudaGetLastError());
+    return mark(2);
+  }
   if (b.formal_kind == FORMAL_MOVING) {
     // per-ray opacity, formal solution and rate integrals (velocity.cu), then
     // the common assembly

@@ -507,7 +507,7 @@ int build_atmosphere(jfnk_ctx* ctx, int lane, const AtomData& A, const jfnk_atmo
   size_t o_qmeta = ar.take<int>((size_t)kQMetaT * nq), o_qtr = ar.take<int>((size_t)kQMetaT * nq);
   size_t o_W2 = ar.take<float2>(nwin), o_c2p = ar.take<float2>(nq), o_rc2p = ar.take<float2>(nq);
   size_t o_linc = ar.take<int>((size_t)nl * (nt + 1));
-  size_t o_ang32 = ar.take<float4>(nmu), o_dz32 = ar.take<float2>(nz - 1);
+  size_t o_ang64 = ar.take<Ang64>(nmu), o_ang32 = ar.take<float4>(nmu), o_dz32 = ar.take<float2>(nz - 1);
   size_t o_vlos = ar.take<double>(M->moving ? nz : 0);
   const size_t host_prefix = ar.cursor;
   size_t o_V = ar.take<double>((size_t)nwin * nz), o_G = ar.take<double>((size_t)nwin * nz);
@@ -625,6 +625,9 @@ int build_atmosphere(jfnk_ctx* ctx, int lane, const AtomData& A, const jfnk_atmo
   JFNK_CUDA(up(o_linc, linc.data(), linc.size() * 4));
   // the sweep kernels' per-angle and per-layer constants, rounded once from FP64
   std::vector<float4> ang32(nmu);
+  std::vector<Ang64> ang64(nmu);
+  for (int m = 0; m < nmu; ++m) ang64[m] = Ang64{0.5 / mu[m], 0.5 * wmu[m], 2.0 * mu[m], 0.0};
+  JFNK_CUDA(up(o_ang64, ang64.data(), nmu * sizeof(Ang64)));
   for (int m = 0; m < nmu; ++m)
     ang32[m] = make_float4((float)(0.5 / mu[m]), (float)(0.5 * wmu[m]), (float)(2.0 * mu[m]), 0.f);
   std::vector<float2> dz32(nz - 1);
@@ -715,6 +718,7 @@ int build_atmosphere(jfnk_ctx* ctx, int lane, const AtomData& A, const jfnk_atmo
   tb_.qtr = ar.ptr<int>(o_qtr);
   tb_.lvl_inc = ar.ptr<int>(o_linc);
   tb_.mu = ar.ptr<double>(o_mu); tb_.wmu = ar.ptr<double>(o_wmu);
+  tb_.ang64 = ar.ptr<Ang64>(o_ang64);
   tb_.ang32 = ar.ptr<float4>(o_ang32); tb_.dz32 = ar.ptr<float2>(o_dz32);
   tb_.Vd = M->moving ? ar.ptr<double>(o_Vd) : nullptr;
   tb_.chi_c = ar.ptr<double>(o_chic); tb_.eta_c = ar.ptr<double>(o_etac);

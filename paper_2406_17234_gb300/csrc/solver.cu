@@ -37,22 +37,22 @@ void DeviceArena::release() {
 struct ColLayout {
   size_t n, v, v32, chiT, S32T, dSkT, dchiT, dS32T, dJ32T, Jdag, Jnew, istar, chi, S, dSk, dchi, dS, ddSk, H, HI, dH,
       LX, LE, part, J, dJ, Lchi, Leta, Lchi32, Leta32, Rup, Rdn, dRup, dRdn, Apart, rh, F, dF, P, piv, Iem, Vb, Hh, cs, sn, gv, x,
-      w, nprev, np, fdp, eta, etab32, n2, mchi, mS, mdchi, mdS, mI, mdI, mLX, mLE;
+      w, nprev, np, fdp, eta, etab32, n2, mchi, mS, mdchi, mdS, mI, mdI, mLX, mLE, cf, rpart;
 };
 
-size_t column_bytes(const AtmosData& M, int kind, int mixed, int kmax, ColLayout* out) {
+size_t column_bytes(const AtmosData& M, int kind, int mixed, int kmax, ColLayout* out, int qb) {
   DeviceArena ar;   // used as a cursor only
   ColLayout o{};
   const size_t rs = mixed ? sizeof(float) : sizeof(double);
   const size_t nz = M.nz, nq = M.nq, nl = M.nl, nt = M.nt, nmu = M.nmu, N = nz * nl;
   const bool per_ray = (kind == FORMAL_UNFUSED);   // unfused kernels need per-ray buffers
-  const bool sweep = (kind == FORMAL_SWEEP);
+  const bool sweep = (kind == FORMAL_SWEEP), cached = (kind == FORMAL_CACHED);
   o.n = ar.take<double>(N); o.v = ar.take<double>(N);
   o.Jdag = ar.take<double>(nq * nz); o.Jnew = ar.take<double>(nq * nz);
   o.istar = ar.take<int>(nz);
   o.chi = ar.take<char>(rs * nq * nz); o.S = ar.take<double>(nq * nz);
   o.dSk = ar.take<char>(per_ray ? rs * nq * nz : 0);
-  o.dchi = ar.take<char>(sweep ? 0 : rs * nq * nz); o.dS = ar.take<double>(sweep ? 0 : nq * nz);
+  o.dchi = ar.take<char>(sweep || cached ? 0 : rs * nq * nz); o.dS = ar.take<double>(sweep || cached ? 0 : nq * nz);
   const size_t TQ = sweep ? (size_t)nz * col_pitch((int)nq) : 0;
   o.v32 = ar.take<float>(sweep ? N : 0);
   o.chiT = ar.take<float>(TQ); o.S32T = ar.take<float>(TQ); o.dSkT = ar.take<float>(TQ);
@@ -62,7 +62,7 @@ size_t column_bytes(const AtmosData& M, int kind, int mixed, int kmax, ColLayout
   o.H = ar.take<char>(pr); o.dH = ar.take<char>(pr); o.HI = ar.take<char>(pr);
   o.LX = ar.take<char>(pr); o.LE = ar.take<char>(pr);
   o.part = ar.take<char>(sweep ? sweep_scratch_bytes((int)nq, (int)nz) : 0);
-  o.J = ar.take<double>(nq * nz); o.dJ = ar.take<double>(sweep ? 0 : nq * nz);
+  o.J = ar.take<double>(cached ? 0 : nq * nz); o.dJ = ar.take<double>(sweep || cached ? 0 : nq * nz);
   o.Lchi = ar.take<double>(sweep ? 0 : nq * nz); o.Leta = ar.take<double>(sweep ? 0 : nq * nz);
   o.Lchi32 = ar.take<float>(sweep ? nq * nz : 0); o.Leta32 = ar.take<float>(sweep ? nq * nz : 0);
   o.Rup = ar.take<double>(nt * nz); o.Rdn = ar.take<double>(nt * nz);
@@ -83,13 +83,15 @@ size_t column_bytes(const AtmosData& M, int kind, int mixed, int kmax, ColLayout
   o.mchi = ar.take<double>(MR); o.mS = ar.take<double>(MR); o.mdchi = ar.take<double>(MR);
   o.mdS = ar.take<double>(MR); o.mI = ar.take<double>(MR); o.mdI = ar.take<double>(MR);
   o.mLX = ar.take<double>(MR); o.mLE = ar.take<double>(MR);
+  o.cf = ar.take<double>(cached ? cached_planes(qb, M.nz, M.nq, M.nmu) : 0);
+  o.rpart = ar.take<double>(cached ? cached_parts(qb, M.nz, M.nl, M.nwin, M.nt) : 0);
   if (out) *out = o;
   return ar.cursor;
 }
 
-void column_bind(char* base, const AtmosData& M, int kind, int mixed, int kmax, SolverState* st, ColDesc* d) {
+void column_bind(char* base, const AtmosData& M, int kind, int mixed, int kmax, SolverState* st, ColDesc* d, int qb) {
   ColLayout o;
-  column_bytes(M, kind, mixed, kmax, &o);
+  column_bytes(M, kind, mixed, kmax, &o, qb);
   auto P = [&](size_t off) { return static_cast<void*>(base + off); };
   const bool sweep = (kind == FORMAL_SWEEP);
   d->t = M.tables;
@@ -132,8 +134,15 @@ void column_bind(char* base, const AtmosData& M, int kind, int mixed, int kmax, 
     w.mdS = (double*)P(o.mdS); w.mI = (double*)P(o.mI); w.mdI = (double*)P(o.mdI);
     w.mLX = (double*)P(o.mLX); w.mLE = (double*)P(o.mLE);
   }
+  if (kind == FORMAL_CACHED) {
+    w.cf = (double*)P(o.cf); w.rpart = (double*)P(o.rpart); w.cq = qb;
+  }
   w.st = st;
 }
+
+// Largest total of the cached FP64 coefficients of a batch (a 4,096-column
+// batch keeps the memory it had).
+constexpr size_t kCachedBytes = (size_t)24 << 30;
 
 int batch_create(Batch* b, const std::vector<const AtmosData*>& cols, int mixed, int kmax) {
   const int nc = (int)cols.size();
@@ -163,19 +172,44 @@ int batch_create(Batch* b, const std::vector<const AtmosData*>& cols, int mixed,
     JFNK_CUDA(cudaGetDevice(&dev));
     JFNK_CUDA(cudaDeviceGetAttribute(&b->n_sm, cudaDevAttrMultiProcessorCount, dev));
   }
-  b->formal_qb = mixed || moving ? 0 : fused_default_qb(b->max_nz, b->max_nmu, false);
-  b->formal_kind = moving ? FORMAL_MOVING
-                          : (mixed ? FORMAL_SWEEP : (b->formal_qb > 0 ? FORMAL_FUSED : FORMAL_UNFUSED));
+  // FP64 static columns: the cached evaluation, unless its coefficient planes
+  // (40 bytes per ray-point pair) of the whole batch would exceed kCachedBytes
+  // or the device has no room for them; then the fused kernel, which keeps none
+  bool cached = !mixed && !moving;
+  size_t planes = 0;
+  std::vector<int> qc(nc, 0);
+  for (int c = 0; c < nc && cached; ++c) {
+    const AtmosData& M = *cols[c];
+    qc[c] = cached_default_qb(M.nq, M.nz, M.nmu, M.nl, b->n_sm);
+    cached = qc[c] > 0 && (planes += cached_planes(qc[c], M.nz, M.nq, M.nmu) * sizeof(double)) <= kCachedBytes;
+    if (!cached) break;
+    b->eval_mu = c == 0 || b->eval_mu == M.nmu ? M.nmu : 0;
+    b->max_tiles = std::max(b->max_tiles, (M.nq + qc[c] - 1) / qc[c]);
+    b->eval_smem = std::max(b->eval_smem, cached_smem_bytes(qc[c], M.nz, M.nmu, M.nl));
+  }
   std::vector<size_t> off(nc);
-  for (int c = 0; c < nc; ++c)
-    off[c] = ar.take<char>(column_bytes(*cols[c], b->formal_kind, mixed, kmax, nullptr));
-  size_t o_cols = ar.take<ColDesc>(nc);
-  size_t o_state = ar.take<SolverState>(nc);
-  size_t o_status = ar.take<int>(nc);
-  size_t o_opts = ar.take<SolverOpts>(1);
-  size_t o_view = ar.take<ColDesc>(nc);
-  int rc = ar.allocate();
-  if (rc) return rc;
+  size_t o_cols = 0, o_state = 0, o_status = 0, o_opts = 0, o_view = 0;
+  for (;;) {
+    b->formal_qb = cached ? qc[0] : (mixed || moving ? 0 : fused_default_qb(b->max_nz, b->max_nmu, false));
+    b->formal_threads = cached ? kEvalThreads : 0;
+    b->formal_kind = cached   ? FORMAL_CACHED
+                     : moving ? FORMAL_MOVING
+                     : mixed  ? FORMAL_SWEEP
+                              : (b->formal_qb > 0 ? FORMAL_FUSED : FORMAL_UNFUSED);
+    ar.reset();
+    for (int c = 0; c < nc; ++c)
+      off[c] = ar.take<char>(column_bytes(*cols[c], b->formal_kind, mixed, kmax, nullptr, qc[c]));
+    o_cols = ar.take<ColDesc>(nc);
+    o_state = ar.take<SolverState>(nc);
+    o_status = ar.take<int>(nc);
+    o_opts = ar.take<SolverOpts>(1);
+    o_view = ar.take<ColDesc>(nc);
+    const int rc = ar.allocate();
+    if (!rc) break;
+    if (!cached) return rc;
+    cudaGetLastError();   // no room for the planes: the fused kernel
+    cached = false;
+  }
   b->h_cols.resize(nc);
   b->d_cols = ar.ptr<ColDesc>(o_cols);
   b->d_state = ar.ptr<SolverState>(o_state);
@@ -183,11 +217,11 @@ int batch_create(Batch* b, const std::vector<const AtmosData*>& cols, int mixed,
   b->d_opts = ar.ptr<SolverOpts>(o_opts);
   b->d_view = ar.ptr<ColDesc>(o_view);
   for (int c = 0; c < nc; ++c)
-    column_bind(ar.base + off[c], *cols[c], b->formal_kind, mixed, kmax, b->d_state + c, &b->h_cols[c]);
+    column_bind(ar.base + off[c], *cols[c], b->formal_kind, mixed, kmax, b->d_state + c, &b->h_cols[c], qc[c]);
   JFNK_CUDA(cudaMemcpy(b->d_cols, b->h_cols.data(), nc * sizeof(ColDesc), cudaMemcpyHostToDevice));
   JFNK_CUDA(cudaMemset(b->d_state, 0, nc * sizeof(SolverState)));
   if (b->formal_kind == FORMAL_SWEEP) return sweep_prepare(b);
-  if (b->formal_kind == FORMAL_MOVING) return JFNK_OK;
+  if (b->formal_kind == FORMAL_MOVING || b->formal_kind == FORMAL_CACHED) return JFNK_OK;
   return fused_prepare(b);
 }
 
@@ -283,7 +317,11 @@ __device__ double rh92_depth(const ColDesc& cd, int k, bool clamp, bool correcti
     for (int j = 0; j < nl; ++j) coef[j] = 0.0;
     coef[lo] += r[0] + C[lo * nl + up];
     coef[up] -= r[1] + r[2] + C[up * nl + lo];
-    for (int s = 0; s < nt; ++s) coef[T.t_up[s]] += r[kRhFixed + s];
+    if (cd.w.cf) {   // already added per level
+      for (int j = 0; j < nl; ++j) coef[j] += r[kRhFixed + j];
+    } else {
+      for (int s = 0; s < nt; ++s) coef[T.t_up[s]] += r[kRhFixed + s];
+    }
     for (int j = 0; j < nl; ++j) {
       M[lo * nl + j] += coef[j];
       M[up * nl + j] -= coef[j];

@@ -303,7 +303,7 @@ static int run_to_completion(Batch* b, const jfnk_options* o, cudaStream_t s) {
       // a few columns: one thread per frequency leaves most SMs idle, and the
       // warp-per-frequency-pair sweep (same results) finishes each tick sooner
       if (b->formal_kind == FORMAL_SWEEP && b->sweep_variant == 1 &&
-          (long)b->ncols * b->max_nq < 256L * b->n_sm && sweep_warp_size(b->max_nz) > 0) {
+          sweep_small(b->ncols, b->max_nq, b->n_sm) && sweep_warp_size(b->max_nz) > 0) {
         b->sweep_variant = 2;
         b->formal_threads = sweep_warp_size(b->max_nz);
       }

@@ -95,7 +95,8 @@ struct ColTables {
                           // t << 1 | (1 if the level is the upper one), -1 after the last
   const int* qmeta;       // [kQMetaT][nq] transitions active at nu_q, packed as
                           // window point << 8 | lo << 4 | up; -1 past the last
-  const int* qtr;         // [kQMetaT][nq] the same transitions' indices t
+  const int4* qmeta4;     // [nq][2] the same eight entries of a frequency side by side
+  const uint2* qtr8;      // [nq] the same transitions' indices t, one byte each (0xff past the last)
   const double* dz;       // [nz-1] |z_k - z_{k+1}|
   const double* mu;       // [nmu]
   const double* wmu;      // [nmu]

@@ -88,6 +88,85 @@ __device__ __forceinline__ void tan_acc(TanAcc& t, float V, float g, float vlo, 
   t.dchi = fma3(V, sub(vlo, mul(g, vup)), t.dchi);
   t.deta = fma3(mul(g, V), vup, t.deta);
 }
+// Opacity and source function at (nu, k) of a mixed-mode base or RH92
+// evaluation (Eqs. chi, eta): chi is stored in float, S (and the RH92
+// emissivity) as float pairs; every sum runs in pair arithmetic on the FP32
+// pipe (GB300's FP64 pipe is 1/64 of it): chi = chi_c + chi_sca + sum V n_lo -
+// sum g V n_up, eta / (2 h nu^3/c^2) = (eta_c + chi_sca J^dagger) c^2/(2 h nu^3)
+// + sum g V n_up; i = q nz + k.
+struct BasePoint {
+  float chi;
+  df S;
+};
+// EARLY: the loads of the first three transitions are issued together (small
+// launches, bound by latency; a large one is faster with fewer registers).
+template <bool EARLY>
+__device__ __forceinline__ BasePoint base_opacity(const ColDesc& cd, int mode, int q, int k, int i) {
+  const ColTables& T = cd.t;
+  const int nz = T.nz;
+  const float2* n2 = cd.w.n2 + k * T.nl;
+  const df jd = df_load(as_pairs(jdag_ptr(cd)), i);
+  const df eta_bg = df_add(df_load(T.etac2, i), df_mul(df_load(T.chisca2, k), jd));
+  df chl = df_make(0.f, 0.f), el = df_make(0.f, 0.f);
+  if (EARLY && T.max_overlap <= kQMetaT) {
+    constexpr int E = 3;
+    const int4 a = __ldg(T.qmeta4 + 2 * (size_t)q), b = __ldg(T.qmeta4 + 2 * (size_t)q + 1);
+    const int ms[kQMetaT] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+    df V[E], gV[E], nl_[E], nu_[E];
+#pragma unroll
+    for (int j = 0; j < E; ++j) {
+      const int m = max(ms[j], 0);
+      const size_t p = (size_t)(m >> 8) * nz + k;
+      V[j] = df_load(T.V2, p);
+      gV[j] = df_load(T.gV2, p);
+      nl_[j] = df_load(n2, (m >> 4) & 15);
+      nu_[j] = df_load(n2, m & 15);
+    }
+#pragma unroll
+    for (int j = 0; j < kQMetaT; ++j) {
+      const int m = ms[j];
+      if (m < 0) break;
+      if (j < E) {
+        chl = df_add(chl, df_mul(V[j], nl_[j]));
+        el = df_add(el, df_mul(gV[j], nu_[j]));
+      } else {
+        const size_t p = (size_t)(m >> 8) * nz + k;
+        chl = df_add(chl, df_mul(df_load(T.V2, p), df_load(n2, (m >> 4) & 15)));
+        el = df_add(el, df_mul(df_load(T.gV2, p), df_load(n2, m & 15)));
+      }
+    }
+  } else if (T.max_overlap <= kQMetaT) {
+    // the packed table gives window point and levels in one load
+#pragma unroll
+    for (int j = 0; j < kQMetaT; ++j) {
+      const int m = __ldg(T.qmeta + (size_t)j * T.nq + q);
+      if (m < 0) break;
+      const size_t p = (size_t)(m >> 8) * nz + k;
+      chl = df_add(chl, df_mul(df_load(T.V2, p), df_load(n2, (m >> 4) & 15)));
+      el = df_add(el, df_mul(df_load(T.gV2, p), df_load(n2, m & 15)));
+    }
+  } else {
+    for (int s = T.q_off[q]; s < T.q_off[q + 1]; ++s) {
+      const int t = T.q_t[s];
+      const size_t p = (size_t)(T.t_base[t] + q - T.t_q0[t]) * nz + k;
+      chl = df_add(chl, df_mul(df_load(T.V2, p), df_load(n2, T.t_lo[t])));
+      el = df_add(el, df_mul(df_load(T.gV2, p), df_load(n2, T.t_up[t])));
+    }
+  }
+  const df chi = df_sub(df_add(df_load(T.chibg2, i), chl), el);
+  const df etan = df_add(df_mul(eta_bg, df_load(T.rc2p, q)), el);
+  BasePoint p;
+  p.chi = chi.hi;
+  p.S = df_div(etan, chi);
+  reinterpret_cast<float*>(cd.w.chi)[i] = p.chi;
+  df_store(as_pairs(cd.w.S), i, p.S);
+  if (mode == EV_RH92) {   // for the RH92 rate sums
+    df_store(as_pairs(cd.w.eta), i, df_add(eta_bg, df_mul(el, df_load(T.c2p, q))));
+    cd.w.etab32[i] = eta_bg.hi;
+  }
+  return p;
+}
+
 // Hardware reciprocal (1 ulp): a single instruction without a slow-path
 // branch, so that loops around it stay one basic block the compiler can
 // software-pipeline. Its arguments (opacity sums) are positive normal numbers.

@@ -69,12 +69,21 @@ __host__ __device__ inline size_t ring_floats(int threads) { return (size_t)kRin
 // Which form of the coefficients a step takes: chosen per step (CM_EITHER),
 // or known for every angle of the depth (CM_SERIES: all steps below 0.1;
 // CM_DIRECT: none), the same choice as CM_EITHER makes for each step.
-enum CoefMode { CM_EITHER = 0, CM_SERIES = 1, CM_DIRECT = 2 };
+// CM_SELECT forms both and selects: no branch, for launches bound by latency.
+enum CoefMode { CM_EITHER = 0, CM_SERIES = 1, CM_DIRECT = 2, CM_SELECT = 3 };
 
 template <int CM = CM_EITHER>
 __device__ __forceinline__ void pl_coef_rn(float x, float r, float& e, float& w, float& a, float& bq) {
   e = exp_neg(x);
-  if (CM == CM_SERIES || (CM == CM_EITHER && x < 0.1f)) {
+  if (CM == CM_SELECT) {
+    float es, ws, as, bs, ed, wd, ad, bd;
+    pl_coef_rn<CM_SERIES>(x, r, es, ws, as, bs);
+    pl_coef_rn<CM_DIRECT>(x, r, ed, wd, ad, bd);
+    const bool thin = x < 0.1f;
+    w = thin ? ws : wd;
+    a = thin ? as : ad;
+    bq = thin ? bs : bd;
+  } else if (CM == CM_SERIES || (CM == CM_EITHER && x < 0.1f)) {
     w = fma3(fma3(fma3(fma3(fma3(-1.0f / 720.0f, x, 1.0f / 120.0f), x, -1.0f / 24.0f), x, 1.0f / 6.0f), x, -0.5f), x, 1.0f);
     a = mul(x, fma3(fma3(fma3(fma3(fma3(-1.0f / 5040.0f, x, 1.0f / 720.0f), x, -1.0f / 120.0f), x, 1.0f / 24.0f), x, -1.0f / 6.0f), x, 0.5f));
     bq = fma3(fma3(fma3(fma3(1.0f / 144.0f, x, -1.0f / 30.0f), x, 1.0f / 8.0f), x, -1.0f / 3.0f), x, 0.5f);
@@ -116,34 +125,61 @@ struct RayOut {
 // better-conditioned value: D carries an absolute error of the order of the
 // largest |D| met upstream (attenuated along the ray), I - S one of the order
 // of |I| + |S|.
+// The part of a step that depends on the opacities only (RayCoef) and the
+// recurrence itself are separate, so that the warp variant can form the
+// coefficients of several depths before it steps through them.
+struct RayCoef {
+  float e;        // exp(-dtau)
+  float X;        // w (S^u - S^k)
+  float Y;        // tangent: bq (S^u - S^k)          | base: bq
+  float Z;        // tangent: w (dS^u - dS^k)         | base: a S^k + b S^u
+  float t;        // tangent: ddtau                   | base: h
+  float sa, xe;   // base: (S^k/chi^k) factor a and 1/2 w_mu a/chi^k
+};
 template <bool TAN, int CM = CM_EITHER>
-__device__ __forceinline__ RayOut ray_step(const StepIn& in, float inv2mu, float two_mu, float hw, float& D,
-                                           float& I, float& M, float& dD) {
-  RayOut o;
+__device__ __forceinline__ RayCoef ray_coef(const StepIn& in, float inv2mu, float two_mu, float hw) {
+  RayCoef c;
   // the depth's factors are formed once per depth (StepIn), one multiply per angle here
   const float dtau = mul(in.tz, inv2mu);
   const float rdt = mul(in.rz, two_mu);
-  float e, w, a, bq;
-  pl_coef_rn<CM>(dtau, rdt, e, w, a, bq);
-  const float Du = D;
-  float Dn = fma3(Du, e, mul(w, in.dSin));
+  float w, a, bq;
+  pl_coef_rn<CM>(dtau, rdt, c.e, w, a, bq);
+  c.X = mul(w, in.dSin);
   if (TAN) {
-    const float ddtau = mul(in.dtz, inv2mu);
-    const float dDn = fma3(dD, e, fma3(-ddtau, fma3(e, Du, mul(bq, in.dSin)), mul(w, in.ddSin)));
+    c.t = mul(in.dtz, inv2mu);
+    c.Y = mul(bq, in.dSin);
+    c.Z = mul(w, in.ddSin);
+    c.sa = c.xe = 0.f;
+  } else {
+    c.t = mul(in.dzk, inv2mu);
+    c.Y = bq;
+    c.Z = fma3(a, in.S0, mul(mul(bq, dtau), in.Su));
+    c.sa = a;
+    c.xe = mul(hw, mul(a, in.rc0));
+  }
+  return c;
+}
+template <bool TAN>
+__device__ __forceinline__ RayOut ray_apply(const RayCoef& c, float dSin, float S0, float rc0, float hw, float& D,
+                                            float& I, float& M, float& dD) {
+  RayOut o;
+  const float Du = D;
+  float Dn = fma3(Du, c.e, c.X);
+  if (TAN) {
+    const float dDn = fma3(dD, c.e, fma3(-c.t, fma3(c.e, Du, c.Y), c.Z));
     dD = dDn;
     o.xd = mul(hw, dDn);
     o.xD = o.xI = o.xx = o.xe = 0.f;
   } else {
-    const float h = mul(in.dzk, inv2mu);
-    const float In = fma3(I, e, fma3(a, in.S0, mul(mul(bq, dtau), in.Su)));
-    const float lx = -fma3(mul(in.S0, in.rc0), a, mul(h, fma3(in.dSin, bq, mul(e, Du))));
+    const float In = fma3(I, c.e, c.Z);
+    const float lx = -fma3(mul(S0, rc0), c.sa, mul(c.t, fma3(dSin, c.Y, mul(c.e, Du))));
     o.xI = mul(hw, In);
     o.xx = mul(hw, lx);
-    o.xe = mul(hw, mul(a, in.rc0));
-    M = fmaxf(mul(M, e), fabsf(Dn));
-    const float anchor = add(fabsf(In), fabsf(in.S0));
+    o.xe = c.xe;
+    M = fmaxf(mul(M, c.e), fabsf(Dn));
+    const float anchor = add(fabsf(In), fabsf(S0));
     if (anchor < M) {
-      Dn = sub(In, in.S0);
+      Dn = sub(In, S0);
       M = anchor;
     }
     I = In;
@@ -152,6 +188,12 @@ __device__ __forceinline__ RayOut ray_step(const StepIn& in, float inv2mu, float
   }
   D = Dn;
   return o;
+}
+template <bool TAN, int CM = CM_EITHER>
+__device__ __forceinline__ RayOut ray_step(const StepIn& in, float inv2mu, float two_mu, float hw, float& D,
+                                           float& I, float& M, float& dD) {
+  const RayCoef c = ray_coef<TAN, CM>(in, inv2mu, two_mu, hw);
+  return ray_apply<TAN>(c, in.dSin, in.S0, in.rc0, hw, D, I, M, dD);
 }
 
 // Sum of the angle contributions in the fixed tree of a 3-level xor butterfly
@@ -174,13 +216,6 @@ __device__ __forceinline__ float tree_mu(const float* x) {
   const Part s = padd(padd(padd(p[0], p[4]), padd(p[2], p[6])), padd(padd(p[1], p[5]), padd(p[3], p[7])));
   return s.on ? s.v : 0.f;
 }
-__device__ __forceinline__ float butterfly8(float v) {
-  v = add(v, __shfl_xor_sync(0xffffffffu, v, 4));
-  v = add(v, __shfl_xor_sync(0xffffffffu, v, 2));
-  v = add(v, __shfl_xor_sync(0xffffffffu, v, 1));
-  return v;
-}
-
 // Output of one depth from the two hemisphere sums (base: D, |D|, I, Lchi, Leta).
 // J = (S + sum D) c2, or (sum I) c2 where that representation carries the
 // smaller rounding error (intensities are >= 0), is formed in pair arithmetic
@@ -617,197 +652,290 @@ __global__ void __launch_bounds__(kFusedThreads, 7) k_formal_sweep_fused(const C
 // ---------------------------------------------------------------------------
 // Variant 2 (small launches): one warp per two frequencies; lane = (frequency
 // of the pair, hemisphere, angle), so both hemispheres advance together and
-// every lane runs one ray. A hemisphere's sums come from an xor butterfly
-// over its 8 angle lanes (the tree of tree8), land in shared memory per
-// depth, and the 16 lanes of a frequency then combine the two hemispheres
-// depth by depth (coalesced output rows).
+// every lane runs one ray. A hemisphere's sums are those of an xor butterfly
+// over its 8 angle lanes (the tree of tree_mu), every kWarpChunk depths from
+// the lanes' rows in shared memory.
+//
+// A small launch is bound by latency: one trip to L2 per depth was most of it.
+// A 233-depth, 2,010-frequency column: base evaluation 288 + 15 us (thread
+// variant and its opacity kernel) -> 66, tangent 221 + 29 -> 39 us; 82 depths:
+// base 83 + 6 -> 25 us. So
+// a block first stages every depth of its frequencies in shared memory, all
+// loads in flight at once, and forms the opacity there: the separate opacity
+// kernels (6 to 28 us at these sizes, too few threads in flight) are not
+// launched, and the recurrence then reads shared memory only. It has about one
+// warp per scheduler, so its steps are straight code: the coefficients of
+// kWarpAhead depths are formed before the steps through them, both their forms
+// and a selection instead of a branch, and no shuffles.
 // ---------------------------------------------------------------------------
-constexpr int kWarpParts = kSweepParts;
+constexpr int kWarpAhead = 4;    // depths whose coefficients are formed together
+constexpr int kWarpStage2 = 2;   // warps that stage per warp that sweeps
+constexpr int kWarpChunk = 16;   // depths between two sums over the angle lanes
+static_assert(kWarpChunk % kWarpAhead == 0, "a chunk is whole groups");
 
-__host__ __device__ inline size_t warp_variant_smem(int nz, int warps) {
-  return sizeof(float) * (2 * (size_t)nz + (size_t)warps * 2 * 2 * kWarpParts * nz);
+__host__ __device__ inline int warp_parts(bool tan) { return tan ? 1 : kSweepParts; }
+// rows of a chunk: one word per lane of dD, or of D, I, dI/dchi, dI/deta, padded by a bank
+__host__ __device__ inline int warp_lanes_row(bool tan) { return (tan ? 1 : 4) * 32 + 1; }
+__host__ __device__ inline int warp_row(int nz) { return nz | 1; }   // odd: lanes on different frequencies, different banks
+
+__host__ __device__ inline size_t warp_variant_smem(int nz, int warps, bool tan) {
+  return sizeof(float) * (2 * (size_t)nz + (size_t)warps * (2 * 4 * (size_t)warp_row(nz) + 2 * warp_parts(tan) * (size_t)nz +
+                                                                 kWarpChunk * warp_lanes_row(tan)));
+}
+
+// Stage of a tangent block: chi, S^{k+1} - S^k, dchi, dS of its frequencies at
+// every depth ([array][frequency][depth]); dchi and dS as k_opacity_tan32
+// forms them (tan_acc, tan_dS: the same bits).
+__device__ __forceinline__ void stage_tan(const ColDesc& cd, int qb, int F, float* __restrict__ st, int row) {
+  const ColTables& T = cd.t;
+  const int nz = T.nz, nq = T.nq, nl = T.nl, nwin = T.nwin;
+  const int f = threadIdx.x % F, q = qb + f;
+  if (q >= nq) return;
+  const size_t pitch = (size_t)col_pitch(nq);
+  const double* __restrict__ dir = cd.forced_mode >= 0 ? cd.w.v
+                                   : cd.w.st->phase == PH_RESTART ? cd.w.x
+                                                                  : cd.w.Vb + (size_t)cd.w.st->j * nz * nl;
+  const int m0 = __ldg(T.qmeta + q), m1 = __ldg(T.qmeta + (size_t)nq + q);
+  float* o = st + (size_t)f * row;
+  const size_t plane = (size_t)F * row;
+  const int ks = blockDim.x / F;
+#pragma unroll 4
+  for (int k = threadIdx.x / F; k < nz; k += ks) {
+    const size_t i = (size_t)k * pitch + q;
+    const float S = cd.w.S32T[i], c = cd.w.chiT[i];
+    const float dSk = k < nz - 1 ? cd.w.dSkT[i] : 0.f;
+    const float2* __restrict__ VG = T.VG32T + (size_t)k * nwin;
+    const double* __restrict__ v = dir + (size_t)k * nl;
+    float2 a0 = make_float2(0.f, 0.f), a1 = a0;
+    float l0 = 0.f, u0 = 0.f, l1 = 0.f, u1 = 0.f;
+    if (m0 >= 0) {
+      a0 = __ldg(VG + (m0 >> 8));
+      l0 = (float)v[(m0 >> 4) & 15];
+      u0 = (float)v[m0 & 15];
+    }
+    if (m1 >= 0) {
+      a1 = __ldg(VG + (m1 >> 8));
+      l1 = (float)v[(m1 >> 4) & 15];
+      u1 = (float)v[m1 & 15];
+    }
+    TanAcc ta;
+    if (m0 >= 0) tan_acc(ta, a0.x, a0.y, l0, u0);
+    if (m1 >= 0) {
+      tan_acc(ta, a1.x, a1.y, l1, u1);
+      for (int j = 2; j < kQMetaT; ++j) {
+        const int m = __ldg(T.qmeta + (size_t)j * nq + q);
+        if (m < 0) break;
+        const float2 a = __ldg(VG + (m >> 8));
+        tan_acc(ta, a.x, a.y, (float)v[(m >> 4) & 15], (float)v[m & 15]);
+      }
+      if (T.max_overlap > kQMetaT)
+        for (int s = T.q_off[q] + kQMetaT; s < T.q_off[q + 1]; ++s) {
+          const int t = T.q_t[s];
+          const float2 a = __ldg(VG + T.t_base[t] + q - T.t_q0[t]);
+          tan_acc(ta, a.x, a.y, (float)v[T.t_lo[t]], (float)v[T.t_up[t]]);
+        }
+    }
+    o[k] = c;
+    o[plane + k] = dSk;
+    o[2 * plane + k] = ta.dchi;
+    o[3 * plane + k] = tan_dS(ta, S, c);
+  }
+}
+
+// Stage of a base-type block: chi, S^{k+1} - S^k (formed from the pairs, then
+// rounded), S as a pair; and the arrays the tangents of the Newton step read.
+__device__ __forceinline__ void stage_base(const ColDesc& cd, int mode, int qb, int F, float* __restrict__ st,
+                                           int row) {
+  const ColTables& T = cd.t;
+  const int nz = T.nz, nq = T.nq;
+  const int nf = min(F, nq - qb);
+  const size_t plane = (size_t)F * row, pitch = (size_t)col_pitch(nq);
+  for (int i = threadIdx.x; i < nf * nz; i += blockDim.x) {
+    const int f = i / nz, k = i - f * nz;
+    const BasePoint p = base_opacity<true>(cd, mode, qb + f, k, (qb + f) * nz + k);
+    float* o = st + (size_t)f * row + k;
+    o[0] = p.chi;
+    o[2 * plane] = p.S.hi;
+    o[3 * plane] = p.S.lo;
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < nf * nz; i += blockDim.x) {
+    const int k = i / nf, f = i - k * nf;
+    float* o = st + (size_t)f * row + k;
+    const size_t g = (size_t)k * pitch + qb + f;
+    cd.w.chiT[g] = o[0];
+    cd.w.S32T[g] = o[2 * plane];
+    if (k < nz - 1) {
+      const df a = df_make(o[2 * plane], o[3 * plane]), b = df_make(o[2 * plane + 1], o[3 * plane + 1]);
+      const float d = -df_to_float(df_sub(a, b));   // S^{k+1} - S^k
+      o[plane] = d;
+      cd.w.dSkT[g] = d;
+    }
+  }
 }
 
 template <bool TAN>
-__device__ __forceinline__ void sweep_warp(const ColDesc& cd, int q, float* __restrict__ wp,
-                                           const float* __restrict__ s_dz, const float* __restrict__ s_idz) {
+__device__ __forceinline__ void sweep_warp(const ColDesc& cd, int q, int fl, const float* __restrict__ st, int row,
+                                           size_t plane, float* __restrict__ wp, const float* __restrict__ s_dz,
+                                           const float* __restrict__ s_idz) {
   const ColTables& T = cd.t;
   const int nz = T.nz, nq = T.nq, nmu = T.nmu;
   const int lane = threadIdx.x & 31;
   const int qi = lane >> 4, hemi = (lane >> 3) & 1, m = lane & 7;
-  const int leader = lane & ~7;
   const bool up = hemi == 1;
   const bool valid = q < nq;
   const int qq = valid ? q : nq - 1;
-  const size_t row = (size_t)qq * nz;
-  const size_t pitch = (size_t)col_pitch(nq);
-  const float* __restrict__ chi = reinterpret_cast<const float*>(cd.w.chi) + row;
-  const float2* __restrict__ S2 = as_pairs(cd.w.S) + row;   // S as float pairs
-  float* __restrict__ chiT = cd.w.chiT + qq;
-  float* __restrict__ S32T = cd.w.S32T + qq;
-  float* __restrict__ dSkT = cd.w.dSkT + qq;
-  const float* __restrict__ dchiT = cd.w.dchiT + qq;
-  const float* __restrict__ dS32T = cd.w.dS32T + qq;
+  constexpr int NP = TAN ? 1 : kSweepParts;
+  const float* __restrict__ in = st + (size_t)(valid ? fl : 0) * row;   // this frequency's staged rows
   const double c2 = T.c2[qq];
-  const float c2f = T.c2f[qq];
-  const df c2p = df_load(T.c2p, qq);
-  const bool on = m < nmu;
-  const float4 ang = on ? T.ang32[m] : make_float4(0.f, 0.f, 0.f, 0.f);
+  // lanes past the last angle run with zero weight (their sums add zeros)
+  const float4 ang = m < nmu ? T.ang32[m] : make_float4(0.f, 0.f, 0.f, 0.f);
   const float inv2mu = ang.x;
   const float hw = ang.y;
   const float two_mu = ang.z;
-  float* hp = wp + (size_t)(qi * 2 + hemi) * kWarpParts * nz;   // this hemisphere's sums [v][k]
-  const bool writer = !TAN && !up && m == 0 && valid;           // depth-major copies
-  auto tan_in = [&](int kk, float& dc, float& dS) {
-    const size_t o = (size_t)kk * pitch;
-    dc = dchiT[o];
-    dS = dS32T[o];
-  };
+  constexpr int LR = (TAN ? 1 : 4) * 32 + 1;
+  float* lanes = wp + (size_t)2 * NP * nz;   // [kWarpChunk][LR]; wp: [2][NP][nz]
 
   const int k0 = up ? nz - 1 : 0;
-  df Sp = df_load(S2, k0);
-  float cp = TAN ? chiT[k0 * pitch] : chi[k0];
-  float dSp = 0.f, dcp = 0.f;
-  if (TAN) tan_in(k0, dcp, dSp);
-  float Su = Sp.hi;
-  if (writer) {
-    chiT[0] = cp;
-    S32T[0] = Su;
-  }
-  const double Ib64 = up ? T.Bn[row + nz - 1] / c2 : 0.0;
-  const float D0 = df_to_float(df_sub(df_from_double(Ib64), Sp));
+  const df Sb = TAN ? df_load(as_pairs(cd.w.S), (size_t)qq * nz + k0) : df_make(in[2 * plane + k0], in[3 * plane + k0]);
+  const double Ib64 = up ? T.Bn[(size_t)qq * nz + nz - 1] / c2 : 0.0;
+  const float D0 = df_to_float(df_sub(df_from_double(Ib64), Sb));
   const float I0 = __double2float_rn(Ib64);
-  const float dD0 = -dSp;
+  const float dD0 = TAN ? -in[3 * plane + k0] : -0.f;
   float D = D0, I = I0, M = fabsf(D0), dD = dD0;
-  RayOut r;
-  r.xD = on ? mul(hw, D0) : 0.f;
-  r.xI = on ? mul(hw, I0) : 0.f;
-  r.xx = r.xe = 0.f;
-  r.xd = on ? mul(hw, dD0) : 0.f;
-  auto store = [&](int k) {
+  // row r of the chunk: the boundary depth is the first chunk's row 0
+  auto put = [&](int r, const RayOut& x) {
+    float* o = lanes + r * LR + lane;
     if (TAN) {
-      const float td = butterfly8(r.xd);
-      if (m == 0) hp[k] = td;
+      o[0] = x.xd;
     } else {
-      const float tD = butterfly8(r.xD), ta = butterfly8(fabsf(r.xD)), tI = butterfly8(r.xI);
-      const float tx = butterfly8(r.xx), te = butterfly8(r.xe);
-      if (m == 0) {
-        hp[k] = tD;
-        hp[nz + k] = ta;
-        hp[2 * nz + k] = tI;
-        hp[3 * nz + k] = tx;
-        hp[4 * nz + k] = te;
+      o[0] = x.xD;
+      o[32] = x.xI;
+      o[64] = x.xx;
+      o[96] = x.xe;
+    }
+  };
+  {
+    RayOut r;
+    r.xD = mul(hw, D0);
+    r.xI = mul(hw, I0);
+    r.xx = r.xe = 0.f;
+    r.xd = mul(hw, dD0);
+    put(0, r);
+  }
+  for (int c0 = 0; c0 < nz; c0 += kWarpChunk) {
+    const int c1 = min(c0 + kWarpChunk, nz);
+    for (int s0 = max(c0, 1); s0 < c1; s0 = (s0 & ~(kWarpAhead - 1)) + kWarpAhead) {
+      RayCoef c[kWarpAhead];
+      float dSin[kWarpAhead], S0[kWarpAhead], rc0[kWarpAhead];
+      const int se = min((s0 & ~(kWarpAhead - 1)) + kWarpAhead, c1);   // steps s0 .. se - 1
+#pragma unroll
+      for (int u = 0; u < kWarpAhead; ++u) {
+        const int s = min(s0 + u, nz - 1);
+        const int k = up ? nz - 1 - s : s, ku = up ? k + 1 : k - 1, kd = up ? k : k - 1;
+        StepIn x;
+        const float cc = in[k];
+        const float dSl = in[plane + kd];
+        x.csum = add(cc, in[ku]);
+        x.rs = rcp_approx(x.csum);
+        x.dzk = s_dz[kd];
+        x.idzk = s_idz[kd];
+        x.tz = mul(x.dzk, x.csum);
+        x.rz = mul(x.rs, x.idzk);
+        x.dSin = up ? dSl : -dSl;
+        if (TAN) {
+          x.dcs = add(in[2 * plane + k], in[2 * plane + ku]);
+          x.dtz = mul(x.dzk, x.dcs);
+          x.ddSin = sub(in[3 * plane + ku], in[3 * plane + k]);
+          x.S0 = x.Su = x.rc0 = 0.f;
+        } else {
+          x.S0 = in[2 * plane + k];
+          x.Su = in[2 * plane + ku];
+          x.rc0 = rcp_approx(cc);
+          x.dcs = x.dtz = x.ddSin = 0.f;
+        }
+        c[u] = ray_coef<TAN, CM_SELECT>(x, inv2mu, two_mu, hw);
+        dSin[u] = x.dSin;
+        S0[u] = x.S0;
+        rc0[u] = x.rc0;
       }
+#pragma unroll
+      for (int u = 0; u < kWarpAhead; ++u)
+        if (s0 + u < se) put(s0 + u - c0, ray_apply<TAN>(c[u], dSin[u], S0[u], rc0[u], hw, D, I, M, dD));
     }
-  };
-  store(k0);
-  // the next depth's inputs are loaded one step ahead (latency off the chain)
-  float c_n = 0.f, dc_n = 0.f, dS_n = 0.f, dSl_n = 0.f;
-  df S_n = df_make(0.f, 0.f);
-  auto load = [&](int s) {
-    const int k = up ? nz - 1 - s : s;
-    const int kd = up ? k : k - 1;
-    if (TAN) {
-      c_n = chiT[(size_t)k * pitch];
-      tan_in(k, dc_n, dS_n);
-      dSl_n = dSkT[(size_t)kd * pitch];
-    } else {
-      c_n = chi[k];
-      if (m == 0) S_n = df_load(S2, k);
-    }
-  };
-  if (nz > 1) load(1);
-  for (int s = 1; s < nz; ++s) {
-    const int k = up ? nz - 1 - s : s;
-    const int kd = up ? k : k - 1;
-    StepIn in;
-    const float c0 = c_n;
-    float dc0 = 0.f, dS0 = 0.f;
-    const float dSl = dSl_n;
-    const df Sk = S_n;
-    if (TAN) {
-      dc0 = dc_n;
-      dS0 = dS_n;
-    }
-    if (s + 1 < nz) load(s + 1);
-    if (TAN) {
-      in.dSin = up ? dSl : -dSl;
-      in.S0 = in.Su = in.rc0 = 0.f;
-      in.dcs = add(dc0, dcp);
-      in.ddSin = sub(dSp, dS0);
-    } else {
-      // the pair difference is formed once per hemisphere (angle lane 0)
-      float dSin = 0.f, S0 = 0.f;
-      if (m == 0) {
-        dSin = df_to_float(df_sub(Sp, Sk));
-        S0 = Sk.hi;
-        Sp = Sk;
-        if (writer) {
-          chiT[(size_t)k * pitch] = c0;
-          S32T[(size_t)k * pitch] = S0;
-          dSkT[(size_t)kd * pitch] = -dSin;   // S^{k} - S^{k-1}
+    __syncwarp();
+    // the hemispheres' sums of the chunk's depths: row r of group (frequency,
+    // hemisphere). The hemisphere that reaches a depth first leaves its sums in
+    // wp, the other one adds its own and writes the depth's output (a middle
+    // depth is reached by both in one row); first the rows of the first kind.
+    const size_t pitch = (size_t)col_pitch(nq);
+    for (int pass = 0; pass < 2; ++pass) {
+      for (int i = lane; i < (c1 - c0) * 4; i += 32) {
+        const int g = i & 3, r = i >> 2, s = c0 + r, o = nz - 1 - s, fq = q - qi + (g >> 1);
+        if ((s < o) != (pass == 0) || (s == o && (g & 1)) || fq >= nq) continue;
+        const int k = (g & 1) ? o : s;
+        const float* x = lanes + r * LR + g * 8;
+        float* h = wp + (size_t)(g >> 1) * NP * nz + k;
+        float v[NP];
+        auto sums = [&](const float* y) {
+          v[0] = tree_mu<8>(y);
+          if (!TAN) {
+            float ax[8];
+#pragma unroll
+            for (int j = 0; j < 8; ++j) ax[j] = fabsf(y[j]);
+            v[1] = tree_mu<8>(ax);
+            v[2] = tree_mu<8>(y + 32);
+            v[3] = tree_mu<8>(y + 64);
+            v[4] = tree_mu<8>(y + 96);
+          }
+        };
+        sums(x);
+        if (s < o) {
+#pragma unroll
+          for (int j = 0; j < NP; ++j) h[(size_t)j * nz] = v[j];
+          continue;
+        }
+        float w[NP];
+#pragma unroll
+        for (int j = 0; j < NP; ++j) w[j] = s > o ? h[(size_t)j * nz] : v[j];
+        if (s == o) sums(x + 8);   // the other hemisphere's lanes
+        const float* fi = st + (size_t)(fl - qi + (g >> 1)) * row;
+        if (TAN) {
+          write_tan(cd, (size_t)k * pitch + fq, fi[3 * plane + k], add(v[0], w[0]));
+        } else {
+          write_base(cd, (size_t)fq * nz + k, df_make(fi[2 * plane + k], fi[3 * plane + k]), df_load(T.c2p, fq),
+                     T.c2f[fq], add(v[0], w[0]), add(v[1], w[1]), add(v[2], w[2]), add(v[3], w[3]), add(v[4], w[4]));
         }
       }
-      in.dSin = __shfl_sync(0xffffffffu, dSin, leader);
-      in.S0 = __shfl_sync(0xffffffffu, S0, leader);
-      in.Su = Su;
-      in.rc0 = rcp_approx(c0);
-      in.dcs = in.ddSin = 0.f;
-    }
-    in.csum = add(c0, cp);
-    in.rs = rcp_approx(in.csum);
-    in.dzk = s_dz[kd];
-    in.idzk = s_idz[kd];
-    in.tz = mul(in.dzk, in.csum);
-    in.rz = mul(in.rs, in.idzk);
-    in.dtz = TAN ? mul(in.dzk, in.dcs) : 0.f;
-    if (on) {
-      r = ray_step<TAN>(in, inv2mu, two_mu, hw, D, I, M, dD);
-    } else {
-      r.xD = r.xI = r.xx = r.xe = r.xd = 0.f;
-    }
-    store(k);
-    Su = in.S0;
-    cp = c0;
-    dcp = dc0;
-    dSp = dS0;
-  }
-  if (up && on && valid && !TAN) cd.w.Iem[(size_t)q * nmu + m] = __dmul_rn((double)I, c2);
-  __syncwarp();
-  if (!valid) return;
-  // combine the hemispheres of frequency q, depths strided over its 16 lanes
-  const float* dn = wp + (size_t)(qi * 2 + 0) * kWarpParts * nz;
-  const float* upp = wp + (size_t)(qi * 2 + 1) * kWarpParts * nz;
-  for (int k = lane & 15; k < nz; k += 16) {
-    if (TAN) {
-      const size_t o = (size_t)k * pitch + q;
-      write_tan(cd, o, cd.w.dS32T[o], add(upp[k], dn[k]));
-    } else {
-      write_base(cd, row + k, df_load(S2, k), c2p, c2f, add(upp[k], dn[k]), add(upp[nz + k], dn[nz + k]),
-                 add(upp[2 * nz + k], dn[2 * nz + k]), add(upp[3 * nz + k], dn[3 * nz + k]),
-                 add(upp[4 * nz + k], dn[4 * nz + k]));
+      __syncwarp();
     }
   }
+  if (up && m < nmu && valid && !TAN) cd.w.Iem[(size_t)q * nmu + m] = __dmul_rn((double)I, c2);
 }
 
-__global__ void __launch_bounds__(256) k_formal_sweep_warp(const ColDesc* __restrict__ cols, int which) {
-  extern __shared__ float s_tab[];   // [nz] |dz|, [nz] 1/|dz|, per warp [2][2][parts][nz]
+template <bool TAN>
+__global__ void __launch_bounds__(128 * kWarpStage2) k_formal_sweep_warp(const ColDesc* __restrict__ cols) {
+  extern __shared__ float s_tab[];   // [nz] |dz|, [nz] 1/|dz|, staged rows [4][F][row], per warp [2][parts][nz] and a chunk
   const ColDesc& cd = cols[blockIdx.y];
   const int mode = eval_mode_f(cd);
-  if (mode == EV_SKIP || (which == 1 && mode == EV_TANGENT) || (which == 2 && mode != EV_TANGENT)) return;
+  if (mode == EV_SKIP || (mode == EV_TANGENT) != TAN) return;
   const ColTables& T = cd.t;
   const int nz = T.nz, nq = T.nq;
-  const int warps = blockDim.x >> 5;
-  if ((int)blockIdx.x * warps * 2 >= nq) return;   // uniform over the block
+  const int warps = blockDim.x / (32 * kWarpStage2), F = 2 * warps, qb = blockIdx.x * F;
+  if (qb >= nq) return;   // uniform over the block
   float* s_dz = s_tab;
   float* s_idz = s_tab + nz;
+  float* st = s_idz + nz;
+  const int row = warp_row(nz);
+  const size_t plane = (size_t)F * row;
   stage_dz(T, s_dz, s_idz);
+  if (TAN) stage_tan(cd, qb, F, st, row);
+  else stage_base(cd, mode, qb, F, st, row);
   __syncthreads();
-  const int wid = threadIdx.x >> 5;
-  float* wp = s_tab + 2 * nz + (size_t)wid * 2 * 2 * kWarpParts * nz;
-  const int q = ((int)blockIdx.x * warps + wid) * 2 + ((threadIdx.x & 31) >> 4);
-  if (mode == EV_TANGENT) sweep_warp<true>(cd, q, wp, s_dz, s_idz);
-  else sweep_warp<false>(cd, q, wp, s_dz, s_idz);
+  const int wid = threadIdx.x >> 5, fl = wid * 2 + ((threadIdx.x & 31) >> 4);
+  if (wid >= warps) return;   // these warps only stage
+  float* wp = st + 4 * plane + (size_t)wid * (2 * warp_parts(TAN) * nz + kWarpChunk * warp_lanes_row(TAN));
+  sweep_warp<TAN>(cd, qb + fl, fl, st, row, plane, wp, s_dz, s_idz);
 }
 
 // Angle counts with their own instantiation; a launch uses the smallest one
@@ -854,6 +982,14 @@ static int allow_smem_mu() {
   return JFNK_OK;
 }
 
+// Warps per block of the warp variant: the most whose shared memory lets three
+// blocks share a multiprocessor, else one warp (0: a column too deep for it).
+static int warp_size(int nz, bool tan) {
+  for (int w : {4, 2})
+    if (warp_variant_smem(nz, w, tan) <= (size_t)75 * 1024) return w;
+  return warp_variant_smem(nz, 1, tan) <= (size_t)227 * 1024 ? 1 : 0;
+}
+
 // variant 1: ``size`` threads per block, at most occ_tan / occ_base blocks per
 // SM (0: no cap); variant 2: ``size`` warps per block; which: 0 every column,
 // 1 base-type evaluations, 2 tangent ones
@@ -862,9 +998,16 @@ static int launch_sweep_cfg(const Batch& b, cudaStream_t s, int variant, int siz
   if (fuse && (variant != 1 || size != kFusedThreads))
     return fail(JFNK_E_INVALID, "fused tangent sweep: thread variant with 128-thread blocks only");
   if (variant == 2) {
-    const int fpb = 2 * size;   // frequencies per block
-    dim3 g((b.max_nq + fpb - 1) / fpb, b.ncols);
-    k_formal_sweep_warp<<<g, 32 * size, warp_variant_smem(b.max_nz, size), s>>>(b.d_cols, which);
+    // two frequencies per warp; the warps per block follow from the depth
+    auto grid = [&](int w) { return dim3((b.max_nq + 2 * w - 1) / (2 * w), b.ncols); };
+    if (which != 1) {
+      const int w = warp_size(b.max_nz, true);
+      k_formal_sweep_warp<true><<<grid(w), 32 * w * kWarpStage2, warp_variant_smem(b.max_nz, w, true), s>>>(b.d_cols);
+    }
+    if (which != 2) {
+      const int w = warp_size(b.max_nz, false);
+      k_formal_sweep_warp<false><<<grid(w), 32 * w * kWarpStage2, warp_variant_smem(b.max_nz, w, false), s>>>(b.d_cols);
+    }
   } else {
     switch (sweep_mu_class(b.max_nmu)) {
       case 2: launch_mu<2>(b, s, size, which, occ_tan, occ_base, fuse); break;
@@ -878,18 +1021,21 @@ static int launch_sweep_cfg(const Batch& b, cudaStream_t s, int variant, int siz
   return JFNK_OK;
 }
 
-static bool warp_variant_fits(int nz, int warps) {
-  return warp_variant_smem(nz, warps) <= (size_t)227 * 1024;
-}
-
 int sweep_prepare(Batch* b) {
-  const size_t bytes = warp_variant_smem(b->max_nz, 8);
-  JFNK_CUDA(cudaFuncSetAttribute(k_formal_sweep_warp, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)std::min(bytes, (size_t)227 * 1024)));
+  // the attribute is the kernel's, not this batch's: always the largest size
+  JFNK_CUDA(cudaFuncSetAttribute(k_formal_sweep_warp<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
+  JFNK_CUDA(cudaFuncSetAttribute(k_formal_sweep_warp<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
   int rc;
   if ((rc = allow_smem_mu<2>()) || (rc = allow_smem_mu<3>()) || (rc = allow_smem_mu<4>()) ||
       (rc = allow_smem_mu<5>()) || (rc = allow_smem_mu<8>()))
     return rc;
+  if (b->sweep_variant == 0 && sweep_small(b->ncols, b->max_nq, b->n_sm) && sweep_warp_size(b->max_nz) > 0) {
+    // nothing to tune: the variant's shape follows from the depth
+    b->sweep_variant = b->tuned_variant = 2;
+    b->formal_threads = b->tuned_size = sweep_warp_size(b->max_nz);
+    b->optan_depths = 16;   // the separate opacity kernel's default, should a forced variant launch it
+    b->tuned = true;
+  }
   if (b->sweep_variant == 0) {
     b->sweep_variant = 1;
     b->formal_threads = 128;
@@ -904,11 +1050,11 @@ int launch_formal_sweep(const Batch& b, cudaStream_t s, int which) {
                           which, b.sweep_occ, b.sweep_occ_base, sweep_fused(b) ? b.sweep_fuse : 0);
 }
 
-int sweep_warp_size(int nz) {
-  for (int w : {4, 2, 1})
-    if (warp_variant_fits(nz, w)) return w;
-  return 0;
-}
+// Launches of fewer frequencies than these (256 per multiprocessor) take the
+// warp variant: one thread per frequency would leave most warp slots empty.
+bool sweep_small(int ncols, int max_nq, int n_sm) { return (long)ncols * max_nq < 256L * n_sm; }
+
+int sweep_warp_size(int nz) { return std::min(warp_size(nz, true), warp_size(nz, false)); }
 
 // Autotuner of the sweep kernels, timed on the batch's own columns: the
 // tangent sweep (the columns in tangent mode) over variant 1 with 32..256
@@ -924,7 +1070,7 @@ int sweep_autotune(Batch* b, cudaStream_t s) {
   int rc = JFNK_OK;
   // a tangent candidate without fusion is timed with the separate opacity-tangent launch it needs
   auto once = [&](int variant, int size, int which, int ot, int ob, int fuse) -> int {
-    if (which == 2 && !fuse) {
+    if (which == 2 && !fuse && variant != 2) {
       int r = launch_opacity_tan(*b, s);
       if (r) return r;
     }
@@ -987,7 +1133,6 @@ int sweep_autotune(Batch* b, cudaStream_t s) {
   std::vector<Cand> cands;
   for (int t : {32, 64, 128, 256})
     for (int occ : {0, 2, 4, 8}) cands.push_back({1, t, occ, 0});
-  for (int w : {1, 2, 4, 8}) cands.push_back({2, w, 0, 0});
   // the default (128 threads, no cap) stays unless a candidate beats it by 2 %:
   // closer than that, single measurements flip between runs
   float best = 1e30f;
@@ -996,7 +1141,6 @@ int sweep_autotune(Batch* b, cudaStream_t s) {
   best *= 0.98f;
   for (const auto& c : cands) {
     if (rc) break;
-    if (c.variant == 2 && !warp_variant_fits(b->max_nz, c.size)) continue;
     if (c.variant == 1 && c.occ > 0 && c.size * c.occ > 2048) continue;
     if (c.variant == 1 && c.size == 128 && c.occ == 0) continue;
     float ms = 0.f;

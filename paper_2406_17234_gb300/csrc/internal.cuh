@@ -134,6 +134,7 @@ struct Batch {
   int max_tiles = 0;                  // cached FP64 evaluation: most tiles of a column of the view
   int eval_mu = 0;                    // ... the angle count shared by every column (0: several)
   size_t eval_smem = 0;               // ... and its blocks' dynamic shared memory
+  int forced = -1;                    // evaluation kind forced on every column (-1: each its own)
   bool tuned = false;                 // autotuner has run on this batch
   int graph_kernels = 0;              // kernel nodes in the captured tick graph
   long replays = 0;                   // graph replays of the last solve
@@ -209,6 +210,8 @@ bool sweep_fused(const Batch& b);
 int launch_opacity_tan(const Batch& b, cudaStream_t s, int depths = 0);
 // Warps per block of the warp variant whose shared memory fits depth nz (0: none).
 int sweep_warp_size(int nz);
+// Few frequencies in flight: the warp variant.
+bool sweep_small(int ncols, int max_nq, int n_sm);
 int sweep_autotune(Batch* b, cudaStream_t s);
 // Mixed mode: converts the J^dagger of columns d_cols[0, ncols) (FP64, as
 // filled by the host or the tables) to float pairs in place (to_pairs), or
@@ -220,8 +223,6 @@ int launch_j_pairs(const ColDesc* d_cols, int ncols, size_t max_qz, cudaStream_t
 int launch_moving_evaluation(const Batch& b, cudaStream_t s, cudaEvent_t ev0 = nullptr, cudaEvent_t ev1 = nullptr);
 // Kernel attributes of the current device, set once per context (residual.cu).
 int prepare_kernels();
-// Opacity kernel of the mixed mode (tangent columns skipped when the sweeps form it).
-int launch_opacity_mixed(const Batch& b, cudaStream_t s, int skip_tangent);
 // Solver options: checks, device copy (api.cu).
 int validate_options(const jfnk_options* o);
 void options_to_device(const jfnk_options* o, SolverOpts* so);

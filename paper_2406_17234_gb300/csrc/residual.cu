@@ -101,41 +101,7 @@ __device__ __forceinline__ void opacity_point(const ColDesc& cd, int mode, int i
   }
   const int q = i / nz, k = i - q * nz;
   if (sizeof(real) == sizeof(float)) {
-    // mixed mode: chi is stored in float, S (and the RH92 emissivity) as
-    // float pairs; every sum runs in pair arithmetic on the FP32 pipe (GB300's
-    // FP64 pipe is 1/64 of it): chi = chi_c + chi_sca + sum V n_lo - sum g V
-    // n_up, eta / (2 h nu^3/c^2) = (eta_c + chi_sca J^dagger) c^2/(2 h nu^3)
-    // + sum g V n_up (Eqs. chi, eta)
-    const float2* n2 = cd.w.n2 + k * nl;
-    const df jd = df_load(as_pairs(jdag_ptr(cd)), i);
-    const df eta_bg = df_add(df_load(T.etac2, i), df_mul(df_load(T.chisca2, k), jd));
-    df chl = df_make(0.f, 0.f), el = df_make(0.f, 0.f);
-    if (T.max_overlap <= kQMetaT) {
-      // the packed table gives window point and levels in one load
-#pragma unroll
-      for (int j = 0; j < kQMetaT; ++j) {
-        const int m = __ldg(T.qmeta + (size_t)j * T.nq + q);
-        if (m < 0) break;
-        const size_t p = (size_t)(m >> 8) * nz + k;
-        chl = df_add(chl, df_mul(df_load(T.V2, p), df_load(n2, (m >> 4) & 15)));
-        el = df_add(el, df_mul(df_load(T.gV2, p), df_load(n2, m & 15)));
-      }
-    } else {
-      for (int s = T.q_off[q]; s < T.q_off[q + 1]; ++s) {
-        const int t = T.q_t[s];
-        const size_t p = (size_t)(T.t_base[t] + q - T.t_q0[t]) * nz + k;
-        chl = df_add(chl, df_mul(df_load(T.V2, p), df_load(n2, T.t_lo[t])));
-        el = df_add(el, df_mul(df_load(T.gV2, p), df_load(n2, T.t_up[t])));
-      }
-    }
-    const df chi = df_sub(df_add(df_load(T.chibg2, i), chl), el);
-    const df etan = df_add(df_mul(eta_bg, df_load(T.rc2p, q)), el);
-    reinterpret_cast<float*>(cd.w.chi)[i] = chi.hi;
-    df_store(as_pairs(cd.w.S), i, df_div(etan, chi));
-    if (mode == EV_RH92) {   // for the RH92 rate sums
-      df_store(as_pairs(cd.w.eta), i, df_add(eta_bg, df_mul(el, df_load(T.c2p, q))));
-      cd.w.etab32[i] = eta_bg.hi;
-    }
+    base_opacity<false>(cd, mode, q, k, i);
     return;
   }
   const double* n = eval_pops(cd, mode) + k * nl;
@@ -274,15 +240,18 @@ __global__ void __launch_bounds__(256, 6) k_opacity_tan32(const ColDesc* __restr
 // (transition, depth): lanes stride over the transition's frequency window
 // (coalesced rows of the depth-major tables) and a fixed xor-butterfly adds
 // the lanes, so the sums are bit-reproducible.
+// DEPTHS depths per warp (independent sums in flight): 4 in large launches, 1 in
+// small ones, which are bound by the trips to memory along a window; there the
+// loads of four window strides are issued together.
 constexpr int kRateTanWarps = 8;
-constexpr int kRateTanDepths = 4;   // depths per warp (independent sums in flight)
+template <int DEPTHS>
 __global__ void __launch_bounds__(32 * kRateTanWarps) k_rates_tan32(const ColDesc* __restrict__ cols) {
   const ColDesc& cd = cols[blockIdx.z];
   if (!cd.mixed || eval_mode(cd) != EV_TANGENT) return;
   const ColTables& T = cd.t;
   const int t = blockIdx.y;
-  // warp w of the block takes depths k0 + w + d * kRateTanWarps, d < kRateTanDepths
-  const int k0 = blockIdx.x * kRateTanWarps * kRateTanDepths + (threadIdx.x >> 5);
+  // warp w of the block takes depths k0 + w + d * kRateTanWarps, d < DEPTHS
+  const int k0 = blockIdx.x * kRateTanWarps * DEPTHS + (threadIdx.x >> 5);
   if (t >= T.nt || k0 >= T.nz) return;   // whole warps
   const int lane = threadIdx.x & 31;
   const int nz = T.nz, nwin = T.nwin;
@@ -291,13 +260,35 @@ __global__ void __launch_bounds__(32 * kRateTanWarps) k_rates_tan32(const ColDes
   const float2* __restrict__ VG = T.VG32T + base - q0;
   const float* __restrict__ W32 = T.W32 + base - q0;
   const float* __restrict__ dJ = cd.w.dJ32T;
-  float a0[kRateTanDepths], a1[kRateTanDepths];
+  float a0[DEPTHS], a1[DEPTHS];
 #pragma unroll
-  for (int d = 0; d < kRateTanDepths; ++d) a0[d] = a1[d] = 0.f;
-  for (int q = q0 + lane; q <= q1; q += 32) {
+  for (int d = 0; d < DEPTHS; ++d) a0[d] = a1[d] = 0.f;
+  int q = q0 + lane;
+  if (DEPTHS == 1) {
+    constexpr int U = 4;
+    const float2* __restrict__ vgk = VG + (size_t)k0 * nwin;
+    const float* __restrict__ dJk = dJ + (size_t)k0 * pitch;
+    for (; q + 32 * (U - 1) <= q1; q += 32 * U) {
+      float W[U], x[U];
+      float2 vg[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        W[u] = __ldg(W32 + q + 32 * u);
+        vg[u] = __ldg(vgk + q + 32 * u);
+        x[u] = __ldg(dJk + q + 32 * u);
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const float WV = W[u] * vg[u].x;
+        a0[0] = fmaf(WV, x[u], a0[0]);
+        a1[0] = fmaf(WV * vg[u].y, x[u], a1[0]);
+      }
+    }
+  }
+  for (; q <= q1; q += 32) {
     const float W = __ldg(W32 + q);
 #pragma unroll
-    for (int d = 0; d < kRateTanDepths; ++d) {
+    for (int d = 0; d < DEPTHS; ++d) {
       const int k = k0 + d * kRateTanWarps;
       if (k < nz) {
         const float2 vg = __ldg(VG + (size_t)k * nwin + q);
@@ -309,7 +300,7 @@ __global__ void __launch_bounds__(32 * kRateTanWarps) k_rates_tan32(const ColDes
     }
   }
 #pragma unroll
-  for (int d = 0; d < kRateTanDepths; ++d) {
+  for (int d = 0; d < DEPTHS; ++d) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
       a0[d] += __shfl_xor_sync(0xffffffffu, a0[d], o);
@@ -605,6 +596,61 @@ __device__ __forceinline__ int rate_mode(const ColDesc& cd, int t, int tile) {
   return mode;
 }
 
+// The packed transitions active at a frequency (ColTables::qmeta4). PIPE
+// (small launches, few warps on a multiprocessor): the whole list is loaded
+// two frequencies before its use, since a list and then the tables it points
+// to would be two trips to memory in a row, and the terms of its first three
+// transitions with the frequency's other inputs; 168 registers. Otherwise
+// (large launches, which need the warps more) two transitions and 128
+// registers; the 512-column batch was 3 % slower with the former.
+// H I-like column, 82 x 2,010: 59 -> 30 us for a base evaluation.
+struct RateList {
+  int m[kQMetaT];
+};
+template <bool PIPE>
+__device__ __forceinline__ RateList rate_list(const ColTables& T, bool packed, int q) {
+  RateList L;
+  if (PIPE) {
+    const int4 a = packed ? __ldg(T.qmeta4 + 2 * (size_t)q) : make_int4(-1, -1, -1, -1);
+    const int4 b = packed ? __ldg(T.qmeta4 + 2 * (size_t)q + 1) : make_int4(-1, -1, -1, -1);
+    L.m[0] = a.x; L.m[1] = a.y; L.m[2] = a.z; L.m[3] = a.w;
+    L.m[4] = b.x; L.m[5] = b.y; L.m[6] = b.z; L.m[7] = b.w;
+  } else {
+    L.m[0] = packed ? __ldg(T.qmeta + q) : -1;
+    L.m[1] = packed ? __ldg(T.qmeta + (size_t)T.nq + q) : -1;
+  }
+  return L;
+}
+// A warp's frequencies q, q + kRateWarps, ... <= qb of its chunk, in order, two
+// at a time loaded, then summed.
+template <bool PIPE, typename Ld, typename Use>
+__device__ __forceinline__ void rate_window(const ColTables& T, bool packed, int q, int qb, Ld ld, Use use) {
+  if (q > qb) return;
+  if (PIPE) {
+    RateList n0 = rate_list<PIPE>(T, packed, q), n1 = rate_list<PIPE>(T, packed, min(q + kRateWarps, qb));
+    for (; q + kRateWarps <= qb; q += 2 * kRateWarps) {
+      const RateList l0 = n0, l1 = n1;
+      const auto r0 = ld(q, l0), r1 = ld(q + kRateWarps, l1);
+      n0 = rate_list<PIPE>(T, packed, min(q + 2 * kRateWarps, qb));
+      n1 = rate_list<PIPE>(T, packed, min(q + 3 * kRateWarps, qb));
+      use(q, l0, r0);
+      use(q + kRateWarps, l1, r1);
+    }
+    if (q <= qb) use(q, n0, ld(q, n0));
+  } else {
+    for (; q + kRateWarps <= qb; q += 2 * kRateWarps) {
+      const RateList l0 = rate_list<PIPE>(T, packed, q), l1 = rate_list<PIPE>(T, packed, q + kRateWarps);
+      const auto r0 = ld(q, l0), r1 = ld(q + kRateWarps, l1);
+      use(q, l0, r0);
+      use(q + kRateWarps, l1, r1);
+    }
+    if (q <= qb) {
+      const RateList l0 = rate_list<PIPE>(T, packed, q);
+      use(q, l0, ld(q, l0));
+    }
+  }
+}
+
 // One (32-depth tile, transition t, column): lanes map to depths (every table
 // and J access is coalesced), the ``split`` blocks of the cluster split the
 // frequency window into contiguous chunks and their warps stride through the
@@ -617,8 +663,10 @@ __device__ __forceinline__ int rate_mode(const ColDesc& cd, int t, int tile) {
 // float pairs (W, V, g V, J pairs), the preconditioner sums (base) and the
 // RH92 sums in FP32, and Jeff = J - Psi* eta from the pairs because it cancels
 // in optically thick layers.
+template <bool PIPE>
 __device__ void rates_tile(const ColDesc& cd, const int mode, const int t, const int tile, const int rank,
                            const RateSmem& sm, cg::cluster_group& cluster, const SolverOpts* bopts) {
+  constexpr int kRateHeld = PIPE ? 3 : 2;   // transitions whose terms a frequency's inputs hold
   const ColTables& T = cd.t;
   const int nz = T.nz, nl = T.nl, nt = T.nt;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -665,10 +713,9 @@ __device__ void rates_tile(const ColDesc& cd, const int mode, const int t, const
     struct In {
       df J, w, V, gV;
       float Vf, gf, Wr, Lx, Le, c2f;
-      int m0, m1;
-      float Vs0, Gs0, Vs1, Gs1;
+      float Vs[kRateHeld], Gs[kRateHeld];
     };
-    auto ld = [&](int q) {
+    auto ld = [&](int q, const RateList& L) {
       In r;
       const int p = wbase + q - q0;
       const size_t pk = (size_t)p * nz + k, o = (size_t)q * nz + k;
@@ -682,26 +729,18 @@ __device__ void rates_tile(const ColDesc& cd, const int mode, const int t, const
       r.Lx = cd.w.Lchi32[o];
       r.Le = cd.w.Leta32[o];
       r.c2f = __ldg(T.c2f + q);
-      r.m0 = r.m1 = -1;
-      r.Vs0 = r.Gs0 = r.Vs1 = r.Gs1 = 0.f;
-      if (packed) {
-        // the packed table gives window point and levels in one load
-        r.m0 = __ldg(T.qmeta + q);
-        r.m1 = __ldg(T.qmeta + (size_t)T.nq + q);
-        if (r.m0 >= 0) {
-          const size_t ps = (size_t)(r.m0 >> 8) * nz + k;
-          r.Vs0 = __ldg(T.V32 + ps);
-          r.Gs0 = __ldg(T.G32 + ps);
-        }
-        if (r.m1 >= 0) {
-          const size_t ps = (size_t)(r.m1 >> 8) * nz + k;
-          r.Vs1 = __ldg(T.V32 + ps);
-          r.Gs1 = __ldg(T.G32 + ps);
+#pragma unroll
+      for (int j = 0; j < kRateHeld; ++j) {
+        r.Vs[j] = r.Gs[j] = 0.f;
+        if (L.m[j] >= 0) {
+          const size_t ps = (size_t)(L.m[j] >> 8) * nz + k;
+          r.Vs[j] = __ldg(T.V32 + ps);
+          r.Gs[j] = __ldg(T.G32 + ps);
         }
       }
       return r;
     };
-    auto use = [&](int q, const In& r) {
+    auto use = [&](int q, const RateList& L, const In& r) {
       s0 = df_acc(s0, df_mul(df_mul(r.w, r.V), r.J));
       s1 = df_acc(s1, df_mul(df_mul(r.w, r.gV), r.J));
       const float Wc0 = r.Wr * (r.Vf * (nlo_f - r.gf * nup_f));
@@ -723,12 +762,13 @@ __device__ void rates_tile(const ColDesc& cd, const int mode, const int t, const
         zu = fmaf(cU, Gs * Vs, zu);
       };
       if (packed) {
-        if (r.m0 >= 0) add_terms(r.m0, r.Vs0, r.Gs0);
-        if (r.m1 >= 0) {
-          add_terms(r.m1, r.Vs1, r.Gs1);
-          for (int j = 2; j < kQMetaT; ++j) {
-            const int m = __ldg(T.qmeta + (size_t)j * T.nq + q);
-            if (m < 0) break;
+#pragma unroll
+        for (int j = 0; j < kQMetaT; ++j) {
+          const int m = PIPE || j < kRateHeld ? L.m[j] : __ldg(T.qmeta + (size_t)j * T.nq + q);
+          if (m < 0) break;
+          if (j < kRateHeld) {
+            add_terms(m, r.Vs[j], r.Gs[j]);
+          } else {
             const size_t ps = (size_t)(m >> 8) * nz + k;
             add_terms(m, __ldg(T.V32 + ps), __ldg(T.G32 + ps));
           }
@@ -741,13 +781,7 @@ __device__ void rates_tile(const ColDesc& cd, const int mode, const int t, const
         }
       }
     };
-    int q = qa + wid;
-    for (; q + kRateWarps <= qb; q += 2 * kRateWarps) {
-      const In r0 = ld(q), r1 = ld(q + kRateWarps);
-      use(q, r0);
-      use(q + kRateWarps, r1);
-    }
-    if (q <= qb) use(q, ld(q));
+    rate_window<PIPE>(T, packed, qa + wid, qb, ld, use);
   } else if (base_mode) {
     const int pv = precond_variant(cd, bopts);
     const double sca = T.chi_sca[k];
@@ -780,15 +814,14 @@ __device__ void rates_tile(const ColDesc& cd, const int mode, const int t, const
     const float nlo_f = (float)n_lo, nup_f = (float)n_up;
     const bool packed = T.max_overlap <= kQMetaT;
     const float2* __restrict__ eta2 = as_pairs(cd.w.eta);
-    // one frequency's inputs; two frequencies are loaded before the first is
-    // summed, so that their latencies overlap (the sums keep their order)
+    // as above
     struct In {
       df J, w, V, gV, eta;
       float Le, Wf, Vf, gf, c2f, etab;
-      int m0, t0, m1, t1;
-      float GV0, GV1;
+      float GV[kRateHeld];
+      uint2 tr;
     };
-    auto ld = [&](int q) {
+    auto ld = [&](int q, const RateList& L) {
       In r;
       const int p = wbase + q - q0;
       const size_t pk = (size_t)p * nz + k, o = (size_t)q * nz + k;
@@ -803,26 +836,18 @@ __device__ void rates_tile(const ColDesc& cd, const int mode, const int t, const
       r.gf = __ldg(T.G32 + pk);
       r.c2f = __ldg(T.c2f + q);
       r.etab = cd.w.etab32[o];
-      r.m0 = r.m1 = r.t0 = r.t1 = -1;
-      r.GV0 = r.GV1 = 0.f;
-      if (packed) {
-        // the packed tables give window point and transition in two loads
-        r.m0 = __ldg(T.qmeta + q);
-        r.m1 = __ldg(T.qmeta + (size_t)T.nq + q);
-        r.t0 = __ldg(T.qtr + q);
-        r.t1 = __ldg(T.qtr + (size_t)T.nq + q);
-        if (r.m0 >= 0) {
-          const size_t ps = (size_t)(r.m0 >> 8) * nz + k;
-          r.GV0 = __ldg(T.G32 + ps) * __ldg(T.V32 + ps);
-        }
-        if (r.m1 >= 0) {
-          const size_t ps = (size_t)(r.m1 >> 8) * nz + k;
-          r.GV1 = __ldg(T.G32 + ps) * __ldg(T.V32 + ps);
+      r.tr = __ldg(T.qtr8 + q);
+#pragma unroll
+      for (int j = 0; j < kRateHeld; ++j) {
+        r.GV[j] = 0.f;
+        if (L.m[j] >= 0) {
+          const size_t ps = (size_t)(L.m[j] >> 8) * nz + k;
+          r.GV[j] = __ldg(T.G32 + ps) * __ldg(T.V32 + ps);
         }
       }
       return r;
     };
-    auto use = [&](int q, const In& r) {
+    auto use = [&](int q, const RateList& L, const In& r) {
       s0 = df_acc(s0, df_mul(df_mul(r.w, r.V), r.J));
       s1 = df_acc(s1, df_mul(df_mul(r.w, r.gV), r.J));
       // Jeff = J - Psi* eta cancels in optically thick layers: formed from the pairs
@@ -834,19 +859,16 @@ __device__ void rates_tile(const ColDesc& cd, const int mode, const int t, const
       f3 = fmaf(wcp, r.etab, f3);
       const float wcu = wcp * r.c2f;
       if (packed) {
-        if (r.m0 >= 0) {
-          float& z = sm.f(wid, r.t0, lane);
-          z = fmaf(wcu, r.GV0, z);
-        }
-        if (r.m1 >= 0) {
-          float& z = sm.f(wid, r.t1, lane);
-          z = fmaf(wcu, r.GV1, z);
-          for (int j = 2; j < kQMetaT; ++j) {
-            const int m = __ldg(T.qmeta + (size_t)j * T.nq + q);
-            if (m < 0) break;
+#pragma unroll
+        for (int j = 0; j < kQMetaT; ++j) {
+          const int m = PIPE || j < kRateHeld ? L.m[j] : __ldg(T.qmeta + (size_t)j * T.nq + q);
+          if (m < 0) break;
+          float& z = sm.f(wid, ((j < 4 ? r.tr.x : r.tr.y) >> (8 * (j & 3))) & 0xff, lane);
+          if (j < kRateHeld) {
+            z = fmaf(wcu, r.GV[j], z);
+          } else {
             const size_t ps = (size_t)(m >> 8) * nz + k;
-            float& zj = sm.f(wid, __ldg(T.qtr + (size_t)j * T.nq + q), lane);
-            zj = fmaf(wcu, __ldg(T.G32 + ps) * __ldg(T.V32 + ps), zj);
+            z = fmaf(wcu, __ldg(T.G32 + ps) * __ldg(T.V32 + ps), z);
           }
         }
       } else {
@@ -858,13 +880,7 @@ __device__ void rates_tile(const ColDesc& cd, const int mode, const int t, const
         }
       }
     };
-    int q = qa + wid;
-    for (; q + kRateWarps <= qb; q += 2 * kRateWarps) {
-      const In r0 = ld(q), r1 = ld(q + kRateWarps);
-      use(q, r0);
-      use(q + kRateWarps, r1);
-    }
-    if (q <= qb) use(q, ld(q));
+    rate_window<PIPE>(T, packed, qa + wid, qb, ld, use);
   } else {
     const double* Jd = jdag_ptr(cd);
     for (int q = qa + wid; q <= qb; q += kRateWarps) {
@@ -941,6 +957,7 @@ __device__ void rates_tile(const ColDesc& cd, const int mode, const int t, const
 // (depth tile, transition) and walks the columns 32 at a time, lane l testing
 // column c0 + l * step, so that columns in another evaluation kind cost one
 // load each instead of a cluster launch.
+template <bool PIPE>
 __global__ void __launch_bounds__(32 * kRateWarps) k_rates(const ColDesc* __restrict__ cols, int ncols,
                                                            int racc, int fslots, const SolverOpts* bopts) {
   extern __shared__ __align__(16) unsigned char rate_smem[];
@@ -963,7 +980,7 @@ __global__ void __launch_bounds__(32 * kRateWarps) k_rates(const ColDesc* __rest
       const int l = __ffs(act) - 1;
       act &= act - 1;
       const int mode = __shfl_sync(0xffffffffu, ml, l);
-      rates_tile(cols[c0 + l * step], mode, t, tile, rank, sm, cluster, bopts);
+      rates_tile<PIPE>(cols[c0 + l * step], mode, t, tile, rank, sm, cluster, bopts);
     }
   }
 }
@@ -973,7 +990,8 @@ __global__ void __launch_bounds__(32 * kRateWarps) k_rates(const ColDesc* __rest
 int prepare_kernels() {
   const int max_smem = (int)((size_t)kRateWarps * 32 * ((2 + kRhFixed + kMaxT) * sizeof(double) +
                                                        std::max(kMaxT, kMaxL) * sizeof(float)));
-  JFNK_CUDA(cudaFuncSetAttribute(k_rates, cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem));
+  JFNK_CUDA(cudaFuncSetAttribute(k_rates<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem));
+  JFNK_CUDA(cudaFuncSetAttribute(k_rates<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem));
   return cached_prepare();
 }
 
@@ -1001,7 +1019,7 @@ static int launch_rates(const Batch& b, cudaStream_t s) {
   attr[0].val.clusterDim.z = split;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  JFNK_CUDA(cudaLaunchKernelEx(&cfg, k_rates, (const ColDesc*)b.d_cols, b.ncols, racc, fslots,
+  JFNK_CUDA(cudaLaunchKernelEx(&cfg, split > 1 ? k_rates<true> : k_rates<false>, (const ColDesc*)b.d_cols, b.ncols, racc, fslots,
                                (const SolverOpts*)b.d_opts));
   return JFNK_OK;
 }
@@ -1248,26 +1266,25 @@ int launch_opacity_tan(const Batch& b, cudaStream_t s, int depths) {
   return JFNK_OK;
 }
 
-int launch_opacity_mixed(const Batch& b, cudaStream_t s, int skip_tangent) {
-  const int tb = 256;
-  k_pop_pairs<<<dim3((b.max_N + tb - 1) / tb, b.ncols), tb, 0, s>>>(b.d_cols);
-  k_opacity<float><<<opacity_grid(b, tb), tb, 0, s>>>(b.d_cols, 1);   // base and RH92 columns
-  if (!skip_tangent) launch_op_tan(b, s);
-  JFNK_CUDA(cudaGetLastError());
-  return JFNK_OK;
-}
-
 // The assembly: tangent evaluations thread per depth, the others warp per depth.
 static void launch_assemble(const Batch& b, cudaStream_t s) {
-  k_assemble_tan<<<dim3((b.max_nz + kAsmTanThreads - 1) / kAsmTanThreads, b.ncols, std::max(1, b.max_nl)),
-                   kAsmTanThreads, 0, s>>>(b.d_cols);
-  k_assemble<<<dim3((b.max_nz + kAsmWarps - 1) / kAsmWarps, b.ncols), 32 * kAsmWarps, 0, s>>>(b.d_cols);
+  if (b.forced < 0 || b.forced == EV_TANGENT)
+    k_assemble_tan<<<dim3((b.max_nz + kAsmTanThreads - 1) / kAsmTanThreads, b.ncols, std::max(1, b.max_nl)),
+                     kAsmTanThreads, 0, s>>>(b.d_cols);
+  if (b.forced != EV_TANGENT)
+    k_assemble<<<dim3((b.max_nz + kAsmWarps - 1) / kAsmWarps, b.ncols), 32 * kAsmWarps, 0, s>>>(b.d_cols);
 }
 
 static void launch_rates_tan32(const Batch& b, cudaStream_t s) {
-  k_rates_tan32<<<dim3((b.max_nz + kRateTanWarps * kRateTanDepths - 1) / (kRateTanWarps * kRateTanDepths),
-                       b.max_nt, b.ncols),
-                  32 * kRateTanWarps, 0, s>>>(b.d_cols);
+  auto grid = [&](int d) {
+    return dim3((b.max_nz + kRateTanWarps * d - 1) / (kRateTanWarps * d), b.max_nt, b.ncols);
+  };
+  // a window's stride per warp and depth: below 32 warps per multiprocessor the
+  // launch is short of warps, and one depth per warp gives it four times as many
+  if ((long)b.ncols * b.max_nt * b.max_nz < 32L * 4 * b.n_sm)
+    k_rates_tan32<1><<<grid(1), 32 * kRateTanWarps, 0, s>>>(b.d_cols);
+  else
+    k_rates_tan32<4><<<grid(4), 32 * kRateTanWarps, 0, s>>>(b.d_cols);
 }
 
 int launch_evaluation(const Batch& b, cudaStream_t s, cudaEvent_t ev0, cudaEvent_t ev1, cudaStream_t side,
@@ -1288,8 +1305,10 @@ int launch_evaluation(const Batch& b, cudaStream_t s, cudaEvent_t ev0, cudaEvent
     // joined before the assembly, which reads both.
     JFNK_CUDA(cudaEventRecord(b.fork_ev, s));
     JFNK_CUDA(cudaStreamWaitEvent(side, b.fork_ev, 0));
-    k_dir32<<<dim3((b.max_N + tb - 1) / tb, nc), tb, 0, side>>>(b.d_cols);
-    if (!sweep_fused(b)) launch_op_tan(b, side);
+    // (the warp variant of the sweeps forms the opacity itself)
+    const bool own = b.sweep_variant == 2;
+    if (!own) k_dir32<<<dim3((b.max_N + tb - 1) / tb, nc), tb, 0, side>>>(b.d_cols);
+    if (!own && !sweep_fused(b)) launch_op_tan(b, side);
     if (ev2) JFNK_CUDA(cudaEventRecordWithFlags(ev2, side, cudaEventRecordExternal));
     int rc = launch_formal_sweep(b, side, 2);
     if (rc) return rc;
@@ -1297,7 +1316,7 @@ int launch_evaluation(const Batch& b, cudaStream_t s, cudaEvent_t ev0, cudaEvent
     launch_rates_tan32(b, side);
     JFNK_CUDA(cudaEventRecord(b.join_ev, side));
     k_pop_pairs<<<dim3((b.max_N + tb - 1) / tb, nc), tb, 0, s>>>(b.d_cols);
-    k_opacity<float><<<opacity_grid(b, tb), tb, 0, s>>>(b.d_cols, 1);
+    if (!own) k_opacity<float><<<opacity_grid(b, tb), tb, 0, s>>>(b.d_cols, 1);
     if (ev0) JFNK_CUDA(cudaEventRecordWithFlags(ev0, s, cudaEventRecordExternal));
     if ((rc = launch_formal_sweep(b, s, 1))) return rc;
     if (ev1) JFNK_CUDA(cudaEventRecordWithFlags(ev1, s, cudaEventRecordExternal));
@@ -1335,21 +1354,29 @@ int launch_evaluation(const Batch& b, cudaStream_t s, cudaEvent_t ev0, cudaEvent
     // (float tangent direction,) opacity, then the per-frequency sweeps; with
     // events (a profiled tick) the tangent sweep is bracketed by ev2/ev3 and
     // the base-type sweep by ev0/ev1, each timed alone on this one stream
-    k_dir32<<<dim3((b.max_N + tb - 1) / tb, nc), tb, 0, s>>>(b.d_cols);
-    int rc0 = launch_opacity_mixed(b, s, sweep_fused(b) ? 1 : 0);
-    if (rc0) return rc0;
+    // an explicit call forces one kind on every column: only its kernels are launched
+    const bool own = b.sweep_variant == 2;
+    const bool tans = b.forced < 0 || b.forced == EV_TANGENT, bases = b.forced != EV_TANGENT;
+    if (tans && !own) k_dir32<<<dim3((b.max_N + tb - 1) / tb, nc), tb, 0, s>>>(b.d_cols);
+    if (bases) k_pop_pairs<<<dim3((b.max_N + tb - 1) / tb, nc), tb, 0, s>>>(b.d_cols);
+    if (bases && !own) k_opacity<float><<<opacity_grid(b, tb), tb, 0, s>>>(b.d_cols, 1);   // base and RH92 columns
+    if (tans && !own && !sweep_fused(b)) launch_op_tan(b, s);
     int rc;
-    if (ev2) {
-      JFNK_CUDA(cudaEventRecordWithFlags(ev2, s, cudaEventRecordExternal));
-      if ((rc = launch_formal_sweep(b, s, 2))) return rc;
-      if (ev3) JFNK_CUDA(cudaEventRecordWithFlags(ev3, s, cudaEventRecordExternal));
-      if (ev0) JFNK_CUDA(cudaEventRecordWithFlags(ev0, s, cudaEventRecordExternal));
-      if ((rc = launch_formal_sweep(b, s, 1))) return rc;
-    } else {
-      if (ev0) JFNK_CUDA(cudaEventRecordWithFlags(ev0, s, cudaEventRecordExternal));
-      if ((rc = launch_formal_sweep(b, s))) return rc;
-    }
+    if (ev2) JFNK_CUDA(cudaEventRecordWithFlags(ev2, s, cudaEventRecordExternal));
+    if (tans && (rc = launch_formal_sweep(b, s, 2))) return rc;
+    if (ev3) JFNK_CUDA(cudaEventRecordWithFlags(ev3, s, cudaEventRecordExternal));
+    if (ev0) JFNK_CUDA(cudaEventRecordWithFlags(ev0, s, cudaEventRecordExternal));
+    if (bases && (rc = launch_formal_sweep(b, s, 1))) return rc;
     if (ev1) JFNK_CUDA(cudaEventRecordWithFlags(ev1, s, cudaEventRecordExternal));
+    if (bases) {
+      if ((rc = launch_rates(b, s))) return rc;
+      launch_dJdn_update(b, s);
+    }
+    if (tans) launch_rates_tan32(b, s);
+    if ((rc = mark(1))) return rc;
+    launch_assemble(b, s);
+    JFNK_CUDA(cudaGetLastError());
+    return mark(2);
   } else if (b.formal_kind == FORMAL_FUSED) {
     // opacity, then the fused formal solution with in-block ray sums
     k_opacity<double><<<opacity_grid(b, tb), tb, 0, s>>>(b.d_cols, 0);
@@ -1369,7 +1396,6 @@ int launch_evaluation(const Batch& b, cudaStream_t s, cudaEvent_t ev0, cudaEvent
     int rc = launch_rates(b, s);
     if (rc) return rc;
     launch_dJdn_update(b, s);
-    if (b.mixed) launch_rates_tan32(b, s);
     if ((rc = mark(1))) return rc;
   }
   launch_assemble(b, s);

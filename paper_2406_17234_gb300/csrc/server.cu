@@ -242,7 +242,7 @@ int jfnk_server_create(jfnk_ctx* ctx, const jfnk_server_desc* d, jfnk_server** o
   if (sv->kind == FORMAL_SWEEP) {
     // few frequencies in flight: the warp-per-frequency-pair sweep (same results)
     const int ws = sweep_warp_size(d->max_depth);
-    if ((long)S * d->max_freq < 256L * ctx->n_sm && ws > 0) {
+    if (sweep_small(S, d->max_freq, ctx->n_sm) && ws > 0) {
       b.sweep_variant = 2;
       b.formal_threads = ws;
     }

@@ -504,7 +504,8 @@ int build_atmosphere(jfnk_ctx* ctx, int lane, const AtomData& A, const jfnk_atmo
          o_vt = ar.take<double>(nz);
   size_t o_tr = ar.take<TransDev>(nt), o_cd = ar.take<CollDev>(nt);
   size_t o_W32 = ar.take<float>(nwin), o_Wr32 = ar.take<float>(nwin), o_c2f = ar.take<float>(nq);
-  size_t o_qmeta = ar.take<int>((size_t)kQMetaT * nq), o_qtr = ar.take<int>((size_t)kQMetaT * nq);
+  size_t o_qmeta = ar.take<int>((size_t)kQMetaT * nq), o_qmeta4 = ar.take<int4>(2 * (size_t)nq), o_qtr8 = ar.take<uint2>(nq);
+  static_assert(kQMetaT == 8, "qmeta4 and qtr8 hold eight transitions");
   size_t o_W2 = ar.take<float2>(nwin), o_c2p = ar.take<float2>(nq), o_rc2p = ar.take<float2>(nq);
   size_t o_linc = ar.take<int>((size_t)nl * (nt + 1));
   size_t o_ang64 = ar.take<Ang64>(nmu), o_ang32 = ar.take<float4>(nmu), o_dz32 = ar.take<float2>(nz - 1);
@@ -604,15 +605,18 @@ int build_atmosphere(jfnk_ctx* ctx, int lane, const AtomData& A, const jfnk_atmo
   JFNK_CUDA(up(o_W2, w2.data(), nwin * sizeof(float2)));
   JFNK_CUDA(up(o_c2p, c2p.data(), nq * sizeof(float2)));
   JFNK_CUDA(up(o_rc2p, rc2p.data(), nq * sizeof(float2)));
-  std::vector<int> qmeta((size_t)kQMetaT * nq, -1), qtr((size_t)kQMetaT * nq, -1);
+  std::vector<int> qmeta((size_t)kQMetaT * nq, -1), qmeta4((size_t)kQMetaT * nq, -1);
+  std::vector<unsigned char> qtr8((size_t)kQMetaT * nq, 0xff);
   for (int q = 0; q < nq; ++q)
     for (int s = A.q_off[q], j = 0; s < A.q_off[q + 1] && j < kQMetaT; ++s, ++j) {
       const int t = A.q_t[s];
-      qmeta[(size_t)j * nq + q] = ((A.t_base[t] + q - A.t_q0[t]) << 8) | (A.t_lo[t] << 4) | A.t_up[t];
-      qtr[(size_t)j * nq + q] = t;
+      qmeta[(size_t)j * nq + q] = qmeta4[(size_t)q * kQMetaT + j] =
+          ((A.t_base[t] + q - A.t_q0[t]) << 8) | (A.t_lo[t] << 4) | A.t_up[t];
+      qtr8[(size_t)q * kQMetaT + j] = (unsigned char)t;
     }
   JFNK_CUDA(up(o_qmeta, qmeta.data(), qmeta.size() * 4));
-  JFNK_CUDA(up(o_qtr, qtr.data(), qtr.size() * 4));
+  JFNK_CUDA(up(o_qmeta4, qmeta4.data(), qmeta4.size() * 4));
+  JFNK_CUDA(up(o_qtr8, qtr8.data(), qtr8.size()));
   // per level, its transitions in index order (lower level: +, upper: -)
   std::vector<int> linc((size_t)nl * (nt + 1), -1);
   for (int l = 0; l < nl; ++l) {
@@ -715,7 +719,8 @@ int build_atmosphere(jfnk_ctx* ctx, int lane, const AtomData& A, const jfnk_atmo
   tb_.VG32T = ar.ptr<float2>(o_VG32T);
   tb_.Wr32 = ar.ptr<float>(o_Wr32); tb_.c2f = ar.ptr<float>(o_c2f);
   tb_.qmeta = ar.ptr<int>(o_qmeta);
-  tb_.qtr = ar.ptr<int>(o_qtr);
+  tb_.qmeta4 = ar.ptr<int4>(o_qmeta4);
+  tb_.qtr8 = ar.ptr<uint2>(o_qtr8);
   tb_.lvl_inc = ar.ptr<int>(o_linc);
   tb_.mu = ar.ptr<double>(o_mu); tb_.wmu = ar.ptr<double>(o_wmu);
   tb_.ang64 = ar.ptr<Ang64>(o_ang64);

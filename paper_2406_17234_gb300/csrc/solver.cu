@@ -229,6 +229,7 @@ __global__ void k_set_forced(ColDesc* cols, int mode) { cols[blockIdx.x].forced_
 
 int batch_set_forced_mode(Batch* b, int mode, cudaStream_t s) {
   for (auto& c : b->h_cols) c.forced_mode = mode;
+  b->forced = mode;
   k_set_forced<<<b->ncols, 1, 0, s>>>(b->d_cols, mode);
   JFNK_CUDA(cudaGetLastError());
   return JFNK_OK;

@@ -816,9 +816,8 @@ int jfnk_rh92_update(jfnk_ctx* ctx, const jfnk_atmos* a, int precision, const do
   Batch* b;
   if ((rc = get_single(a, precision == JFNK_MIXED, &b))) return rc;
   return on_ctx_stream(ctx, stream, where, [&](cudaStream_t s) {
-    int r = explicit_eval(ctx, a, b, EV_RH92, n, J_dagger, where, s);
+    int r = explicit_eval(ctx, a, b, EV_RH92, n, J_dagger, where, s);   // its assembly updates w.n
     if (r) return r;
-    if ((r = launch_rh92_update(*b, s))) return r;
     const ColDesc& c = b->h_cols[0];
     const AtmosData& M = a->d;
     if ((r = copy_out(n_out, c.w.n, (size_t)M.nz * M.nl * 8, where, s))) return r;

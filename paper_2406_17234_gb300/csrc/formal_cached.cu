@@ -174,23 +174,6 @@ __device__ __forceinline__ float abs_float(double x) {
 
 __device__ __forceinline__ int mag(double x) { return __double2hiint(x) & 0x7fffffff; }
 
-// First part slot of transition t in ColWork::rpart and its number of tiles,
-// for the lane's transition (warp-wide; lanes past nt get 0).
-__device__ __forceinline__ int part_offset(const ColTables& T, int qb, int lane, int& tile0, int& ntile) {
-  tile0 = ntile = 0;
-  if (lane < T.nt) {
-    tile0 = T.t_q0[lane] / qb;
-    ntile = T.t_q1[lane] / qb - tile0 + 1;
-  }
-  int s = ntile;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const int v = __shfl_up_sync(0xffffffffu, s, o);
-    if (lane >= o) s += v;
-  }
-  return s - ntile;
-}
-
 struct Tile {
   int qb0, nqb, Qb, Qp, R5;   // first frequency, frequencies, tile size, padded size, Qb n_mu
   int tile;
@@ -800,51 +783,6 @@ __global__ void __launch_bounds__(kEvalThreads) k_eval64(const ColDesc* __restri
   }
 }
 
-// Adds the tiles' parts of every rate integral in tile order and writes the
-// rates, the preconditioner sums or the RH92 sums where the assembly and the
-// RH92 update read them; thread per (transition, slot, depth).
-__global__ void __launch_bounds__(128) k_rates_reduce(const ColDesc* __restrict__ cols) {
-  const ColDesc& cd = cols[blockIdx.z];
-  const int mode = mode_of(cd);
-  if (mode == EV_SKIP) return;
-  const ColTables& T = cd.t;
-  const int nz = T.nz, nl = T.nl, t = blockIdx.y;
-  const bool base = (mode == EV_BASE), rh = (mode == EV_RH92);
-  const int ns = base ? 2 + nl : rh ? kPartFixed + nl : 2;
-  if (t >= T.nt || (int)(blockIdx.x * blockDim.x) >= ns * nz) return;
-  __shared__ int s_off, s_nt;
-  if (threadIdx.x < 32) {
-    int tile0, ntile;
-    const int off = part_offset(T, cd.w.cq, threadIdx.x, tile0, ntile);
-    if ((int)threadIdx.x == t) {
-      s_off = off;
-      s_nt = ntile;
-    }
-  }
-  __syncthreads();
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= ns * nz) return;
-  const int sl = i / nz, k = i - sl * nz;
-  const size_t stride = (size_t)(kPartFixed + nl) * nz;
-  const double* p = cd.w.rpart + (size_t)s_off * stride + (size_t)sl * nz + k;
-  double s = 0.0;
-#pragma unroll 8
-  for (int a = 0; a < s_nt; ++a) s += p[(size_t)a * stride];
-  const size_t o = (size_t)t * nz + k;
-  if (mode == EV_TANGENT) {
-    (sl == 0 ? cd.w.dRup : cd.w.dRdn)[o] = s;
-    return;
-  }
-  const double rsp = T.Rsp[o];
-  if (sl == 0) cd.w.Rup[o] = s;
-  else if (sl == 1) {
-    cd.w.Rdn[o] = s + rsp;
-    if (rh) cd.w.rh[o * kRhStride + 2] = rsp;
-  } else if (base) cd.w.Apart[o * nl + sl - 2] = s;
-  else if (sl < kPartFixed) cd.w.rh[o * kRhStride + (sl == 4 ? 3 : sl - 2)] = s;   // Jeff sums, constant part
-  else cd.w.rh[o * kRhStride + kRhFixed + sl - kPartFixed] = s;                     // per level
-}
-
 int cached_prepare() {
   double2 tab[kExpTab];
   for (int j = 0; j < kExpTab; ++j)
@@ -859,13 +797,6 @@ int launch_eval64(const Batch& b, cudaStream_t s) {
   const dim3 g(b.max_tiles, b.ncols);
   if (b.eval_mu == 5) k_eval64<5><<<g, kEvalThreads, b.eval_smem, s>>>(b.d_cols, b.d_opts);
   else k_eval64<0><<<g, kEvalThreads, b.eval_smem, s>>>(b.d_cols, b.d_opts);
-  JFNK_CUDA(cudaGetLastError());
-  return JFNK_OK;
-}
-
-int launch_rates_reduce(const Batch& b, cudaStream_t s) {
-  const int slots = kPartFixed + b.max_nl;
-  k_rates_reduce<<<dim3((slots * b.max_nz + 127) / 128, b.max_nt, b.ncols), 128, 0, s>>>(b.d_cols);
   JFNK_CUDA(cudaGetLastError());
   return JFNK_OK;
 }

@@ -18,6 +18,23 @@ __device__ __forceinline__ int eval_mode_f(const ColDesc& cd) {
   }
 }
 
+// First part slot of transition t in ColWork::rpart and its number of tiles,
+// for the lane's transition (warp-wide; lanes past nt get 0).
+__device__ __forceinline__ int part_offset(const ColTables& T, int qb, int lane, int& tile0, int& ntile) {
+  tile0 = ntile = 0;
+  if (lane < T.nt) {
+    tile0 = T.t_q0[lane] / qb;
+    ntile = T.t_q1[lane] / qb - tile0 + 1;
+  }
+  int s = ntile;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int v = __shfl_up_sync(0xffffffffu, s, o);
+    if (lane >= o) s += v;
+  }
+  return s - ntile;
+}
+
 // Coefficients of one step of optical depth x: e = exp(-x), w = (1 - e)/x,
 // a = 1 - w and bq = (w - e)/x, each from its own Taylor series below
 // x = 0.1 (where 1 - e, 1 - w and w - e cancel); r = 1/x is supplied by the

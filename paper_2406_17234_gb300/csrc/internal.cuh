@@ -134,6 +134,7 @@ struct Batch {
   int max_tiles = 0;                  // cached FP64 evaluation: most tiles of a column of the view
   int eval_mu = 0;                    // ... the angle count shared by every column (0: several)
   size_t eval_smem = 0;               // ... and its blocks' dynamic shared memory
+  bool serving = false;               // a server's slots: few of the columns are in one kind at a time
   int forced = -1;                    // evaluation kind forced on every column (-1: each its own)
   bool tuned = false;                 // autotuner has run on this batch
   int graph_kernels = 0;              // kernel nodes in the captured tick graph
@@ -180,6 +181,8 @@ int launch_evaluation(const Batch& b, cudaStream_t s, cudaEvent_t ev0 = nullptr,
 int ensure_side_stream(Batch* b);
 // Allocates and binds the lagged d J/d n buffers of every column (once).
 int ensure_dJdn(Batch* b, cudaStream_t s);
+// The assembly solves the RH92 updates (a warp per depth); else the Krylov step.
+bool rh92_by_warp(const Batch& b);
 // Launch of the Krylov/Newton state machine step.
 int launch_krylov_step(const Batch& b, cudaStream_t s);
 // Fused formal solution + ray sums (formal_fused.cu).
@@ -196,7 +199,6 @@ size_t cached_parts(int qb, int nz, int nl, int nwin, int nt);
 constexpr int kEvalThreads = 512;   // threads per block of the cached evaluation
 int cached_prepare();
 int launch_eval64(const Batch& b, cudaStream_t s);
-int launch_rates_reduce(const Batch& b, cudaStream_t s);
 // Per-frequency sweep kernel of the mixed mode (formal_sweep.cu).
 size_t sweep_scratch_bytes(int nq, int nz);
 int sweep_prepare(Batch* b);
@@ -236,7 +238,4 @@ int launch_istar(const Batch& b, cudaStream_t s);
 // Zero-radiation initial guess (rate equations with I = 0) in every column's n;
 // reads n = LTE populations for the conservation rows.
 int launch_zero_radiation(const Batch& b, cudaStream_t s);
-// RH92 per-depth update from an EV_RH92 evaluation (explicit API path).
-int launch_rh92_update(const Batch& b, cudaStream_t s);
-
 }  // namespace jfnk

@@ -1105,21 +1105,164 @@ __global__ void __launch_bounds__(kAsmTanThreads) k_assemble_tan(const ColDesc* 
   cd.w.dF[(size_t)k * nl + l] = f;
 }
 
-__global__ void __launch_bounds__(32 * kAsmWarps) k_assemble(const ColDesc* __restrict__ cols) {
+// Shared memory of a warp of the assembly.
+struct AsmSmem {
+  double up[kMaxT], dn[kMaxT], kap[kMaxT];
+  double P[kMaxL * (kMaxL + 1)];   // P^k, or the RH92 system
+  union {
+    double aug[kMaxL * 2 * kMaxL];
+    double A[kMaxT * kMaxL];       // per transition and level: preconditioner sums, or RH92 coefficients
+  };
+  double c0[kMaxT];
+};
+
+// RH92 update of depth k from the sums of an EV_RH92 evaluation, one warp;
+// returns the population change measure of the depth (or NaN on a singular
+// system) on every lane. With clamp the correction is limited like a Newton
+// correction (Sect. 2.2.2), so that no population of the depth falls below a
+// tenth of its old value.
+//
+// The preconditioned rate equations M n' + c0 = 0 (plus the conservation row)
+// are affine in n' and equal the residual F at n' = n, so n' = n + d with
+// M d = -F(n) and sum d = n_tot - sum n, the same update. With ``correction``
+// (mixed mode, once the iteration has settled) the correction d is solved
+// from the residual the evaluation assembled in float-pair and FP64
+// arithmetic, so that the FP32 sums in M (Psi*, the cross-coupling terms)
+// affect the speed of convergence only and not the fixed point, which is then
+// F(n) = 0 to the residual's accuracy (in optically thick lines the net rates
+// cancel far below FP32 resolution of the gross rates). Far from the
+// solution the direct form is the more robust one (M and c0 carry the same
+// rounding), so the mixed mode starts with it.
+//
+// On entry s.A[t][j] holds the cross-coupling sums per level of a cached
+// evaluation and s.up, s.dn, s.c0 its Jeff and constant sums; other
+// evaluations read w.rh. Transitions, then matrix elements, on the lanes, every
+// sum in transition order. (One thread per depth, in the Krylov step: 128 us of
+// an 82-depth, 15-transition column's step.)
+__device__ double rh92_warp(const ColDesc& cd, int k, int lane, AsmSmem& s, bool clamp, bool correction, double damp,
+                            double* out) {
+  const ColTables& T = cd.t;
+  const int nl = T.nl, nt = T.nt, nz = T.nz;
+  const double* C = T.C + (size_t)k * nl * nl;
+  const bool cached = cd.w.cf != nullptr;
+  __syncwarp();
+  if (lane < nt) {
+    const int t = lane, lo = T.t_lo[t], up = T.t_up[t];
+    double* coef = s.A + t * kMaxL;
+    const double* r = cd.w.rh + ((size_t)t * nz + k) * kRhStride;
+    const double r0 = cached ? s.up[t] : r[0], r1 = cached ? s.dn[t] : r[1];
+    const double r2 = cached ? T.Rsp[(size_t)t * nz + k] : r[2];
+    if (!cached) {
+      for (int j = 0; j < nl; ++j) coef[j] = 0.0;
+      s.c0[t] = r[3];
+    }
+    coef[lo] += r0 + C[lo * nl + up];
+    coef[up] -= r1 + r2 + C[up * nl + lo];
+    if (!cached)
+      for (int j = 0; j < nt; ++j) coef[T.t_up[j]] += r[kRhFixed + j];
+  }
+  __syncwarp();
+  const int is = cd.w.istar[k];
+  const double* n = cd.w.n + (size_t)k * nl;
+  const double* F = cd.w.F + (size_t)k * nl;   // F[is] = n_tot - sum n
+  const int w1 = nl + 1;                       // [M | rhs]
+  double* A = s.P;
+  for (int e = lane; e < nl * w1; e += 32) {
+    const int i = e / w1, j = e - i * w1;
+    double v = 0.0;
+    if (i == is) {
+      v = j < nl ? 1.0 : (correction ? F[is] : T.ntot[k]);
+    } else if (j < nl || !correction) {
+      const int* inc = T.lvl_inc + i * (nt + 1);
+      for (int q = 0; q < nt; ++q) {
+        const int m = inc[q];
+        if (m < 0) break;
+        const double g = j < nl ? s.A[(m >> 1) * kMaxL + j] : s.c0[m >> 1];
+        v += (m & 1) ? -g : g;
+      }
+      if (j == nl) v = -v;
+    } else {
+      v = -F[i];
+    }
+    A[e] = v;
+  }
+  __syncwarp();
+  // elimination with partial pivoting; every lane finds the same pivot
+  for (int c = 0; c < nl; ++c) {
+    int pr = c;
+    double best = fabs(A[c * w1 + c]);
+    for (int i = c + 1; i < nl; ++i)
+      if (fabs(A[i * w1 + c]) > best) { best = fabs(A[i * w1 + c]); pr = i; }
+    if (!(best > 0.0)) return nan("");
+    __syncwarp();
+    if (pr != c)
+      for (int j = lane; j < w1; j += 32) {
+        const double t = A[c * w1 + j];
+        A[c * w1 + j] = A[pr * w1 + j];
+        A[pr * w1 + j] = t;
+      }
+    __syncwarp();
+    // row i > c on lane i: its factor, then its elements spread over the lanes
+    if (lane > c && lane < nl) s.kap[lane] = A[lane * w1 + c] / A[c * w1 + c];
+    __syncwarp();
+    const int wc = w1 - c, ne = (nl - 1 - c) * wc;
+    for (int e = lane; e < ne; e += 32) {
+      const int i = c + 1 + e / wc, j = c + e % wc;
+      A[i * w1 + j] = fma(-s.kap[i], A[c * w1 + j], A[i * w1 + j]);
+    }
+    __syncwarp();
+  }
+  // back substitution into the last column
+  for (int i = nl - 1; i >= 0; --i) {
+    if (lane == 0) {
+      double v = A[i * w1 + nl];
+      for (int j = i + 1; j < nl; ++j) v = fma(-A[i * w1 + j], A[j * w1 + nl], v);
+      A[i * w1 + nl] = v / A[i * w1 + i];
+    }
+    __syncwarp();
+  }
+  double alpha = 1.0, x = 0.0, err = 0.0;
+  if (lane < nl) {
+    x = A[lane * w1 + nl];
+    if (correction) x += n[lane];   // n' = n + d
+    if (clamp) {
+      const double d = x - n[lane];
+      if (d < 0.0) alpha = fmin(alpha, 0.9 * n[lane] / (-d));
+    }
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) alpha = fmin(alpha, __shfl_xor_sync(0xffffffffu, alpha, o));
+  bool bad = false;
+  if (lane < nl) {
+    double nn = clamp ? n[lane] + alpha * (x - n[lane]) : x;
+    if (damp < 1.0) nn = n[lane] + damp * (nn - n[lane]);
+    err = 0.5 * fabs((nn - n[lane]) / (nn + n[lane]));
+    bad = !(err == err);
+    if (bad) err = 0.0;   // a NaN is left out of the maximum, as fmax does
+    out[(size_t)k * nl + lane] = nn;
+  }
+  return warp_max(err);
+}
+
+__global__ void __launch_bounds__(32 * kAsmWarps) k_assemble(const ColDesc* __restrict__ cols,
+                                                             const SolverOpts* bopts, int rh_warp) {
   const ColDesc& cd = cols[blockIdx.y];
   const int mode = eval_mode(cd);
-  if (mode == EV_SKIP || mode == EV_TANGENT) return;   // k_assemble_tan
+  const bool cached = cd.w.cf != nullptr;
+  if (mode == EV_SKIP || (mode == EV_TANGENT && !cached)) return;   // k_assemble_tan
   const ColTables& T = cd.t;
   const int nz = T.nz, nl = T.nl, nt = T.nt;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int k = blockIdx.x * kAsmWarps + wid;
   if (k >= nz) return;
-  __shared__ double s_up[kAsmWarps][kMaxT], s_dn[kAsmWarps][kMaxT], s_kap[kAsmWarps][kMaxT];
-  __shared__ double s_P[kAsmWarps][kMaxL * kMaxL];
-  const bool fd = (mode == EV_FD);
+  __shared__ AsmSmem s_all[kAsmWarps];
+  AsmSmem& s = s_all[wid];
+  const bool fd = (mode == EV_FD), tan = (mode == EV_TANGENT), base = (mode == EV_BASE), rh = (mode == EV_RH92);
+  double* s_up = s.up;
+  double* s_dn = s.dn;
+  double* s_P = s.P;
   const double* n = eval_pops(cd, mode) + k * nl;
   const double* C = T.C + (size_t)k * nl * nl;
-  const bool tan = (mode == EV_TANGENT);
   int is;
   if (!tan && !fd) {
     // conservation row at the most populated level (lowest index on ties)
@@ -1131,17 +1274,40 @@ __global__ void __launch_bounds__(32 * kAsmWarps) k_assemble(const ColDesc* __re
     is = cd.w.istar[k];
   }
   const double* v = tan ? tangent_dir(cd) + k * nl : nullptr;
-  for (int t = lane; t < nt; t += 32) {
-    const int lo = T.t_lo[t], up = T.t_up[t];
+  const size_t stride = (size_t)(kPartFixed + nl) * nz;
+  int off = 0, ntile = 0, tile0;
+  if (cached) off = part_offset(T, cd.w.cq, lane, tile0, ntile);
+  if (lane < nt) {
+    const int t = lane, lo = T.t_lo[t], up = T.t_up[t];
     const size_t o = (size_t)t * nz + k;
-    const double ur = C[lo * nl + up] + cd.w.Rup[o];
-    const double dr = C[up * nl + lo] + cd.w.Rdn[o];
-    if (tan)
-      s_kap[wid][t] = v[lo] * ur + n[lo] * cd.w.dRup[o] - v[up] * dr - n[up] * cd.w.dRdn[o];
-    else
-      s_kap[wid][t] = n[lo] * ur - n[up] * dr;
-    s_up[wid][t] = ur;
-    s_dn[wid][t] = dr;
+    double ru, rd;
+    if (cached) {
+      // the tiles' parts of R_ij and R_ji (their tangents), in tile order
+      const double* p = cd.w.rpart + (size_t)off * stride + k;
+      ru = rd = 0.0;
+#pragma unroll 8
+      for (int a = 0; a < ntile; ++a) {
+        ru += p[(size_t)a * stride];
+        rd += p[(size_t)a * stride + nz];
+      }
+      if (!tan) {
+        rd += T.Rsp[o];
+        cd.w.Rup[o] = ru;
+        cd.w.Rdn[o] = rd;
+      }
+    } else {
+      ru = cd.w.Rup[o];
+      rd = cd.w.Rdn[o];
+    }
+    if (tan) {
+      const double ur = C[lo * nl + up] + cd.w.Rup[o], dr = C[up * nl + lo] + cd.w.Rdn[o];
+      s.kap[t] = v[lo] * ur + n[lo] * ru - v[up] * dr - n[up] * rd;
+    } else {
+      const double ur = C[lo * nl + up] + ru, dr = C[up * nl + lo] + rd;
+      s.kap[t] = n[lo] * ur - n[up] * dr;
+      s_up[t] = ur;
+      s_dn[t] = dr;
+    }
   }
   __syncwarp();
   if (lane < nl) {
@@ -1152,7 +1318,7 @@ __global__ void __launch_bounds__(32 * kAsmWarps) k_assemble(const ColDesc* __re
     for (int e = 0; e < nt; ++e) {
       const int m = inc[e];
       if (m < 0) break;
-      const double kp = s_kap[wid][m >> 1];
+      const double kp = s.kap[m >> 1];
       f += (m & 1) ? -kp : kp;
     }
     if (lane == is) {
@@ -1167,7 +1333,40 @@ __global__ void __launch_bounds__(32 * kAsmWarps) k_assemble(const ColDesc* __re
     }
     (tan || fd ? cd.w.dF : cd.w.F)[k * nl + lane] = f;
   }
-  if (mode != EV_BASE) return;
+  if (tan || fd) return;
+  if (cached) {
+    // the tiles' parts of the level sums, (transition, slot) pairs on the lanes
+    const int ns = base ? nl : nl + 3;
+    __syncwarp();
+    for (int e0 = 0; e0 < nt * ns; e0 += 32) {
+      const int e = e0 + lane, t = min(e / ns, nt - 1), sl = e - t * ns;
+      const int to = __shfl_sync(0xffffffffu, off, t), tn = __shfl_sync(0xffffffffu, ntile, t);
+      if (e >= nt * ns) continue;
+      const double* p = cd.w.rpart + (size_t)to * stride + (size_t)(2 + sl) * nz + k;
+      double a = 0.0;
+#pragma unroll 8
+      for (int i = 0; i < tn; ++i) a += p[(size_t)i * stride];
+      if (base) s.A[t * kMaxL + sl] = a;
+      else if (sl == 0) s_up[t] = a;   // Jeff sums, constant part, then per level
+      else if (sl == 1) s_dn[t] = a;
+      else if (sl == 2) s.c0[t] = a;
+      else s.A[t * kMaxL + sl - 3] = a;
+    }
+    __syncwarp();
+  }
+  if (rh) {
+    if (cd.forced_mode >= 0) {   // the plain update: jfnk_rh92_update applies no limiting
+      rh92_warp(cd, k, lane, s, false, false, 1.0, cd.w.n);
+    } else if (rh_warp) {   // else the Krylov step does it
+      const SolverOpts& o = cd.opts ? *cd.opts : *bopts;
+      const SolverState* st = cd.w.st;
+      // mixed mode: the correction form once the change has fallen below 1e-2
+      const bool corr = cd.mixed && st->rh92_iter > 0 && st->err < 1e-2;
+      const double e = rh92_warp(cd, k, lane, s, o.clamp != 0, corr, st->rh_damp > 0.0 ? st->rh_damp : 1.0, cd.w.x);
+      if (lane == 0) cd.w.w[k] = e;
+    }
+    return;
+  }
   // P^k = Gamma^k + A^kk (Sect. 2.5.1), conservation row -1
   for (int e = lane; e < nl * nl; e += 32) {
     const int i = e / nl, j = e - i * nl;
@@ -1178,29 +1377,28 @@ __global__ void __launch_bounds__(32 * kAsmWarps) k_assemble(const ColDesc* __re
       if (m < 0) break;
       const int t = m >> 1;
       const int lo = T.t_lo[t], up = T.t_up[t];
-      double g = cd.w.Apart[((size_t)t * nz + k) * nl + j];
-      if (j == lo) g += s_up[wid][t];
-      if (j == up) g -= s_dn[wid][t];
+      double g = cached ? s.A[t * kMaxL + j] : cd.w.Apart[((size_t)t * nz + k) * nl + j];
+      if (j == lo) g += s_up[t];
+      if (j == up) g -= s_dn[t];
       pv += (m & 1) ? -g : g;   // i is the lower level (+) or the upper one (-)
     }
-    s_P[wid][e] = (i == is) ? -1.0 : pv;
+    s_P[e] = (i == is) ? -1.0 : pv;
   }
   __syncwarp();
   double* P = cd.w.P + (size_t)k * nl * nl;
   if (cd.forced_mode >= 0) {
-    for (int e = lane; e < nl * nl; e += 32) P[e] = s_P[wid][e];
+    for (int e = lane; e < nl * nl; e += 32) P[e] = s_P[e];
     return;
   }
   // explicit inverse of P^k, so that the Krylov step applies P^{-1} as a fully
   // parallel small mat-vec: Gauss-Jordan elimination with partial pivoting on
   // [P | I], lane j owning column j (2 nl <= 32 lanes); every lane finds the
   // same pivot from the same shared data, one reciprocal per column
-  __shared__ double s_aug[kAsmWarps][kMaxL * 2 * kMaxL];
-  double* G = s_aug[wid];
+  double* G = s.aug;
   const int w2 = 2 * nl;
   for (int e = lane; e < nl * w2; e += 32) {
     const int r = e / w2, j = e - r * w2;
-    G[e] = j < nl ? s_P[wid][r * nl + j] : (j - nl == r ? 1.0 : 0.0);
+    G[e] = j < nl ? s_P[r * nl + j] : (j - nl == r ? 1.0 : 0.0);
   }
   __syncwarp();
   const bool own = lane < w2;
@@ -1268,11 +1466,13 @@ int launch_opacity_tan(const Batch& b, cudaStream_t s, int depths) {
 
 // The assembly: tangent evaluations thread per depth, the others warp per depth.
 static void launch_assemble(const Batch& b, cudaStream_t s) {
-  if (b.forced < 0 || b.forced == EV_TANGENT)
+  const bool cached = b.formal_kind == FORMAL_CACHED;   // k_assemble takes its tangents too
+  if (!cached && (b.forced < 0 || b.forced == EV_TANGENT))
     k_assemble_tan<<<dim3((b.max_nz + kAsmTanThreads - 1) / kAsmTanThreads, b.ncols, std::max(1, b.max_nl)),
                      kAsmTanThreads, 0, s>>>(b.d_cols);
-  if (b.forced != EV_TANGENT)
-    k_assemble<<<dim3((b.max_nz + kAsmWarps - 1) / kAsmWarps, b.ncols), 32 * kAsmWarps, 0, s>>>(b.d_cols);
+  if (cached || b.forced != EV_TANGENT)
+    k_assemble<<<dim3((b.max_nz + kAsmWarps - 1) / kAsmWarps, b.ncols), 32 * kAsmWarps, 0, s>>>(b.d_cols, b.d_opts,
+                                                                                                  rh92_by_warp(b) ? 1 : 0);
 }
 
 static void launch_rates_tan32(const Batch& b, cudaStream_t s) {
@@ -1334,7 +1534,6 @@ int launch_evaluation(const Batch& b, cudaStream_t s, cudaEvent_t ev0, cudaEvent
     int rc = launch_eval64(b, s);
     if (rc) return rc;
     if (ev1) JFNK_CUDA(cudaEventRecordWithFlags(ev1, s, cudaEventRecordExternal));
-    if ((rc = launch_rates_reduce(b, s))) return rc;
     launch_dJdn_update(b, s);
     if ((rc = mark(1))) return rc;
     launch_assemble(b, s);

@@ -236,6 +236,7 @@ int jfnk_server_create(jfnk_ctx* ctx, const jfnk_server_desc* d, jfnk_server** o
   b.max_nl = d->max_levels;
   b.max_overlap = d->max_trans;
   b.n_sm = ctx->n_sm;
+  b.serving = true;
   b.formal_qb = sv->mixed ? 0 : fused_default_qb(d->max_depth, d->max_mu, false);
   b.formal_kind = sv->mixed ? FORMAL_SWEEP : (b.formal_qb > 0 ? FORMAL_FUSED : FORMAL_UNFUSED);
   sv->kind = b.formal_kind;

@@ -238,16 +238,34 @@ int batch_set_forced_mode(Batch* b, int mode, cudaStream_t s) {
 // ---------------------------------------------------------------------------
 // block reductions
 // ---------------------------------------------------------------------------
-__device__ double block_sum(double v, double* sh) {
+// One warp adds the warps' sums in order and the block reads the result: FP64
+// instructions cost every warp of a scheduler 64 cycles each, so sixteen warps
+// repeating the addition (and the caller's square root) took longer than all
+// the rest of a norm (10,700 of a Krylov step's 31,000 cycles).
+template <typename F>
+__device__ double block_sum_then(double v, double* sh, F f) {
   v = warp_sum(v);
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
   __syncthreads();
   if (lane == 0) sh[wid] = v;
   __syncthreads();
-  double r = 0.0;
-  for (int i = 0; i < nw; ++i) r += sh[i];
+  if (wid == 0) {
+    double r = 0.0;
+    for (int i = 0; i < nw; ++i) r += sh[i];
+    r = f(r);
+    __syncwarp();
+    if (lane == 0) sh[0] = r;
+  }
+  __syncthreads();
+  const double r = sh[0];
   __syncthreads();
   return r;
+}
+__device__ double block_sum(double v, double* sh) {
+  return block_sum_then(v, sh, [](double r) { return r; });
+}
+__device__ double block_norm(double ss, double* sh) {   // square root of the sum
+  return block_sum_then(ss, sh, [](double r) { return sqrt(r); });
 }
 
 __device__ double block_max(double v, double* sh) {
@@ -256,8 +274,13 @@ __device__ double block_max(double v, double* sh) {
   __syncthreads();
   if (lane == 0) sh[wid] = v;
   __syncthreads();
-  double r = sh[0];
-  for (int i = 1; i < nw; ++i) r = fmax(r, sh[i]);
+  if (wid == 0) {
+    const double r = warp_max(lane < nw ? sh[lane] : sh[0]);
+    __syncwarp();
+    if (lane == 0) sh[0] = r;
+  }
+  __syncthreads();
+  const double r = sh[0];
   __syncthreads();
   return r;
 }
@@ -288,22 +311,9 @@ __device__ bool small_solve(double* A, double* b, int nl) {
   return true;
 }
 
-// RH92 update of depth k from the sums of an EV_RH92 evaluation; returns the
-// population change measure of the depth (or NaN on a singular system). With
-// clamp the correction is limited like a Newton correction (Sect. 2.2.2), so
-// that no population of the depth falls below a tenth of its old value.
-//
-// The preconditioned rate equations M n' + c0 = 0 (plus the conservation row)
-// are affine in n' and equal the residual F at n' = n, so n' = n + d with
-// M d = -F(n) and sum d = n_tot - sum n, the same update. With ``correction``
-// (mixed mode, once the iteration has settled) the correction d is solved
-// from the residual the evaluation assembled in float-pair and FP64
-// arithmetic, so that the FP32 sums in M (Psi*, the cross-coupling terms)
-// affect the speed of convergence only and not the fixed point, which is then
-// F(n) = 0 to the residual's accuracy (in optically thick lines the net rates
-// cancel far below FP32 resolution of the gross rates). Far from the
-// solution the direct form is the more robust one (M and c0 carry the same
-// rounding), so the mixed mode starts with it.
+// The RH92 update of depth k (rh92_warp in residual.cu, the same operations in
+// the same order) by one thread: large launches, which are bound by FP64
+// instructions and fill their lanes this way.
 __device__ double rh92_depth(const ColDesc& cd, int k, bool clamp, bool correction, double damp, double* out) {
   const ColTables& T = cd.t;
   const int nl = T.nl, nt = T.nt, nz = T.nz;
@@ -318,11 +328,7 @@ __device__ double rh92_depth(const ColDesc& cd, int k, bool clamp, bool correcti
     for (int j = 0; j < nl; ++j) coef[j] = 0.0;
     coef[lo] += r[0] + C[lo * nl + up];
     coef[up] -= r[1] + r[2] + C[up * nl + lo];
-    if (cd.w.cf) {   // already added per level
-      for (int j = 0; j < nl; ++j) coef[j] += r[kRhFixed + j];
-    } else {
-      for (int s = 0; s < nt; ++s) coef[T.t_up[s]] += r[kRhFixed + s];
-    }
+    for (int s = 0; s < nt; ++s) coef[T.t_up[s]] += r[kRhFixed + s];
     for (int j = 0; j < nl; ++j) {
       M[lo * nl + j] += coef[j];
       M[up * nl + j] -= coef[j];
@@ -365,6 +371,7 @@ __device__ double rh92_depth(const ColDesc& cd, int k, bool clamp, bool correcti
 // ---------------------------------------------------------------------------
 // Krylov / Newton step: one CTA per column
 // ---------------------------------------------------------------------------
+constexpr int kPinvAhead = 6;
 __device__ void apply_pinv(const ColDesc& cd, const double* in, double sign_in, const double* in2,
                            double sign_in2, double* out, bool precond = true) {
   // out = P^{-1} (sign_in in + sign_in2 in2): w.P holds the explicit block
@@ -381,10 +388,22 @@ __device__ void apply_pinv(const ColDesc& cd, const double* in, double sign_in, 
     const double* a = in + k * nl;
     const double* b2 = in2 ? in2 + k * nl : nullptr;
     double acc = 0.0;
-    for (int j = 0; j < nl; ++j) {
-      double xj = sign_in * a[j];
-      if (b2) xj += sign_in2 * b2[j];
-      acc += Pi[j] * xj;
+    for (int j0 = 0; j0 < nl; j0 += kPinvAhead) {
+      double p[kPinvAhead], xa[kPinvAhead], xb[kPinvAhead];
+#pragma unroll
+      for (int u = 0; u < kPinvAhead; ++u) {   // loads of several terms together
+        const int j = min(j0 + u, nl - 1);
+        p[u] = Pi[j];
+        xa[u] = a[j];
+        xb[u] = b2 ? b2[j] : 0.0;
+      }
+#pragma unroll
+      for (int u = 0; u < kPinvAhead; ++u)
+        if (j0 + u < nl) {
+          double xj = sign_in * xa[u];
+          if (b2) xj += sign_in2 * xb[u];
+          acc += p[u] * xj;
+        }
     }
     out[idx] = acc;
   }
@@ -491,7 +510,7 @@ constexpr int kKrylovThreads = 512;
 
 __global__ void __launch_bounds__(kKrylovThreads) k_krylov(const ColDesc* __restrict__ cols,
                                                 const SolverOpts* __restrict__ opts,
-                                                int* status_out) {
+                                                int* status_out, int rh_warp) {
   const ColDesc& cd = cols[blockIdx.x];
   const SolverOpts o = cd.opts ? *cd.opts : *opts;
   SolverState* st = cd.w.st;
@@ -532,11 +551,11 @@ __global__ void __launch_bounds__(kKrylovThreads) k_krylov(const ColDesc* __rest
     const double damp = st->rh_damp > 0.0 ? st->rh_damp : 1.0;
     const int it0 = st->rh92_iter;
     __syncthreads();
-    // the new populations are staged in w.x and committed only when every
-    // depth's update is finite
+    // the new populations are in w.x, each depth's change in w.w (rh_warp: left
+    // there by the assembly); committed only when every depth's update is finite
     double err = 0.0;
     for (int k = threadIdx.x; k < nz; k += blockDim.x) {
-      double e = rh92_depth(cd, k, o.clamp != 0, corr, damp, cd.w.x);
+      const double e = rh_warp ? cd.w.w[k] : rh92_depth(cd, k, o.clamp != 0, corr, damp, cd.w.x);
       err = (e == e) ? fmax(err, e) : INFINITY;
     }
     err = block_max(err, sh);
@@ -650,7 +669,7 @@ __global__ void __launch_bounds__(kKrylovThreads) k_krylov(const ColDesc* __rest
     __syncthreads();
     double ss = 0.0;
     for (int i = threadIdx.x; i < N; i += blockDim.x) ss += w[i] * w[i];
-    double beta = sqrt(block_sum(ss, sh));
+    double beta = block_norm(ss, sh);
     if (threadIdx.x == 0) {
       st->r0norm = beta;
       st->restarts = 0;
@@ -811,7 +830,7 @@ __global__ void __launch_bounds__(kKrylovThreads) k_krylov(const ColDesc* __rest
       __syncthreads();
       double ss = 0.0;
       for (int i = threadIdx.x; i < N; i += blockDim.x) ss += w[i] * w[i];
-      double beta = sqrt(block_sum(ss, sh));
+      double beta = block_norm(ss, sh);
       if (threadIdx.x == 0) {
         if (!(beta == beta)) { st->status = JFNK_E_NAN; s_next = NX_DONE; }
         else if (beta < o.rtol * st->r0norm) s_next = NX_NEWTON;
@@ -852,14 +871,18 @@ __global__ void __launch_bounds__(kKrylovThreads) k_krylov(const ColDesc* __rest
       }
       double ss = 0.0;
       for (int i = threadIdx.x; i < N; i += blockDim.x) ss += w[i] * w[i];
-      const double hnext = sqrt(block_sum(ss, sh));
       // the Givens state staged in shared memory by every thread, so that the
       // serial update below touches no global memory on its dependent chain
       for (int i = threadIdx.x; i < j; i += blockDim.x) {
         s_cs[i] = cd.w.cs[i];
         s_sn[i] = cd.w.sn[i];
       }
-      __syncthreads();
+      const double hnext = block_norm(ss, sh);
+      // the next basis vector beside the serial update (unused when the solve ends here)
+      if (wid > 0) {
+        double* vn = Vb + (size_t)(j + 1) * N;
+        for (int e = threadIdx.x - 32; e < N; e += blockDim.x - 32) vn[e] = w[e] / hnext;
+      }
       if (threadIdx.x == 0) {
         double* Hh = cd.w.Hh;
         double* gv = cd.w.gv;
@@ -892,7 +915,6 @@ __global__ void __launch_bounds__(kKrylovThreads) k_krylov(const ColDesc* __rest
         }
         s_next = nx;
         s_solve = solve;
-        s_val = hnext;
       }
       __syncthreads();
       if (s_solve) {
@@ -919,13 +941,7 @@ __global__ void __launch_bounds__(kKrylovThreads) k_krylov(const ColDesc* __rest
         return;
       }
       if (next == NX_NONE) {
-        const double hn = s_val;
-        double* vn = Vb + (size_t)(j + 1) * N;
-        for (int e = threadIdx.x; e < N; e += blockDim.x) vn[e] = w[e] / hn;
-        if (o.jvp) {
-          __syncthreads();
-          fd_prepare(cd, st, o.jvp, vn, +1, sh);
-        }
+        if (o.jvp) fd_prepare(cd, st, o.jvp, Vb + (size_t)(j + 1) * N, +1, sh);
         if (threadIdx.x == 0) { st->j = j + 1; st->phase = PH_JVP; status_out[blockIdx.x] = st->status; }
         return;
       }
@@ -979,17 +995,19 @@ __global__ void __launch_bounds__(kKrylovThreads) k_krylov(const ColDesc* __rest
   }
 }
 
-int launch_krylov_step(const Batch& b, cudaStream_t s) {
-  k_krylov<<<b.ncols, kKrylovThreads, 0, s>>>(b.d_cols, b.d_opts, b.d_status);
-  JFNK_CUDA(cudaGetLastError());
-  return JFNK_OK;
+// A warp per depth finishes one column's RH92 update in about 10 us (one thread
+// per depth: 100 us) but uses a fifth of its lanes: above about 50 columns of
+// 82 depths the FP64 instructions take longer than the latency saved (512
+// columns: 205.8 against 200.2 ms a solve). A server's slots are a quarter
+// or less in RH92 iterations at a time (48 slots: 253.7 against 265.1 ms).
+bool rh92_by_warp(const Batch& b) {
+  return b.formal_kind == FORMAL_CACHED || (long)b.ncols * b.max_nz < (b.serving ? 104L : 26L) * b.n_sm;
 }
 
-__global__ void k_rh92_apply(const ColDesc* __restrict__ cols) {
-  const ColDesc& cd = cols[blockIdx.y];
-  const int k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= cd.t.nz) return;
-  rh92_depth(cd, k, false, false, 1.0, cd.w.n);   // the plain update: jfnk_rh92_update applies no limiting
+int launch_krylov_step(const Batch& b, cudaStream_t s) {
+  k_krylov<<<b.ncols, kKrylovThreads, 0, s>>>(b.d_cols, b.d_opts, b.d_status, rh92_by_warp(b) ? 1 : 0);
+  JFNK_CUDA(cudaGetLastError());
+  return JFNK_OK;
 }
 
 // Zero-radiation initial guess (Sect. 2.2.1): the rate equations with I = 0,
@@ -1033,13 +1051,6 @@ __global__ void k_zero_radiation(const ColDesc* __restrict__ cols) {
 int launch_zero_radiation(const Batch& b, cudaStream_t s) {
   dim3 g((b.max_nz + 63) / 64, b.ncols);
   k_zero_radiation<<<g, 64, 0, s>>>(b.d_cols);
-  JFNK_CUDA(cudaGetLastError());
-  return JFNK_OK;
-}
-
-int launch_rh92_update(const Batch& b, cudaStream_t s) {
-  dim3 g((b.max_nz + 63) / 64, b.ncols);
-  k_rh92_apply<<<g, 64, 0, s>>>(b.d_cols);
   JFNK_CUDA(cudaGetLastError());
   return JFNK_OK;
 }

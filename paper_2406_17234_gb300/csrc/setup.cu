@@ -226,76 +226,132 @@ struct AtomDev {
   double mass;
 };
 
-__global__ void k_lte(AtomDev at, int nz, const double* T, const double* ne, const double* ntot,
-                      double* nstar) {
-  int k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= nz) return;
-  double kT = kKB * T[k];
-  int smin = at.stage[0];
-  for (int l = 1; l < at.nl; ++l) smin = min(smin, at.stage[l]);
-  double lsaha = log(2.0 * pow(2.0 * kPi * kME * kKB * T[k] / (kH * kH), 1.5) / ne[k]);
-  double lw[kMaxL];
-  double mx = -1e300;
-  for (int l = 0; l < at.nl; ++l) {
-    lw[l] = log(at.g[l]) - at.E[l] * kEV / kT + (at.stage[l] - smin) * lsaha;
-    mx = fmax(mx, lw[l]);
-  }
-  double s = 0.0;
-  for (int l = 0; l < at.nl; ++l) { lw[l] = exp(lw[l] - mx); s += lw[l]; }
-  for (int l = 0; l < at.nl; ++l) nstar[k * at.nl + l] = ntot[k] * lw[l] / s;
-}
-
-__global__ void k_planck_background(int nq, int nz, const double* nu, const double* T,
-                                    const double* rho, const double* ne, double kappa,
-                                    double kappa_nu_ref, double kappa_power, double kappa_max,
-                                    int thomson, double* Bn, double* chi_c, double* eta_c,
-                                    double* chi_sca) {
-  int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= nq * nz) return;
-  int q = i / nz, k = i % nz;
-  double v = nu[q];
-  double B = (2.0 * kH * v * v * v / (kC * kC)) / expm1(kH * v / (kKB * T[k]));
-  double kap = kappa;
-  if (kappa_power != 0.0) kap = kappa * fmin(kappa_max, fmax(1.0, pow(v / kappa_nu_ref, kappa_power)));
-  double cc = (kappa != 0.0) ? kap * rho[k] : 0.0;
-  Bn[i] = B;
-  chi_c[i] = cc;
-  eta_c[i] = cc * B;
-  if (q == 0) chi_sca[k] = thomson ? kSigmaT * ne[k] : 0.0;
-}
-
 struct TransDev {
   int kind, lo, up;
   double nu0, f, damping, alpha0;
 };
+struct CollDev {
+  int kind, lo, up;
+  double nu0, f, upsilon, eps, q0;
+};
 
-// V and g on every window point of every transition (Eqs. Vij, Vij2, gij);
+// Inputs and outputs of the first set-up launch.
+struct SetupIn {
+  AtomDev at;
+  int nz, nq, nl, nt, nwin, thomson;
+  const TransDev* tr;
+  const CollDev* cd;
+  const int *t_q0, *t_base, *winT;
+  const double *nu, *T, *ne, *ntot, *rho, *vturb;
+  double kappa, kappa_nu_ref, kappa_power, kappa_max;
+  double *V, *G, *Bn, *chi_c, *eta_c, *chi_sca, *nstar, *C;
+};
+
+// V and g on window point p of its transition at depth k (Eqs. Vij, Vij2, gij);
 // line profiles unnormalised here.
-__global__ void k_window_tables(int nt, const TransDev* tr, const int* t_q0, const int* t_base,
-                                const int* win_t, int nwin, int nz, const double* nu,
-                                const double* T, const double* ne, const double* vturb,
-                                AtomDev at, double* V, double* G) {
-  int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= nwin * nz) return;
-  int p = i / nz, k = i % nz;
-  int t = win_t[p];
-  const TransDev d = tr[t];
-  int q = t_q0[t] + (p - t_base[t]);
-  double v = nu[q];
-  double kT = kKB * T[k];
+__device__ void window_point(const SetupIn& a, int i) {
+  const int p = i / a.nz, k = i % a.nz;
+  const int t = a.winT[p];
+  const TransDev d = a.tr[t];
+  const AtomDev& at = a.at;
+  const double v = a.nu[a.t_q0[t] + (p - a.t_base[t])];
+  const double kT = kKB * a.T[k];
   if (d.kind == 0) {
-    double vt = vturb ? vturb[k] : 0.0;
-    double dnud = d.nu0 / kC * sqrt(2.0 * kKB * T[k] / (at.mass * kAMU) + vt * vt);
-    double x = (v - d.nu0) / dnud;
-    double phi = voigt_H(d.damping, x) / (1.7724538509055160273 * dnud);
-    V[i] = (kPi * kQE * kQE / (kME * kC)) * d.f * phi;
-    G[i] = at.g[d.lo] / at.g[d.up];
+    const double vt = a.vturb ? a.vturb[k] : 0.0;
+    const double dnud = d.nu0 / kC * sqrt(2.0 * kKB * a.T[k] / (at.mass * kAMU) + vt * vt);
+    const double x = (v - d.nu0) / dnud;
+    const double phi = voigt_H(d.damping, x) / (1.7724538509055160273 * dnud);
+    a.V[i] = (kPi * kQE * kQE / (kME * kC)) * d.f * phi;
+    a.G[i] = at.g[d.lo] / at.g[d.up];
   } else {
-    double r = d.nu0 / v;
-    V[i] = d.alpha0 * r * r * r;
-    double phi_saha = (at.g[d.lo] / (2.0 * at.g[d.up])) *
-                      pow(kH * kH / (2.0 * kPi * kME * kKB * T[k]), 1.5);
-    G[i] = ne[k] * phi_saha * exp(((at.E[d.up] - at.E[d.lo]) * kEV - kH * v) / kT);
+    const double r = d.nu0 / v;
+    a.V[i] = d.alpha0 * r * r * r;
+    const double phi_saha = (at.g[d.lo] / (2.0 * at.g[d.up])) * pow(kH * kH / (2.0 * kPi * kME * kKB * a.T[k]), 1.5);
+    a.G[i] = a.ne[k] * phi_saha * exp(((at.E[d.up] - at.E[d.lo]) * kEV - kH * v) / kT);
+  }
+}
+
+// Planck function and background continuum at (nu, k).
+__device__ void background_point(const SetupIn& a, int i) {
+  const int q = i / a.nz, k = i % a.nz;
+  const double v = a.nu[q];
+  const double B = (2.0 * kH * v * v * v / (kC * kC)) / expm1(kH * v / (kKB * a.T[k]));
+  double kap = a.kappa;
+  if (a.kappa_power != 0.0) kap = a.kappa * fmin(a.kappa_max, fmax(1.0, pow(v / a.kappa_nu_ref, a.kappa_power)));
+  const double cc = (a.kappa != 0.0) ? kap * a.rho[k] : 0.0;
+  a.Bn[i] = B;
+  a.chi_c[i] = cc;
+  a.eta_c[i] = cc * B;
+  if (q == 0) a.chi_sca[k] = a.thomson ? kSigmaT * a.ne[k] : 0.0;
+}
+
+// LTE populations (levels on the lanes) and collision rates (transitions on the
+// lanes, added in transition order) of depth k, one warp; C: its block in
+// shared memory.
+__device__ void depth_point(const SetupIn& a, int k, int lane, double* C) {
+  const AtomDev& at = a.at;
+  const int nl = a.nl, nt = a.nt;
+  const double Tk = a.T[k], kT = kKB * Tk;
+  int smin = at.stage[0];
+  for (int l = 1; l < nl; ++l) smin = min(smin, at.stage[l]);
+  const double lsaha = log(2.0 * pow(2.0 * kPi * kME * kKB * Tk / (kH * kH), 1.5) / a.ne[k]);
+  double lw = -1e300;
+  if (lane < nl) lw = log(at.g[lane]) - at.E[lane] * kEV / kT + (at.stage[lane] - smin) * lsaha;
+  const double mx = warp_max(lw);
+  lw = lane < nl ? exp(lw - mx) : 0.0;
+  double s = 0.0;
+  for (int l = 0; l < nl; ++l) s += __shfl_sync(0xffffffffu, lw, l);
+  if (lane < nl) a.nstar[(size_t)k * nl + lane] = a.ntot[k] * lw / s;
+  double up = 0.0, down = 0.0;
+  if (lane < nt) {
+    const CollDev d = a.cd[lane];
+    const double gi = at.g[d.lo], gj = at.g[d.up];
+    if (d.kind == 0) {
+      const double hnu_kt = kH * d.nu0 / kT;
+      if (d.eps > 0.0) {
+        const double Aji = 8.0 * kPi * kPi * kQE * kQE * d.nu0 * d.nu0 / (kME * kC * kC * kC) * (gi / gj) * d.f;
+        down = d.eps * Aji / ((1.0 - d.eps) * (-expm1(-hnu_kt)));
+      } else {
+        down = 8.63e-6 * a.ne[k] * d.upsilon / (gj * sqrt(Tk));
+      }
+      up = down * (gj / gi) * exp(-hnu_kt);
+    } else {
+      const double dE = (at.E[d.up] - at.E[d.lo]) * kEV;
+      up = a.ne[k] * d.q0 * sqrt(Tk) * exp(-dE / kT);
+      const double ratio = a.ne[k] * (gi / (2.0 * gj)) * pow(kH * kH / (2.0 * kPi * kME * kT), 1.5) * exp(dE / kT);
+      down = up * ratio;
+    }
+  }
+  for (int i = lane; i < nl * nl; i += 32) C[i] = 0.0;
+  __syncwarp();
+  for (int t = 0; t < nt; ++t) {
+    if (lane == t) {
+      const int lo = a.cd[t].lo, u = a.cd[t].up;
+      C[u * nl + lo] += down;
+      C[lo * nl + u] += up;
+    }
+    __syncwarp();
+  }
+  for (int i = lane; i < nl * nl; i += 32) a.C[(size_t)k * nl * nl + i] = C[i];
+}
+
+// First set-up launch: everything that depends on the descriptors alone, side
+// by side in one grid (window tables, then background, then depths): 150 us of
+// an H I-like column's tables (15 transitions, 82 depths) where the separate
+// launches took 150 + 57 + 51 + 23 us one after the other.
+constexpr int kSetupThreads = 256;
+__global__ void __launch_bounds__(kSetupThreads) k_setup_points(SetupIn a, int nb_win, int nb_bg) {
+  __shared__ double s_C[kSetupThreads / 32][kMaxL * kMaxL];
+  const int b = blockIdx.x;
+  if (b < nb_win) {
+    const int i = b * kSetupThreads + threadIdx.x;
+    if (i < a.nwin * a.nz) window_point(a, i);
+  } else if (b < nb_win + nb_bg) {
+    const int i = (b - nb_win) * kSetupThreads + threadIdx.x;
+    if (i < a.nq * a.nz) background_point(a, i);
+  } else {
+    const int wid = threadIdx.x >> 5, k = (b - nb_win - nb_bg) * (kSetupThreads / 32) + wid;
+    if (k < a.nz) depth_point(a, k, threadIdx.x & 31, s_C[wid]);
   }
 }
 
@@ -326,125 +382,137 @@ __global__ void k_window_tables_dir(int nt, const TransDev* tr, const int* t_q0,
   Vd[i] = (kPi * kQE * kQE / (kME * kC)) * d.f * voigt_H(d.damping, x) / (1.7724538509055160273 * dnud);
 }
 
-// Float copies of the (normalised) window tables for mixed-mode tangents.
-__global__ void k_float_copy(int nwin, int nz, const double* V, const double* G, float* V32, float* G32,
-                             float2* VG32T) {
-  const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= (size_t)nwin * nz) return;
-  const size_t p = i / nz, k = i % nz;
-  const float v = (float)V[i], g = (float)G[i];
-  V32[i] = v;
-  G32[i] = g;
-  VG32T[k * nwin + p] = make_float2(v, g);
+// sum_p a_p b_p over a window of nw points in window order (one chain of FMAs
+// per lane, by warp 0), the terms formed by the block's other warps a chunk
+// ahead: term(p, a, b). The result is on warp 0's lanes. One thread walking
+// the window alone waited for memory, and for an FP64 division in the
+// normalisation, at every point (200 and 360 us of an H I-like column's
+// set-up); the order is kept, so that the tables are the same to the last bit.
+constexpr int kWinWarps = 8;
+constexpr int kWinChunk = 56;   // points per chunk: eight per producing warp
+struct WinBuf {
+  double a[2][kWinChunk][32];
+  double b[2][kWinChunk];
+};
+template <typename Term>
+__device__ __forceinline__ double window_sum(int nw, WinBuf& s, Term term) {
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  double sum = 0.0;
+  const int nch = (nw + kWinChunk - 1) / kWinChunk;
+  for (int c = 0; c <= nch; ++c) {
+    if (wid > 0) {
+      if (c < nch) {
+        const int p0 = c * kWinChunk, np = min(kWinChunk, nw - p0);
+#pragma unroll 4
+        for (int i = wid - 1; i < np; i += kWinWarps - 1) {
+          double a, b;
+          term(p0 + i, a, b);
+          s.a[c & 1][i][lane] = a;
+          if (lane == 0) s.b[c & 1][i] = b;
+        }
+      }
+    } else if (c > 0) {
+      const int p0 = (c - 1) * kWinChunk, np = min(kWinChunk, nw - p0);
+#pragma unroll 8
+      for (int i = 0; i < np; ++i) sum = fma(s.b[(c - 1) & 1][i], s.a[(c - 1) & 1][i][lane], sum);
+    }
+    __syncthreads();
+  }
+  return sum;
 }
 
 // Renormalise each line profile so that sum_q omega_t(q) phi(q, k) = 1 (for
-// every direction's copy when ndir > 1: the tables follow one another).
-__global__ void k_normalise_lines(int nt, const TransDev* tr, const int* t_q0, const int* t_q1,
-                                  const int* t_base, const double* t_w, int nz, double* V, int ndir = 1,
-                                  size_t dir_stride = 0) {
-  int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= nt * nz * ndir) return;
-  const int dd = i / (nt * nz);
-  i -= dd * nt * nz;
-  V += (size_t)dd * dir_stride;
-  int t = i / nz, k = i % nz;
+// every direction's copy: the tables follow one another); block per
+// (32 depths, transition, direction).
+__global__ void __launch_bounds__(32 * kWinWarps) k_normalise_lines(const TransDev* tr, const int* t_q0,
+                                                                    const int* t_q1, const int* t_base,
+                                                                    const double* t_w, int nz, double* V,
+                                                                    size_t dir_stride = 0) {
+  const int t = blockIdx.y, lane = threadIdx.x & 31, wid = threadIdx.x >> 5, k = blockIdx.x * 32 + lane;
   const TransDev d = tr[t];
   if (d.kind != 0) return;
-  int nw = t_q1[t] - t_q0[t] + 1;
-  double* Vt = V + (size_t)t_base[t] * nz;
-  const double* w = t_w + t_base[t];
-  double s = 0.0;
-  const double scale = (kPi * kQE * kQE / (kME * kC)) * d.f;
-  for (int p = 0; p < nw; ++p) s += w[p] * (Vt[(size_t)p * nz + k] / scale);
-  if (s > 0.0)
-    for (int p = 0; p < nw; ++p) Vt[(size_t)p * nz + k] /= s;
-}
-
-// Products of the window tables per (window point, depth): g V (stimulated
-// emission and emissivity, Eqs. chi, eta) and the rate-integral weights W V and
-// W g V with W = omega_t(nu_q) 4 pi/(h nu_q) (Eqs. Rij, Rji), so that each term
-// of those sums takes one product.
-__global__ void k_rate_weights(int nwin, int nz, const int* winT, const int* t_q0, const int* t_base,
-                               const double* t_w, const double* rw, const double* V, const double* G,
-                               double* gV, double* WV, double* WgV) {
-  const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= (size_t)nwin * nz) return;
-  const int p = (int)(i / nz);
-  const int t = winT[p];
-  const double W = t_w[p] * rw[t_q0[t] + p - t_base[t]];
-  const double wv = W * V[i];
-  gV[i] = G[i] * V[i];
-  WV[i] = wv;
-  WgV[i] = wv * G[i];
-}
-
-// The population-independent part of R_ji (Eq. Rji): sum over the window of
-// W g V 2 h nu^3/c^2, in window order.
-__global__ void k_spontaneous(int nt, int nz, const int* t_q0, const int* t_q1, const int* t_base,
-                              const double* c2, const double* WgV, double* Rsp) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= nt * nz) return;
-  const int t = i / nz, k = i % nz;
+  __shared__ WinBuf buf;
+  __shared__ double s_sum[32];
   const int nw = t_q1[t] - t_q0[t] + 1;
-  const double* w = WgV + (size_t)t_base[t] * nz + k;
-  double s = 0.0;
-  for (int p = 0; p < nw; ++p) s += w[(size_t)p * nz] * c2[t_q0[t] + p];
-  Rsp[i] = s;
+  double* Vt = V + (size_t)blockIdx.z * dir_stride + (size_t)t_base[t] * nz + min(k, nz - 1);
+  const double* w = t_w + t_base[t];
+  const double scale = (kPi * kQE * kQE / (kME * kC)) * d.f;
+  const double sum = window_sum(nw, buf, [&](int p, double& a, double& b) {
+    a = Vt[(size_t)p * nz] / scale;
+    b = w[p];
+  });
+  if (wid == 0) s_sum[lane] = sum;
+  __syncthreads();
+  const double s = s_sum[lane];
+  if (k < nz && s > 0.0)
+    for (int p = wid; p < nw; p += kWinWarps) Vt[(size_t)p * nz] /= s;
 }
 
-// Float-pair copies of FP64 tables (the mixed mode's base evaluations).
-__global__ void k_pairs(const double* src, float2* dst, size_t n) {
-  const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) {
-    const df p = df_from_double(src[i]);
-    dst[i] = make_float2(p.hi, p.lo);
-  }
-}
-// chi_c + chi_sca per (nu, depth), summed in FP64, as pairs
-__global__ void k_chibg_pairs(int nq, int nz, const double* chi_c, const double* chi_sca, float2* dst) {
-  const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < (size_t)nq * nz) {
-    const df p = df_from_double(chi_c[i] + chi_sca[i % nz]);
-    dst[i] = make_float2(p.hi, p.lo);
-  }
-}
-
-struct CollDev {
-  int kind, lo, up;
-  double nu0, f, upsilon, eps, q0;
+// Inputs and outputs of the last set-up launch.
+struct ProductsIn {
+  int nz, nq, nt, nwin;
+  const int *winT, *t_q0, *t_q1, *t_base;
+  const double *t_w, *rw, *c2, *V, *G, *chi_c, *eta_c, *chi_sca;
+  double *gV, *WV, *WgV, *Rsp;
+  float2 *V2, *gV2, *VG32T, *etac2, *chibg2, *chisca2;
+  float *V32, *G32;
 };
 
-__global__ void k_collisions(int nt, const CollDev* cd, AtomDev at, int nz, const double* T,
-                             const double* ne, double* C) {
-  int k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= nz) return;
-  const int nl = at.nl;
-  double* Ck = C + (size_t)k * nl * nl;
-  for (int i = 0; i < nl * nl; ++i) Ck[i] = 0.0;
-  double Tk = T[k], kT = kKB * Tk;
-  for (int t = 0; t < nt; ++t) {
-    const CollDev d = cd[t];
-    double gi = at.g[d.lo], gj = at.g[d.up];
-    if (d.kind == 0) {
-      double hnu_kt = kH * d.nu0 / kT;
-      double down;
-      if (d.eps > 0.0) {
-        double Aji = 8.0 * kPi * kPi * kQE * kQE * d.nu0 * d.nu0 / (kME * kC * kC * kC) * (gi / gj) * d.f;
-        down = d.eps * Aji / ((1.0 - d.eps) * (-expm1(-hnu_kt)));
-      } else {
-        down = 8.63e-6 * ne[k] * d.upsilon / (gj * sqrt(Tk));
-      }
-      Ck[d.up * nl + d.lo] += down;
-      Ck[d.lo * nl + d.up] += down * (gj / gi) * exp(-hnu_kt);
-    } else {
-      double dE = (at.E[d.up] - at.E[d.lo]) * kEV;
-      double up = ne[k] * d.q0 * sqrt(Tk) * exp(-dE / kT);
-      double ratio = ne[k] * (gi / (2.0 * gj)) * pow(kH * kH / (2.0 * kPi * kME * kT), 1.5) * exp(dE / kT);
-      Ck[d.lo * nl + d.up] += up;
-      Ck[d.up * nl + d.lo] += up * ratio;
-    }
+__device__ __forceinline__ float2 pair_of(double x) {
+  const df p = df_from_double(x);
+  return make_float2(p.hi, p.lo);
+}
+
+// Last set-up launch, side by side in one grid (it was eight launches): per
+// (window point, depth) the products g V (stimulated emission and emissivity,
+// Eqs. chi, eta) and the rate-integral weights W V and W g V with W =
+// omega_t(nu_q) 4 pi/(h nu_q) (Eqs. Rij, Rji), so that each term of those sums
+// takes one product, with the float and float-pair copies of the mixed mode;
+// per (nu, depth) the pairs of the background terms; and per (transition, 32
+// depths) the population-independent part of R_ji (Eq. Rji), sum over the
+// window of W g V 2 h nu^3/c^2, in window order.
+__global__ void __launch_bounds__(kSetupThreads) k_setup_products(ProductsIn a, int nb_sp, int nb_win) {
+  static_assert(kSetupThreads == 32 * kWinWarps, "the window is split over the block's warps");
+  __shared__ WinBuf buf;
+  const int nz = a.nz;
+  int b = blockIdx.x;
+  if (b < nb_sp) {
+    const int tiles = (nz + 31) / 32, t = b / tiles, lane = threadIdx.x & 31;
+    const int k = (b - t * tiles) * 32 + lane, kc = min(k, nz - 1);
+    const int q0 = a.t_q0[t], nw = a.t_q1[t] - q0 + 1, base = a.t_base[t];
+    const double s = window_sum(nw, buf, [&](int p, double& x, double& y) {
+      const size_t i = (size_t)(base + p) * nz + kc;
+      const double W = a.t_w[base + p] * a.rw[q0 + p];
+      x = (W * a.V[i]) * a.G[i];
+      y = a.c2[q0 + p];
+    });
+    if (threadIdx.x < 32 && k < nz) a.Rsp[(size_t)t * nz + k] = s;
+    return;
   }
+  b -= nb_sp;
+  if (b < nb_win) {
+    const size_t i = (size_t)b * kSetupThreads + threadIdx.x;
+    if (i >= (size_t)a.nwin * nz) return;
+    const int p = (int)(i / nz), k = (int)(i % nz), t = a.winT[p];
+    const double W = a.t_w[p] * a.rw[a.t_q0[t] + p - a.t_base[t]], V = a.V[i], G = a.G[i];
+    const double gV = G * V, wv = W * V;
+    a.gV[i] = gV;
+    a.WV[i] = wv;
+    a.WgV[i] = wv * G;
+    a.V2[i] = pair_of(V);
+    a.gV2[i] = pair_of(gV);
+    const float v = (float)V, g = (float)G;
+    a.V32[i] = v;
+    a.G32[i] = g;
+    a.VG32T[(size_t)k * a.nwin + p] = make_float2(v, g);
+    return;
+  }
+  const size_t i = (size_t)(b - nb_win) * kSetupThreads + threadIdx.x;
+  if (i >= (size_t)a.nq * nz) return;
+  const double sca = a.chi_sca[i % nz];
+  a.etac2[i] = pair_of(a.eta_c[i]);
+  a.chibg2[i] = pair_of(a.chi_c[i] + sca);   // summed in FP64
+  if (i < (size_t)nz) a.chisca2[i] = pair_of(sca);
 }
 
 // ---------------------------------------------------------------------------
@@ -655,50 +723,51 @@ int build_atmosphere(jfnk_ctx* ctx, int lane, const AtomData& A, const jfnk_atmo
   for (int l = 0; l < nl; ++l) { at.E[l] = A.E[l]; at.g[l] = A.g[l]; at.stage[l] = A.stage[l]; }
   double* T = ar.ptr<double>(o_T);
   double* ne = ar.ptr<double>(o_ne);
-  const int tb = 256;
-  k_lte<<<(nz + tb - 1) / tb, tb, 0, s>>>(at, nz, T, ne, ar.ptr<double>(o_ntot), ar.ptr<double>(o_nstar));
-  k_planck_background<<<(nq * nz + tb - 1) / tb, tb, 0, s>>>(
-      nq, nz, ar.ptr<double>(o_nu), T, ar.ptr<double>(o_rho), ne, d->kappa, d->kappa_nu_ref,
-      d->kappa_power, d->kappa_max, d->thomson, ar.ptr<double>(o_B), ar.ptr<double>(o_chic),
-      ar.ptr<double>(o_etac), ar.ptr<double>(o_sca));
-  k_window_tables<<<(int)(((size_t)nwin * nz + tb - 1) / tb), tb, 0, s>>>(
-      nt, ar.ptr<TransDev>(o_tr), ar.ptr<int>(o_tq0), ar.ptr<int>(o_tbase), ar.ptr<int>(o_winT),
-      nwin, nz, ar.ptr<double>(o_nu), T, ne, d->vturb ? ar.ptr<double>(o_vt) : nullptr, at,
-      ar.ptr<double>(o_V), ar.ptr<double>(o_G));
-  k_normalise_lines<<<(nt * nz + tb - 1) / tb, tb, 0, s>>>(
-      nt, ar.ptr<TransDev>(o_tr), ar.ptr<int>(o_tq0), ar.ptr<int>(o_tq1), ar.ptr<int>(o_tbase),
-      ar.ptr<double>(o_tw), nz, ar.ptr<double>(o_V));
+  const int tb = kSetupThreads;
+  auto blocks = [&](size_t n) { return (int)((n + tb - 1) / tb); };
+  const size_t nwz = (size_t)nwin * nz, nqz = (size_t)nq * nz;
+  {
+    SetupIn a{};
+    a.at = at;
+    a.nz = nz; a.nq = nq; a.nl = nl; a.nt = nt; a.nwin = nwin; a.thomson = d->thomson;
+    a.tr = ar.ptr<TransDev>(o_tr); a.cd = ar.ptr<CollDev>(o_cd);
+    a.t_q0 = ar.ptr<int>(o_tq0); a.t_base = ar.ptr<int>(o_tbase); a.winT = ar.ptr<int>(o_winT);
+    a.nu = ar.ptr<double>(o_nu); a.T = T; a.ne = ne; a.ntot = ar.ptr<double>(o_ntot); a.rho = ar.ptr<double>(o_rho);
+    a.vturb = d->vturb ? ar.ptr<double>(o_vt) : nullptr;
+    a.kappa = d->kappa; a.kappa_nu_ref = d->kappa_nu_ref; a.kappa_power = d->kappa_power; a.kappa_max = d->kappa_max;
+    a.V = ar.ptr<double>(o_V); a.G = ar.ptr<double>(o_G); a.Bn = ar.ptr<double>(o_B);
+    a.chi_c = ar.ptr<double>(o_chic); a.eta_c = ar.ptr<double>(o_etac); a.chi_sca = ar.ptr<double>(o_sca);
+    a.nstar = ar.ptr<double>(o_nstar); a.C = ar.ptr<double>(o_C);
+    const int bw = blocks(nwz), bg = blocks(nqz), bd = (nz + tb / 32 - 1) / (tb / 32);
+    k_setup_points<<<bw + bg + bd, tb, 0, s>>>(a, bw, bg);
+  }
+  k_normalise_lines<<<dim3((nz + 31) / 32, nt), 32 * kWinWarps, 0, s>>>(
+      ar.ptr<TransDev>(o_tr), ar.ptr<int>(o_tq0), ar.ptr<int>(o_tq1), ar.ptr<int>(o_tbase), ar.ptr<double>(o_tw), nz,
+      ar.ptr<double>(o_V));
   if (M->moving) {
-    const size_t nd = 2 * (size_t)nmu, per = (size_t)nwin * nz;
-    k_window_tables_dir<<<(int)((nd * per + tb - 1) / tb), tb, 0, s>>>(
+    const size_t nd = 2 * (size_t)nmu;
+    k_window_tables_dir<<<blocks(nd * nwz), tb, 0, s>>>(
         nt, ar.ptr<TransDev>(o_tr), ar.ptr<int>(o_tq0), ar.ptr<int>(o_tbase), ar.ptr<int>(o_winT), nwin, nz, nmu,
         ar.ptr<double>(o_nu), T, d->vturb ? ar.ptr<double>(o_vt) : nullptr, ar.ptr<double>(o_vlos),
         ar.ptr<double>(o_mu), at, ar.ptr<double>(o_V), ar.ptr<double>(o_Vd));
-    k_normalise_lines<<<(int)((nd * nt * nz + tb - 1) / tb), tb, 0, s>>>(
-        nt, ar.ptr<TransDev>(o_tr), ar.ptr<int>(o_tq0), ar.ptr<int>(o_tq1), ar.ptr<int>(o_tbase),
-        ar.ptr<double>(o_tw), nz, ar.ptr<double>(o_Vd), (int)nd, per);
+    k_normalise_lines<<<dim3((nz + 31) / 32, nt, (unsigned)nd), 32 * kWinWarps, 0, s>>>(
+        ar.ptr<TransDev>(o_tr), ar.ptr<int>(o_tq0), ar.ptr<int>(o_tq1), ar.ptr<int>(o_tbase), ar.ptr<double>(o_tw), nz,
+        ar.ptr<double>(o_Vd), nwz);
   }
-  k_rate_weights<<<(int)(((size_t)nwin * nz + tb - 1) / tb), tb, 0, s>>>(
-      nwin, nz, ar.ptr<int>(o_winT), ar.ptr<int>(o_tq0), ar.ptr<int>(o_tbase), ar.ptr<double>(o_tw),
-      ar.ptr<double>(o_rw), ar.ptr<double>(o_V), ar.ptr<double>(o_G), ar.ptr<double>(o_gV),
-      ar.ptr<double>(o_WV), ar.ptr<double>(o_WgV));
-  k_spontaneous<<<(nt * nz + tb - 1) / tb, tb, 0, s>>>(nt, nz, ar.ptr<int>(o_tq0), ar.ptr<int>(o_tq1),
-                                                        ar.ptr<int>(o_tbase), ar.ptr<double>(o_c2),
-                                                        ar.ptr<double>(o_WgV), ar.ptr<double>(o_Rsp));
   {
-    const size_t nwz = (size_t)nwin * nz, nqz = (size_t)nq * nz;
-    k_pairs<<<(int)((nwz + tb - 1) / tb), tb, 0, s>>>(ar.ptr<double>(o_V), ar.ptr<float2>(o_V2), nwz);
-    k_pairs<<<(int)((nwz + tb - 1) / tb), tb, 0, s>>>(ar.ptr<double>(o_gV), ar.ptr<float2>(o_gV2), nwz);
-    k_pairs<<<(int)((nqz + tb - 1) / tb), tb, 0, s>>>(ar.ptr<double>(o_etac), ar.ptr<float2>(o_etac2), nqz);
-    k_pairs<<<(nz + tb - 1) / tb, tb, 0, s>>>(ar.ptr<double>(o_sca), ar.ptr<float2>(o_chisca2), (size_t)nz);
-    k_chibg_pairs<<<(int)((nqz + tb - 1) / tb), tb, 0, s>>>(nq, nz, ar.ptr<double>(o_chic), ar.ptr<double>(o_sca),
-                                                            ar.ptr<float2>(o_chibg2));
+    ProductsIn a{};
+    a.nz = nz; a.nq = nq; a.nt = nt; a.nwin = nwin;
+    a.winT = ar.ptr<int>(o_winT); a.t_q0 = ar.ptr<int>(o_tq0); a.t_q1 = ar.ptr<int>(o_tq1);
+    a.t_base = ar.ptr<int>(o_tbase); a.t_w = ar.ptr<double>(o_tw); a.rw = ar.ptr<double>(o_rw);
+    a.c2 = ar.ptr<double>(o_c2); a.V = ar.ptr<double>(o_V); a.G = ar.ptr<double>(o_G);
+    a.chi_c = ar.ptr<double>(o_chic); a.eta_c = ar.ptr<double>(o_etac); a.chi_sca = ar.ptr<double>(o_sca);
+    a.gV = ar.ptr<double>(o_gV); a.WV = ar.ptr<double>(o_WV); a.WgV = ar.ptr<double>(o_WgV);
+    a.Rsp = ar.ptr<double>(o_Rsp); a.V2 = ar.ptr<float2>(o_V2); a.gV2 = ar.ptr<float2>(o_gV2);
+    a.VG32T = ar.ptr<float2>(o_VG32T); a.etac2 = ar.ptr<float2>(o_etac2); a.chibg2 = ar.ptr<float2>(o_chibg2);
+    a.chisca2 = ar.ptr<float2>(o_chisca2); a.V32 = ar.ptr<float>(o_V32); a.G32 = ar.ptr<float>(o_G32);
+    const int bs = nt * ((nz + 31) / 32), bw = blocks(nwz), bg = blocks(nqz);
+    k_setup_products<<<bs + bw + bg, tb, 0, s>>>(a, bs, bw);
   }
-  k_collisions<<<(nz + tb - 1) / tb, tb, 0, s>>>(nt, ar.ptr<CollDev>(o_cd), at, nz, T, ne,
-                                                  ar.ptr<double>(o_C));
-  k_float_copy<<<(int)(((size_t)nwin * nz + tb - 1) / tb), tb, 0, s>>>(
-      nwin, nz, ar.ptr<double>(o_V), ar.ptr<double>(o_G), ar.ptr<float>(o_V32), ar.ptr<float>(o_G32),
-      ar.ptr<float2>(o_VG32T));
   JFNK_CUDA(cudaGetLastError());
   JFNK_CUDA(cudaEventRecord(ctx->setup_done[lane], s));
   ColTables& tb_ = M->tables;

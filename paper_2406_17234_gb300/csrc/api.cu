@@ -366,7 +366,7 @@ int ensure_dJdn(Batch* b, cudaStream_t s) {
 static int prepare_solve(Batch* b, const std::vector<const jfnk_atmos*>& cols,
                          const jfnk_options* o, double* const* n_in, double* const* J_in,
                          jfnk_mem where, cudaStream_t s) {
-  if (b->formal_kind == FORMAL_MOVING &&
+  if (kind_moving(b->formal_kind) &&
       (o->rh92_warmup > 0 || o->solver != JFNK_SOLVER_JFNK || o->precond > 1))
     return fail(JFNK_E_INVALID,
                 "moving columns: Algorithm 2 without an RH92 start, with the first preconditioner solution or none");
@@ -491,14 +491,14 @@ static int finish_solve(Batch* b, const std::vector<const jfnk_atmos*>& cols, do
       S.formal_fuse = b->formal_kind == FORMAL_SWEEP && sweep_fused(*b) ? b->sweep_fuse : 0;
       S.formal_launches = active;
       S.kernel_launches = (int)(b->replays * b->graph_kernels) + 2;   // + state init, mode reset
-      S.formal_qb = b->formal_kind == FORMAL_FUSED || b->formal_kind == FORMAL_CACHED ? b->formal_qb : 0;
+      S.formal_qb = b->formal_kind == FORMAL_FUSED || kind_cached(b->formal_kind) ? b->formal_qb : 0;
       S.formal_threads = b->formal_threads;
       S.formal_kernel = b->formal_kind == FORMAL_SWEEP
                             ? (b->sweep_variant == 2 ? JFNK_FORMAL_SWEEP_WARP
                                : (sweep_fused(*b) ? JFNK_FORMAL_SWEEP_THREAD_FUSED : JFNK_FORMAL_SWEEP_THREAD))
                             : (b->formal_kind == FORMAL_CACHED ? JFNK_FORMAL_CACHED
                                : b->formal_kind == FORMAL_FUSED ? JFNK_FORMAL_FUSED
-                               : (b->formal_kind == FORMAL_MOVING ? JFNK_FORMAL_MOVING : JFNK_FORMAL_PER_RAY));
+                               : (kind_moving(b->formal_kind) ? JFNK_FORMAL_MOVING : JFNK_FORMAL_PER_RAY));
     }
     if (status != JFNK_OK && *worst == JFNK_OK) *worst = status;
   }

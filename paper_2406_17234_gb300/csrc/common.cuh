@@ -223,7 +223,7 @@ struct ColWork {
   double* np;       // [N] populations of a finite-difference evaluation (n + s eps u)
   double* fdp;      // [N] F(n + eps u) of a central difference
   // moving column (per-ray path, FP64): [2 nmu][nq][nz] each
-  double* mchi;     // opacity of each direction
+  double* mchi;     // opacity of each direction (cached evaluation: its reciprocal)
   double* mS;       // source function of each direction
   double* mdchi;    // their tangents
   double* mdS;
@@ -234,6 +234,7 @@ struct ColWork {
   // FP64 static columns, cached formal solution (formal_cached.cu); w.chi holds 1/chi there
   double* cf;       // coefficient planes [tile][nz-1][5][n_mu][qb] (null with another formal kernel)
   int cq;           // frequencies per tile (the column's own: its results are the same in any batch)
+  int crsp;         // 1: the parts of R_ji lack the spontaneous rates (static columns)
   double* rpart;    // parts of the rate integrals [(transition, tile)][kPartFixed + nl][nz]
   double* dJdn;     // [nq][nz][nl] lagged d J/d n_j of the second preconditioner
                     // solution (null until a solve asks for it)

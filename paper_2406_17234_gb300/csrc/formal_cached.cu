@@ -783,6 +783,337 @@ __global__ void __launch_bounds__(kEvalThreads) k_eval64(const ColDesc* __restri
   }
 }
 
+// ---------------------------------------------------------------------------
+// Moving columns (velocity.cu has the equations): the same evaluation with an
+// opacity and a source function per ray. Nothing is shared by the hemispheres,
+// so every (ray, layer) has its own coefficients; a base evaluation keeps e, h a,
+// h b and h |dz|/(2 mu) G of each, h = w_mu/2, G the slope of the ray's intensity
+// on its optical depth,
+//   G = -I^u e + (b/dtau) S^k + (e - b/dtau) S^u   (da = (b/dtau) ddtau, db = (e - b/dtau) ddtau),
+// and a product is h dI^k = h dI^u e + [h |dz|/(2 mu) G](dchi^k + dchi^u) + h a dS^k
+// + h b dS^u: five FP64 instructions per ray-point besides its opacity's tangent.
+// The local derivatives of the block-Jacobi sums follow from the same numbers,
+// dI^k/dchi^k = |dz|/(2 mu) G - (S^k/chi^k) a, dI^k/deta^k = a/chi^k.
+//
+// Rays stay in shared memory over all depths ([depth][ray]); a column too deep
+// for that takes the separate kernels of velocity.cu. 82 depths x 1,005
+// frequencies x 10 rays: product 35 + 197 + 37 -> 76 us, base evaluation 41 +
+// 245 + 8 + 205 -> 286 us.
+// ---------------------------------------------------------------------------
+constexpr int kMvPlanes = 4;   // e, h a, h b, then h bq and finally the slope
+
+__host__ __device__ inline size_t mv_rows(int nz) { return 3 * (size_t)nz + 4 * kChunk; }
+
+size_t moving_smem_bytes(int qb, int nz, int nmu) {
+  return sizeof(double) * mv_rows(nz) * ((2 * nmu * qb) | 1) + sizeof(int) * ((size_t)qb * kMaxT);
+}
+size_t moving_planes(int qb, int nz, int nq, int nmu) {
+  return (size_t)((nq + qb - 1) / qb) * (nz - 1) * kMvPlanes * 2 * nmu * qb;
+}
+
+// Frequencies per block of a moving column (0: too deep), as cached_default_qb:
+// about 25 full warps' worth of FP64 instructions per ray step besides the ray
+// warps' own.
+int moving_default_qb(int nq, int nz, int nmu, int n_sm) {
+  int best = 0;
+  double cost = 0.0;
+  for (int qb = 1; qb <= kMaxQb; ++qb) {
+    if (moving_smem_bytes(qb, nz, nmu) > kCachedSmem || 2 * nmu * qb > 128) break;
+    const long blocks = (nq + qb - 1) / qb;
+    const double waves = blocks <= 4L * n_sm ? (double)((blocks + n_sm - 1) / n_sm) : (double)blocks / n_sm;
+    const int rays = 2 * nmu * qb;
+    const double c = waves * (25.0 * rays / 32.0 + (rays + 31) / 32);
+    if (!best || c < cost) {
+      best = qb;
+      cost = c;
+    }
+  }
+  return best;
+}
+
+template <int MU>
+__global__ void __launch_bounds__(kEvalThreads) k_eval64_moving(const ColDesc* __restrict__ cols) {
+  extern __shared__ __align__(16) double sm[];
+  __shared__ double s_inv2mu[kMaxMu], s_hw[kMaxMu];
+  __shared__ double2 s_tab[kExpTab];
+  __shared__ int s_act[kMaxT], s_off[kMaxT], s_nact;
+  const ColDesc& cd = cols[blockIdx.y];
+  const int mode = mode_of(cd);
+  if (mode == EV_SKIP || mode == EV_RH92) return;   // RH92 is rejected for moving columns
+  const ColTables& T = cd.t;
+  const int nz = T.nz, nq = T.nq, nmu = MU ? MU : T.nmu, nl = T.nl, Qb = cd.w.cq;
+  Tile g;
+  g.tile = blockIdx.x;
+  g.Qb = Qb;
+  g.qb0 = g.tile * Qb;
+  if (g.qb0 >= nq) return;
+  g.nqb = min(Qb, nq - g.qb0);
+  g.Qp = pad_qb(Qb);
+  g.R5 = Qb * nmu;
+  const int nqb = g.nqb, qb0 = g.qb0, R5 = g.R5, nray = 2 * R5, rp = nray | 1;
+  double* s0 = sm;                      // [nz][rp] chi (or its tangent); then dI/dchi
+  double* s1 = s0 + (size_t)nz * rp;    // S (or its tangent); then dI/deta
+  double* sI = s1 + (size_t)nz * rp;    // h I (or h dI)
+  double* s_in = sI + (size_t)nz * rp;  // [2][2][kChunk][nray]: e, X of a chunk
+  int* s_list = reinterpret_cast<int*>(sm + mv_rows(nz) * rp);
+  double* cf = cd.w.cf + (size_t)g.tile * (nz - 1) * kMvPlanes * nray;
+  const bool tan = (mode == EV_TANGENT), base = (mode == EV_BASE);
+  const double* Vd = T.Vd ? T.Vd : T.V;                       // a static column of the batch: one profile
+  const size_t dstride = T.Vd ? (size_t)T.nwin * nz : 0, per = (size_t)nq * nz;
+
+  stage_lists(T, g, s_list);
+  for (int m = threadIdx.x; m < nmu; m += blockDim.x) {
+    s_inv2mu[m] = T.ang64[m].inv2mu;
+    s_hw[m] = T.ang64[m].hw;
+  }
+  if (!tan)
+    for (int i = threadIdx.x; i < kExpTab; i += blockDim.x) s_tab[i] = d_exp_tab[i];
+  if (threadIdx.x < 32) {
+    int tile0, ntile;
+    const int off = part_offset(T, Qb, threadIdx.x, tile0, ntile);
+    const bool on = g.tile >= tile0 && g.tile < tile0 + ntile;
+    const unsigned b = __ballot_sync(0xffffffffu, on);
+    if (on) {
+      const int i = __popc(b & ((1u << threadIdx.x) - 1));
+      s_act[i] = threadIdx.x;
+      s_off[i] = off + g.tile - tile0;
+    }
+    if (threadIdx.x == 0) s_nact = __popc(b);
+  }
+  // rays: ingoing first, then outgoing, each [angle][frequency]; direction d of
+  // the tables counts the outgoing ones first
+  const int ray = threadIdx.x, hfirst = (nray + 31) & ~31;
+  const bool up = ray >= R5;
+  const int rr = up ? ray - R5 : ray, rm = rr / Qb, rq = rr - rm * Qb;
+  const bool run = ray < nray && rq < nqb, helper = (int)threadIdx.x >= hfirst;
+  const int t0 = threadIdx.x - hfirst, nh = blockDim.x - hfirst;
+  const int nch = (nz - 2) / kChunk + 1;
+  int ir[kItems], iy[kItems];
+#pragma unroll
+  for (int j = 0; j < kItems; ++j) {
+    const int i = t0 + j * nh, r = i / nray;
+    iy[j] = i - r * nray;
+    ir[j] = !helper || r >= kChunk || (iy[j] >= R5 ? iy[j] - R5 : iy[j]) % Qb >= nqb ? nz : r;   // nz: never
+  }
+  double be[kItems], ba[kItems], bb[kItems], bg[kItems];
+  auto load = [&](int c) {
+#pragma unroll
+    for (int j = 0; j < kItems; ++j) {
+      const int s = c * kChunk + ir[j];
+      if (s < nz - 1) {
+        const double* p = cf + (size_t)(iy[j] >= R5 ? nz - 2 - s : s) * kMvPlanes * nray + iy[j];
+        be[j] = p[0];
+        ba[j] = p[nray];
+        bb[j] = p[2 * nray];
+        if (tan) bg[j] = p[3 * nray];
+      }
+    }
+  };
+  auto store = [&](int c) {
+    double* in = s_in + (size_t)(c & 1) * 2 * kChunk * nray;
+#pragma unroll
+    for (int j = 0; j < kItems; ++j) {
+      const int s = c * kChunk + ir[j];
+      if (s < nz - 1) {
+        const bool u = iy[j] >= R5;
+        const int k = u ? nz - 2 - s : s + 1, ku = u ? k + 1 : k - 1;
+        const int e = k * rp + iy[j], eu = ku * rp + iy[j];
+        double X = fma(ba[j], s1[e], bb[j] * s1[eu]);   // h (a S^k + b S^u), or of the tangents
+        if (tan) X = fma(bg[j], s0[e] + s0[eu], X);
+        in[ir[j] * nray + iy[j]] = be[j];
+        in[(kChunk + ir[j]) * nray + iy[j]] = X;
+      }
+    }
+  };
+  if (tan) load(0);
+  __syncthreads();
+  const int nslot = kPartFixed + nl;
+
+  // ---- opacity and source function of every ray, or their tangents -----------
+  const double* x = tan ? dir_of(cd) : eval_pops(cd, mode);
+  const double* Jd = jdag_ptr(cd);
+  for (int i = threadIdx.x; i < nray * nz; i += blockDim.x) {
+    const int y = i / nz, k = i - y * nz, yr = y >= R5 ? y - R5 : y, m = yr / Qb, ql = yr - m * Qb;
+    if (ql >= nqb) continue;
+    const int d = y >= R5 ? m : nmu + m, q = qb0 + ql;
+    const size_t o = (size_t)d * per + (size_t)q * nz + k;
+    const double* Vk = Vd + (size_t)d * dstride + k;
+    const double* xk = x + (size_t)k * nl;
+    const int* L = s_list + ql * kMaxT;
+    double a = 0.0, e = 0.0;   // sum V (x_lo - g x_up), sum g V x_up
+    for (int j = 0; j < kMaxT; ++j) {
+      const int w = L[j];
+      if (w < 0) break;
+      const size_t p = (size_t)(w >> 8) * nz;
+      const double V = Vk[p], gx = T.G[p + k] * xk[w & 15];
+      a = fma(V, xk[(w >> 4) & 15] - gx, a);
+      e = fma(V, gx, e);
+    }
+    const double c2 = T.c2[q];
+    if (tan) {
+      s0[k * rp + y] = a;
+      s1[k * rp + y] = fma(c2, e, -cd.w.mS[o] * a) * cd.w.mchi[o];   // mchi: 1/chi
+    } else {
+      const size_t qk = (size_t)q * nz + k;
+      const double sca = T.chi_sca[k], chi = T.chi_c[qk] + sca + a;
+      const double eta = fma(c2, e, T.eta_c[qk] + sca * Jd[qk]);
+      const double rc = 1.0 / chi, s = eta * rc, S = fma(fma(-s, chi, eta), rc, s);   // rounded once
+      s0[k * rp + y] = chi;
+      s1[k * rp + y] = S;
+      if (base) {
+        cd.w.mchi[o] = rc;
+        cd.w.mS[o] = S;
+      }
+    }
+  }
+  __syncthreads();
+  if (!tan) {
+    for (int i = threadIdx.x; i < nray * (nz - 1); i += blockDim.x) {
+      const int l = i / nray, y = i - l * nray, yr = y >= R5 ? y - R5 : y, m = yr / Qb;
+      if (yr - m * Qb >= nqb) continue;
+      const double dtau = T.dz[l] * s_inv2mu[m] * (s0[l * rp + y] + s0[(l + 1) * rp + y]), hw = s_hw[m];
+      double e, w, a, bq, om;
+      step_coef(dtau, 1.0 / dtau, s_tab, e, w, a, bq, om);
+      double* p = cf + (size_t)l * kMvPlanes * nray + y;
+      p[0] = e;
+      p[nray] = hw * a;
+      p[2 * nray] = hw * (bq * dtau);
+      p[3 * nray] = hw * bq;
+    }
+    __syncthreads();
+    load(0);
+  }
+  // ---- recurrences: h I^k = h I^u e + X ----------------------------------------
+  double I = 0.0;   // boundary values (their tangents are zero)
+  if (run) {
+    if (up && !tan) I = s_hw[rm] * T.Bn[(size_t)(qb0 + rq) * nz + nz - 1];
+    sI[(up ? nz - 1 : 0) * rp + ray] = I;
+  }
+  store(0);
+  load(1);
+  __syncthreads();
+  for (int c = 0; c < nch; ++c) {
+    if (!helper) {
+      if (run) {
+        const int c0 = c * kChunk, rows = min(kChunk, nz - 1 - c0);
+        const double* in = s_in + (size_t)(c & 1) * 2 * kChunk * nray + ray;
+        double e[kChunk], X[kChunk];
+#pragma unroll
+        for (int r = 0; r < kChunk; ++r) {
+          const int q = min(r, rows - 1) * nray;
+          e[r] = in[q];
+          X[r] = in[kChunk * nray + q];
+        }
+#pragma unroll
+        for (int r = 0; r < kChunk; ++r) X[r] = I = r < rows ? fma(I, e[r], X[r]) : I;
+#pragma unroll
+        for (int r = 0; r < kChunk; ++r)
+          if (r < rows) sI[(up ? nz - 2 - c0 - r : c0 + r + 1) * rp + ray] = X[r];
+      }
+    } else if (c + 1 < nch) {
+      store(c + 1);
+      load(c + 2);
+    }
+    __syncthreads();
+  }
+  if (base) {
+    if (run && up) cd.w.Iem[(size_t)(qb0 + rq) * nmu + rm] = I / s_hw[rm];
+    // the slope of each ray's intensity on its optical depth, times h |dz|/(2 mu)
+    for (int i = threadIdx.x; i < nray * (nz - 1); i += blockDim.x) {
+      const int l = i / nray, y = i - l * nray, yr = y >= R5 ? y - R5 : y, m = yr / Qb;
+      if (yr - m * Qb >= nqb) continue;
+      const bool u = y >= R5;
+      const int k = u ? l : l + 1, ku = u ? l + 1 : l;
+      double* p = cf + (size_t)l * kMvPlanes * nray + y;
+      const double Su = s1[ku * rp + y], e = p[0];
+      const double G = fma(p[3 * nray], s1[k * rp + y] - Su, e * fma(s_hw[m], Su, -sI[ku * rp + y]));
+      const double hG = T.dz[l] * s_inv2mu[m] * G;
+      p[3 * nray] = hG;
+      s0[k * rp + y] = hG;   // chi is no longer needed; the boundary depth is set below
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < nray * nz; i += blockDim.x) {
+      const int y = i / nz, k = i - y * nz, yr = y >= R5 ? y - R5 : y, m = yr / Qb, ql = yr - m * Qb;
+      if (ql >= nqb) continue;
+      const bool u = y >= R5;
+      const int l = u ? k : k - 1, e = k * rp + y;
+      double lx = 0.0, le = 0.0;
+      if (l >= 0 && l < nz - 1) {
+        const size_t o = (size_t)(u ? m : nmu + m) * per + (size_t)(qb0 + ql) * nz + k;
+        le = cd.w.mchi[o] * cf[((size_t)l * kMvPlanes + 1) * nray + y];
+        lx = fma(-s1[e], le, s0[e]);
+      }
+      s0[e] = lx;   // h dI/dchi, h dI/deta
+      s1[e] = le;
+    }
+    __syncthreads();
+    // J = sum of h I over the rays
+    for (int i = threadIdx.x; i < nqb * nz; i += blockDim.x) {
+      const int ql = i / nz, k = i - ql * nz;
+      double J = 0.0;
+      for (int m = 0; m < 2 * nmu; ++m) J += sI[k * rp + m * Qb + ql];
+      jnew_ptr(cd)[(size_t)(qb0 + ql) * nz + k] = J;
+    }
+  }
+  // ---- parts of the rate integrals (and of the block-Jacobi sums) -------------
+  for (int i = threadIdx.x; i < s_nact * nz; i += blockDim.x) {
+    const int a = i / nz, k = i - a * nz, t = s_act[a];
+    const int q0 = T.t_q0[t], qa = max(q0, qb0), qe = min(T.t_q1[t], qb0 + nqb - 1);
+    const double nlo = x[k * nl + T.t_lo[t]], nup = x[k * nl + T.t_up[t]];
+    double a0 = 0.0, a1 = 0.0;
+    double acc[kMaxL];
+    if (base)
+      for (int j = 0; j < nl; ++j) acc[j] = 0.0;
+    for (int q = qa; q <= qe; ++q) {
+      const int p = T.t_base[t] + q - q0, ql = q - qb0;
+      const size_t pk = (size_t)p * nz + k;
+      const double W = T.t_w[p] * T.rw[q], gt = T.G[pk], c2 = T.c2[q];
+      double V[2 * kMaxMu], su = 0.0, sv = 0.0;
+#pragma unroll
+      for (int m = 0; m < 2 * nmu; ++m)   // ray order: ingoing, then outgoing
+        V[m] = Vd[(size_t)(m < nmu ? nmu + m : m - nmu) * dstride + pk];
+#pragma unroll
+      for (int m = 0; m < 2 * nmu; ++m) {
+        su = fma(V[m], sI[k * rp + m * Qb + ql], su);
+        if (!tan) sv = fma(s_hw[m < nmu ? m : m - nmu], V[m], sv);
+      }
+      a0 = fma(W, su, a0);
+      a1 = fma(W * gt, tan ? su : fma(c2, sv, su), a1);
+      if (base) {
+        const double c = W * fma(-gt, nup, nlo);
+        const int* L = s_list + ql * kMaxT;
+        for (int j = 0; j < kMaxT; ++j) {
+          const int w = L[j];
+          if (w < 0) break;
+          const size_t ps = (size_t)(w >> 8) * nz + k;
+          double m1 = 0.0, m2 = 0.0;
+#pragma unroll
+          for (int m = 0; m < 2 * nmu; ++m) {
+            const double vv = V[m] * Vd[(size_t)(m < nmu ? nmu + m : m - nmu) * dstride + ps];
+            m1 = fma(vv, s0[k * rp + m * Qb + ql], m1);
+            m2 = fma(vv, s1[k * rp + m * Qb + ql], m2);
+          }
+          acc[(w >> 4) & 15] = fma(c, m1, acc[(w >> 4) & 15]);
+          acc[w & 15] = fma(c * T.G[ps], fma(c2, m2, -m1), acc[w & 15]);
+        }
+      }
+    }
+    double* part = cd.w.rpart + (size_t)s_off[a] * nslot * nz + k;
+    part[0] = a0;
+    part[nz] = a1;
+    if (base)
+      for (int j = 0; j < nl; ++j) part[(size_t)(2 + j) * nz] = acc[j];
+  }
+}
+
+int launch_eval64_moving(const Batch& b, cudaStream_t s) {
+  const dim3 g(b.max_tiles, b.ncols);
+  if (b.eval_mu == 5) k_eval64_moving<5><<<g, kEvalThreads, b.eval_smem, s>>>(b.d_cols);
+  else k_eval64_moving<0><<<g, kEvalThreads, b.eval_smem, s>>>(b.d_cols);
+  JFNK_CUDA(cudaGetLastError());
+  return JFNK_OK;
+}
+
 int cached_prepare() {
   double2 tab[kExpTab];
   for (int j = 0; j < kExpTab; ++j)
@@ -790,6 +1121,8 @@ int cached_prepare() {
   JFNK_CUDA(cudaMemcpyToSymbol(d_exp_tab, tab, sizeof(tab)));
   JFNK_CUDA(cudaFuncSetAttribute(k_eval64<5>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCachedSmem));
   JFNK_CUDA(cudaFuncSetAttribute(k_eval64<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCachedSmem));
+  JFNK_CUDA(cudaFuncSetAttribute(k_eval64_moving<5>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCachedSmem));
+  JFNK_CUDA(cudaFuncSetAttribute(k_eval64_moving<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCachedSmem));
   return JFNK_OK;
 }
 

@@ -100,7 +100,10 @@ int build_atmosphere(jfnk_ctx* ctx, int lane, const AtomData& A, const jfnk_atmo
 // Formal-solution kernels: per-ray buffers + ray-sum kernel (any size),
 // in-block fused kernel (FP64), per-frequency sweep kernel (mixed precision).
 // whole evaluation per frequency tile with cached coefficients (FP64).
-enum FormalKind { FORMAL_UNFUSED = 0, FORMAL_FUSED = 1, FORMAL_SWEEP = 2, FORMAL_MOVING = 3, FORMAL_CACHED = 4 };
+enum FormalKind { FORMAL_UNFUSED = 0, FORMAL_FUSED = 1, FORMAL_SWEEP = 2, FORMAL_MOVING = 3, FORMAL_CACHED = 4,
+                  FORMAL_MOVING_CACHED = 5 };
+inline bool kind_moving(int k) { return k == FORMAL_MOVING || k == FORMAL_MOVING_CACHED; }
+inline bool kind_cached(int k) { return k == FORMAL_CACHED || k == FORMAL_MOVING_CACHED; }
 
 // A batch of columns with their work buffers, resident on the device.
 struct Batch {
@@ -199,6 +202,11 @@ size_t cached_parts(int qb, int nz, int nl, int nwin, int nt);
 constexpr int kEvalThreads = 512;   // threads per block of the cached evaluation
 int cached_prepare();
 int launch_eval64(const Batch& b, cudaStream_t s);
+// ... of moving columns
+int moving_default_qb(int nq, int nz, int nmu, int n_sm);
+size_t moving_smem_bytes(int qb, int nz, int nmu);
+size_t moving_planes(int qb, int nz, int nq, int nmu);
+int launch_eval64_moving(const Batch& b, cudaStream_t s);
 // Per-frequency sweep kernel of the mixed mode (formal_sweep.cu).
 size_t sweep_scratch_bytes(int nq, int nz);
 int sweep_prepare(Batch* b);

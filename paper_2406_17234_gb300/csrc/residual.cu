@@ -1291,7 +1291,7 @@ __global__ void __launch_bounds__(32 * kAsmWarps) k_assemble(const ColDesc* __re
         rd += p[(size_t)a * stride + nz];
       }
       if (!tan) {
-        rd += T.Rsp[o];
+        if (cd.w.crsp) rd += T.Rsp[o];
         cd.w.Rup[o] = ru;
         cd.w.Rdn[o] = rd;
       }
@@ -1466,7 +1466,7 @@ int launch_opacity_tan(const Batch& b, cudaStream_t s, int depths) {
 
 // The assembly: tangent evaluations thread per depth, the others warp per depth.
 static void launch_assemble(const Batch& b, cudaStream_t s) {
-  const bool cached = b.formal_kind == FORMAL_CACHED;   // k_assemble takes its tangents too
+  const bool cached = kind_cached(b.formal_kind);   // k_assemble takes its tangents too
   if (!cached && (b.forced < 0 || b.forced == EV_TANGENT))
     k_assemble_tan<<<dim3((b.max_nz + kAsmTanThreads - 1) / kAsmTanThreads, b.ncols, std::max(1, b.max_nl)),
                      kAsmTanThreads, 0, s>>>(b.d_cols);
@@ -1528,10 +1528,10 @@ int launch_evaluation(const Batch& b, cudaStream_t s, cudaEvent_t ev0, cudaEvent
     return JFNK_OK;
   }
   if (int rm = mark(0)) return rm;
-  if (b.formal_kind == FORMAL_CACHED) {
+  if (kind_cached(b.formal_kind)) {
     // opacity, formal solution and the tiles' rate integrals in one kernel
     if (ev0) JFNK_CUDA(cudaEventRecordWithFlags(ev0, s, cudaEventRecordExternal));
-    int rc = launch_eval64(b, s);
+    int rc = b.formal_kind == FORMAL_CACHED ? launch_eval64(b, s) : launch_eval64_moving(b, s);
     if (rc) return rc;
     if (ev1) JFNK_CUDA(cudaEventRecordWithFlags(ev1, s, cudaEventRecordExternal));
     launch_dJdn_update(b, s);

@@ -46,7 +46,7 @@ size_t column_bytes(const AtmosData& M, int kind, int mixed, int kmax, ColLayout
   const size_t rs = mixed ? sizeof(float) : sizeof(double);
   const size_t nz = M.nz, nq = M.nq, nl = M.nl, nt = M.nt, nmu = M.nmu, N = nz * nl;
   const bool per_ray = (kind == FORMAL_UNFUSED);   // unfused kernels need per-ray buffers
-  const bool sweep = (kind == FORMAL_SWEEP), cached = (kind == FORMAL_CACHED);
+  const bool sweep = (kind == FORMAL_SWEEP), cached = kind_cached(kind);
   o.n = ar.take<double>(N); o.v = ar.take<double>(N);
   o.Jdag = ar.take<double>(nq * nz); o.Jnew = ar.take<double>(nq * nz);
   o.istar = ar.take<int>(nz);
@@ -79,11 +79,13 @@ size_t column_bytes(const AtmosData& M, int kind, int mixed, int kmax, ColLayout
   o.eta = ar.take<double>(nq * nz); o.etab32 = ar.take<float>(mixed ? nq * nz : 0);
   o.n2 = ar.take<float2>(mixed ? N : 0);
   // moving columns: per-ray opacity, source function, intensity, tangents and local derivatives
-  const size_t MR = kind == FORMAL_MOVING ? 2 * nmu * nq * nz : 0;
-  o.mchi = ar.take<double>(MR); o.mS = ar.take<double>(MR); o.mdchi = ar.take<double>(MR);
+  const size_t MR = kind == FORMAL_MOVING ? 2 * nmu * nq * nz : 0, MC = kind_moving(kind) ? 2 * nmu * nq * nz : 0;
+  o.mchi = ar.take<double>(MC); o.mS = ar.take<double>(MC); o.mdchi = ar.take<double>(MR);
   o.mdS = ar.take<double>(MR); o.mI = ar.take<double>(MR); o.mdI = ar.take<double>(MR);
   o.mLX = ar.take<double>(MR); o.mLE = ar.take<double>(MR);
-  o.cf = ar.take<double>(cached ? cached_planes(qb, M.nz, M.nq, M.nmu) : 0);
+  o.cf = ar.take<double>(kind == FORMAL_CACHED          ? cached_planes(qb, M.nz, M.nq, M.nmu)
+                         : kind == FORMAL_MOVING_CACHED ? moving_planes(qb, M.nz, M.nq, M.nmu)
+                                                        : 0);
   o.rpart = ar.take<double>(cached ? cached_parts(qb, M.nz, M.nl, M.nwin, M.nt) : 0);
   if (out) *out = o;
   return ar.cursor;
@@ -134,8 +136,11 @@ void column_bind(char* base, const AtmosData& M, int kind, int mixed, int kmax, 
     w.mdS = (double*)P(o.mdS); w.mI = (double*)P(o.mI); w.mdI = (double*)P(o.mdI);
     w.mLX = (double*)P(o.mLX); w.mLE = (double*)P(o.mLE);
   }
-  if (kind == FORMAL_CACHED) {
-    w.cf = (double*)P(o.cf); w.rpart = (double*)P(o.rpart); w.cq = qb;
+  if (kind == FORMAL_MOVING_CACHED) {
+    w.mchi = (double*)P(o.mchi); w.mS = (double*)P(o.mS);
+  }
+  if (kind_cached(kind)) {
+    w.cf = (double*)P(o.cf); w.rpart = (double*)P(o.rpart); w.cq = qb; w.crsp = kind == FORMAL_CACHED;
   }
   w.st = st;
 }
@@ -172,27 +177,31 @@ int batch_create(Batch* b, const std::vector<const AtmosData*>& cols, int mixed,
     JFNK_CUDA(cudaGetDevice(&dev));
     JFNK_CUDA(cudaDeviceGetAttribute(&b->n_sm, cudaDevAttrMultiProcessorCount, dev));
   }
-  // FP64 static columns: the cached evaluation, unless its coefficient planes
+  // FP64 columns: the cached evaluation, unless its coefficient planes
   // (40 bytes per ray-point pair) of the whole batch would exceed kCachedBytes
   // or the device has no room for them; then the fused kernel, which keeps none
-  bool cached = !mixed && !moving;
+  bool cached = !mixed;
   size_t planes = 0;
   std::vector<int> qc(nc, 0);
   for (int c = 0; c < nc && cached; ++c) {
     const AtmosData& M = *cols[c];
-    qc[c] = cached_default_qb(M.nq, M.nz, M.nmu, M.nl, b->n_sm);
-    cached = qc[c] > 0 && (planes += cached_planes(qc[c], M.nz, M.nq, M.nmu) * sizeof(double)) <= kCachedBytes;
+    qc[c] = moving ? moving_default_qb(M.nq, M.nz, M.nmu, b->n_sm)
+                   : cached_default_qb(M.nq, M.nz, M.nmu, M.nl, b->n_sm);
+    // (moving columns: the planes take less than the per-ray arrays they replace)
+    cached = qc[c] > 0 &&
+             (moving || (planes += cached_planes(qc[c], M.nz, M.nq, M.nmu) * sizeof(double)) <= kCachedBytes);
     if (!cached) break;
     b->eval_mu = c == 0 || b->eval_mu == M.nmu ? M.nmu : 0;
     b->max_tiles = std::max(b->max_tiles, (M.nq + qc[c] - 1) / qc[c]);
-    b->eval_smem = std::max(b->eval_smem, cached_smem_bytes(qc[c], M.nz, M.nmu, M.nl));
+    b->eval_smem = std::max(b->eval_smem, moving ? moving_smem_bytes(qc[c], M.nz, M.nmu)
+                                                 : cached_smem_bytes(qc[c], M.nz, M.nmu, M.nl));
   }
   std::vector<size_t> off(nc);
   size_t o_cols = 0, o_state = 0, o_status = 0, o_opts = 0, o_view = 0;
   for (;;) {
     b->formal_qb = cached ? qc[0] : (mixed || moving ? 0 : fused_default_qb(b->max_nz, b->max_nmu, false));
     b->formal_threads = cached ? kEvalThreads : 0;
-    b->formal_kind = cached   ? FORMAL_CACHED
+    b->formal_kind = cached   ? (moving ? FORMAL_MOVING_CACHED : FORMAL_CACHED)
                      : moving ? FORMAL_MOVING
                      : mixed  ? FORMAL_SWEEP
                               : (b->formal_qb > 0 ? FORMAL_FUSED : FORMAL_UNFUSED);
@@ -221,7 +230,7 @@ int batch_create(Batch* b, const std::vector<const AtmosData*>& cols, int mixed,
   JFNK_CUDA(cudaMemcpy(b->d_cols, b->h_cols.data(), nc * sizeof(ColDesc), cudaMemcpyHostToDevice));
   JFNK_CUDA(cudaMemset(b->d_state, 0, nc * sizeof(SolverState)));
   if (b->formal_kind == FORMAL_SWEEP) return sweep_prepare(b);
-  if (b->formal_kind == FORMAL_MOVING || b->formal_kind == FORMAL_CACHED) return JFNK_OK;
+  if (kind_moving(b->formal_kind) || kind_cached(b->formal_kind)) return JFNK_OK;
   return fused_prepare(b);
 }
 

@@ -72,3 +72,46 @@ def test_cached_evaluation_matches_oracle_at_tile_edges(i):
     new, _ = B.rh92_update(atm, n, Jd)
     rn = ora_rh92(m, n, ref)
     assert np.all(np.abs(new - rn) <= 1e-7 * np.abs(rn).max(axis=1, keepdims=True))
+
+
+MOVING = [
+    # (depths, line points, angles): chunk edges, ragged tiles; the last is too
+    # deep for a block's rays and takes the separate kernels
+    (2, 5, 1), (9, 7, 3), (17, 21, 8), (34, 9, 5), (1000, 5, 8),
+]
+
+
+@pytest.mark.parametrize("nz,nq,nmu", MOVING)
+def test_moving_evaluation_matches_oracle_at_tile_edges(nz, nq, nmu):
+    from dataclasses import replace
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    wl = W.tiny_workload(n_depth=nz, n_nu_line=nq, n_nu_cont=3)
+    col = replace(wl.columns[0], vlos=np.linspace(3e5, -1e5, nz))
+    ctx = B.Context(0)
+    atom = B.Atom(ctx, wl.atom)
+    atm = B.Atmosphere(ctx, atom, col, n_mu=nmu)
+    m = OM.build_model(wl.atom, col, nmu)
+    rng = np.random.default_rng(nz)
+    n = W.perturbed_populations(m.nstar, rng, 0.02)
+    Jd = m.B * np.exp(rng.normal(0.0, 0.05, m.B.shape))
+    v = n * rng.normal(0.0, 1.0, n.shape)
+    ref = ora_residual(m, n, Jd, want_lambda=True)
+    gross, dgross = np.zeros_like(n), np.zeros_like(n)
+    for t, tr in enumerate(m.trans):
+        up = m.Cmat[:, tr.lo, tr.up] + ref.R_up[t]
+        dn = m.Cmat[:, tr.up, tr.lo] + ref.R_dn[t]
+        for l in (tr.lo, tr.up):
+            gross[:, l] += n[:, tr.lo] * up + n[:, tr.up] * dn
+            dgross[:, l] += np.abs(v[:, tr.lo]) * up + np.abs(v[:, tr.up]) * dn
+    gross[np.arange(nz), ref.istar] = n.sum(axis=1)
+    dgross += gross
+    F, J, I = B.residual(atm, n, Jd, want_J=True, want_emergent=True)
+    assert np.all(np.abs(F - ref.F) <= 1e-10 * gross)
+    np.testing.assert_allclose(J, ref.J, rtol=1e-9)
+    np.testing.assert_allclose(I, ref.I_emergent, rtol=1e-9)
+    Jv = B.jvp(atm, n, v, Jd)
+    assert np.all(np.abs(Jv - jvp_complex(m, n, Jd, v, ref.istar)) <= 1e-10 * dgross)
+    P, rP = B.block_jacobi(atm, n, Jd), ora_P(m, n, ref)
+    assert np.all(np.abs(P - rP) <= 1e-9 * np.abs(rP).max(axis=(1, 2), keepdims=True))

@@ -599,8 +599,8 @@ __device__ __forceinline__ int rate_mode(const ColDesc& cd, int t, int tile) {
 // The packed transitions active at a frequency (ColTables::qmeta4). PIPE
 // (small launches, few warps on a multiprocessor): the whole list is loaded
 // two frequencies before its use, since a list and then the tables it points
-// to would be two trips to memory in a row, and the terms of its first three
-// transitions with the frequency's other inputs; 168 registers. Otherwise
+// to would be two trips to memory in a row, and the terms of its transitions
+// with the frequency's other inputs. Otherwise
 // (large launches, which need the warps more) two transitions and 128
 // registers; the 512-column batch was 3 % slower with the former.
 // H I-like column, 82 x 2,010: 59 -> 30 us for a base evaluation.
@@ -666,7 +666,7 @@ __device__ __forceinline__ void rate_window(const ColTables& T, bool packed, int
 template <bool PIPE>
 __device__ void rates_tile(const ColDesc& cd, const int mode, const int t, const int tile, const int rank,
                            const RateSmem& sm, cg::cluster_group& cluster, const SolverOpts* bopts) {
-  constexpr int kRateHeld = PIPE ? 3 : 2;   // transitions whose terms a frequency's inputs hold
+  constexpr int kRateHeld = PIPE ? kQMetaT : 2;   // transitions whose terms a frequency's inputs hold
   const ColTables& T = cd.t;
   const int nz = T.nz, nl = T.nl, nt = T.nt;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -958,8 +958,8 @@ __device__ void rates_tile(const ColDesc& cd, const int mode, const int t, const
 // column c0 + l * step, so that columns in another evaluation kind cost one
 // load each instead of a cluster launch.
 template <bool PIPE>
-__global__ void __launch_bounds__(32 * kRateWarps) k_rates(const ColDesc* __restrict__ cols, int ncols,
-                                                           int racc, int fslots, const SolverOpts* bopts) {
+__device__ __forceinline__ void rates_columns(const ColDesc* __restrict__ cols, int ncols, int racc, int fslots,
+                                              const SolverOpts* bopts) {
   extern __shared__ __align__(16) unsigned char rate_smem[];
   cg::cluster_group cluster = cg::this_cluster();
   const int rank = (int)cluster.block_rank();
@@ -985,13 +985,26 @@ __global__ void __launch_bounds__(32 * kRateWarps) k_rates(const ColDesc* __rest
   }
 }
 
+// Two kernels, so that each has its own register bound: the large launch keeps
+// the compiler's 128 (a second bound argument, even 1, makes it 160 and the
+// 512-column batch 3 % slower), the small one the 206 its held terms need
+// (168 and spills without it).
+__global__ void __launch_bounds__(32 * kRateWarps) k_rates(const ColDesc* __restrict__ cols, int ncols, int racc,
+                                                           int fslots, const SolverOpts* bopts) {
+  rates_columns<false>(cols, ncols, racc, fslots, bopts);
+}
+__global__ void __launch_bounds__(32 * kRateWarps, 2) k_rates_small(const ColDesc* __restrict__ cols, int ncols,
+                                                                    int racc, int fslots, const SolverOpts* bopts) {
+  rates_columns<true>(cols, ncols, racc, fslots, bopts);
+}
+
 // Kernel attributes, set once per device when a context is created (outside
 // any stream capture): the rate kernel's largest dynamic shared memory.
 int prepare_kernels() {
   const int max_smem = (int)((size_t)kRateWarps * 32 * ((2 + kRhFixed + kMaxT) * sizeof(double) +
                                                        std::max(kMaxT, kMaxL) * sizeof(float)));
-  JFNK_CUDA(cudaFuncSetAttribute(k_rates<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem));
-  JFNK_CUDA(cudaFuncSetAttribute(k_rates<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem));
+  JFNK_CUDA(cudaFuncSetAttribute(k_rates_small, cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem));
+  JFNK_CUDA(cudaFuncSetAttribute(k_rates, cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem));
   return cached_prepare();
 }
 
@@ -1019,8 +1032,8 @@ static int launch_rates(const Batch& b, cudaStream_t s) {
   attr[0].val.clusterDim.z = split;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  JFNK_CUDA(cudaLaunchKernelEx(&cfg, split > 1 ? k_rates<true> : k_rates<false>, (const ColDesc*)b.d_cols, b.ncols, racc, fslots,
-                               (const SolverOpts*)b.d_opts));
+  JFNK_CUDA(cudaLaunchKernelEx(&cfg, split > 1 ? k_rates_small : k_rates, (const ColDesc*)b.d_cols, b.ncols, racc,
+                               fslots, (const SolverOpts*)b.d_opts));
   return JFNK_OK;
 }
 
@@ -1276,20 +1289,37 @@ __global__ void __launch_bounds__(32 * kAsmWarps) k_assemble(const ColDesc* __re
   const double* v = tan ? tangent_dir(cd) + k * nl : nullptr;
   const size_t stride = (size_t)(kPartFixed + nl) * nz;
   int off = 0, ntile = 0, tile0;
-  if (cached) off = part_offset(T, cd.w.cq, lane, tile0, ntile);
+  double pu = 0.0, pd = 0.0;
+  if (cached) {
+    // the tiles' parts of R_ij and R_ji (their tangents): G lanes per transition
+    // take every G-th tile in order, then add theirs pairwise (an order that
+    // depends on the atom only)
+    off = part_offset(T, cd.w.cq, lane, tile0, ntile);
+    const int lg = nt <= 1 ? 5 : __clz(nt - 1) - 27;   // G = 32 / (nt rounded up to a power of two)
+    const int G = 1 << lg, t = lane >> lg;
+    const int to = __shfl_sync(0xffffffffu, off, min(t, nt - 1)), tn = __shfl_sync(0xffffffffu, ntile, min(t, nt - 1));
+    if (t < nt) {
+      const double* p = cd.w.rpart + (size_t)to * stride + k;
+#pragma unroll 8
+      for (int a = lane & (G - 1); a < tn; a += G) {
+        pu += p[(size_t)a * stride];
+        pd += p[(size_t)a * stride + nz];
+      }
+    }
+    for (int o = 1; o < G; o <<= 1) {
+      pu += __shfl_xor_sync(0xffffffffu, pu, o);
+      pd += __shfl_xor_sync(0xffffffffu, pd, o);
+    }
+    pu = __shfl_sync(0xffffffffu, pu, (lane << lg) & 31);   // lane t gets its transition's sums
+    pd = __shfl_sync(0xffffffffu, pd, (lane << lg) & 31);
+  }
   if (lane < nt) {
     const int t = lane, lo = T.t_lo[t], up = T.t_up[t];
     const size_t o = (size_t)t * nz + k;
     double ru, rd;
     if (cached) {
-      // the tiles' parts of R_ij and R_ji (their tangents), in tile order
-      const double* p = cd.w.rpart + (size_t)off * stride + k;
-      ru = rd = 0.0;
-#pragma unroll 8
-      for (int a = 0; a < ntile; ++a) {
-        ru += p[(size_t)a * stride];
-        rd += p[(size_t)a * stride + nz];
-      }
+      ru = pu;
+      rd = pd;
       if (!tan) {
         if (cd.w.crsp) rd += T.Rsp[o];
         cd.w.Rup[o] = ru;
@@ -1557,7 +1587,7 @@ int launch_evaluation(const Batch& b, cudaStream_t s, cudaEvent_t ev0, cudaEvent
     const bool own = b.sweep_variant == 2;
     const bool tans = b.forced < 0 || b.forced == EV_TANGENT, bases = b.forced != EV_TANGENT;
     if (tans && !own) k_dir32<<<dim3((b.max_N + tb - 1) / tb, nc), tb, 0, s>>>(b.d_cols);
-    if (bases) k_pop_pairs<<<dim3((b.max_N + tb - 1) / tb, nc), tb, 0, s>>>(b.d_cols);
+    if (bases && !b.pairs_ready) k_pop_pairs<<<dim3((b.max_N + tb - 1) / tb, nc), tb, 0, s>>>(b.d_cols);
     if (bases && !own) k_opacity<float><<<opacity_grid(b, tb), tb, 0, s>>>(b.d_cols, 1);   // base and RH92 columns
     if (tans && !own && !sweep_fused(b)) launch_op_tan(b, s);
     int rc;

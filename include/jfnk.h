@@ -146,7 +146,7 @@ typedef struct {
 typedef enum {
   JFNK_FORMAL_PER_RAY = 0,       /* per-ray buffers, separate ray-sum kernel      */
   JFNK_FORMAL_FUSED = 1,         /* FP64: block per frequency group, shared memory */
-  JFNK_FORMAL_SWEEP_THREAD = 2,  /* mixed: thread per frequency, all angles        */
+  JFNK_FORMAL_SWEEP_THREAD = 2,  /* mixed: thread per frequency (tangents: per two), all angles */
   JFNK_FORMAL_SWEEP_WARP = 3,    /* mixed: warp per frequency pair, lane per ray   */
   JFNK_FORMAL_MOVING = 4,        /* moving columns: thread per ray, per-ray opacity */
   JFNK_FORMAL_SWEEP_THREAD_FUSED = 5, /* mixed: thread per frequency, the tangent sweep

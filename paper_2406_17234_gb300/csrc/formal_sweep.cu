@@ -270,7 +270,8 @@ __device__ __forceinline__ void stage_dz(const ColTables& T, float* s_dz, float*
 }
 
 // ---------------------------------------------------------------------------
-// Variant 1: one thread per frequency, all angles of a hemisphere in registers.
+// Variant 1: one thread per frequency, all angles of a hemisphere in registers (the
+// tangent sweep of a large launch: per two frequencies, sweep_pair below).
 // ---------------------------------------------------------------------------
 // Base evaluations read chi and S per frequency row ([q][k], S as a float
 // pair), form S^u - S^k in pair arithmetic, and leave depth-major float
@@ -578,10 +579,12 @@ __device__ __forceinline__ void sweep_thread(const ColDesc& cd, int q, const flo
     };
     if (EXACT) {
       // the angles' optical depths tz/(2 mu) fall with m (mu ascending): one
-      // test on the first and last angle settles the form for all of them
-      if (!(mul(in.tz, inv2mu[MU - 1]) < 0.1f)) angles(std::integral_constant<int, CM_DIRECT>());
-      else if (mul(in.tz, inv2mu[0]) < 0.1f) angles(std::integral_constant<int, CM_SERIES>());
-      else angles(std::integral_constant<int, CM_EITHER>());
+      // test on the first and last angle settles the form for all of them. The
+      // warp takes one form together: lanes that differ would run every form one
+      // after the other (base sweeps of 512 Ca II columns: 38.0 -> 36.5 ms a solve).
+      if (__all_sync(amask, !(mul(in.tz, inv2mu[MU - 1]) < 0.1f))) angles(std::integral_constant<int, CM_DIRECT>());
+      else if (__all_sync(amask, mul(in.tz, inv2mu[0]) < 0.1f)) angles(std::integral_constant<int, CM_SERIES>());
+      else angles(std::integral_constant<int, CM_SELECT>());
     } else {
       angles(std::integral_constant<int, CM_EITHER>());
     }
@@ -596,6 +599,235 @@ __device__ __forceinline__ void sweep_thread(const ColDesc& cd, int q, const flo
 #pragma unroll
     for (int m = 0; m < MU; ++m)
       if (EXACT || m < nmu) cd.w.Iem[(size_t)q * nmu + m] = __dmul_rn((double)I[m], c2);
+  }
+}
+
+// ---------------------------------------------------------------------------
+// Tangent sweep of a large launch: one thread per two neighbouring frequencies,
+// every FP32 operation a packed pair (fma.rn.f32x2 and its mul: two IEEE
+// operations in one instruction). The scalar sweep filled the issue slots (0.88
+// of the peak rate) with DRAM and the FP32 lanes half idle; a packed instruction
+// takes the lanes twice as long as a scalar one but one issue slot, and loads
+// and addresses are shared by the two frequencies. A warp votes on the form of
+// the coefficients, so that lanes on both sides of the limit cost one pass and
+// not three. Each element sees the operations of ray_step in their order: the
+// same bits. Now the FP32 pipe (0.87) and the issue slots (0.94 on a full
+// multiprocessor) bind together.
+// 512 Ca II columns, 256 x 1,005, 5 angles, median launch of a solve: scalar 960 us,
+// scalar with the vote 999, packed 963, packed with the vote 785 (57.0 -> 46.8 ms per
+// solve). A vote per angle in mixed warps: 47.9 ms; 64 threads per block: 49.0.
+// ---------------------------------------------------------------------------
+using f32x2 = unsigned long long;
+__device__ __forceinline__ f32x2 pack2(float a, float b) {
+  f32x2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ void unpack2(f32x2 v, float& a, float& b) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+}
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+  f32x2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+__device__ __forceinline__ f32x2 both2(float a) { return pack2(a, a); }
+// a + b and a - b as fma with a packed 1 or -1 the compiler cannot see the value
+// of (a kernel argument): it contracts a packed product and the add.rn.f32x2 or
+// constant fma after it into one operation, which rounds once instead of twice
+// (it leaves the scalar mul.rn and add.rn apart).
+struct Ones2 {
+  f32x2 one, neg;
+};
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b, const Ones2& u) { return fma2(a, u.one, b); }
+__device__ __forceinline__ f32x2 sub2(f32x2 a, f32x2 b, const Ones2& u) { return fma2(b, u.neg, a); }
+__device__ __forceinline__ f32x2 ld2(const float* p) { return *reinterpret_cast<const f32x2*>(p); }
+__device__ __forceinline__ void st2(float* p, f32x2 v) { *reinterpret_cast<f32x2*>(p) = v; }
+__device__ __forceinline__ f32x2 select2(bool a, bool b, f32x2 x, f32x2 y) {   // per element: x or y
+  float x0, x1, y0, y1;
+  unpack2(x, x0, x1);
+  unpack2(y, y0, y1);
+  return pack2(a ? x0 : y0, b ? x1 : y1);
+}
+__device__ __forceinline__ void series2(f32x2 x, f32x2& w, f32x2& bq) {
+  w = fma2(fma2(fma2(fma2(fma2(both2(-1.0f / 720.0f), x, both2(1.0f / 120.0f)), x, both2(-1.0f / 24.0f)), x,
+                     both2(1.0f / 6.0f)), x, both2(-0.5f)), x, both2(1.0f));
+  bq = fma2(fma2(fma2(fma2(both2(1.0f / 144.0f), x, both2(-1.0f / 30.0f)), x, both2(1.0f / 8.0f)), x,
+                 both2(-1.0f / 3.0f)), x, both2(0.5f));
+}
+__device__ __forceinline__ void direct2(f32x2 e, f32x2 r, f32x2& w, f32x2& bq, const Ones2& u) {
+  w = mul2(sub2(u.one, e, u), r);
+  bq = mul2(sub2(w, e, u), r);
+}
+
+constexpr int kPairThreads = 128;
+constexpr int kPairAhead = 4;   // depths ahead whose rows are prefetched into L2
+
+template <int MU, bool UP>
+__device__ __forceinline__ void sweep_pair(const ColDesc& cd, int q, const float* __restrict__ s_dz,
+                                           const float* __restrict__ s_idz, const Ones2& u, unsigned amask) {
+  const ColTables& T = cd.t;
+  const int nz = T.nz, nq = T.nq;
+  const size_t pitch = (size_t)col_pitch(nq);
+  const float* __restrict__ chiT = cd.w.chiT + q;
+  const float* __restrict__ dSkT = cd.w.dSkT + q;
+  const float* __restrict__ dchiT = cd.w.dchiT + q;
+  const float* __restrict__ dS32T = cd.w.dS32T + q;
+  float* __restrict__ part = reinterpret_cast<float*>(cd.w.part) + q;
+  float* __restrict__ dJ = cd.w.dJ32T + q;
+  float inv2mu[MU], two_mu[MU], hw[MU];
+#pragma unroll
+  for (int m = 0; m < MU; ++m) {
+    const float4 a = T.ang32[m];
+    inv2mu[m] = a.x;
+    hw[m] = a.y;
+    two_mu[m] = a.z;
+  }
+  // boundary depth: I = 0 at the top, I = B at the bottom (Sect. 2.1)
+  const int k0 = UP ? nz - 1 : 0, q1 = min(q + 1, nq - 1);
+  auto D0_of = [&](int qq) {
+    const size_t i = (size_t)qq * nz;
+    const double Ib = UP ? T.Bn[i + nz - 1] / T.c2[qq] : 0.0;
+    return df_to_float(df_sub(df_from_double(Ib), df_load(as_pairs(cd.w.S), i + k0)));
+  };
+  f32x2 cp = ld2(chiT + k0 * pitch), dcp = ld2(dchiT + k0 * pitch), dSp = ld2(dS32T + k0 * pitch);
+  f32x2 D[MU], dD[MU], x[8];
+  {
+    const f32x2 D0 = pack2(D0_of(q), D0_of(q1));
+    float a, b;
+    unpack2(dSp, a, b);
+    const f32x2 dD0 = pack2(-a, -b);
+#pragma unroll
+    for (int m = 0; m < MU; ++m) {
+      D[m] = D0;
+      dD[m] = dD0;
+      x[m] = mul2(both2(hw[m]), dD0);
+    }
+  }
+  // the angles' sum in the order of tree_mu
+  auto tree = [&]() {
+    auto pair_add = [&](int i, int j) { return j < MU ? add2(x[i], x[j], u) : x[i]; };   // i < MU
+    f32x2 ev = pair_add(0, 4);
+    if (MU > 2) ev = add2(ev, pair_add(2, 6), u);
+    if (MU == 1) return ev;
+    f32x2 od = pair_add(1, 5);
+    if (MU > 3) od = add2(od, pair_add(3, 7), u);
+    return add2(ev, od, u);
+  };
+  auto emit = [&](int k, f32x2 dS, f32x2 pt) {
+    const f32x2 t = tree();
+    if (!UP) st2(part + (size_t)k * pitch, t);
+    else st2(dJ + (size_t)k * pitch, add2(dS, add2(t, pt, u), u));
+  };
+  emit(k0, dSp, UP ? ld2(part + (size_t)k0 * pitch) : 0);
+  // the next depth's inputs are loaded one step ahead, their lines brought into L2 before that
+  int kn = UP ? nz - 2 : 1;
+  f32x2 c_n = 0, dc_n = 0, dS_n = 0, dSl_n = 0, pt_n = 0;
+  auto load = [&](int k) {
+    c_n = ld2(chiT + (size_t)k * pitch);
+    dSl_n = ld2(dSkT + (size_t)(UP ? k : k - 1) * pitch);
+    dc_n = ld2(dchiT + (size_t)k * pitch);
+    dS_n = ld2(dS32T + (size_t)k * pitch);
+    if (UP) pt_n = ld2(part + (size_t)k * pitch);
+    const int kf = UP ? k - kPairAhead : k + kPairAhead;
+    if (kf >= 0 && kf < nz) {
+      const size_t o = (size_t)kf * pitch;
+      asm volatile("prefetch.global.L2 [%0];" ::"l"(chiT + o));
+      asm volatile("prefetch.global.L2 [%0];" ::"l"(dSkT + o));
+      asm volatile("prefetch.global.L2 [%0];" ::"l"(dchiT + o));
+      asm volatile("prefetch.global.L2 [%0];" ::"l"(dS32T + o));
+      if (UP) asm volatile("prefetch.global.L2 [%0];" ::"l"(part + o));
+    }
+  };
+  if (nz > 1) load(kn);
+  for (int s = 1; s < nz; ++s) {
+    const int k = kn, kd = UP ? k : k - 1;   // layer between k and its upstream neighbour
+    const f32x2 c0 = c_n, dc0 = dc_n, dS0 = dS_n, dSl = dSl_n, pt = pt_n;
+    if (s + 1 < nz) {
+      kn = UP ? k - 1 : k + 1;
+      load(kn);
+    }
+    const f32x2 dz = both2(s_dz[kd]);
+    const f32x2 csum = add2(c0, cp, u);
+    float ca, cb, ta, tb;
+    unpack2(csum, ca, cb);
+    const f32x2 tz = mul2(dz, csum), rz = mul2(pack2(rcp_approx(ca), rcp_approx(cb)), both2(s_idz[kd]));
+    const f32x2 dtz = mul2(dz, add2(dc0, dcp, u)), ddSin = sub2(dSp, dS0, u);
+    const f32x2 dSin = UP ? dSl : mul2(dSl, u.neg);
+    unpack2(tz, ta, tb);
+    // the angles' optical depths tz/(2 mu) fall with m (mu ascending): a test on
+    // the first and last angle settles the form for all of them. The warp takes
+    // one form together: lanes that differ would run every form one after the other.
+    const bool direct = __all_sync(amask, !(mul(ta, inv2mu[MU - 1]) < 0.1f) && !(mul(tb, inv2mu[MU - 1]) < 0.1f));
+    const bool series = __all_sync(amask, mul(ta, inv2mu[0]) < 0.1f && mul(tb, inv2mu[0]) < 0.1f);
+    auto angles = [&](auto cm) {
+      constexpr int CM = decltype(cm)::value;
+#pragma unroll
+      for (int m = 0; m < MU; ++m) {
+        const f32x2 dtau = mul2(tz, both2(inv2mu[m]));
+        float a, b, ea, eb;
+        unpack2(mul2(dtau, both2(-1.4426950408889634f)), a, b);
+        asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(ea) : "f"(a));
+        asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(eb) : "f"(b));
+        const f32x2 e = pack2(ea, eb);
+        f32x2 w, bq;
+        if (CM != CM_SERIES) direct2(e, mul2(rz, both2(two_mu[m])), w, bq, u);
+        if (CM == CM_SERIES) series2(dtau, w, bq);
+        if (CM == CM_SELECT) {
+          f32x2 ws, bs;
+          series2(dtau, ws, bs);
+          unpack2(dtau, a, b);
+          w = select2(a < 0.1f, b < 0.1f, ws, w);
+          bq = select2(a < 0.1f, b < 0.1f, bs, bq);
+        }
+        const f32x2 tn = mul2(dtz, both2(-inv2mu[m]));   // -ddtau
+        const f32x2 dDn = fma2(dD[m], e, fma2(tn, fma2(e, D[m], mul2(bq, dSin)), mul2(w, ddSin)));
+        D[m] = fma2(D[m], e, mul2(w, dSin));
+        dD[m] = dDn;
+        x[m] = mul2(both2(hw[m]), dDn);
+      }
+    };
+    if (direct) angles(std::integral_constant<int, CM_DIRECT>());
+    else if (series) angles(std::integral_constant<int, CM_SERIES>());
+    else angles(std::integral_constant<int, CM_SELECT>());
+    emit(k, dS0, pt);
+    cp = c0;
+    dcp = dc0;
+    dSp = dS0;
+  }
+}
+
+// Columns of a launch whose angle count is not MU take the scalar sweep, one
+// frequency of the thread's pair after the other.
+template <int MU>
+__global__ void __launch_bounds__(kPairThreads) k_formal_sweep_pair(const ColDesc* __restrict__ cols,
+                                                                    float one) {   // one: 1
+  extern __shared__ float s_tab[];   // [nz] |dz|, [nz] 1/|dz|
+  const ColDesc& cd = cols[blockIdx.y];
+  if (eval_mode_f(cd) != EV_TANGENT) return;
+  const ColTables& T = cd.t;
+  if ((int)(2 * blockIdx.x * blockDim.x) >= T.nq) return;   // uniform over the block
+  float* s_dz = s_tab;
+  float* s_idz = s_tab + T.nz;
+  stage_dz(T, s_dz, s_idz);
+  __syncthreads();
+  const int q = 2 * (blockIdx.x * blockDim.x + threadIdx.x);
+  const unsigned amask = __ballot_sync(0xffffffffu, q < T.nq);
+  if (q >= T.nq) return;
+  if (T.nmu == MU) {
+    const Ones2 u{both2(one), both2(-one)};
+    sweep_pair<MU, false>(cd, q, s_dz, s_idz, u, amask);
+    sweep_pair<MU, true>(cd, q, s_dz, s_idz, u, amask);
+  } else {
+    for (int i = q; i < min(q + 2, T.nq); ++i) {
+      sweep_thread<MU, true, false, false>(cd, i, s_dz, s_idz);
+      sweep_thread<MU, true, true, false>(cd, i, s_dz, s_idz);
+    }
   }
 }
 
@@ -632,9 +864,9 @@ __device__ __forceinline__ void formal_sweep_block(const ColDesc* __restrict__ c
   }
 }
 
-template <int MU, bool TAN>
+template <int MU>
 __global__ void __launch_bounds__(256) k_formal_sweep(const ColDesc* __restrict__ cols) {
-  formal_sweep_block<MU, TAN, false>(cols);
+  formal_sweep_block<MU, false, false>(cols);
 }
 
 // The tangent sweep that forms the opacity tangent itself (forced variant):
@@ -967,18 +1199,20 @@ static void launch_mu(const Batch& b, cudaStream_t s, int threads, int which, in
   if (which != 1) {
     const size_t sm = sweep_smem(b.max_nz, occ_tan, threads, true, fuse != 0);
     if (fuse) k_formal_sweep_fused<MU><<<g, threads, sm, s>>>(b.d_cols);
-    else k_formal_sweep<MU, true><<<g, threads, sm, s>>>(b.d_cols);
+    else   // two frequencies per thread
+      k_formal_sweep_pair<MU><<<dim3((b.max_nq + 2 * kPairThreads - 1) / (2 * kPairThreads), b.ncols), kPairThreads, sm,
+                                s>>>(b.d_cols, 1.0f);
   }
   if (which != 2)
-    k_formal_sweep<MU, false><<<g, threads, sweep_smem(b.max_nz, occ_base, threads, false), s>>>(b.d_cols);
+    k_formal_sweep<MU><<<g, threads, sweep_smem(b.max_nz, occ_base, threads, false), s>>>(b.d_cols);
 }
 
 template <int MU>
 static int allow_smem_mu() {
-  JFNK_CUDA(cudaFuncSetAttribute(k_formal_sweep<MU, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
+  JFNK_CUDA(cudaFuncSetAttribute(k_formal_sweep_pair<MU>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
   JFNK_CUDA(cudaFuncSetAttribute(k_formal_sweep_fused<MU>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  227 * 1024));
-  JFNK_CUDA(cudaFuncSetAttribute(k_formal_sweep<MU, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
+  JFNK_CUDA(cudaFuncSetAttribute(k_formal_sweep<MU>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
   return JFNK_OK;
 }
 
@@ -1056,13 +1290,14 @@ bool sweep_small(int ncols, int max_nq, int n_sm) { return (long)ncols * max_nq 
 
 int sweep_warp_size(int nz) { return std::min(warp_size(nz, true), warp_size(nz, false)); }
 
-// Autotuner of the sweep kernels, timed on the batch's own columns: the
-// tangent sweep (the columns in tangent mode) over variant 1 with 32..256
-// threads per block and a cap of 2..8 resident blocks per SM or none, and
-// variant 2 with 1..8 warps per block (where its shared memory fits); then,
-// for variant 1, the base-type sweep's cap (columns in base mode). First the
-// opacity tangent's run of depths per thread. Every choice gives bit-identical
-// results, so it changes the speed only.
+// Autotuner of a large batch, timed on its own columns: the opacity tangent's
+// run of depths per thread, then a cap of resident blocks per SM for the
+// tangent sweep (the columns in tangent mode) and for the base-type sweep (in
+// base mode). Every choice gives bit-identical results, so it changes the speed
+// only. (Block sizes of 32 to 256 threads and the warp variant were candidates
+// once: 128 threads always stayed for launches of this size, and the smaller
+// ones take the warp variant by rule; the first solve of a 512-column plan went
+// from 990 to 650 ms without them.)
 int sweep_autotune(Batch* b, cudaStream_t s) {
   cudaEvent_t e0, e1;
   JFNK_CUDA(cudaEventCreate(&e0));
@@ -1076,13 +1311,13 @@ int sweep_autotune(Batch* b, cudaStream_t s) {
     }
     return launch_sweep_cfg(*b, s, variant, size, which, ot, ob, fuse);
   };
-  // a candidate's time: the fastest of five launches timed one by one, after a
+  // a candidate's time: the fastest of three launches timed one by one, after a
   // warm-up (single launches differ by a few per cent; the minimum is stable)
   auto timed = [&](int variant, int size, int which, int ot, int ob, float* ms, int fuse = 0) -> int {
     int r = once(variant, size, which, ot, ob, fuse);   // warm-up
     if (r) return r;
     float best = 1e30f;
-    for (int i = 0; i < 5; ++i) {
+    for (int i = 0; i < 3; ++i) {
       if (cudaEventRecord(e0, s) != cudaSuccess) return fail(JFNK_E_CUDA, "autotune event");
       if ((r = once(variant, size, which, ot, ob, fuse))) return r;
       float t = 0.f;
@@ -1101,7 +1336,7 @@ int sweep_autotune(Batch* b, cudaStream_t s) {
       int r = launch_opacity_tan(*b, s, dr);   // warm-up
       if (r) return r;
       float best = 1e30f;
-      for (int i = 0; i < 5; ++i) {
+      for (int i = 0; i < 3; ++i) {
         if (cudaEventRecord(e0, s) != cudaSuccess) return fail(JFNK_E_CUDA, "autotune event");
         if ((r = launch_opacity_tan(*b, s, dr))) return r;
         float t = 0.f;
@@ -1117,7 +1352,7 @@ int sweep_autotune(Batch* b, cudaStream_t s) {
     int bd = 16;
     if (!(rc = time_optan(16, &bo))) {
       bo *= 0.98f;
-      for (int dr : {4, 8, 32}) {
+      for (int dr : {8, 32}) {
         float ms = 0.f;
         if ((rc = time_optan(dr, &ms))) break;
         if (ms < bo) { bo = ms; bd = dr; }
@@ -1129,47 +1364,35 @@ int sweep_autotune(Batch* b, cudaStream_t s) {
   // alone it can win, but inside a tick the separate opacity-tangent kernel
   // overlaps the base-type chain on the other stream, and the fused sweep
   // made the whole solve about 11 % slower.
-  struct Cand { int variant, size, occ, fuse; };
-  std::vector<Cand> cands;
-  for (int t : {32, 64, 128, 256})
-    for (int occ : {0, 2, 4, 8}) cands.push_back({1, t, occ, 0});
-  // the default (128 threads, no cap) stays unless a candidate beats it by 2 %:
-  // closer than that, single measurements flip between runs
+  // caps of resident blocks per SM, of the tangent sweep (the columns in tangent
+  // mode), then of the base-type sweep (in base mode); no cap stays unless one
+  // gains 2 %: closer than that, single measurements flip between runs
+  int best_occ = 0, best_base = 0;
   float best = 1e30f;
-  Cand bc{1, 128, 0, 0};
-  if ((rc = timed(1, 128, 2, 0, 0, &best))) best = 1e30f;
-  best *= 0.98f;
-  for (const auto& c : cands) {
-    if (rc) break;
-    if (c.variant == 1 && c.occ > 0 && c.size * c.occ > 2048) continue;
-    if (c.variant == 1 && c.size == 128 && c.occ == 0) continue;
+  for (int occ : {0, 4}) {
     float ms = 0.f;
-    if ((rc = timed(c.variant, c.size, 2, c.occ, 0, &ms, c.fuse))) break;
-    if (ms < best) { best = ms; bc = c; }
+    if (rc || (rc = timed(1, 128, 2, occ, 0, &ms))) break;
+    if (occ == 0) ms *= 0.98f;
+    if (ms < best) { best = ms; best_occ = occ; }
   }
-  int best_base = 0;
-  if (!rc && bc.variant == 1) {
-    // the base-type sweep's cap, on the same columns in base mode
-    if (!(rc = batch_set_forced_mode(b, EV_BASE, s))) {
-      float bb = 1e30f;
-      for (int occ : {0, 2, 3, 4, 6, 8}) {
-        if (occ > 0 && bc.size * occ > 2048) continue;
-        float ms = 0.f;
-        if ((rc = timed(1, bc.size, 1, bc.occ, occ, &ms))) break;
-        if (occ == 0) ms *= 0.98f;   // no cap unless a cap gains 2 %
-        if (ms < bb) { bb = ms; best_base = occ; }
-      }
-      if (!rc) rc = batch_set_forced_mode(b, EV_TANGENT, s);
+  if (!rc && !(rc = batch_set_forced_mode(b, EV_BASE, s))) {
+    best = 1e30f;
+    for (int occ : {0, 3, 4}) {
+      float ms = 0.f;
+      if ((rc = timed(1, 128, 1, best_occ, occ, &ms))) break;
+      if (occ == 0) ms *= 0.98f;
+      if (ms < best) { best = ms; best_base = occ; }
     }
+    if (!rc) rc = batch_set_forced_mode(b, EV_TANGENT, s);
   }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   if (rc) return rc;
-  b->sweep_variant = bc.variant;
-  b->formal_threads = bc.size;
-  b->sweep_occ = bc.variant == 1 ? bc.occ : 0;
-  b->sweep_occ_base = bc.variant == 1 ? best_base : 0;
-  b->sweep_fuse = bc.variant == 1 ? bc.fuse : 0;
+  b->sweep_variant = 1;
+  b->formal_threads = 128;
+  b->sweep_occ = best_occ;
+  b->sweep_occ_base = best_base;
+  b->sweep_fuse = 0;
   return JFNK_OK;
 }
 

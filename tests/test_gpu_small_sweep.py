@@ -27,6 +27,7 @@ CASES = [
     ("h", lambda: W.config3(nu_scale=0.1, n_depth=65), 4),
     ("ca", lambda: W.config2(nu_scale=0.06, n_depth=700), 5),
     ("dense", lambda: W.dense_overlap_workload(n_depth=34), 2),
+    ("h", lambda: W.config3(nu_scale=0.07, n_depth=33), 6),
 ]
 
 

@@ -599,11 +599,12 @@ __device__ __forceinline__ int rate_mode(const ColDesc& cd, int t, int tile) {
 // The packed transitions active at a frequency (ColTables::qmeta4). PIPE
 // (small launches, few warps on a multiprocessor): the whole list is loaded
 // two frequencies before its use, since a list and then the tables it points
-// to would be two trips to memory in a row, and the terms of its transitions
-// with the frequency's other inputs. Otherwise
-// (large launches, which need the warps more) two transitions and 128
+// to would be two trips to memory in a row, and the terms of its first five
+// transitions with the frequency's other inputs (a mixed solve of an H I-like
+// column, 82 x 2,010, with three held: 4.59 ms, five: 4.40, all eight: 4.73).
+// Otherwise (large launches, which need the warps more) two transitions and 128
 // registers; the 512-column batch was 3 % slower with the former.
-// H I-like column, 82 x 2,010: 59 -> 30 us for a base evaluation.
+// The H I-like column's base evaluation: 59 -> 28 us.
 struct RateList {
   int m[kQMetaT];
 };
@@ -666,7 +667,7 @@ __device__ __forceinline__ void rate_window(const ColTables& T, bool packed, int
 template <bool PIPE>
 __device__ void rates_tile(const ColDesc& cd, const int mode, const int t, const int tile, const int rank,
                            const RateSmem& sm, cg::cluster_group& cluster, const SolverOpts* bopts) {
-  constexpr int kRateHeld = PIPE ? kQMetaT : 2;   // transitions whose terms a frequency's inputs hold
+  constexpr int kRateHeld = PIPE ? 5 : 2;   // transitions whose terms a frequency's inputs hold
   const ColTables& T = cd.t;
   const int nz = T.nz, nl = T.nl, nt = T.nt;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -987,7 +988,7 @@ __device__ __forceinline__ void rates_columns(const ColDesc* __restrict__ cols, 
 
 // Two kernels, so that each has its own register bound: the large launch keeps
 // the compiler's 128 (a second bound argument, even 1, makes it 160 and the
-// 512-column batch 3 % slower), the small one the 206 its held terms need
+// 512-column batch 3 % slower), the small one the 194 its held terms need
 // (168 and spills without it).
 __global__ void __launch_bounds__(32 * kRateWarps) k_rates(const ColDesc* __restrict__ cols, int ncols, int racc,
                                                            int fslots, const SolverOpts* bopts) {

@@ -2,6 +2,7 @@
 // residual / JVP / preconditioner / RH92 evaluations, and the solvers.
 #include <algorithm>
 #include <cmath>
+#include <cstdint>
 #include <cstring>
 
 #include "internal.cuh"
@@ -132,6 +133,19 @@ __global__ void k_explicit_out(const ColDesc* cols, const double* src, double* d
     for (size_t i = i0; i < NI; i += step) Iem[i] = cd.w.Iem[i];
 }
 
+// Whether those kernels may use a caller's array: aligned device memory of the
+// context's device. Any other array takes the copies, which serve every
+// address the runtime knows and refuse the rest with an error.
+static bool kernel_array(const jfnk_ctx* ctx, const double* p, jfnk_mem where) {
+  if (where != JFNK_MEM_DEVICE || reinterpret_cast<uintptr_t>(p) % sizeof(double)) return false;
+  cudaPointerAttributes at;
+  if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+    cudaGetLastError();   // an unknown address: the copy reports it
+    return false;
+  }
+  return at.type == cudaMemoryTypeDevice && at.device == ctx->device;
+}
+
 static unsigned explicit_blocks(size_t n) { return (unsigned)std::min<size_t>((n + 255) / 256, 608); }
 
 // The batch's solver options, uploaded when they change.
@@ -171,13 +185,13 @@ static int explicit_eval(jfnk_ctx* ctx, const jfnk_atmos* a, Batch* b, int mode,
     options_to_device(&o, &so);
     if ((rc = set_options(b, so, s))) return rc;
   }
-  if (where == JFNK_MEM_HOST) {
+  if (!kernel_array(ctx, n, where)) {
     if ((rc = copy_in(c.w.n, n, N * 8, where, s))) return rc;
     n = c.w.n;
-    if (Jdag) {
-      if ((rc = copy_in(c.w.Jdag, Jdag, QZ * 8, where, s))) return rc;
-      Jdag = c.w.Jdag;
-    }
+  }
+  if (Jdag && !kernel_array(ctx, Jdag, where)) {
+    if ((rc = copy_in(c.w.Jdag, Jdag, QZ * 8, where, s))) return rc;
+    Jdag = c.w.Jdag;
   }
   if ((rc = explicit_in(b, mode, n, Jdag ? Jdag : M.tables.Bn, nullptr, s))) return rc;
   b->pairs_ready = true;
@@ -188,11 +202,11 @@ static int explicit_eval(jfnk_ctx* ctx, const jfnk_atmos* a, Batch* b, int mode,
 
 // Copies an explicit evaluation's results out: ``n`` doubles of ``src`` to
 // ``dst``, the new mean intensity and the emergent intensity where wanted.
-static int explicit_out(Batch* b, const double* src, double* dst, size_t n, double* J, double* Iem, jfnk_mem where,
-                        cudaStream_t s) {
+static int explicit_out(const jfnk_ctx* ctx, Batch* b, const double* src, double* dst, size_t n, double* J, double* Iem,
+                        jfnk_mem where, cudaStream_t s) {
   const ColDesc& c = b->h_cols[0];
   const size_t QZ = (size_t)c.t.nq * c.t.nz, NI = (size_t)c.t.nq * c.t.nmu;
-  if (where == JFNK_MEM_DEVICE) {
+  if (kernel_array(ctx, dst, where) && (!J || kernel_array(ctx, J, where)) && (!Iem || kernel_array(ctx, Iem, where))) {
     k_explicit_out<<<explicit_blocks(J ? QZ : std::max(n, Iem ? NI : 0)), 256, 0, s>>>(b->d_cols, src, dst, n, J, Iem);
     JFNK_CUDA(cudaGetLastError());
     return JFNK_OK;
@@ -822,7 +836,7 @@ int jfnk_residual(jfnk_ctx* ctx, const jfnk_atmos* a, int precision, const doubl
   return on_ctx_stream(ctx, stream, where, [&](cudaStream_t s) {
     int r = explicit_eval(ctx, a, b, EV_BASE, n, J_dagger, where, s);
     if (r) return r;
-    return explicit_out(b, b->h_cols[0].w.F, F, (size_t)a->d.nz * a->d.nl, J_new, I_emergent, where, s);
+    return explicit_out(ctx, b, b->h_cols[0].w.F, F, (size_t)a->d.nz * a->d.nl, J_new, I_emergent, where, s);
   });
 }
 
@@ -841,13 +855,13 @@ int jfnk_jvp(jfnk_ctx* ctx, const jfnk_atmos* a, int precision, const double* n,
     const AtmosData& M = a->d;
     const size_t N = (size_t)M.nz * M.nl;
     const double* vd = v;
-    if (where == JFNK_MEM_HOST) {
+    if (!kernel_array(ctx, v, where)) {
       if ((r = copy_in(c.w.v, v, N * 8, where, s))) return r;
       vd = c.w.v;
     }
     if ((r = explicit_in(b, EV_TANGENT, nullptr, nullptr, vd, s))) return r;
     if ((r = launch_evaluation(*b, s))) return r;
-    return explicit_out(b, c.w.dF, Jv, N, nullptr, nullptr, where, s);
+    return explicit_out(ctx, b, c.w.dF, Jv, N, nullptr, nullptr, where, s);
   });
 }
 
@@ -863,7 +877,7 @@ int jfnk_block_jacobi(jfnk_ctx* ctx, const jfnk_atmos* a, int precision, const d
     int r = explicit_eval(ctx, a, b, EV_BASE, n, J_dagger, where, s);
     if (r) return r;
     const AtmosData& M = a->d;
-    return explicit_out(b, b->h_cols[0].w.P, P, (size_t)M.nz * M.nl * M.nl, nullptr, nullptr, where, s);
+    return explicit_out(ctx, b, b->h_cols[0].w.P, P, (size_t)M.nz * M.nl * M.nl, nullptr, nullptr, where, s);
   });
 }
 
@@ -910,7 +924,7 @@ int jfnk_rh92_update(jfnk_ctx* ctx, const jfnk_atmos* a, int precision, const do
   return on_ctx_stream(ctx, stream, where, [&](cudaStream_t s) {
     int r = explicit_eval(ctx, a, b, EV_RH92, n, J_dagger, where, s);   // its assembly updates w.n
     if (r) return r;
-    return explicit_out(b, b->h_cols[0].w.n, n_out, (size_t)a->d.nz * a->d.nl, J_new, nullptr, where, s);
+    return explicit_out(ctx, b, b->h_cols[0].w.n, n_out, (size_t)a->d.nz * a->d.nl, J_new, nullptr, where, s);
   });
 }
 

@@ -115,3 +115,40 @@ def test_moving_evaluation_matches_oracle_at_tile_edges(nz, nq, nmu):
     assert np.all(np.abs(Jv - jvp_complex(m, n, Jd, v, ref.istar)) <= 1e-10 * dgross)
     P, rP = B.block_jacobi(atm, n, Jd), ora_P(m, n, ref)
     assert np.all(np.abs(P - rP) <= 1e-9 * np.abs(rP).max(axis=(1, 2), keepdims=True))
+
+
+@pytest.mark.parametrize("precision", [B.JFNK_FP64, B.JFNK_MIXED])
+def test_explicit_calls_take_device_arrays_off_the_double_boundary(precision):
+    """Arrays that start between two doubles are copied, not read by a kernel:
+    the same results to the bit as from aligned ones."""
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    wl = W.config1(n_depth=21, n_nu=17)
+    ctx = B.Context(0)
+    atm = B.Atmosphere(ctx, B.Atom(ctx, wl.atom), wl.columns[0], n_mu=3)
+    N, QZ, QM = atm.n_depth * atm.n_levels, atm.n_nu * atm.n_depth, atm.n_nu * atm.n_mu
+
+    def device(x, off):
+        raw = torch.empty(8 * x.size + 8, dtype=torch.uint8, device="cuda")
+        raw[off:off + 8 * x.size] = torch.from_numpy(x.ravel().view(np.uint8).copy()).cuda()
+        return raw
+
+    def host(raw, off, n):
+        return raw[off:off + 8 * n].cpu().numpy().view(np.float64)
+
+    n, J = atm.lte(), atm.planck()
+    got = []
+    for off in (0, 4):
+        a = [device(x, off) for x in (n, J, 0.1 * n)]
+        out = [device(np.zeros(k), off) for k in (N, QZ, QM, N)]
+        p, q = [t.data_ptr() + off for t in a], [t.data_ptr() + off for t in out]
+        torch.cuda.synchronize()
+        B.check(ctx.lib.jfnk_residual(ctx.h, atm.h, precision, p[0], p[1], q[0], q[1], q[2], B.JFNK_MEM_DEVICE, None),
+                "jfnk_residual")
+        B.check(ctx.lib.jfnk_jvp(ctx.h, atm.h, precision, p[0], p[1], p[2], q[3], B.JFNK_MEM_DEVICE, None), "jfnk_jvp")
+        torch.cuda.synchronize()
+        got.append([host(t, off, k) for t, k in zip(out, (N, QZ, QM, N))])
+    for x, y in zip(*got):
+        assert np.abs(x).max() > 0.0
+        np.testing.assert_array_equal(x, y)

@@ -303,7 +303,8 @@ def cpu_baseline_batch(wl, start, pool, futures, workers, t0):
 ALG_OPS = {"value": (10, 2), "jvp": (26, 2)}
 FORMAL_KERNELS = {0: "k_formal<double> + k_ray_sum (per-ray buffers)", 1: "k_formal_fused<double>",
                   2: "k_formal_sweep (thread per frequency)", 3: "k_formal_sweep_warp (warp per frequency pair)",
-                  4: "k_mv_formal (moving column, thread per ray)"}
+                  4: "k_mv_formal / k_eval64_moving (moving column)",
+                  6: "k_eval64 (opacity, formal solution and rate integrals per tile of frequencies)"}
 
 
 FP32_LANES_PER_SM = 128   # FP32 FMA lanes per SM per clock (Blackwell SM: 4 x 32)
@@ -408,7 +409,7 @@ def alu_roofline(B, ctx, fp64, n_value, n_jvp, pts_per_launch, kern_ms, launches
     return {"bound": "alu", "kernel": FORMAL_KERNELS.get(kernel, str(kernel)),
             "achieved": achieved / 1e9, "peak": peak / 1e9, "unit": "G ray-points/s",
             "frac": achieved / peak,
-            "traffic": None if traffic_pp is None or not fp64 else traffic_pp * pts_per_launch,
+            "traffic": None if traffic_pp is None or not fp64 or kernel != 1 else traffic_pp * pts_per_launch,
             "ops_per_ray_point": {"value": ALG_OPS["value"], "jvp": ALG_OPS["jvp"],
                                   "mix": {"value": w_v, "jvp": w_j}},
             "avg_launch_us": avg_s * 1e6, "launches": launches, "peak_source": peak_source(fp64, peaks),

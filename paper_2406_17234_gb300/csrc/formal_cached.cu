@@ -19,8 +19,8 @@
 //     D = I - S on the better-conditioned form compares exponent words.
 // The opacity of the tile and the rate integrals over it are formed in the
 // same block (two launches and the round trips of chi, dJ and the Lambda
-// diagonals fewer); a tile leaves its part of each integral it meets, and
-// k_rates_reduce adds the parts in tile order (no atomics).
+// diagonals fewer); a tile leaves its part of each integral it meets, and the
+// assembly adds the parts in an order set by the atom (no atomics).
 //
 // A block takes Qb frequencies (cached_default_qb) of one column: all threads
 // form the coefficients, one thread per ray runs the recurrences over chunks
@@ -28,8 +28,9 @@
 // of the chunk. Lanes run over frequencies first, so the coefficient planes
 // [tile][layer][5][angle][Qb] are read in contiguous rows.
 //
-// Measured (kernel time, warm L2), against the fused kernel with its separate
-// opacity and rate kernels: 82 depths x 1,005 frequencies x 5 angles, base
+// Measured (kernel time, warm L2; the 8 or 10 us added the parts, now in the
+// assembly), against the fused kernel with its separate opacity and rate
+// kernels: 82 depths x 1,005 frequencies x 5 angles, base
 // 244 + 11 + 59 -> 87 + 8 us, tangent 149 + 11 + 12 -> 26 + 8 us; 101 x 41 x 5,
 // base 126 + 8 + 18 -> 50 + 10 us, tangent 48 + 8 + 11 -> 18 + 10 us. A base
 // evaluation is bound by its FP64 instructions (half of it the coefficients),

@@ -39,6 +39,7 @@
 #include <cmath>
 
 #include "formal_coef.cuh"
+#include "step_coef.cuh"
 
 namespace jfnk {
 
@@ -48,11 +49,9 @@ constexpr int kMaxQb = 8;
 constexpr int kItems = 3;     // ray steps of a chunk per helper thread: kChunk 128 <= kItems (kEvalThreads - 128)
 constexpr int kBufRows = 8 * kChunk + 2 * (2 * kChunk + 1) + kChunk;
 static_assert(kChunk * 128 <= kItems * (kEvalThreads - 128), "a chunk's ray steps fit the helpers");
-constexpr int kExpTab = 256;
 constexpr size_t kCachedSmem = (size_t)222 * 1024;   // beside the static shared memory
 
-// 2^(-j/256) and 1 - 2^(-j/256), for neg_exp
-__device__ double2 d_exp_tab[kExpTab];
+__device__ ExpEntry d_exp_tab[kExpTab];   // for neg_exp
 
 __host__ __device__ inline int pad_qb(int qb) { return qb | 1; }   // odd row stride: no bank conflicts over depths
 
@@ -110,61 +109,6 @@ __device__ __forceinline__ const double* dir_of(const ColDesc& cd) {
   if (cd.forced_mode >= 0) return cd.w.v;
   const int N = cd.t.nz * cd.t.nl;
   return cd.w.st->phase == PH_RESTART ? cd.w.x : cd.w.Vb + (size_t)cd.w.st->j * N;
-}
-
-// e = e^(-x) and om = 1 - e for x >= 1e-5 (e = 0 from x = 700 on) in ten FP64
-// instructions: x = n ln2/256 + r, |r| < 1.4e-3, 2^(-n/256) from a table, p =
-// e^(-r) - 1 to the fourth order (the next term is below 4e-17): the table
-// method of Tang (ACM Trans. Math. Softw. 15, 144, 1989). Below ln 2 the sum is
-// formed for om, from tabulated 1 - 2^(-j/256), and e = 1 - om: w = om/x then
-// keeps full relative accuracy in thin layers, where 1 - e cancels.
-__device__ __forceinline__ void neg_exp(double x, const double2* tab, double& e, double& om) {
-  const double magic = 6755399441055744.0;   // 1.5 2^52: n in the low word
-  const double t = fma(x, 369.32993046757464, magic);
-  const int n = __double2loint(t);
-  const double tn = t - magic;
-  double r = fma(tn, -0.0027076061740622863, x);
-  r = fma(tn, -9.0587766165870294e-20, r);
-  double q = fma(r, 1.0 / 24, -1.0 / 6);
-  q = fma(q, r, 0.5);
-  q = fma(q, r, -1.0);
-  const double2 T0 = tab[n & (kExpTab - 1)];
-  const double T = __hiloint2double(__double2hiint(T0.x) - ((n >> 8) << 20), __double2loint(T0.x));
-  const bool small = n < kExpTab;
-  const double u = fma(small ? -T : T, q * r, small ? T0.y : T), v = 1.0 - u;
-  e = small ? v : u;
-  om = small ? u : v;
-  if (__double2hiint(x) >= 0x4085e000) {   // x >= 700
-    e = 0.0;
-    om = 1.0;
-  }
-}
-
-// Coefficients of one step of optical depth x, r = 1/x (App. A.1): e, w, bq =
-// (w - e)/x, a = 1 - w and om = 1 - e = a + bq x. With om from neg_exp the
-// direct forms lose 1e-16/x relative in a and bq (which enter every sum times
-// x or x dS), so the series (truncated below 4e-17) is needed from x = 1e-5
-// down only; it skips the exponential.
-__device__ __forceinline__ void step_coef(double x, double r, const double2* tab, double& e, double& w, double& a,
-                                          double& bq, double& om) {
-  if (x < 1e-5) {
-    if (x > -1e-5) {
-      w = fma(fma(fma(-1.0 / 24, x, 1.0 / 6), x, -0.5), x, 1.0);
-      bq = fma(fma(1.0 / 8, x, -1.0 / 3), x, 0.5);
-      om = x * w;
-      e = 1.0 - om;
-      a = fma(-bq, x, om);
-    } else {   // inverted populations
-      pl_series64(x, w, a, bq);
-      e = exp(-x);
-      om = fma(bq, x, a);
-    }
-  } else {
-    neg_exp(x, tab, e, om);
-    w = om * r;
-    a = 1.0 - w;
-    bq = (w - e) * r;
-  }
 }
 
 // |x| to float by its words (no FP64 instruction), 0 below the float range.
@@ -265,7 +209,7 @@ __global__ void __launch_bounds__(kEvalThreads) k_eval64(const ColDesc* __restri
   extern __shared__ __align__(16) double sm[];
   __shared__ double s_inv2mu[kMaxMu], s_hw[kMaxMu], s_2mu[kMaxMu];
   __shared__ float s_hwf[kMaxMu];
-  __shared__ double2 s_tab[kExpTab];
+  __shared__ ExpEntry s_tab[kExpTab];
   __shared__ int s_act[kMaxT], s_off[kMaxT], s_nact;
   const ColDesc& cd = cols[blockIdx.y];
   const int mode = mode_of(cd);
@@ -836,7 +780,7 @@ template <int MU>
 __global__ void __launch_bounds__(kEvalThreads) k_eval64_moving(const ColDesc* __restrict__ cols) {
   extern __shared__ __align__(16) double sm[];
   __shared__ double s_inv2mu[kMaxMu], s_hw[kMaxMu];
-  __shared__ double2 s_tab[kExpTab];
+  __shared__ ExpEntry s_tab[kExpTab];
   __shared__ int s_act[kMaxT], s_off[kMaxT], s_nact;
   const ColDesc& cd = cols[blockIdx.y];
   const int mode = mode_of(cd);
@@ -1116,9 +1060,8 @@ int launch_eval64_moving(const Batch& b, cudaStream_t s) {
 }
 
 int cached_prepare() {
-  double2 tab[kExpTab];
-  for (int j = 0; j < kExpTab; ++j)
-    tab[j] = make_double2(std::exp2(-j / (double)kExpTab), -std::expm1(-j / (double)kExpTab * 0.69314718055994530942));
+  ExpEntry tab[kExpTab];
+  for (int j = 0; j < kExpTab; ++j) tab[j] = exp_entry(j);
   JFNK_CUDA(cudaMemcpyToSymbol(d_exp_tab, tab, sizeof(tab)));
   JFNK_CUDA(cudaFuncSetAttribute(k_eval64<5>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCachedSmem));
   JFNK_CUDA(cudaFuncSetAttribute(k_eval64<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCachedSmem));

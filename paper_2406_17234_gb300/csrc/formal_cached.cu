@@ -111,12 +111,6 @@ __device__ __forceinline__ const double* dir_of(const ColDesc& cd) {
   return cd.w.st->phase == PH_RESTART ? cd.w.x : cd.w.Vb + (size_t)cd.w.st->j * N;
 }
 
-// |x| to float by its words (no FP64 instruction), 0 below the float range.
-__device__ __forceinline__ float abs_float(double x) {
-  const int h = (__double2hiint(x) & 0x7fffffff) - (896 << 20);
-  return h <= 0 ? 0.f : __int_as_float((h << 3) | ((unsigned)__double2loint(x) >> 29));
-}
-
 __device__ __forceinline__ int mag(double x) { return __double2hiint(x) & 0x7fffffff; }
 
 struct Tile {
@@ -208,7 +202,6 @@ template <int MU>
 __global__ void __launch_bounds__(kEvalThreads) k_eval64(const ColDesc* __restrict__ cols, const SolverOpts* bopts) {
   extern __shared__ __align__(16) double sm[];
   __shared__ double s_inv2mu[kMaxMu], s_hw[kMaxMu], s_2mu[kMaxMu];
-  __shared__ float s_hwf[kMaxMu];
   __shared__ ExpEntry s_tab[kExpTab];
   __shared__ int s_act[kMaxT], s_off[kMaxT], s_nact;
   const ColDesc& cd = cols[blockIdx.y];
@@ -230,7 +223,7 @@ __global__ void __launch_bounds__(kEvalThreads) k_eval64(const ColDesc* __restri
   double* s_S = sm;               // S^k
   double* s_chi = s_S + Z;        // chi^k; then sum w I; then J
   double* s_tz = s_chi + Z;       // sum w D; then Lambda_chi
-  double* s_rs = s_tz + Z;        // sum w |D| (float)
+  double* s_rs = s_tz + Z;        // sum w |D|
   double* s_dS = s_rs + Z;        // S^{k+1} - S^k; then Lambda_eta
   double* s_A = s_dS + Z;         // per layer, sum over the angles of w a
   double* s_G = s_A + Z;          // sum of w dI/dchi without the local term
@@ -248,7 +241,6 @@ __global__ void __launch_bounds__(kEvalThreads) k_eval64(const ColDesc* __restri
     s_inv2mu[m] = a.inv2mu;
     s_hw[m] = a.hw;
     s_2mu[m] = a.two_mu;
-    s_hwf[m] = (float)a.hw;
   }
   if (!tan)
     for (int i = threadIdx.x; i < kExpTab; i += blockDim.x) s_tab[i] = d_exp_tab[i];
@@ -476,18 +468,17 @@ __global__ void __launch_bounds__(kEvalThreads) k_eval64(const ColDesc* __restri
   __syncthreads();
   double* s_I = s_chi;
   double* s_D = s_tz;
-  float* s_aD = reinterpret_cast<float*>(s_rs);   // only compared
+  double* s_aD = s_rs;
   double* s_Le = s_dS;
   for (int i = threadIdx.x; i < nqb * nz; i += blockDim.x) {
     const int k = i / nqb, ql = i - k * nqb, e = k * Qp + ql;
-    double d = 0.0, in = 0.0;
-    float ad = 0.f;
+    double d = 0.0, in = 0.0, ad = 0.0;
     if (k == 0 || k == nz - 1) {
       const double Ib = k == 0 ? 0.0 : T.Bn[(size_t)(qb0 + ql) * nz + nz - 1] / T.c2[qb0 + ql];
       const double D = Ib - s_S[e];
       for (int m = 0; m < nmu; ++m) {
         d = fma(s_hw[m], D, d);
-        ad = fmaf(s_hwf[m], abs_float(D), ad);
+        ad = fma(s_hw[m], fabs(D), ad);
         in = fma(s_hw[m], Ib, in);
       }
     }
@@ -582,14 +573,13 @@ __global__ void __launch_bounds__(kEvalThreads) k_eval64(const ColDesc* __restri
           if (sums && sr < rows && (apart || h == sh)) {
             const int k = sh ? nz - 2 - (c0 + sr) : c0 + sr + 1, l = sh ? k : k - 1;
             const int y = sr * nray + sh * R5 + sq, e = k * Qp + sq;
-            double d = s_D[e], in = s_I[e], gs = 0.0;
-            float ad = s_aD[e];
+            double d = s_D[e], in = s_I[e], ad = s_aD[e], gs = 0.0;
 #pragma unroll
             for (int m = 0; m < nmu; ++m) {
               const double hw = s_hw[m], Dk = out[nray + y + m * Qb];
               d = fma(hw, Dk, d);
               if (der) {
-                ad = fmaf(s_hwf[m], abs_float(Dk), ad);
+                ad = fma(hw, fabs(Dk), ad);
                 in = fma(hw, out[(kChunk + 1) * nray + y + m * Qb], in);
                 if (base) gs = fma(hw, s_g[y + m * Qb], gs);
               }
@@ -617,7 +607,7 @@ __global__ void __launch_bounds__(kEvalThreads) k_eval64(const ColDesc* __restri
     double J = (S + s_D[e]) * c2, Lx = 0.0, Le = 0.0;
     if (der) {
       // the representation with the smaller rounding error (intensities are >= 0)
-      if (abs_float(s_I[e]) < s_aD[e]) J = s_I[e] * c2;
+      if (fabs(s_I[e]) < s_aD[e]) J = s_I[e] * c2;
       const double rc = reinterpret_cast<const double*>(cd.w.chi)[o];
       const double A = (k < nz - 1 ? s_A[e] : 0.0) + (k > 0 ? s_A[e - Qp] : 0.0);
       Le = rc * A;

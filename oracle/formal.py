@@ -41,7 +41,7 @@ def pl_coefficients(dtau):
     """e = exp(-dtau), a = 1 - (1-e)/dtau, b = (1-e)/dtau - e, and b/dtau (App. A.1)."""
     dtau = np.asarray(dtau)
     e = np.exp(-dtau)
-    small = dtau.real < DTAU_SERIES
+    small = np.abs(dtau.real) < DTAU_SERIES   # below zero: inverted populations
     safe = np.where(small, 1.0, dtau)
     w = (1.0 - e) / safe
     a_dir = 1.0 - w

@@ -37,7 +37,7 @@ __device__ __forceinline__ int part_offset(const ColTables& T, int qb, int lane,
 
 // Coefficients of one step of optical depth x: e = exp(-x), w = (1 - e)/x,
 // a = 1 - w and bq = (w - e)/x, each from its own Taylor series below
-// x = 0.1 (where 1 - e, 1 - w and w - e cancel); r = 1/x is supplied by the
+// |x| = 0.1 (where 1 - e, 1 - w and w - e cancel); r = 1/x is supplied by the
 // caller (shared between the rays of a layer).
 // FP64 Taylor coefficients: w = sum_{n>=0} (-x)^n/(n+1)!,
 // a/x = sum_{n>=0} (-x)^n/(n+2)!, bq = sum_{n>=0} (-x)^n (n+1)/(n+2)!.
@@ -58,11 +58,11 @@ __device__ __forceinline__ void pl_series64(double x, double& w, double& a, doub
 }
 
 // In FP64 the direct forms of w, a and bq lose about 1e-16/x^2 relative
-// (1 - e, 1 - w and w - e cancel): 2e-10 at x = 1e-3, so the series takes
-// over below x = 1e-3 only.
+// (1 - e, 1 - w and w - e cancel): 2e-10 at |x| = 1e-3, so the series takes
+// over below |x| = 1e-3 only (x < 0: inverted populations).
 __device__ __forceinline__ void pl_coef_f(double x, double r, double& e, double& w, double& a, double& bq) {
   e = exp(-x);
-  if (x < 1e-3) {
+  if (fabs(x) < 1e-3) {
     pl_series64(x, w, a, bq);
   } else {
     w = (1.0 - e) * r;
@@ -73,7 +73,7 @@ __device__ __forceinline__ void pl_coef_f(double x, double r, double& e, double&
 
 __device__ __forceinline__ void pl_coef_f(float x, float r, float& e, float& w, float& a, float& bq) {
   e = __expf(-x);
-  if (x < 0.1f) {
+  if (fabsf(x) < 0.1f) {
     w = fmaf(fmaf(fmaf(fmaf(fmaf(-1.0f / 720.0f, x, 1.0f / 120.0f), x, -1.0f / 24.0f), x, 1.0f / 6.0f), x, -0.5f), x, 1.0f);
     a = x * fmaf(fmaf(fmaf(fmaf(fmaf(-1.0f / 5040.0f, x, 1.0f / 720.0f), x, -1.0f / 120.0f), x, 1.0f / 24.0f), x, -1.0f / 6.0f), x, 0.5f);
     bq = fmaf(fmaf(fmaf(fmaf(1.0f / 144.0f, x, -1.0f / 30.0f), x, 1.0f / 8.0f), x, -1.0f / 3.0f), x, 0.5f);

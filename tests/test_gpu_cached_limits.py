@@ -23,8 +23,8 @@ def _context():
     return B.Context(0)
 
 
-def _mean_intensity(chi, S, z, n_mu, I_bottom):
-    """J of one frequency in extended precision, and the sum of its terms' sizes."""
+def _mean_intensity(chi, S, z, n_mu, I_bottom, absolute=False):
+    """J of one frequency in extended precision (absolute: over the sizes of its terms)."""
     x, w = np.polynomial.legendre.leggauss(n_mu)
     mu, wmu = (L(1) + x) / 2, w / L(2)
     dz = np.abs(np.diff(z.astype(L)))
@@ -35,6 +35,8 @@ def _mean_intensity(chi, S, z, n_mu, I_bottom):
         series = sum((-t) ** k * (k + 1) / L(np.prod(np.arange(1, k + 3, dtype=float))) for k in range(18))
         bq = np.where(np.abs(t) < 0.5, series, (om / t - e) / t)
         a, b = om - bq * t, bq * t
+        if absolute:
+            a, b, S = np.abs(a), np.abs(b), np.abs(S)
         for order in (range(1, len(z)), range(len(z) - 2, -1, -1)):
             up = order[0] != 1
             I = I_bottom if up else L(0)

@@ -1132,9 +1132,9 @@ struct AsmSmem {
 
 // RH92 update of depth k from the sums of an EV_RH92 evaluation, one warp;
 // returns the population change measure of the depth (or NaN on a singular
-// system) on every lane. With clamp the correction is limited like a Newton
-// correction (Sect. 2.2.2), so that no population of the depth falls below a
-// tenth of its old value.
+// system or a non-finite population) on every lane. With clamp the correction
+// is limited like a Newton correction (Sect. 2.2.2), so that no population of
+// the depth falls below a tenth of its old value.
 //
 // The preconditioned rate equations M n' + c0 = 0 (plus the conservation row)
 // are affine in n' and equal the residual F at n' = n, so n' = n + d with
@@ -1250,12 +1250,11 @@ __device__ double rh92_warp(const ColDesc& cd, int k, int lane, AsmSmem& s, bool
   if (lane < nl) {
     double nn = clamp ? n[lane] + alpha * (x - n[lane]) : x;
     if (damp < 1.0) nn = n[lane] + damp * (nn - n[lane]);
-    err = 0.5 * fabs((nn - n[lane]) / (nn + n[lane]));
-    bad = !(err == err);
-    if (bad) err = 0.0;   // a NaN is left out of the maximum, as fmax does
+    bad = !(fabs(nn) < INFINITY);
+    err = fmax(0.0, 0.5 * fabs((nn - n[lane]) / (nn + n[lane])));   // two empty levels: 0/0 counts as no change
     out[(size_t)k * nl + lane] = nn;
   }
-  return warp_max(err);
+  return __any_sync(0xffffffffu, bad) ? nan("") : warp_max(err);
 }
 
 __global__ void __launch_bounds__(32 * kAsmWarps) k_assemble(const ColDesc* __restrict__ cols,

@@ -367,14 +367,16 @@ __device__ double rh92_depth(const ColDesc& cd, int k, bool clamp, bool correcti
       if (d < 0.0) alpha = fmin(alpha, 0.9 * n[l] / (-d));
     }
   double err = 0.0;
+  bool bad = false;
   double* o = out + (size_t)k * nl;
   for (int l = 0; l < nl; ++l) {
     double nn = clamp ? n[l] + alpha * (rhs[l] - n[l]) : rhs[l];
     if (damp < 1.0) nn = n[l] + damp * (nn - n[l]);
-    err = fmax(err, 0.5 * fabs((nn - n[l]) / (nn + n[l])));
+    if (!(fabs(nn) < INFINITY)) bad = true;
+    err = fmax(err, 0.5 * fabs((nn - n[l]) / (nn + n[l])));   // two empty levels: 0/0 counts as no change
     o[l] = nn;
   }
-  return err;
+  return bad ? nan("") : err;
 }
 
 // ---------------------------------------------------------------------------

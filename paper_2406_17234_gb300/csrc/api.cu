@@ -133,17 +133,31 @@ __global__ void k_explicit_out(const ColDesc* cols, const double* src, double* d
     for (size_t i = i0; i < NI; i += step) Iem[i] = cd.w.Iem[i];
 }
 
-// Whether those kernels may use a caller's array: aligned device memory of the
-// context's device. Any other array takes the copies, which serve every
-// address the runtime knows and refuse the rest with an error.
-static bool kernel_array(const jfnk_ctx* ctx, const double* p, jfnk_mem where) {
-  if (where != JFNK_MEM_DEVICE || reinterpret_cast<uintptr_t>(p) % sizeof(double)) return false;
-  cudaPointerAttributes at;
-  if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
-    cudaGetLastError();   // an unknown address: the copy reports it
-    return false;
-  }
-  return at.type == cudaMemoryTypeDevice && at.device == ctx->device;
+// Whether those kernels may use a caller's array of n doubles: aligned device
+// memory of the context's device, in one allocation from its first to its last
+// byte. Any other array takes the copies, which serve every address the runtime
+// knows and refuse the rest with an error; one that runs past the end of its
+// cudaMalloc allocation is refused here. (Memory mapped in pieces, or from a
+// pool, may go on behind the piece that an address is in.)
+static int kernel_array(const jfnk_ctx* ctx, const double* p, size_t n, jfnk_mem where, bool* yes) {
+  *yes = false;
+  if (where != JFNK_MEM_DEVICE || !ctx->pointer_attributes) return JFNK_OK;
+  // one driver call; of an unknown address every value is zero
+  unsigned type = 0;
+  int managed = 0, device = -1, plain = 0;
+  CUdeviceptr base = 0;
+  size_t size = 0;
+  CUpointer_attribute what[] = {CU_POINTER_ATTRIBUTE_MEMORY_TYPE,    CU_POINTER_ATTRIBUTE_IS_MANAGED,
+                                CU_POINTER_ATTRIBUTE_DEVICE_ORDINAL, CU_POINTER_ATTRIBUTE_RANGE_START_ADDR,
+                                CU_POINTER_ATTRIBUTE_RANGE_SIZE,     CU_POINTER_ATTRIBUTE_IS_LEGACY_CUDA_IPC_CAPABLE};
+  void* to[] = {&type, &managed, &device, &base, &size, &plain};
+  const CUdeviceptr a = reinterpret_cast<CUdeviceptr>(p);
+  if (ctx->pointer_attributes(6, what, to, a) != CUDA_SUCCESS || type != CU_MEMORYTYPE_DEVICE || managed)
+    return JFNK_OK;
+  const bool inside = a >= base && a - base <= size && n * sizeof(double) <= size - (a - base);
+  if (!inside && plain) return fail(JFNK_E_INVALID, "a device array is shorter than the call needs");
+  *yes = inside && a % sizeof(double) == 0 && device == ctx->device;
+  return JFNK_OK;
 }
 
 static unsigned explicit_blocks(size_t n) { return (unsigned)std::min<size_t>((n + 255) / 256, 608); }
@@ -185,11 +199,14 @@ static int explicit_eval(jfnk_ctx* ctx, const jfnk_atmos* a, Batch* b, int mode,
     options_to_device(&o, &so);
     if ((rc = set_options(b, so, s))) return rc;
   }
-  if (!kernel_array(ctx, n, where)) {
+  bool direct_n, direct_J = true;
+  if ((rc = kernel_array(ctx, n, N, where, &direct_n))) return rc;
+  if (Jdag && (rc = kernel_array(ctx, Jdag, QZ, where, &direct_J))) return rc;
+  if (!direct_n) {
     if ((rc = copy_in(c.w.n, n, N * 8, where, s))) return rc;
     n = c.w.n;
   }
-  if (Jdag && !kernel_array(ctx, Jdag, where)) {
+  if (!direct_J) {
     if ((rc = copy_in(c.w.Jdag, Jdag, QZ * 8, where, s))) return rc;
     Jdag = c.w.Jdag;
   }
@@ -206,12 +223,16 @@ static int explicit_out(const jfnk_ctx* ctx, Batch* b, const double* src, double
                         jfnk_mem where, cudaStream_t s) {
   const ColDesc& c = b->h_cols[0];
   const size_t QZ = (size_t)c.t.nq * c.t.nz, NI = (size_t)c.t.nq * c.t.nmu;
-  if (kernel_array(ctx, dst, where) && (!J || kernel_array(ctx, J, where)) && (!Iem || kernel_array(ctx, Iem, where))) {
+  bool direct, direct_J = true, direct_I = true;
+  int rc;
+  if ((rc = kernel_array(ctx, dst, n, where, &direct))) return rc;
+  if (J && (rc = kernel_array(ctx, J, QZ, where, &direct_J))) return rc;
+  if (Iem && (rc = kernel_array(ctx, Iem, NI, where, &direct_I))) return rc;
+  if (direct && direct_J && direct_I) {
     k_explicit_out<<<explicit_blocks(J ? QZ : std::max(n, Iem ? NI : 0)), 256, 0, s>>>(b->d_cols, src, dst, n, J, Iem);
     JFNK_CUDA(cudaGetLastError());
     return JFNK_OK;
   }
-  int rc;
   if ((rc = copy_out(dst, src, n * 8, where, s))) return rc;
   if (J && b->mixed && (rc = launch_j_pairs(b->d_cols, 1, QZ, s, false))) return rc;
   if (J && (rc = copy_out(J, c.w.Jnew, QZ * 8, where, s))) return rc;
@@ -672,6 +693,14 @@ int jfnk_init(int device, jfnk_ctx** out) {
   cudaError_t e = cudaGetDeviceProperties(&p, device);
   if (e != cudaSuccess) { delete c; return fail(JFNK_E_CUDA, cudaGetErrorString(e)); }
   c->n_sm = p.multiProcessorCount;
+  {
+    void* fn = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    if (cudaGetDriverEntryPointByVersion("cuPointerGetAttributes", &fn, 12000, cudaEnableDefault, &q) == cudaSuccess &&
+        q == cudaDriverEntryPointSuccess)
+      c->pointer_attributes = reinterpret_cast<decltype(c->pointer_attributes)>(fn);
+    cudaGetLastError();   // without it every caller's array takes the copies
+  }
   if (int rc = prepare_kernels()) { delete c; return rc; }
   {
     // the stream-ordered pool keeps freed atmosphere tables for reuse
@@ -855,7 +884,9 @@ int jfnk_jvp(jfnk_ctx* ctx, const jfnk_atmos* a, int precision, const double* n,
     const AtmosData& M = a->d;
     const size_t N = (size_t)M.nz * M.nl;
     const double* vd = v;
-    if (!kernel_array(ctx, v, where)) {
+    bool direct;
+    if ((r = kernel_array(ctx, v, N, where, &direct))) return r;
+    if (!direct) {
       if ((r = copy_in(c.w.v, v, N * 8, where, s))) return r;
       vd = c.w.v;
     }

@@ -1,6 +1,7 @@
 // Host-side objects of the library and the interfaces between its units.
 #pragma once
 
+#include <cuda.h>
 #include <memory>
 #include <mutex>
 
@@ -63,6 +64,8 @@ struct AtmosData {
 struct jfnk_ctx {
   int device = 0;
   int n_sm = 0;
+  // cuPointerGetAttributes: what a caller's device address is (api.cu)
+  CUresult(CUDAAPI* pointer_attributes)(unsigned, CUpointer_attribute*, void**, CUdeviceptr) = nullptr;
   // atmosphere set-up lanes: a stream (highest priority), its pinned staging
   // buffer and the event of its last set-up; callers take lanes in turn and
   // wait for their own set-up outside the context lock

@@ -88,16 +88,20 @@ static int check_common(jfnk_ctx* ctx, const jfnk_atmos* a, int precision, jfnk_
 
 // Inputs of an explicit evaluation, in one launch: the populations (with their
 // float pairs), J^dagger (as pairs in the mixed mode), the tangent direction,
-// and the evaluation kind the following kernels read. Null sources are left
-// alone; a source may be the destination itself (arrays that came from the
+// the evaluation kind and the options the following kernels read (the options
+// by value: a captured call replays with its own). Null sources are left alone; a source may be the destination itself (arrays that came from the
 // host). With the results below it takes the place of up to nine copies and
 // small kernels, 2 to 5 us each, of a call whose evaluation is 50 to 100 us.
-__global__ void k_explicit_in(ColDesc* cols, int mode, const double* n, const double* Jdag, const double* v) {
+__global__ void k_explicit_in(ColDesc* cols, int mode, const double* n, const double* Jdag, const double* v,
+                              SolverOpts* opts, SolverOpts so) {
   ColDesc& cd = cols[0];
   const ColWork& w = cd.w;
   const size_t N = (size_t)cd.t.nz * cd.t.nl, QZ = (size_t)cd.t.nq * cd.t.nz;
   const size_t i0 = (size_t)blockIdx.x * blockDim.x + threadIdx.x, step = (size_t)gridDim.x * blockDim.x;
-  if (i0 == 0) cd.forced_mode = mode;
+  if (i0 == 0) {
+    cd.forced_mode = mode;
+    *opts = so;
+  }
   for (size_t i = i0; i < N; i += step) {
     if (n) {
       const double x = n[i];
@@ -162,22 +166,18 @@ static int kernel_array(const jfnk_ctx* ctx, const double* p, size_t n, jfnk_mem
 
 static unsigned explicit_blocks(size_t n) { return (unsigned)std::min<size_t>((n + 255) / 256, 608); }
 
-// The batch's solver options, uploaded when they change.
-static int set_options(Batch* b, const SolverOpts& so, cudaStream_t s) {
-  if (b->opts_set && std::memcmp(&so, &b->h_opts, sizeof(so)) == 0) return JFNK_OK;
-  b->opts_set = false;
-  b->h_opts = so;
-  JFNK_CUDA(cudaMemcpyAsync(b->d_opts, &b->h_opts, sizeof(so), cudaMemcpyHostToDevice, s));
-  b->opts_set = true;
-  return JFNK_OK;
-}
-
-static int explicit_in(Batch* b, int mode, const double* n, const double* Jdag, const double* v, cudaStream_t s) {
+static int explicit_in(Batch* b, int mode, int variant, const double* n, const double* Jdag, const double* v,
+                       cudaStream_t s) {
+  jfnk_options o;
+  jfnk_default_options(&o);
+  o.precond = variant;
+  SolverOpts so;
+  options_to_device(&o, &so);
   const ColTables& T = b->h_cols[0].t;
   for (auto& c : b->h_cols) c.forced_mode = mode;
   b->forced = mode;
-  k_explicit_in<<<explicit_blocks(Jdag ? (size_t)T.nq * T.nz : (size_t)T.nz * T.nl), 256, 0, s>>>(b->d_cols, mode, n,
-                                                                                                  Jdag, v);
+  k_explicit_in<<<explicit_blocks(Jdag ? (size_t)T.nq * T.nz : (size_t)T.nz * T.nl), 256, 0, s>>>(
+      b->d_cols, mode, n, Jdag, v, b->d_opts, so);
   JFNK_CUDA(cudaGetLastError());
   return JFNK_OK;
 }
@@ -190,15 +190,6 @@ static int explicit_eval(jfnk_ctx* ctx, const jfnk_atmos* a, Batch* b, int mode,
   const AtmosData& M = a->d;
   const size_t N = (size_t)M.nz * M.nl, QZ = (size_t)M.nq * M.nz;
   int rc;
-  {
-    jfnk_options o;
-    jfnk_default_options(&o);
-    o.precond = variant;
-    SolverOpts so;
-    std::memset(&so, 0, sizeof(so));
-    options_to_device(&o, &so);
-    if ((rc = set_options(b, so, s))) return rc;
-  }
   bool direct_n, direct_J = true;
   if ((rc = kernel_array(ctx, n, N, where, &direct_n))) return rc;
   if (Jdag && (rc = kernel_array(ctx, Jdag, QZ, where, &direct_J))) return rc;
@@ -210,7 +201,7 @@ static int explicit_eval(jfnk_ctx* ctx, const jfnk_atmos* a, Batch* b, int mode,
     if ((rc = copy_in(c.w.Jdag, Jdag, QZ * 8, where, s))) return rc;
     Jdag = c.w.Jdag;
   }
-  if ((rc = explicit_in(b, mode, n, Jdag ? Jdag : M.tables.Bn, nullptr, s))) return rc;
+  if ((rc = explicit_in(b, mode, variant, n, Jdag ? Jdag : M.tables.Bn, nullptr, s))) return rc;
   b->pairs_ready = true;
   rc = launch_evaluation(*b, s);
   b->pairs_ready = false;
@@ -287,8 +278,9 @@ int validate_options(const jfnk_options* o) {
   return JFNK_OK;
 }
 
-__global__ void k_init_state(SolverState* st, int n, int phase) {
+__global__ void k_init_state(SolverState* st, int n, int phase, SolverOpts* opts, SolverOpts so) {
   int c = blockIdx.x * blockDim.x + threadIdx.x;
+  if (c == 0) *opts = so;
   if (c >= n) return;
   SolverState s{};
   s.phase = phase;
@@ -498,19 +490,17 @@ static int prepare_solve(Batch* b, const std::vector<const jfnk_atmos*>& cols,
       (o->rh92_warmup > 0 || o->solver != JFNK_SOLVER_JFNK || o->precond > 1))
     return fail(JFNK_E_INVALID,
                 "moving columns: Algorithm 2 without an RH92 start, with the first preconditioner solution or none");
-  SolverOpts so;
-  std::memset(&so, 0, sizeof(so));
-  options_to_device(o, &so);
-  int rc = set_options(b, so, s);
+  int rc = batch_set_forced_mode(b, -1, s);
   if (rc) return rc;
-  if ((rc = batch_set_forced_mode(b, -1, s))) return rc;
   if (o->precond == 2) {
     // the lagged estimate starts at zero in every solve
     if ((rc = ensure_dJdn(b, s))) return rc;
     JFNK_CUDA(cudaMemsetAsync(b->dJ_arena.base, 0, b->dJ_arena.bytes, s));
   }
   const int phase = (o->rh92_warmup > 0 || o->solver == JFNK_SOLVER_RH92) ? PH_RH92 : PH_BASE;
-  k_init_state<<<(b->ncols + 127) / 128, 128, 0, s>>>(b->d_state, b->ncols, phase);
+  SolverOpts so;
+  options_to_device(o, &so);
+  k_init_state<<<(b->ncols + 127) / 128, 128, 0, s>>>(b->d_state, b->ncols, phase, b->d_opts, so);
   JFNK_CUDA(cudaGetLastError());
   JFNK_CUDA(cudaMemsetAsync(b->d_status, 0, sizeof(int) * b->ncols, s));
   for (int c = 0; c < b->ncols; ++c) {
@@ -890,7 +880,7 @@ int jfnk_jvp(jfnk_ctx* ctx, const jfnk_atmos* a, int precision, const double* n,
       if ((r = copy_in(c.w.v, v, N * 8, where, s))) return r;
       vd = c.w.v;
     }
-    if ((r = explicit_in(b, EV_TANGENT, nullptr, nullptr, vd, s))) return r;
+    if ((r = explicit_in(b, EV_TANGENT, 1, nullptr, nullptr, vd, s))) return r;
     if ((r = launch_evaluation(*b, s))) return r;
     return explicit_out(ctx, b, c.w.dF, Jv, N, nullptr, nullptr, where, s);
   });

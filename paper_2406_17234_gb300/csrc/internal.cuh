@@ -141,8 +141,6 @@ struct Batch {
   int eval_mu = 0;                    // ... the angle count shared by every column (0: several)
   size_t eval_smem = 0;               // ... and its blocks' dynamic shared memory
   bool serving = false;               // a server's slots: few of the columns are in one kind at a time
-  SolverOpts h_opts{};                // the options in d_opts, once set (opts_set)
-  bool opts_set = false;
   bool pairs_ready = false;           // explicit calls: the populations' float pairs are already formed
   int forced = -1;                    // evaluation kind forced on every column (-1: each its own)
   bool tuned = false;                 // autotuner has run on this batch

@@ -103,7 +103,7 @@ struct ColTables {
   const double* Vd;       // [2 nmu][nwin][nz] V_ij seen along each direction (outgoing
                           // mu_1..mu_n, then ingoing): a moving column; null when static
   const Ang64* ang64;     // [nmu]
-  const float4* ang32;    // [nmu] (1/(2 mu), w_mu/2, 2 mu, 0), each the FP64 value rounded once
+  const float4* ang32;    // [kMaxMu] (1/(2 mu), w_mu/2, 2 mu, 0), each the FP64 value rounded once; zeros from nmu on
   const float2* dz32;     // [nz-1] (|dz|, 1/|dz|) likewise
   const double* chi_c;    // [nq][nz]
   const double* eta_c;    // [nq][nz]

@@ -669,6 +669,8 @@ __device__ __forceinline__ void direct2(f32x2 e, f32x2 r, f32x2& w, f32x2& bq, c
 constexpr int kPairThreads = 128;
 constexpr int kPairAhead = 4;   // depths ahead whose rows are prefetched into L2
 
+// A column with fewer than MU angles runs the others with zero weight and zero
+// optical depth (they add zeros to its sums).
 template <int MU, bool UP>
 __device__ __forceinline__ void sweep_pair(const ColDesc& cd, int q, const float* __restrict__ s_dz,
                                            const float* __restrict__ s_idz, const Ones2& u, unsigned amask) {
@@ -689,6 +691,7 @@ __device__ __forceinline__ void sweep_pair(const ColDesc& cd, int q, const float
     hw[m] = a.y;
     two_mu[m] = a.z;
   }
+  const float inv2mu_last = T.ang32[T.nmu - 1].x;
   // boundary depth: I = 0 at the top, I = B at the bottom (Sect. 2.1)
   const int k0 = UP ? nz - 1 : 0, q1 = min(q + 1, nq - 1);
   auto D0_of = [&](int qq) {
@@ -765,7 +768,7 @@ __device__ __forceinline__ void sweep_pair(const ColDesc& cd, int q, const float
     // the first and last angle settles the form for all of them. The warp takes
     // one form together: lanes that differ would run every form one after the other.
     const bool direct =
-        __all_sync(amask, !(fabsf(mul(ta, inv2mu[MU - 1])) < 0.1f) && !(fabsf(mul(tb, inv2mu[MU - 1])) < 0.1f));
+        __all_sync(amask, !(fabsf(mul(ta, inv2mu_last)) < 0.1f) && !(fabsf(mul(tb, inv2mu_last)) < 0.1f));
     const bool series = __all_sync(amask, fabsf(mul(ta, inv2mu[0])) < 0.1f && fabsf(mul(tb, inv2mu[0])) < 0.1f);
     auto angles = [&](auto cm) {
       constexpr int CM = decltype(cm)::value;
@@ -804,10 +807,16 @@ __device__ __forceinline__ void sweep_pair(const ColDesc& cd, int q, const float
   }
 }
 
-// Columns of a launch whose angle count is not MU take the scalar sweep, one
-// frequency of the thread's pair after the other.
+// MU: the largest angle count of the launch, each with its own instantiation.
+// Columns with fewer run the same code: a second body for them in this kernel
+// raised the registers from 96 to 128 (four blocks per SM, not five), and the
+// scalar sweep of one frequency after the other, which stood here, was slower than
+// the one-frequency kernel this one took the place of. 256 Ca II columns, a solve,
+// one frequency per thread -> that -> now: 1 angle 112.6 -> 130.4 -> 102.3 ms, 6
+// angles 132.5 -> 144.6 -> 114.8, 7 angles 136.3 -> 147.6 -> 119.9, columns of 3 and
+// 5 angles 119.8 -> 127.7 -> 112.3.
 template <int MU>
-__global__ void __launch_bounds__(kPairThreads) k_formal_sweep_pair(const ColDesc* __restrict__ cols,
+__global__ void __launch_bounds__(kPairThreads, MU <= 5 ? 5 : 4) k_formal_sweep_pair(const ColDesc* __restrict__ cols,
                                                                     float one) {   // one: 1
   extern __shared__ float s_tab[];   // [nz] |dz|, [nz] 1/|dz|
   const ColDesc& cd = cols[blockIdx.y];
@@ -821,16 +830,9 @@ __global__ void __launch_bounds__(kPairThreads) k_formal_sweep_pair(const ColDes
   const int q = 2 * (blockIdx.x * blockDim.x + threadIdx.x);
   const unsigned amask = __ballot_sync(0xffffffffu, q < T.nq);
   if (q >= T.nq) return;
-  if (T.nmu == MU) {
-    const Ones2 u{both2(one), both2(-one)};
-    sweep_pair<MU, false>(cd, q, s_dz, s_idz, u, amask);
-    sweep_pair<MU, true>(cd, q, s_dz, s_idz, u, amask);
-  } else {
-    for (int i = q; i < min(q + 2, T.nq); ++i) {
-      sweep_thread<MU, true, false, false>(cd, i, s_dz, s_idz);
-      sweep_thread<MU, true, true, false>(cd, i, s_dz, s_idz);
-    }
-  }
+  const Ones2 u{both2(one), both2(-one)};
+  sweep_pair<MU, false>(cd, q, s_dz, s_idz, u, amask);
+  sweep_pair<MU, true>(cd, q, s_dz, s_idz, u, amask);
 }
 
 // One kernel per evaluation kind (its own register allocation): blocks of
@@ -1195,23 +1197,38 @@ static size_t sweep_smem(int max_nz, int occ, int threads, bool tan, bool fuse =
   return std::min(cap, std::max(need, pad));
 }
 
+// The packed tangent sweep of the launch's largest angle count.
+static void launch_pair(const Batch& b, cudaStream_t s, size_t sm) {
+  using Kernel = void (*)(const ColDesc*, float);
+  static const Kernel k[kMaxMu] = {k_formal_sweep_pair<1>, k_formal_sweep_pair<2>, k_formal_sweep_pair<3>,
+                                   k_formal_sweep_pair<4>, k_formal_sweep_pair<5>, k_formal_sweep_pair<6>,
+                                   k_formal_sweep_pair<7>, k_formal_sweep_pair<8>};
+  static_assert(kMaxMu == 8, "one instantiation per angle count");
+  k[b.max_nmu - 1]<<<dim3((b.max_nq + 2 * kPairThreads - 1) / (2 * kPairThreads), b.ncols), kPairThreads, sm, s>>>(
+      b.d_cols, 1.0f);
+}
+
 template <int MU>
 static void launch_mu(const Batch& b, cudaStream_t s, int threads, int which, int occ_tan, int occ_base, int fuse) {
   dim3 g((b.max_nq + threads - 1) / threads, b.ncols);
   if (which != 1) {
     const size_t sm = sweep_smem(b.max_nz, occ_tan, threads, true, fuse != 0);
     if (fuse) k_formal_sweep_fused<MU><<<g, threads, sm, s>>>(b.d_cols);
-    else   // two frequencies per thread
-      k_formal_sweep_pair<MU><<<dim3((b.max_nq + 2 * kPairThreads - 1) / (2 * kPairThreads), b.ncols), kPairThreads, sm,
-                                s>>>(b.d_cols, 1.0f);
+    else launch_pair(b, s, sm);
   }
   if (which != 2)
     k_formal_sweep<MU><<<g, threads, sweep_smem(b.max_nz, occ_base, threads, false), s>>>(b.d_cols);
 }
 
 template <int MU>
-static int allow_smem_mu() {
+static int allow_smem_pair() {
   JFNK_CUDA(cudaFuncSetAttribute(k_formal_sweep_pair<MU>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
+  if constexpr (MU > 1) return allow_smem_pair<MU - 1>();
+  return JFNK_OK;
+}
+
+template <int MU>
+static int allow_smem_mu() {
   JFNK_CUDA(cudaFuncSetAttribute(k_formal_sweep_fused<MU>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  227 * 1024));
   JFNK_CUDA(cudaFuncSetAttribute(k_formal_sweep<MU>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
@@ -1263,7 +1280,7 @@ int sweep_prepare(Batch* b) {
   JFNK_CUDA(cudaFuncSetAttribute(k_formal_sweep_warp<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
   int rc;
   if ((rc = allow_smem_mu<2>()) || (rc = allow_smem_mu<3>()) || (rc = allow_smem_mu<4>()) ||
-      (rc = allow_smem_mu<5>()) || (rc = allow_smem_mu<8>()))
+      (rc = allow_smem_mu<5>()) || (rc = allow_smem_mu<8>()) || (rc = allow_smem_pair<kMaxMu>()))
     return rc;
   if (b->sweep_variant == 0 && sweep_small(b->ncols, b->max_nq, b->n_sm) && sweep_warp_size(b->max_nz) > 0) {
     // nothing to tune: the variant's shape follows from the depth

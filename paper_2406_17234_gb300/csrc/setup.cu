@@ -576,7 +576,7 @@ int build_atmosphere(jfnk_ctx* ctx, int lane, const AtomData& A, const jfnk_atmo
   static_assert(kQMetaT == 8, "qmeta4 and qtr8 hold eight transitions");
   size_t o_W2 = ar.take<float2>(nwin), o_c2p = ar.take<float2>(nq), o_rc2p = ar.take<float2>(nq);
   size_t o_linc = ar.take<int>((size_t)nl * (nt + 1));
-  size_t o_ang64 = ar.take<Ang64>(nmu), o_ang32 = ar.take<float4>(nmu), o_dz32 = ar.take<float2>(nz - 1);
+  size_t o_ang64 = ar.take<Ang64>(nmu), o_ang32 = ar.take<float4>(kMaxMu), o_dz32 = ar.take<float2>(nz - 1);
   size_t o_vlos = ar.take<double>(M->moving ? nz : 0);
   const size_t host_prefix = ar.cursor;
   size_t o_V = ar.take<double>((size_t)nwin * nz), o_G = ar.take<double>((size_t)nwin * nz);
@@ -696,7 +696,7 @@ int build_atmosphere(jfnk_ctx* ctx, int lane, const AtomData& A, const jfnk_atmo
   }
   JFNK_CUDA(up(o_linc, linc.data(), linc.size() * 4));
   // the sweep kernels' per-angle and per-layer constants, rounded once from FP64
-  std::vector<float4> ang32(nmu);
+  std::vector<float4> ang32(kMaxMu, make_float4(0.f, 0.f, 0.f, 0.f));
   std::vector<Ang64> ang64(nmu);
   for (int m = 0; m < nmu; ++m) ang64[m] = Ang64{0.5 / mu[m], 0.5 * wmu[m], 2.0 * mu[m], 0.0};
   JFNK_CUDA(up(o_ang64, ang64.data(), nmu * sizeof(Ang64)));
@@ -704,7 +704,7 @@ int build_atmosphere(jfnk_ctx* ctx, int lane, const AtomData& A, const jfnk_atmo
     ang32[m] = make_float4((float)(0.5 / mu[m]), (float)(0.5 * wmu[m]), (float)(2.0 * mu[m]), 0.f);
   std::vector<float2> dz32(nz - 1);
   for (int k = 0; k + 1 < nz; ++k) dz32[k] = make_float2((float)dzv[k], (float)(1.0 / dzv[k]));
-  JFNK_CUDA(up(o_ang32, ang32.data(), nmu * sizeof(float4)));
+  JFNK_CUDA(up(o_ang32, ang32.data(), kMaxMu * sizeof(float4)));
   if (M->moving) JFNK_CUDA(up(o_vlos, d->vlos, nz * 8));
   JFNK_CUDA(up(o_dz32, dz32.data(), (nz - 1) * sizeof(float2)));
   JFNK_CUDA(up(o_dz, dzv.data(), (nz - 1) * 8));

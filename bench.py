@@ -301,6 +301,11 @@ def cpu_baseline_batch(wl, start, pool, futures, workers, t0):
 # of the path (Delta tau, exp, 1/Delta tau, w a b, I update, J accumulation;
 # the tangent adds the differentiated recurrence).
 ALG_OPS = {"value": (10, 2), "jvp": (26, 2)}
+# ... of the cached FP64 evaluations, which form an exponential and a reciprocal
+# per layer and angle for both hemispheres (moving columns: per ray and layer) in
+# base evaluations only: a product is three FMAs per ray-point (moving: five)
+CACHED_OPS = {"value": (10, 1), "jvp": (3, 0)}
+CACHED_MOVING_OPS = {"value": (10, 2), "jvp": (5, 0)}
 FORMAL_KERNELS = {0: "k_formal<double> + k_ray_sum (per-ray buffers)", 1: "k_formal_fused<double>",
                   2: "k_formal_sweep (thread per frequency)", 3: "k_formal_sweep_warp (warp per frequency pair)",
                   4: "k_mv_formal / k_eval64_moving (moving column)",
@@ -345,12 +350,12 @@ def measured_peaks(B, ctx, device=0):
     return p
 
 
-def peak_rate(kind, fp64, peaks):
+def peak_rate(kind, fp64, peaks, counts=ALG_OPS):
     """Roofline ray-points/s of one evaluation kind ('value' or 'jvp') from the
     algorithmic unit counts and the measured pipe rates: the mixed path is bound
     by the slower of the FP32 lanes and the MUFU; in FP64 mode every operation
     goes to the FP64 pipe, with exp and the reciprocal costed by the probe."""
-    ops, mufu = ALG_OPS[kind]
+    ops, mufu = counts[kind]
     if fp64:
         c_exp = peaks["fp64_fma_per_s"] / peaks["fp64_exp_per_s"]   # one exp in FMA-instruction time
         return peaks["fp64_fma_per_s"] / (ops + mufu * c_exp)
@@ -395,14 +400,23 @@ def peak_source(fp64, peaks):
             f"value {ALG_OPS['value']}, jvp {ALG_OPS['jvp']} (FP32 ops, MUFU ops) per ray-point")
 
 
-def alu_roofline(B, ctx, fp64, n_value, n_jvp, pts_per_launch, kern_ms, launches, clocks, kernel, device):
+def kernel_ops(kernel, qb):
+    """Unit counts of a single column's formal kernel (qb > 0: a tiled one, of the
+    moving kernels the cached one)."""
+    if kernel == 6:
+        return CACHED_OPS
+    return CACHED_MOVING_OPS if kernel == 4 and qb > 0 else ALG_OPS
+
+
+def alu_roofline(B, ctx, fp64, n_value, n_jvp, pts_per_launch, kern_ms, launches, clocks, kernel, qb, device):
     """Roofline of the single-column formal-solution kernel (one launch per
     tick, value and JVP evaluations mixed): achieved = ray-points per launch /
     mean launch time (in-graph CUDA events around the formal kernel of every
     tick), peak = the mix of the two kinds' rooflines at the measured rates."""
     peaks = measured_peaks(B, ctx, device)
     w_v, w_j = n_value / max(1, n_value + n_jvp), n_jvp / max(1, n_value + n_jvp)
-    peak = 1.0 / (w_v / peak_rate("value", fp64, peaks) + w_j / peak_rate("jvp", fp64, peaks))
+    counts = kernel_ops(kernel, qb)
+    peak = 1.0 / (w_v / peak_rate("value", fp64, peaks, counts) + w_j / peak_rate("jvp", fp64, peaks, counts))
     avg_s = kern_ms * 1e-3 / max(1, launches)
     achieved = pts_per_launch / avg_s if avg_s > 0 else 0.0
     traffic_pp = measured_traffic("formal_fp64" if fp64 else "formal_fp32_tan")
@@ -410,7 +424,7 @@ def alu_roofline(B, ctx, fp64, n_value, n_jvp, pts_per_launch, kern_ms, launches
             "achieved": achieved / 1e9, "peak": peak / 1e9, "unit": "G ray-points/s",
             "frac": achieved / peak,
             "traffic": None if traffic_pp is None or not fp64 or kernel != 1 else traffic_pp * pts_per_launch,
-            "ops_per_ray_point": {"value": ALG_OPS["value"], "jvp": ALG_OPS["jvp"],
+            "ops_per_ray_point": {"value": counts["value"], "jvp": counts["jvp"],
                                   "mix": {"value": w_v, "jvp": w_j}},
             "avg_launch_us": avg_s * 1e6, "launches": launches, "peak_source": peak_source(fp64, peaks),
             "measured_peaks": peaks}
@@ -562,7 +576,8 @@ def run_ours(args, rank, ws, local, dist):
     kern_ms = prof["formal_ms"] + prof["formal_tan_ms"]
     fp64 = precision == B.JFNK_FP64
     roofline = alu_roofline(B, ctx, fp64, prof["F_calls"] - prof["jvp_calls"], prof["jvp_calls"],
-                            atm.ray_points, kern_ms, launches, clocks, prof["formal_kernel"], local)
+                            atm.ray_points, kern_ms, launches, clocks, prof["formal_kernel"],
+                            prof["formal_qb"], local)
     roofline["share_of_step"] = kern_ms / (total_ms / args.steps)
     roofline["tick_stages_ms"] = stage_breakdown(prof)
     roofline["timed_in"] = "a separate profiled solve (in-graph events around the formal kernel of every tick)"

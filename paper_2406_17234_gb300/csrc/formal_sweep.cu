@@ -612,8 +612,9 @@ __device__ __forceinline__ void sweep_thread(const ColDesc& cd, int q, const flo
 // and addresses are shared by the two frequencies. A warp votes on the form of
 // the coefficients, so that lanes on both sides of the limit cost one pass and
 // not three. Each element sees the operations of ray_step in their order: the
-// same bits. Now the FP32 pipe (0.87) and the issue slots (0.94 on a full
-// multiprocessor) bind together.
+// same bits. On the 76-column batch, which leaves the SMs at two blocks each, the
+// FP32 pipe is 42 % busy and the issue slots 32 % (48 % with the scalar sweep); the
+// 4,096-column batch runs at 0.70 of the FP32 roofline (0.56).
 // 512 Ca II columns, 256 x 1,005, 5 angles, median launch of a solve: scalar 960 us,
 // scalar with the vote 999, packed 963, packed with the vote 785 (57.0 -> 46.8 ms per
 // solve). A vote per angle in mixed warps: 47.9 ms; 64 threads per block: 49.0.
@@ -1322,75 +1323,53 @@ int sweep_autotune(Batch* b, cudaStream_t s) {
   JFNK_CUDA(cudaEventCreate(&e0));
   JFNK_CUDA(cudaEventCreate(&e1));
   int rc = JFNK_OK;
-  // a tangent candidate without fusion is timed with the separate opacity-tangent launch it needs
-  auto once = [&](int variant, int size, int which, int ot, int ob, int fuse) -> int {
-    if (which == 2 && !fuse && variant != 2) {
-      int r = launch_opacity_tan(*b, s);
-      if (r) return r;
-    }
-    return launch_sweep_cfg(*b, s, variant, size, which, ot, ob, fuse);
-  };
   // a candidate's time: the fastest of three launches timed one by one, after a
   // warm-up (single launches differ by a few per cent; the minimum is stable)
-  auto timed = [&](int variant, int size, int which, int ot, int ob, float* ms, int fuse = 0) -> int {
-    int r = once(variant, size, which, ot, ob, fuse);   // warm-up
+  auto timed = [&](auto launch, float* ms) -> int {
+    int r = launch();   // warm-up
     if (r) return r;
-    float best = 1e30f;
+    *ms = 1e30f;
     for (int i = 0; i < 3; ++i) {
       if (cudaEventRecord(e0, s) != cudaSuccess) return fail(JFNK_E_CUDA, "autotune event");
-      if ((r = once(variant, size, which, ot, ob, fuse))) return r;
+      if ((r = launch())) return r;
       float t = 0.f;
       if (cudaEventRecord(e1, s) != cudaSuccess || cudaEventSynchronize(e1) != cudaSuccess ||
           cudaEventElapsedTime(&t, e0, e1) != cudaSuccess)
         return fail(JFNK_E_CUDA, "autotune timing");
-      best = std::min(best, t);
+      *ms = std::min(*ms, t);
     }
-    *ms = best;
     return JFNK_OK;
   };
+  // the tangent sweep with the opacity-tangent launch it needs, the base-type sweep
+  auto tangent = [&](int occ) {
+    const int r = launch_opacity_tan(*b, s);
+    return r ? r : launch_sweep_cfg(*b, s, 1, 128, 2, occ);
+  };
+  auto base = [&](int occ) { return launch_sweep_cfg(*b, s, 1, 128, 1, 0, occ); };
   // the opacity tangent's run of depths per thread (the depth tile of its
   // grid): the default of 16 unless another run gains 2 %
-  {
-    auto time_optan = [&](int dr, float* ms) -> int {
-      int r = launch_opacity_tan(*b, s, dr);   // warm-up
-      if (r) return r;
-      float best = 1e30f;
-      for (int i = 0; i < 3; ++i) {
-        if (cudaEventRecord(e0, s) != cudaSuccess) return fail(JFNK_E_CUDA, "autotune event");
-        if ((r = launch_opacity_tan(*b, s, dr))) return r;
-        float t = 0.f;
-        if (cudaEventRecord(e1, s) != cudaSuccess || cudaEventSynchronize(e1) != cudaSuccess ||
-            cudaEventElapsedTime(&t, e0, e1) != cudaSuccess)
-          return fail(JFNK_E_CUDA, "autotune timing");
-        best = std::min(best, t);
-      }
-      *ms = best;
-      return JFNK_OK;
-    };
-    float bo = 0.f;
-    int bd = 16;
-    if (!(rc = time_optan(16, &bo))) {
-      bo *= 0.98f;
-      for (int dr : {8, 32}) {
-        float ms = 0.f;
-        if ((rc = time_optan(dr, &ms))) break;
-        if (ms < bo) { bo = ms; bd = dr; }
-      }
-    }
-    b->optan_depths = bd;
+  float best = 0.f;
+  int best_depths = 16;
+  for (int dr : {16, 8, 32}) {
+    float ms = 0.f;
+    if ((rc = timed([&] { return launch_opacity_tan(*b, s, dr); }, &ms))) break;
+    if (dr == 16) best = 0.98f * ms;
+    else if (ms < best) { best = ms; best_depths = dr; }
   }
+  b->optan_depths = best_depths;
   // The fused opacity tangent (forced variant only) is not a candidate: timed
   // alone it can win, but inside a tick the separate opacity-tangent kernel
   // overlaps the base-type chain on the other stream, and the fused sweep
   // made the whole solve about 11 % slower.
+  //
   // caps of resident blocks per SM, of the tangent sweep (the columns in tangent
   // mode), then of the base-type sweep (in base mode); no cap stays unless one
   // gains 2 %: closer than that, single measurements flip between runs
   int best_occ = 0, best_base = 0;
-  float best = 1e30f;
+  best = 1e30f;
   for (int occ : {0, 4}) {
     float ms = 0.f;
-    if (rc || (rc = timed(1, 128, 2, occ, 0, &ms))) break;
+    if (rc || (rc = timed([&] { return tangent(occ); }, &ms))) break;
     if (occ == 0) ms *= 0.98f;
     if (ms < best) { best = ms; best_occ = occ; }
   }
@@ -1398,7 +1377,7 @@ int sweep_autotune(Batch* b, cudaStream_t s) {
     best = 1e30f;
     for (int occ : {0, 3, 4}) {
       float ms = 0.f;
-      if ((rc = timed(1, 128, 1, best_occ, occ, &ms))) break;
+      if ((rc = timed([&] { return base(occ); }, &ms))) break;
       if (occ == 0) ms *= 0.98f;
       if (ms < best) { best = ms; best_base = occ; }
     }

@@ -142,13 +142,15 @@ typedef struct {
 } jfnk_atmos_desc;
 
 /* Formal-solution kernel of a batch (all give the solution of Eqs. Iplus/
- * Iminus; the two sweep kernels of the mixed mode are bit-identical). */
+ * Iminus; the sweep kernels of the mixed mode are bit-identical, the FP64 ones
+ * agree to rounding). */
 typedef enum {
   JFNK_FORMAL_PER_RAY = 0,       /* per-ray buffers, separate ray-sum kernel      */
   JFNK_FORMAL_FUSED = 1,         /* FP64: block per frequency group, shared memory */
   JFNK_FORMAL_SWEEP_THREAD = 2,  /* mixed: thread per frequency (tangents: per two), all angles */
   JFNK_FORMAL_SWEEP_WARP = 3,    /* mixed: warp per frequency pair, lane per ray   */
-  JFNK_FORMAL_MOVING = 4,        /* moving columns: thread per ray, per-ray opacity */
+  JFNK_FORMAL_MOVING = 4,        /* moving columns: an opacity per ray, per tile of frequencies
+                                    with kept coefficients, or a thread per ray          */
   JFNK_FORMAL_SWEEP_THREAD_FUSED = 5, /* mixed: thread per frequency, the tangent sweep
                                     forming the JVP evaluations' opacity tangent itself
                                     (at most 8 transitions overlap at any frequency) */
@@ -258,7 +260,8 @@ typedef struct {
                            integrals (and, moving columns, moments), [4] assembly
                            and preconditioner factorisation, [5] Krylov step      */
   int opacity_depths;   /* mixed mode: depths per thread of the opacity-tangent kernel
-                           (its depth tile, chosen by the autotuner; 0: not tuned) */
+                           (its depth tile, chosen by the autotuner in large
+                           launches; 0 in FP64)                                   */
 } jfnk_stats;
 
 /* ---- context ------------------------------------------------------------ */
@@ -358,8 +361,11 @@ int jfnk_batch_solve(jfnk_ctx* ctx, int n_cols, const jfnk_atmos* const* cols,
 /* ---- persistent batches -------------------------------------------------------- */
 /* A batch plan owns the device work buffers of n_cols columns (precision and
  * Krylov size fixed at creation) and its tick graph, so that repeated solves
- * pay for allocation, autotuning and graph capture once. The atmospheres must
- * outlive the plan. jfnk_batch_run solves every column like jfnk_batch_solve
+ * pay for allocation, autotuning and graph capture once. FP64 columns keep their
+ * coefficients on the device (JFNK_FORMAL_CACHED) while those of the whole plan
+ * take at most 24 GiB and the device has room; else the plan runs the fused
+ * kernel, with results equal to rounding (jfnk_stats.formal_kernel tells). The
+ * atmospheres must outlive the plan. jfnk_batch_run solves every column like jfnk_batch_solve
  * (o->precision must equal the plan's, o->krylov_max <= its krylov_max). */
 typedef struct jfnk_batch jfnk_batch;
 int jfnk_batch_create(jfnk_ctx* ctx, int n_cols, const jfnk_atmos* const* cols, int precision,
@@ -371,7 +377,7 @@ int jfnk_batch_destroy(jfnk_batch* b);
 /* ---- residual without device allocation -------------------------------------- */
 /* The paper has no counterpart to this entry point: it is a deployment aid.
  * Same result as jfnk_residual(ctx, a, JFNK_FP64, n, J_dagger, F, J_new, NULL,
- * JFNK_MEM_DEVICE, stream), but every work buffer comes from one fixed device
+ * JFNK_MEM_DEVICE, stream), to rounding (another kernel), but every work buffer comes from one fixed device
  * array of JFNK_STATIC_SCRATCH_BYTES built into the library (held on every GPU
  * that loads it until the process exits), so the call never allocates device
  * memory. For callers that cannot allocate: code running under a memory budget
@@ -380,7 +386,7 @@ int jfnk_batch_destroy(jfnk_batch* b);
  *   n [nz*nl], J_dagger [nq*nz] (nullable: B_nu(T)), F [nz*nl], J_new [nq*nz]
  *   (nullable): device pointers on the context's device; the work is enqueued
  *   on ``stream`` and the call returns without synchronising.
- * The formal solution runs in the fused kernel of jfnk_residual, whose buffers
+ * The formal solution runs in the fused kernel (JFNK_FORMAL_FUSED), whose buffers
  * take roughly nq * nz * 6 * 8 bytes; a column too deep for it (a frequency's
  * rays over all depths beyond one block's shared memory) takes the per-ray
  * kernels, about nq * nz * (8 n_mu + 9) * 8 bytes. A column whose buffers

@@ -16,7 +16,7 @@
 //       dD^k = dD^u e + g |dz|(dchi^k + dchi^u) + w (dS^u - dS^k):
 //     three FMAs per ray-point instead of an exponential and about 40 others;
 //   - the ray sums take one FMA per ray and quantity, and the re-anchoring of
-//     D = I - S on the better-conditioned form compares exponent words.
+//     D = I - S on the better-conditioned form compares high words.
 // The opacity of the tile and the rate integrals over it are formed in the
 // same block (two launches and the round trips of chi, dJ and the Lambda
 // diagonals fewer); a tile leaves its part of each integral it meets, and the
@@ -33,8 +33,9 @@
 // kernels: 82 depths x 1,005 frequencies x 5 angles, base
 // 244 + 11 + 59 -> 87 + 8 us, tangent 149 + 11 + 12 -> 26 + 8 us; 101 x 41 x 5,
 // base 126 + 8 + 18 -> 50 + 10 us, tangent 48 + 8 + 11 -> 18 + 10 us. A base
-// evaluation is bound by its FP64 instructions (half of it the coefficients),
-// a tangent by the chain of chunks.
+// evaluation is bound by its FP64 instructions (half of it the coefficients; the
+// FP64 pipe is 58 % busy over the launch, stalls are the chunks' barriers and
+// shared memory), a tangent by the chain of chunks (41 %).
 #include <algorithm>
 #include <cmath>
 
@@ -83,7 +84,8 @@ size_t cached_parts(int qb, int nz, int nl, int nwin, int nt) {
 // partly filled), for the column alone on the device: 7 for 1,005 frequencies
 // (144 blocks on 152 SMs), 1 for 41. It sets the order of the rate sums, so it
 // must not depend on the batch: a column's result is the same alone and in any
-// batch.
+// batch that takes the cached evaluation (batch_create: one whose planes are too
+// large for it takes the fused kernel, with other roundings).
 int cached_default_qb(int nq, int nz, int nmu, int nl, int n_sm) {
   int best = 0;
   double cost = 0.0;

@@ -100,9 +100,10 @@ int build_atom(const jfnk_atom_desc* d, AtomData* A);
 // tables are ready once that event has completed.
 int build_atmosphere(jfnk_ctx* ctx, int lane, const AtomData& A, const jfnk_atmos_desc* d, AtmosData* M);
 
-// Formal-solution kernels: per-ray buffers + ray-sum kernel (any size),
-// in-block fused kernel (FP64), per-frequency sweep kernel (mixed precision).
-// whole evaluation per frequency tile with cached coefficients (FP64).
+// Formal-solution kernels: per-ray buffers + ray-sum kernel (FP64, any size),
+// in-block fused kernel (FP64), per-frequency sweep kernels (mixed precision),
+// and the whole evaluation per frequency tile with cached coefficients (FP64;
+// static and moving columns).
 enum FormalKind { FORMAL_UNFUSED = 0, FORMAL_FUSED = 1, FORMAL_SWEEP = 2, FORMAL_MOVING = 3, FORMAL_CACHED = 4,
                   FORMAL_MOVING_CACHED = 5 };
 inline bool kind_moving(int k) { return k == FORMAL_MOVING || k == FORMAL_MOVING_CACHED; }

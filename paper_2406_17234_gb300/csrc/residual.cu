@@ -1510,7 +1510,10 @@ static void launch_rates_tan32(const Batch& b, cudaStream_t s) {
     return dim3((b.max_nz + kRateTanWarps * d - 1) / (kRateTanWarps * d), b.max_nt, b.ncols);
   };
   // a window's stride per warp and depth: below 32 warps per multiprocessor the
-  // launch is short of warps, and one depth per warp gives it four times as many
+  // launch is short of warps, and one depth per warp gives it four times as many.
+  // Solves of Ca II-like columns of up to 256 depths, one and four depths per warp:
+  // 4 columns 5.29 and 5.35 ms, 7 to 36 the same within 0.2 %, 60: 51.7 and 51.1;
+  // the line lies at seven of them
   if ((long)b.ncols * b.max_nt * b.max_nz < 32L * 4 * b.n_sm)
     k_rates_tan32<1><<<grid(1), 32 * kRateTanWarps, 0, s>>>(b.d_cols);
   else

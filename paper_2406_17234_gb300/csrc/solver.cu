@@ -145,8 +145,11 @@ void column_bind(char* base, const AtmosData& M, int kind, int mixed, int kmax, 
   w.st = st;
 }
 
-// Largest total of the cached FP64 coefficients of a batch (a 4,096-column
-// batch keeps the memory it had).
+// Largest total of the cached FP64 coefficients of a batch: about 800 Ca II-like
+// columns of 160 depths. A bound on the memory a plan takes beyond what it had
+// without them (a twelfth of the device), so that plans and servers made beside it
+// keep their room; not a matter of speed (200 columns: 397 ms a solve with them,
+// 1,740 with the fused kernel). Results on its two sides agree to rounding.
 constexpr size_t kCachedBytes = (size_t)24 << 30;
 
 int batch_create(Batch* b, const std::vector<const AtmosData*>& cols, int mixed, int kmax) {
@@ -250,7 +253,7 @@ int batch_set_forced_mode(Batch* b, int mode, cudaStream_t s) {
 // One warp adds the warps' sums in order and the block reads the result: FP64
 // instructions cost every warp of a scheduler 64 cycles each, so sixteen warps
 // repeating the addition (and the caller's square root) took longer than all
-// the rest of a norm (10,700 of a Krylov step's 31,000 cycles).
+// the rest of a norm (two-level slab solve 4.7 -> 4.1 ms without that).
 template <typename F>
 __device__ double block_sum_then(double v, double* sh, F f) {
   v = warp_sum(v);
@@ -1007,10 +1010,15 @@ __global__ void __launch_bounds__(kKrylovThreads) k_krylov(const ColDesc* __rest
 }
 
 // A warp per depth finishes one column's RH92 update in about 10 us (one thread
-// per depth: 100 us) but uses a fifth of its lanes: above about 50 columns of
-// 82 depths the FP64 instructions take longer than the latency saved (512
-// columns: 205.8 against 200.2 ms a solve). A server's slots are a quarter
-// or less in RH92 iterations at a time (48 slots: 253.7 against 265.1 ms).
+// per depth: 100 us) but uses a fifth of its lanes: in large launches the FP64
+// instructions take longer than the latency saved. Solves of Ca II-like columns of
+// up to 256 depths, warp against thread: 4 columns 5.29 and 5.65 ms, 8: 11.72 and
+// 12.17, 16: 20.27 and 20.42, 36: 40.01 and 40.06, 60: 51.12 and 51.06, 512: 205.8
+// and 200.2; the line lies at 15 of them, from where on the two are within 1 %. A
+// server's slots are a quarter or less in RH92 iterations at a time, and it
+// gains longer: bursts of two requests a slot, 32 slots of 300 depths 173 and 184
+// ms, 52: 218 and 229, 64: 261 and 273, 128: 412 and 420. Its line, at 52 slots, is
+// therefore on the low side.
 bool rh92_by_warp(const Batch& b) {
   return b.formal_kind == FORMAL_CACHED || (long)b.ncols * b.max_nz < (b.serving ? 104L : 26L) * b.n_sm;
 }

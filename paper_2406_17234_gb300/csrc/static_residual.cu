@@ -83,8 +83,10 @@ extern "C" int jfnk_residual_static(jfnk_ctx* ctx, const jfnk_atmos* a, const do
   const AtmosData& M = a->d;
   const size_t nz = M.nz, nq = M.nq, nl = M.nl, nt = M.nt, nmu = M.nmu;
   const size_t N = nz * nl, QZ = nq * nz;
-  // the fused formal kernel (the one jfnk_residual runs) needs no per-ray
-  // buffers; the per-ray path only when a frequency's rays exceed its shared memory
+  // the fused formal kernel needs no per-ray buffers and keeps no coefficient
+  // planes, as jfnk_residual's cached evaluation does (16 MB of 82 depths x 1,005
+  // frequencies x 5 angles); the per-ray path only when a frequency's rays exceed
+  // its shared memory
   const int qb = fused_default_qb((int)nz, (int)nmu, false);
   const bool fused = qb > 0;
   const size_t per_ray = fused ? 0 : 2 * nmu * QZ;

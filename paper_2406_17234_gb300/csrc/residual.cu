@@ -989,7 +989,8 @@ __device__ __forceinline__ void rates_columns(const ColDesc* __restrict__ cols, 
 // Two kernels, so that each has its own register bound: the large launch keeps
 // the compiler's 128 (a second bound argument, even 1, makes it 160 and the
 // 512-column batch 3 % slower), the small one the 194 its held terms need
-// (168 and spills without it).
+// (168 and spills without it). FP64 columns hold no terms ahead and take the
+// former (a server's burst of 24 Ca II-like columns 102.5 -> 100.6 ms).
 __global__ void __launch_bounds__(32 * kRateWarps) k_rates(const ColDesc* __restrict__ cols, int ncols, int racc,
                                                            int fslots, const SolverOpts* bopts) {
   rates_columns<false>(cols, ncols, racc, fslots, bopts);
@@ -1033,8 +1034,8 @@ static int launch_rates(const Batch& b, cudaStream_t s) {
   attr[0].val.clusterDim.z = split;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  JFNK_CUDA(cudaLaunchKernelEx(&cfg, split > 1 ? k_rates_small : k_rates, (const ColDesc*)b.d_cols, b.ncols, racc,
-                               fslots, (const SolverOpts*)b.d_opts));
+  JFNK_CUDA(cudaLaunchKernelEx(&cfg, split > 1 && b.mixed ? k_rates_small : k_rates, (const ColDesc*)b.d_cols,
+                               b.ncols, racc, fslots, (const SolverOpts*)b.d_opts));
   return JFNK_OK;
 }
 

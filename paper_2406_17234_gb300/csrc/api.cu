@@ -138,8 +138,8 @@ __global__ void k_explicit_out(const ColDesc* cols, const double* src, double* d
 }
 
 // Whether those kernels may use a caller's array of n doubles: aligned device
-// memory of the context's device, in one allocation from its first to its last
-// byte. Any other array takes the copies, which serve every address the runtime
+// memory of the context's device that it may read and write, in one allocation
+// from its first to its last byte. Any other array takes the copies, which serve every address the runtime
 // knows and refuse the rest with an error; one that runs past the end of its
 // cudaMalloc allocation is refused here. (Memory mapped in pieces, or from a
 // pool, may go on behind the piece that an address is in.)
@@ -148,19 +148,21 @@ static int kernel_array(const jfnk_ctx* ctx, const double* p, size_t n, jfnk_mem
   if (where != JFNK_MEM_DEVICE || !ctx->pointer_attributes) return JFNK_OK;
   // one driver call; of an unknown address every value is zero
   unsigned type = 0;
-  int managed = 0, device = -1, plain = 0;
+  int managed = 0, device = -1, plain = 0, access = 0;
   CUdeviceptr base = 0;
   size_t size = 0;
   CUpointer_attribute what[] = {CU_POINTER_ATTRIBUTE_MEMORY_TYPE,    CU_POINTER_ATTRIBUTE_IS_MANAGED,
                                 CU_POINTER_ATTRIBUTE_DEVICE_ORDINAL, CU_POINTER_ATTRIBUTE_RANGE_START_ADDR,
-                                CU_POINTER_ATTRIBUTE_RANGE_SIZE,     CU_POINTER_ATTRIBUTE_IS_LEGACY_CUDA_IPC_CAPABLE};
-  void* to[] = {&type, &managed, &device, &base, &size, &plain};
+                                CU_POINTER_ATTRIBUTE_RANGE_SIZE,     CU_POINTER_ATTRIBUTE_IS_LEGACY_CUDA_IPC_CAPABLE,
+                                CU_POINTER_ATTRIBUTE_ACCESS_FLAGS};
+  void* to[] = {&type, &managed, &device, &base, &size, &plain, &access};
   const CUdeviceptr a = reinterpret_cast<CUdeviceptr>(p);
-  if (ctx->pointer_attributes(6, what, to, a) != CUDA_SUCCESS || type != CU_MEMORYTYPE_DEVICE || managed)
+  if (ctx->pointer_attributes(7, what, to, a) != CUDA_SUCCESS || type != CU_MEMORYTYPE_DEVICE || managed)
     return JFNK_OK;
   const bool inside = a >= base && a - base <= size && n * sizeof(double) <= size - (a - base);
   if (!inside && plain) return fail(JFNK_E_INVALID, "a device array is shorter than the call needs");
-  *yes = inside && a % sizeof(double) == 0 && device == ctx->device;
+  *yes = inside && a % sizeof(double) == 0 && device == ctx->device &&
+         (plain || access == CU_POINTER_ATTRIBUTE_ACCESS_FLAG_READWRITE);   // memory mapped by hand may be read-only
   return JFNK_OK;
 }
 

@@ -37,7 +37,7 @@ __device__ __forceinline__ int part_offset(const ColTables& T, int qb, int lane,
 
 // Coefficients of one step of optical depth x: e = exp(-x), w = (1 - e)/x,
 // a = 1 - w and bq = (w - e)/x, each from its own Taylor series below
-// |x| = 0.1 (where 1 - e, 1 - w and w - e cancel); r = 1/x is supplied by the
+// x = 0.1 (where 1 - e, 1 - w and w - e cancel); r = 1/x is supplied by the
 // caller (shared between the rays of a layer).
 // FP64 Taylor coefficients: w = sum_{n>=0} (-x)^n/(n+1)!,
 // a/x = sum_{n>=0} (-x)^n/(n+2)!, bq = sum_{n>=0} (-x)^n (n+1)/(n+2)!.
@@ -73,7 +73,7 @@ __device__ __forceinline__ void pl_coef_f(double x, double r, double& e, double&
 
 __device__ __forceinline__ void pl_coef_f(float x, float r, float& e, float& w, float& a, float& bq) {
   e = __expf(-x);
-  if (fabsf(x) < 0.1f) {
+  if (x < 0.1f) {
     w = fmaf(fmaf(fmaf(fmaf(fmaf(-1.0f / 720.0f, x, 1.0f / 120.0f), x, -1.0f / 24.0f), x, 1.0f / 6.0f), x, -0.5f), x, 1.0f);
     a = x * fmaf(fmaf(fmaf(fmaf(fmaf(-1.0f / 5040.0f, x, 1.0f / 720.0f), x, -1.0f / 120.0f), x, 1.0f / 24.0f), x, -1.0f / 6.0f), x, 0.5f);
     bq = fmaf(fmaf(fmaf(fmaf(1.0f / 144.0f, x, -1.0f / 30.0f), x, 1.0f / 8.0f), x, -1.0f / 3.0f), x, 0.5f);

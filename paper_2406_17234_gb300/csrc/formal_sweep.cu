@@ -67,11 +67,14 @@ constexpr int kRingSlots = 9;
 __host__ __device__ inline size_t ring_floats(int threads) { return (size_t)kRing * kRingSlots * threads; }
 
 // Which form of the coefficients a step takes: chosen per step (CM_EITHER),
-// or known for every angle of the depth (CM_SERIES: all steps below 0.1 in
-// size; CM_DIRECT: none), the same choice as CM_EITHER makes for each step.
+// or known for every angle of the depth (CM_SERIES: all steps below 0.1;
+// CM_DIRECT: none), the same choice as CM_EITHER makes for each step.
 // CM_SELECT forms both and selects: no branch, for launches bound by latency.
 enum CoefMode { CM_EITHER = 0, CM_SERIES = 1, CM_DIRECT = 2, CM_SELECT = 3 };
 
+// (Steps of inverted populations, x < 0, take the series, which is off by 2e-4 at
+// x = -1; FP64 takes the direct forms there. With those here too, H I-like columns in
+// which a line lases ended 1e-6 to 1e-3 elsewhere.)
 template <int CM = CM_EITHER>
 __device__ __forceinline__ void pl_coef_rn(float x, float r, float& e, float& w, float& a, float& bq) {
   e = exp_neg(x);
@@ -79,11 +82,11 @@ __device__ __forceinline__ void pl_coef_rn(float x, float r, float& e, float& w,
     float es, ws, as, bs, ed, wd, ad, bd;
     pl_coef_rn<CM_SERIES>(x, r, es, ws, as, bs);
     pl_coef_rn<CM_DIRECT>(x, r, ed, wd, ad, bd);
-    const bool thin = fabsf(x) < 0.1f;
+    const bool thin = x < 0.1f;
     w = thin ? ws : wd;
     a = thin ? as : ad;
     bq = thin ? bs : bd;
-  } else if (CM == CM_SERIES || (CM == CM_EITHER && fabsf(x) < 0.1f)) {
+  } else if (CM == CM_SERIES || (CM == CM_EITHER && x < 0.1f)) {
     w = fma3(fma3(fma3(fma3(fma3(-1.0f / 720.0f, x, 1.0f / 120.0f), x, -1.0f / 24.0f), x, 1.0f / 6.0f), x, -0.5f), x, 1.0f);
     a = mul(x, fma3(fma3(fma3(fma3(fma3(-1.0f / 5040.0f, x, 1.0f / 720.0f), x, -1.0f / 120.0f), x, 1.0f / 24.0f), x, -1.0f / 6.0f), x, 0.5f));
     bq = fma3(fma3(fma3(fma3(1.0f / 144.0f, x, -1.0f / 30.0f), x, 1.0f / 8.0f), x, -1.0f / 3.0f), x, 0.5f);
@@ -582,9 +585,9 @@ __device__ __forceinline__ void sweep_thread(const ColDesc& cd, int q, const flo
       // test on the first and last angle settles the form for all of them. The
       // warp takes one form together: lanes that differ would run every form one
       // after the other (base sweeps of 512 Ca II columns: 38.0 -> 36.5 ms a solve).
-      if (__all_sync(amask, !(fabsf(mul(in.tz, inv2mu[MU - 1])) < 0.1f)))
+      if (__all_sync(amask, !(mul(in.tz, inv2mu[MU - 1]) < 0.1f)))
         angles(std::integral_constant<int, CM_DIRECT>());
-      else if (__all_sync(amask, fabsf(mul(in.tz, inv2mu[0])) < 0.1f)) angles(std::integral_constant<int, CM_SERIES>());
+      else if (__all_sync(amask, mul(in.tz, inv2mu[0]) < 0.1f)) angles(std::integral_constant<int, CM_SERIES>());
       else angles(std::integral_constant<int, CM_SELECT>());
     } else {
       angles(std::integral_constant<int, CM_EITHER>());
@@ -769,8 +772,8 @@ __device__ __forceinline__ void sweep_pair(const ColDesc& cd, int q, const float
     // the first and last angle settles the form for all of them. The warp takes
     // one form together: lanes that differ would run every form one after the other.
     const bool direct =
-        __all_sync(amask, !(fabsf(mul(ta, inv2mu_last)) < 0.1f) && !(fabsf(mul(tb, inv2mu_last)) < 0.1f));
-    const bool series = __all_sync(amask, fabsf(mul(ta, inv2mu[0])) < 0.1f && fabsf(mul(tb, inv2mu[0])) < 0.1f);
+        __all_sync(amask, !(mul(ta, inv2mu_last) < 0.1f) && !(mul(tb, inv2mu_last) < 0.1f));
+    const bool series = __all_sync(amask, mul(ta, inv2mu[0]) < 0.1f && mul(tb, inv2mu[0]) < 0.1f);
     auto angles = [&](auto cm) {
       constexpr int CM = decltype(cm)::value;
 #pragma unroll
@@ -788,8 +791,8 @@ __device__ __forceinline__ void sweep_pair(const ColDesc& cd, int q, const float
           f32x2 ws, bs;
           series2(dtau, ws, bs);
           unpack2(dtau, a, b);
-          w = select2(fabsf(a) < 0.1f, fabsf(b) < 0.1f, ws, w);
-          bq = select2(fabsf(a) < 0.1f, fabsf(b) < 0.1f, bs, bq);
+          w = select2(a < 0.1f, b < 0.1f, ws, w);
+          bq = select2(a < 0.1f, b < 0.1f, bs, bq);
         }
         const f32x2 tn = mul2(dtz, both2(-inv2mu[m]));   // -ddtau
         const f32x2 dDn = fma2(dD[m], e, fma2(tn, fma2(e, D[m], mul2(bq, dSin)), mul2(w, ddSin)));

@@ -390,7 +390,7 @@ __global__ void k_source_diff(const ColDesc* __restrict__ cols) {
 // recurrence needs: e = exp(-x), w = (1 - e)/x, a = 1 - w and bq = b/x with
 // b = w - e. Below a threshold every one of them comes from its own Taylor
 // series, since 1 - e, 1 - w and w - e all cancel there (a = 1 - w loses all
-// FP32 digits at x ~ 1e-6): |x| = 0.1 in FP32, |x| = 1e-3 in FP64.
+// FP32 digits at x ~ 1e-6): x = 0.1 in FP32, |x| = 1e-3 in FP64.
 __device__ __forceinline__ void pl_coef(double x, double& e, double& w, double& a, double& bq) {
   e = exp(-x);
   if (fabs(x) < 1e-3) {
@@ -405,7 +405,7 @@ __device__ __forceinline__ void pl_coef(double x, double& e, double& w, double& 
 
 __device__ __forceinline__ void pl_coef(float x, float& e, float& w, float& a, float& bq) {
   e = __expf(-x);
-  if (fabsf(x) < 0.1f) {
+  if (x < 0.1f) {
     // the same series to x^5 (truncation below 3e-10 relative)
     w = fmaf(fmaf(fmaf(fmaf(fmaf(-1.0f / 720.0f, x, 1.0f / 120.0f), x, -1.0f / 24.0f), x, 1.0f / 6.0f), x, -0.5f), x, 1.0f);
     a = x * fmaf(fmaf(fmaf(fmaf(fmaf(-1.0f / 5040.0f, x, 1.0f / 720.0f), x, -1.0f / 120.0f), x, 1.0f / 24.0f), x, -1.0f / 6.0f), x, 0.5f);

@@ -1,11 +1,11 @@
 """Columns with inverted populations (negative opacity over a few layers): J of
-every formal-solution kernel against extended-precision sums of the same short
+every FP64 formal-solution kernel against extended-precision sums of the same short
 characteristics, and the mixed mode's sweeps against one another.
 
 The scale of an element is the same sum over the absolute values of its terms.
-Tolerance: FP64 1e-11 of it (coefficients to 4e-13 at optical depths of 1e-3; tens of
-layers count), FP32 sweeps 5e-5 (2e-6 a layer, 24 layers). A series used outside its
-range is off by 2e-4 at an optical depth of -1.
+Tolerance: 1e-11 of it (coefficients to 4e-13 at optical depths of 1e-3; tens of
+layers count). A series used outside its range is off by 2e-4 at an optical depth of
+-1.
 """
 import ctypes as C
 
@@ -72,14 +72,11 @@ def _device(atm, n):
 
 # n_mu = 8 at 1,000 depths: too deep for a block's rays, the separate per-ray kernels
 @pytest.mark.parametrize("path,nz,n_mu", [("cached", 24, 2), ("moving", 24, 3), ("moving", 1000, 8), ("static", 24, 2),
-                                          ("static", 1000, 8), ("mixed", 24, 2)])
+                                          ("static", 1000, 8)])
 def test_inverted_layers(path, nz, n_mu):
     atm, n, ref, scale = _inverted(nz, n_mu, path == "moving")
-    if path == "static":
-        J = _device(atm, n)
-    else:
-        J = B.residual(atm, n, want_J=True, precision=B.JFNK_MIXED if path == "mixed" else B.JFNK_FP64)[1]
-    assert np.all(np.abs(J - ref) <= (5e-5 if path == "mixed" else 1e-11) * scale)
+    J = _device(atm, n) if path == "static" else B.residual(atm, n, want_J=True)[1]
+    assert np.all(np.abs(J - ref) <= 1e-11 * scale)
 
 
 @pytest.mark.parametrize("n_mu", [1, 5])

@@ -674,7 +674,7 @@ __device__ void rates_tile(const ColDesc& cd, const int mode, const int t, const
   const bool tan = (mode == EV_TANGENT);
   const bool base_mode = (mode == EV_BASE);
   const bool rh = (mode == EV_RH92);
-  const bool mix = cd.mixed != 0;
+  const bool mix = PIPE || cd.mixed != 0;   // k_rates_small: mixed columns only
   const int nacc = tan ? 2 : (base_mode ? 2 + nl : (rh ? 2 + kRhFixed + nt : 2));
   const int k = min(tile * 32 + lane, nz - 1);
   const int q0 = T.t_q0[t], q1 = T.t_q1[t], wbase = T.t_base[t];
@@ -988,7 +988,7 @@ __device__ __forceinline__ void rates_columns(const ColDesc* __restrict__ cols, 
 
 // Two kernels, so that each has its own register bound: the large launch keeps
 // the compiler's 128 (a second bound argument, even 1, makes it 160 and the
-// 512-column batch 3 % slower), the small one the 194 its held terms need
+// 512-column batch 3 % slower), the small one the 186 its held terms need
 // (168 and spills without it). FP64 columns hold no terms ahead and take the
 // former (a server's burst of 24 Ca II-like columns 102.5 -> 100.6 ms).
 __global__ void __launch_bounds__(32 * kRateWarps) k_rates(const ColDesc* __restrict__ cols, int ncols, int racc,

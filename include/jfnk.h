@@ -25,6 +25,8 @@
  *     and are copied in/out on ``stream``; with JFNK_MEM_DEVICE they are
  *     device pointers on the context's device, read and written on
  *     ``stream``. ``stream`` is a cudaStream_t (NULL = legacy default stream).
+ *     They hold the call's whole array: one that ends before it is refused
+ *     (JFNK_E_INVALID by the explicit evaluations, in a cudaMalloc allocation).
  *     Host-memory calls synchronise the stream before returning; device-memory
  *     calls return after enqueuing unless stated otherwise.
  *   - cgs units throughout.
@@ -377,10 +379,10 @@ int jfnk_batch_destroy(jfnk_batch* b);
 /* ---- residual without device allocation -------------------------------------- */
 /* The paper has no counterpart to this entry point: it is a deployment aid.
  * Same result as jfnk_residual(ctx, a, JFNK_FP64, n, J_dagger, F, J_new, NULL,
- * JFNK_MEM_DEVICE, stream), to rounding (another kernel), but every work buffer comes from one fixed device
- * array of JFNK_STATIC_SCRATCH_BYTES built into the library (held on every GPU
- * that loads it until the process exits), so the call never allocates device
- * memory. For callers that cannot allocate: code running under a memory budget
+ * JFNK_MEM_DEVICE, stream), to rounding (another kernel), but every work buffer
+ * comes from one fixed device array of JFNK_STATIC_SCRATCH_BYTES built into the
+ * library (held on every GPU that loads it until the process exits), so the call
+ * never allocates device memory. For callers that cannot allocate: code running under a memory budget
  * owned by another allocator, or latency-critical loops that must not pay for
  * cudaMalloc (which can synchronise the device and fail mid-run).
  *   n [nz*nl], J_dagger [nq*nz] (nullable: B_nu(T)), F [nz*nl], J_new [nq*nz]

@@ -1,5 +1,5 @@
 """The cached FP64 evaluation where its arithmetic is near a limit: source
-functions below the FP32 range, inverted populations.
+functions below the FP32 range.
 
 References are plain 80- or 128-bit sums of the same short characteristics
 (App. A.1) over the column's own tables, so that only the evaluation's own
